@@ -68,7 +68,7 @@ extern "C" {
 
 /* ---- precision ---- */
 #define GBRT_FP32 0  /* FP32 traversal, intersection and shading; float-float ray, hit refined in its object's frame */
-#define GBRT_FP64 1  /* FP64 throughout (the paper's all-double-precision build, Sec. 2) */
+#define GBRT_FP64 1  /* every result and decision as FP64 arithmetic gives it (the paper's all-double-precision build, Sec. 2) */
 
 #define GBRT_CAMERA_ORTHO 0
 #define GBRT_CAMERA_PINHOLE 1
@@ -352,7 +352,7 @@ GBRT_API int gbrt_philox4x32_10(gbrt_ctx* ctx, const uint32_t* ctr, const uint32
  * cudaMalloc here would fail or fragment it), or a latency-critical loop that
  * must not call cudaMalloc/cudaFree (cudaFree synchronises the device).
  * gbrt_render allocates its working buffers in the context on first use;
- * this variant instead keeps them in one fixed device array of about 4.5 MB
+ * this variant instead keeps them in one fixed device array of about 6.8 MB
  * inside the library, which every GPU that loads the library holds until the
  * process exits. It needs no context: the caller passes the scene and grid
  * (prepared earlier), the outputs (device memory) and the stream to use.

@@ -337,6 +337,58 @@ __device__ __forceinline__ bool walk_start(const GridDev& g, V3<R> o, V3<R> d, R
     return true;
 }
 
+// The same set-up for a ray whose origin is relative to the grid's lower
+// corner (FP64 rays: the difference is formed in FP64 and rounded once, so the
+// walk's error stays relative to the grid's extent).
+__device__ __forceinline__ bool walk_start_rel(const GridDev& g, V3<float> o, V3<float> d, float tmax,
+                                               Walk<float>& w) {
+    if (g.empty) return false;
+    const V3<float> inv = inv_dir(d);
+    const float oo[3] = {o.x, o.y, o.z}, dd[3] = {d.x, d.y, d.z}, ii[3] = {inv.x, inv.y, inv.z};
+    float t0 = 0.0f, t1 = tmax;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const float hi = g.hi[k] - g.lo[k];
+        if (dd[k] == 0.0f) {
+            if (oo[k] < 0.0f || oo[k] > hi) return false;
+        } else {
+            const float ta = -oo[k] * ii[k], tb = (hi - oo[k]) * ii[k];
+            t0 = fmaxf(t0, fminf(ta, tb));
+            t1 = fminf(t1, fmaxf(ta, tb));
+        }
+    }
+    const V3<float> f = v3(o.x - (g.bs[0] - g.lo[0]), o.y - (g.bs[1] - g.lo[1]), o.z - (g.bs[2] - g.lo[2]));
+    const float bb = dot(f, d);
+    const V3<float> v = madd(f, -bb, d);
+    const float disc = g.bs[3] * g.bs[3] - dot(v, v);
+    if (!(disc >= 0.0f)) return false;
+    const float sq = sqrtf(disc);
+    t0 = fmaxf(t0, -bb - sq);
+    t1 = fminf(t1, -bb + sq);
+    if (!(t0 <= t1)) return false;
+    int c[3], st[3];
+    float tn[3], td[3];
+    int stride = 1;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const int n = g.n[k];
+        c[k] = min(max((int)floorf((oo[k] + t0 * dd[k]) * g.inv_h[k]), 0), n - 1);
+        const bool up = dd[k] > 0.0f, down = dd[k] < 0.0f;
+        st[k] = up ? stride : (down ? -stride : 0);
+        tn[k] = (up || down) ? ((float)(up ? c[k] + 1 : c[k]) * g.h[k] - oo[k]) * ii[k] : Num<float>::inf();
+        td[k] = (up || down) ? (up ? g.h[k] : -g.h[k]) * ii[k] : Num<float>::inf();
+        stride *= n;
+    }
+    w.stx = st[0], w.sty = st[1], w.stz = st[2];
+    w.tnx = tn[0], w.tny = tn[1], w.tnz = tn[2];
+    w.tdx = td[0], w.tdy = td[1], w.tdz = td[2];
+    w.ncells = (unsigned)g.ncells;
+    w.t1 = t1;
+    w.cell = (c[2] * g.n[1] + c[1]) * g.n[0] + c[0];
+    w.left = g.n[0] + g.n[1] + g.n[2] + 3;
+    return true;
+}
+
 template <class R>
 __device__ __forceinline__ R walk_cell_exit(const Walk<R>& w) {
     R m = w.tnx < w.tny ? w.tnx : w.tny;
@@ -507,7 +559,7 @@ __device__ __forceinline__ int ao_visible(const FrameDev& f, uint32_t q, V3<R> o
 
 // FP64 hit point re-projected onto the surface of object id, and the geometric
 // normal turned to face the incoming ray.
-__device__ __forceinline__ bool reproject64(const SceneDev& s, uint32_t id, V3<double> o, V3<double> d, double t,
+__device__ __forceinline__ void reproject64(const SceneDev& s, uint32_t id, V3<double> o, V3<double> d, double t,
                                             V3<double>& p, V3<double>& n) {
     V3<double> p0, a;
     double L, r;
@@ -519,12 +571,7 @@ __device__ __forceinline__ bool reproject64(const SceneDev& s, uint32_t id, V3<d
     V3<double> v = p - q;
     n = (1.0 / sqrt(dot(v, v))) * v;
     p = madd(q, r, n);
-    // true when the ray met the surface from inside (the normal is turned)
-    if (dot(n, d) > 0.0) {
-        n = v3(-n.x, -n.y, -n.z);
-        return true;
-    }
-    return false;
+    if (dot(n, d) > 0.0) n = v3(-n.x, -n.y, -n.z);
 }
 
 // ---------------------------------------------------------------- shading

@@ -67,6 +67,7 @@ struct Scene {
     int32_t K = 0;
     float4* obj = nullptr;
     double2* obj64 = nullptr;
+    float4* bs = nullptr;
     uint32_t* color = nullptr;
     float* palette = nullptr;
     float4* aabb = nullptr;  // [2 (S + C)]: lo (xyz), hi (xyz) per object
@@ -86,6 +87,7 @@ struct Scene {
         v.pad = 0;
         v.obj = obj;
         v.obj64 = obj64;
+        v.bs = bs;
         v.color = color;
         v.palette = palette;
         return v;

@@ -23,11 +23,15 @@ enum : uint32_t {
 // zero axis and zero length):
 //   obj    float4 [2 (S+C)]  (p0 xyz, radius), (unit axis xyz, length)
 //   obj64  double2[4 (S+C)]  (p0x, p0y), (p0z, radius), (ax, ay), (az, length)
+//   bs     float4 [S+C]      ball around each object (centre, radius): a sphere
+//                            itself, or the ball around a tube with its radius
+//                            negated (16 bytes to reject a candidate from)
 //   color  uint32 [S+C] palette index; palette float [K*3]
 struct SceneDev {
     int32_t S, C, K, pad;
     const float4* obj;
     const double2* obj64;
+    const float4* bs;
     const uint32_t* color;
     const float* palette;
 };
@@ -118,6 +122,9 @@ struct FrameDev {
 //   hit_off   [n + 1] prefix sums of hits per frame
 //   hits      2 records per hit (FP32: float4 pairs; FP64: 4 double2), at
 //             frames[f].hit_base + h:  (origin xyz, pixel)  (normal xyz, object id)
+//   hits32    what the AO walk reads, float4 pairs in both precisions: `hits`
+//             itself in FP32; in FP64 the same layout with the origin relative
+//             to the grid's lower corner
 //   vis       escaped AO samples per hit slot
 //   lmask     per hit slot, bit l set when the shadow ray toward light l escaped
 //   queue     [0] next primary work item, [1] next AO ray, [2] next shading item
@@ -128,6 +135,7 @@ struct BatchDev {
     unsigned long long* job_off;
     unsigned long long* hit_off;
     void* hits;
+    void* hits32;
     unsigned int* vis;
     unsigned int* lmask;
     unsigned long long* queue;

@@ -16,7 +16,7 @@ namespace {
 //   desc       one FrameDev, then tile_off[2] (i64)
 //   vis        GBRT_NOALLOC_MAX_PIXELS x u32
 //   lmask      GBRT_NOALLOC_MAX_PIXELS x u32 (shadow-ray light bits)
-//   hits       GBRT_NOALLOC_MAX_PIXELS x 64 B (large enough for FP64 records)
+//   hits       GBRT_NOALLOC_MAX_PIXELS x 96 B (FP64 records and the AO walk's FP32 ones)
 constexpr size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 constexpr size_t OFF_COUNTERS = 0;
 constexpr size_t OFF_DESC = 256;
@@ -24,7 +24,7 @@ constexpr size_t OFF_TILES = OFF_DESC + align256(sizeof(FrameDev));
 constexpr size_t OFF_VIS = OFF_TILES + 256;
 constexpr size_t OFF_LMASK = OFF_VIS + align256((size_t)GBRT_NOALLOC_MAX_PIXELS * sizeof(uint32_t));
 constexpr size_t OFF_HITS = OFF_LMASK + align256((size_t)GBRT_NOALLOC_MAX_PIXELS * sizeof(uint32_t));
-constexpr size_t SCRATCH_BYTES = OFF_HITS + (size_t)GBRT_NOALLOC_MAX_PIXELS * 64;
+constexpr size_t SCRATCH_BYTES = OFF_HITS + (size_t)GBRT_NOALLOC_MAX_PIXELS * 96;
 
 // Every GPU that loads the library holds this array until the process exits.
 // In host code `g_scratch` is only a host-side stand-in for the symbol; the
@@ -117,6 +117,7 @@ extern "C" GBRT_API int gbrt_render_noalloc(const gbrt_scene* scene, const gbrt_
         bd.hit_count = (unsigned int*)(q + 8);
         bd.err = (unsigned int*)(q + 8) + 1;
         bd.hits = base + OFF_HITS;
+        bd.hits32 = params->precision == GBRT_FP64 ? base + OFF_HITS + (size_t)width * height * 64 : base + OFF_HITS;
         bd.vis = (unsigned int*)(base + OFF_VIS);
         bd.lmask = (unsigned int*)(base + OFF_LMASK);
         bd.hit_cap = (int64_t)width * height;

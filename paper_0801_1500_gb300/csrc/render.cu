@@ -12,7 +12,8 @@
 //              once fewer than `refill` lanes still hold a ray, walks all of
 //              them in lockstep (several cells per iteration), expands the
 //              (ray, object) pairs over the lanes and tests them 32 at a
-//              time;
+//              time; k_ao_walk64 walks the rays of FP64 frames one a lane,
+//              settling in FP32 every pair that FP32 error bounds decide;
 //   k_shade    one thread per hit: Phong + skylight with V = escaped / spp;
 //   k_resolve  (supersampled frames) box-filters the finer raster.
 // Plus the AO probe and the raw Philox kernel.
@@ -291,19 +292,12 @@ __device__ __forceinline__ bool nearest_fp32_refined(const FrameDev& f, int i, i
     return true;
 }
 
-// Hit records: (AO origin xyz, pixel) and (normal xyz, object id). Bit 31 of
-// the pixel word marks a hit from inside the surface (its normal turned
-// toward the axis or centre); pixel indices stay below 2^31.
-constexpr uint32_t HIT_INSIDE = 0x80000000u;
+// Hit records: (AO origin xyz, pixel) and (normal xyz, object id).
 template <class R>
 struct HitIO;
 
 template <>
 struct HitIO<float> {
-    static __device__ __forceinline__ void store(void* hits, int64_t slot, V3<double> o, V3<double> n, uint32_t q,
-                                                 uint32_t id) {
-        store_f(hits, slot, to_f(o), to_f(n), q, id);
-    }
     static __device__ __forceinline__ void store_f(void* hits, int64_t slot, V3<float> o, V3<float> n, uint32_t q,
                                                    uint32_t id) {
         float4* H = (float4*)hits + 2 * slot;
@@ -372,7 +366,6 @@ __device__ __forceinline__ void ao_plan(const BatchDev& b) {
 
 template <int MODE>
 __global__ void __launch_bounds__(256) k_primary(const __grid_constant__ BatchDev b) {
-    typedef typename std::conditional<MODE == GBRT_FP32, float, double>::type R;
     const int lane = threadIdx.x & 31;
     const long long total = b.tile_off[b.nframes];
     bool overflow = false;
@@ -434,11 +427,13 @@ __global__ void __launch_bounds__(256) k_primary(const __grid_constant__ BatchDe
                 const V3<float> off = madd(wa * a, flip ? r - F.eps_f : r + F.eps_f, nf);
                 const V3<float> ao_o = p0 + off;
                 if (flip) nf = v3(-nf.x, -nf.y, -nf.z);
-                HitIO<float>::store_f(b.hits, slot, ao_o, nf, q | (flip ? HIT_INSIDE : 0u), id);
+                HitIO<float>::store_f(b.hits, slot, ao_o, nf, q, id);
             } else {
                 V3<double> p, n;
-                const bool inside_hit = reproject64(F.scene, id, o64, d64, t64, p, n);
-                HitIO<R>::store(b.hits, slot, madd(p, F.eps, n), n, q | (inside_hit ? HIT_INSIDE : 0u), id);
+                reproject64(F.scene, id, o64, d64, t64, p, n);
+                const V3<double> ao_o = madd(p, F.eps, n);
+                HitIO<double>::store(b.hits, slot, ao_o, n, q, id);
+                HitIO<float>::store_f(b.hits32, slot, to_f(ao_o - ld3(F.grid.lo64)), to_f(n), q, id);
             }
             b.vis[slot] = 0u;
             b.lmask[slot] = 0u;
@@ -477,30 +472,11 @@ __global__ void __launch_bounds__(256) k_primary(const __grid_constant__ BatchDe
 
 // ---------------------------------------------------------------- AO pass
 
-// One AO job -- AO sample or direct-light shadow ray -- of the batch's
-// global job index jj (hits of all frames x jobs per hit): the hit slot whose
-// count or light bit it settles, its ray, and the hit's own object when that
-// object cannot be met again (a hit on a convex outer side), else GBRT_MISS.
-template <class R>
-struct AoJob {
-    V3<R> o, d;
-    R tmax;
-    uint32_t lbit;  // 0: an AO sample; 1 << l: the shadow ray toward light l
-    uint32_t self;
-    int64_t vslot;
-    const FrameDev* F;
-};
-
-// False when no ray is cast: the surface faces away from the light (its bit
-// stays clear).
-template <class R>
-__device__ __forceinline__ bool ao_job(const BatchDev& b, unsigned long long jj, AoJob<R>& J) {
-    const int f = b.nframes == 1 ? 0 : find_frame(b.job_off, b.nframes, jj);
-    const FrameDev& F = b.frames[f];
-    J.F = &F;
-    const unsigned long long jl = jj - b.job_off[f];
+// One AO job -- AO sample or direct-light shadow ray -- of frame F: its index
+// jl among the frame's jobs (hits x jobs per hit) names the hit slot whose
+// count or light bit it settles and the sample.
+__device__ __forceinline__ void ao_split(const FrameDev& F, unsigned long long jl, uint32_t& h, uint32_t& smp) {
     const uint32_t jph = (uint32_t)F.jobs_per_hit;
-    uint32_t h;
     if (jl >= 0xFFFFFFFFull) {
         h = (uint32_t)(jl / jph);
     } else if (jph > 1u) {
@@ -511,28 +487,30 @@ __device__ __forceinline__ bool ao_job(const BatchDev& b, unsigned long long jj,
     } else {
         h = (uint32_t)jl;
     }
-    const uint32_t smp = (uint32_t)(jl - (unsigned long long)h * jph);
-    J.vslot = GBRT_INDEX(F.hit_base + (int64_t)h, b.hit_cap);
-    V3<R> n;
-    uint32_t q;
-    HitIO<R>::load(b.hits, J.vslot, J.o, n, q, J.self);
-    // the own object can be skipped only behind a convex outer side
-    if (q & HIT_INSIDE) J.self = GBRT_MISS;
-    q &= ~HIT_INSIDE;
+    smp = (uint32_t)(jl - (unsigned long long)h * jph);
+}
+
+// Direction of job smp of a hit with normal n and pixel q, and whether a ray
+// is cast at all (a light behind the surface needs none: its bit stays clear).
+// lbit: 0 for an AO sample, 1 << l for the shadow ray toward light l.
+template <class R>
+__device__ __forceinline__ bool ao_direction(const FrameDev& F, uint32_t q, uint32_t smp, V3<R> n, V3<R>& d, R& tmax,
+                                             uint32_t& lbit, bool facing_slack = false) {
     if (smp < (uint32_t)F.spp) {
         uint32_t b1, b2;
         ao_uniforms(q, smp, F.frame, F.seed_lo, F.seed_hi, b1, b2);
-        J.d = cosine_dir(n, b1, b2);
-        J.tmax = ao_maxdist<R>(F);
-        J.lbit = 0u;
+        d = cosine_dir(n, b1, b2);
+        tmax = ao_maxdist<R>(F);
+        lbit = 0u;
         return true;
     }
-    // shadow ray toward light l (none where the surface faces away)
     const int l = (int)(smp - (uint32_t)F.spp);
-    J.d = ShadeP<R>::ldir(F, l);
-    J.tmax = Num<R>::inf();
-    J.lbit = 1u << l;
-    return dot(n, J.d) > R(0);
+    d = ShadeP<R>::ldir(F, l);
+    tmax = Num<R>::inf();
+    lbit = 1u << l;
+    // FP64 frames ask in FP32 (the AO walk): a light within rounding of the
+    // horizon gets its ray, and shading decides in FP64 whether it counts
+    return dot(n, d) > (facing_slack ? R(-1e-5) : R(0));
 }
 
 // A ray that leaves the objects' bounds unoccluded: one more escaped AO
@@ -542,14 +520,18 @@ __device__ __forceinline__ void ao_escape(const BatchDev& b, int64_t vslot, uint
     else atomicAdd(b.vis + vslot, 1u);
 }
 
+// AO rays a warp claims from the global queue at once (its local pool)
+constexpr unsigned AO_CLAIM = 64;
+
+// ---- FP32 frames
+
 // Ray record in shared memory: (origin, tmax) and (direction, -) -- two
-// 128-bit loads per test in the FP32 path.
-template <class R>
+// 128-bit loads per test.
 struct __align__(16) AoRay {
-    V3<R> o;
-    R tmax;
-    V3<R> d;
-    R pad;
+    V3<float> o;
+    float tmax;
+    V3<float> d;
+    float pad;
 };
 
 // Per-warp shared state of the cooperative AO walk.
@@ -557,84 +539,41 @@ struct __align__(16) AoRay {
 //   sd             where each ray's pairs of the current iteration find their
 //                  items (one range per cell taken)
 //   owner          the ray whose pairs start at a position of the current chunk
-//   mbox[lane]     direct-mapped ids this ray already tested (rows padded by
-//                  one word so distinct rays and slots fall in distinct
-//                  banks); a re-test of a missed object cannot hit, so
-//                  skipping it is exact
 //   obj, items     the ray's scene records and grid item list (batches mix
 //                  scenes)
 //   fifo[lane]     cells the ray has stepped to and loaded but not yet taken
-//   q              (FP64 path) surviving (ray, object) pairs waiting for a
-//                  full test batch
 // cells each active ray takes per lockstep iteration: further cells while it
-// holds fewer than AoCfg<R>::min_pairs candidates, at most AO_CELLS
+// holds fewer than AO_MIN_PAIRS candidates, at most AO_CELLS
 constexpr int AO_CELLS = 4;
-// AO rays a warp claims from the global queue at once (its local pool)
-constexpr unsigned AO_CLAIM = 64;
-
-// Per-precision choices. FP32: pairs are tested where they were mapped, one
-// per lane, so a lane whose pair is a re-test would compute and discard it
-// anyway -- no mailbox (a re-test of a missed object misses again, and the
-// hit's own object cannot be met behind a convex outer side, so testing
-// either is exact). FP64: the test occupies the FP64 pipe, so lanes left idle
-// cost more than shared memory -- an 8-slot mailbox drops re-tests, and the
-// surviving pairs are queued and tested in full batches of 32 (in-place tests
-// measured 13% slower there).
-template <class R>
-struct AoCfg;
-template <>
-struct AoCfg<float> {
-    static constexpr int mbox = 0;
-    static constexpr bool queue = false;
-    static constexpr unsigned min_pairs = 8;  // 6: 0.5% slower, 12: 1.5% slower
-};
-template <>
-struct AoCfg<double> {
-    static constexpr int mbox = 8;
-    static constexpr bool queue = true;
-    static constexpr unsigned min_pairs = 4;  // 3: 0.4% slower, 6: 2.1%, 8: 5.0%
-};
-
-template <class R, bool Q = AoCfg<R>::queue>
-struct AoQueue {};
-template <class R>
-struct AoQueue<R, true> {
-    uint2 q[64];  // queued pairs (ray lane, object id)
-};
-
-// per ray: direct-mapped ids it already tested (rows padded by one word so
-// distinct rays and slots fall in distinct banks)
-template <class R, int M = AoCfg<R>::mbox>
-struct AoMbox {
-    uint32_t mbox[32][M + 1];
-};
-template <class R>
-struct AoMbox<R, 0> {};
+// Pairs are tested where they were mapped, one per lane, with no mailbox of
+// tested ids: a re-test of a missed object misses again, and the hit's own
+// object cannot be met behind a convex outer side, so testing either is exact.
+constexpr unsigned AO_MIN_PAIRS = 8;  // 6: 0.5% slower, 12: 1.5% slower
 
 // per ray: its scene records and grid item list, when a batch mixes scenes
 // (UNI: every frame of the batch has the same scene and grid -- the pointers
 // are then kernel-wide)
-template <class R, bool UNI>
+template <bool UNI>
 struct AoPtrs {
-    ObjPtr<R> obj[32];
+    const float4* obj[32];
     const uint32_t* items[32];
 #ifdef GBRT_CHECKED
     int64_t nitems[32];  // the lengths the checked build tests indices against
     int64_t nobj[32];
 #endif
 };
-template <class R>
-struct AoPtrs<R, true> {};
+template <>
+struct AoPtrs<true> {};
 
-// 4 KB a warp at most in the FP32 path: four resident CTAs of 8 warps fit the
+// 4 KB a warp at most: four resident CTAs of 8 warps fit the
 // 132 KB shared-memory configuration, leaving 124 KB of the SM's 256 KB to the
 // L1 that caches the walk's cell, item and object loads. Measured: 5.25 KB a
 // warp (60 KB of L1) 2.5% slower, 5 KB (92 KB of L1, with an 8-slot mailbox
 // and a test queue) 1% slower.
 static_assert(AO_CELLS == 4, "the pair segments of a ray are kept as one uint4 of starts and one of offsets");
-template <class R, bool UNI>
-struct AoWarp : AoQueue<R>, AoMbox<R>, AoPtrs<R, UNI> {
-    AoRay<R> ray[32];
+template <bool UNI>
+struct AoWarp : AoPtrs<UNI> {
+    AoRay ray[32];
     // item index of pair p of ray r: p + sdo[r][g] for the last cell g whose
     // pairs start at or before p (sds[r][g])
     uint4 sds[32];
@@ -644,27 +583,27 @@ struct AoWarp : AoQueue<R>, AoMbox<R>, AoPtrs<R, UNI> {
     // at least one of its at most AO_CELLS cells, so AO_CELLS - 1 wait at most
     uint2 fifo[32][AO_CELLS - 1];
 };
-static_assert(sizeof(AoWarp<float, false>) <= 4096, "the FP32 AO walk's per-warp state outgrew its 4 KB");
+static_assert(sizeof(AoWarp<false>) <= 4096, "the FP32 AO walk's per-warp state outgrew its 4 KB");
 
-template <class R, bool UNI>
-__device__ __forceinline__ ObjPtr<R> ao_obj(const AoWarp<R, UNI>& S, unsigned r, ObjPtr<R> uni) {
+template <bool UNI>
+__device__ __forceinline__ const float4* ao_obj(const AoWarp<UNI>& S, unsigned r, const float4* uni) {
     if constexpr (UNI) return uni;
     else return S.obj[r];
 }
-template <class R, bool UNI>
-__device__ __forceinline__ const uint32_t* ao_items(const AoWarp<R, UNI>& S, unsigned r, const uint32_t* uni) {
+template <bool UNI>
+__device__ __forceinline__ const uint32_t* ao_items(const AoWarp<UNI>& S, unsigned r, const uint32_t* uni) {
     if constexpr (UNI) return uni;
     else return S.items[r];
 }
 #ifdef GBRT_CHECKED
 // ray r's item-buffer length and object count (the checked build's bounds)
-template <class R, bool UNI>
-__device__ __forceinline__ int64_t ao_nitems(const AoWarp<R, UNI>& S, unsigned r, int64_t uni) {
+template <bool UNI>
+__device__ __forceinline__ int64_t ao_nitems(const AoWarp<UNI>& S, unsigned r, int64_t uni) {
     if constexpr (UNI) return uni;
     else return S.nitems[r];
 }
-template <class R, bool UNI>
-__device__ __forceinline__ int64_t ao_nobj(const AoWarp<R, UNI>& S, unsigned r, int64_t uni) {
+template <bool UNI>
+__device__ __forceinline__ int64_t ao_nobj(const AoWarp<UNI>& S, unsigned r, int64_t uni) {
     if constexpr (UNI) return uni;
     else return S.nobj[r];
 }
@@ -675,35 +614,20 @@ __device__ __forceinline__ int64_t ao_nobj(const AoWarp<R, UNI>& S, unsigned r, 
 #define GBRT_AO_OBJ(id, r) (id)
 #endif
 
-// FP64 path: test queued pairs [0, n) (1 <= n <= 32), one per lane (lanes
-// past n redo pair 0 and discard it, so the batch runs without branches);
-// returns the rays hit, as bits.
-template <class R, bool UNI>
-__device__ __forceinline__ unsigned ao_test_batch(AoWarp<R, UNI>& S, int lane, unsigned n, ObjPtr<R> uobj) {
-    const unsigned idx = (unsigned)lane < n ? (unsigned)lane : 0u;
-    const uint2 e = S.q[idx];
-    const unsigned r = e.x;
-    const uint32_t id = e.y;
-    const AoRay<R> ray = S.ray[r];
-    const bool hit = any_hit_object<R>(ao_obj(S, r, uobj), id, ray.o, ray.d, ray.tmax) && (unsigned)lane < n;
-    return __reduce_or_sync(FULL, hit ? (1u << r) : 0u);
-}
-
 // Lockstep cooperative walk: every iteration each active ray takes its next
 // one to AO_CELLS cells (all lanes run the same step code); the warp lays the
 // (ray, item) pairs of those cells out densely with a scan and tests them 32
-// at a time, one pair per lane (the FP64 path skipping the ray's own object
-// and re-tests). UNI: every frame of the batch has the same scene and grid.
-template <class R, bool UNI>
+// at a time, one pair per lane. UNI: every frame of the batch has the same scene and grid.
+template <bool UNI>
 __global__ void __launch_bounds__(256) k_ao_walk(const __grid_constant__ BatchDev b) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    AoWarp<R, UNI>& S = reinterpret_cast<AoWarp<R, UNI>*>(smem_raw)[threadIdx.x >> 5];
+    AoWarp<UNI>& S = reinterpret_cast<AoWarp<UNI>*>(smem_raw)[threadIdx.x >> 5];
     grid_dependency_wait();
-    ObjPtr<R> uobj = nullptr;
+    const float4* uobj = nullptr;
     const uint32_t* uitems = nullptr;
     const uint2* ucells = nullptr;
     if constexpr (UNI) {
-        uobj = Obj<R>::base(b.frames[0].scene);
+        uobj = b.frames[0].scene.obj;
         uitems = b.frames[0].grid.items;
         ucells = b.frames[0].grid.cells;
     }
@@ -716,7 +640,7 @@ __global__ void __launch_bounds__(256) k_ao_walk(const __grid_constant__ BatchDe
     const unsigned long long total = b.job_off[b.nframes];
     const int refill = b.refill;
     bool has = false, exhausted = false, overflow = false;
-    Walk<R> w;
+    Walk<float> w;
     unsigned nf = 0;      // cells waiting in this lane's fifo
     bool wend = false;    // the walk has no further cells
     uint32_t lbit = 0;  // 0: an AO sample; 1 << l: the shadow ray toward light l
@@ -743,38 +667,34 @@ __global__ void __launch_bounds__(256) k_ao_walk(const __grid_constant__ BatchDe
                 const unsigned i = __popc(idle & lt);
                 const unsigned long long jj = i < rem ? pool + i : fresh_base + (i - rem);
                 if (jj < total) {
-                    AoJob<R> J;
-                    const bool cast = ao_job<R>(b, jj, J);
-                    vslot = J.vslot;
-                    lbit = J.lbit;
-                    if (!cast) {
+                    const int f = b.nframes == 1 ? 0 : find_frame(b.job_off, b.nframes, jj);
+                    const FrameDev& F = b.frames[f];
+                    uint32_t h, smp, q, own;
+                    V3<float> o, n, d;
+                    float tmax;
+                    ao_split(F, jj - b.job_off[f], h, smp);
+                    vslot = GBRT_INDEX(F.hit_base + (int64_t)h, b.hit_cap);
+                    HitIO<float>::load(b.hits32, vslot, o, n, q, own);
+                    if (!ao_direction<float>(F, q, smp, n, d, tmax, lbit)) {
                         // the light cannot reach this side: its bit stays clear
-                    } else if (walk_start(J.F->grid, J.o, J.d, R(0), J.tmax, w)) {
+                    } else if (walk_start(F.grid, o, d, 0.0f, tmax, w)) {
                         if constexpr (UNI) {
                             cells = ucells;
                         } else {
-                            cells = J.F->grid.cells;
-                            S.obj[lane] = Obj<R>::base(J.F->scene);
-                            S.items[lane] = J.F->grid.items;
+                            cells = F.grid.cells;
+                            S.obj[lane] = F.scene.obj;
+                            S.items[lane] = F.grid.items;
 #ifdef GBRT_CHECKED
-                            S.nitems[lane] = J.F->grid.nitems;
-                            S.nobj[lane] = (int64_t)J.F->scene.S + J.F->scene.C;
+                            S.nitems[lane] = F.grid.nitems;
+                            S.nobj[lane] = (int64_t)F.scene.S + F.scene.C;
 #endif
                         }
-                        AoRay<R> ray;
-                        ray.o = J.o;
-                        ray.tmax = J.tmax;
-                        ray.d = J.d;
-                        ray.pad = R(0);
+                        AoRay ray;
+                        ray.o = o;
+                        ray.tmax = tmax;
+                        ray.d = d;
+                        ray.pad = 0.0f;
                         S.ray[lane] = ray;
-                        if constexpr (AoCfg<R>::mbox > 0) {
-#pragma unroll
-                            for (int m = 0; m < AoCfg<R>::mbox; ++m) S.mbox[lane][m] = GBRT_MISS;
-                            // the own object starts in the mailbox: it is skipped like a
-                            // re-test while it stays there (testing it is harmless too --
-                            // behind a convex outer side the ray cannot meet it again)
-                            if (J.self != GBRT_MISS) S.mbox[lane][J.self & (AoCfg<R>::mbox - 1)] = J.self;
-                        }
                         // the walk stands on its first cell: its record waits in
                         // the fifo, so every later cell comes from a step
                         S.fifo[lane][0] = __ldg(cells + GBRT_INDEX(w.cell, w.ncells));
@@ -831,7 +751,7 @@ __global__ void __launch_bounds__(256) k_ao_walk(const __grid_constant__ BatchDe
             // below min_pairs candidates: both conditions only turn false
             // (m = 0 when the walk has no cell left: the ray escapes below)
             const unsigned c1 = ng[0], c2 = c1 + ng[1], c3 = c2 + ng[2];
-            constexpr unsigned MP = AoCfg<R>::min_pairs;
+            constexpr unsigned MP = AO_MIN_PAIRS;
             const unsigned m = (avail > 0u) + (avail > 1u && c1 < MP) + (avail > 2u && c2 < MP) + (avail > 3u && c3 < MP);
 #pragma unroll
             for (int g = 1; g < AO_CELLS; ++g) {
@@ -858,11 +778,9 @@ __global__ void __launch_bounds__(256) k_ao_walk(const __grid_constant__ BatchDe
             const unsigned s1 = ex + ng[0], s2 = s1 + ng[1], s3 = s2 + ng[2];
             S.sds[lane] = make_uint4(ex, s1, s2, s3);
             S.sdo[lane] = make_uint4(kg[0] - ex, kg[1] - s1, kg[2] - s2, kg[3] - s3);
-            // 4. map pairs to (ray, object) 32 at a time and test them: in
-            //    place in the FP32 path (lanes past the last pair redo it, so
-            //    the test runs without branches), through the queue in full
-            //    batches of 32 after the mailbox in the FP64 path
-            unsigned qn = 0;
+            // 4. map pairs to (ray, object) 32 at a time and test them in place
+            //    (lanes past the last pair redo it, so the test runs without
+            //    branches)
             for (unsigned base = 0; base < T; base += 32) {
                 // rays mark where their pairs start inside this chunk; a pair's
                 // ray is the last start at or before it. A ray takes part when its
@@ -881,36 +799,13 @@ __global__ void __launch_bounds__(256) k_ao_walk(const __grid_constant__ BatchDe
                 di = p >= st.z ? so.z : di;
                 di = p >= st.w ? so.w : di;
                 const uint32_t id = GBRT_AO_OBJ(__ldg(ao_items(S, r, uitems) + GBRT_AO_ITEM(p + di, r)), r);
-                if constexpr (AoCfg<R>::queue) {
-                    uint32_t* slot = &S.mbox[r][id & (AoCfg<R>::mbox - 1)];
-                    const bool keep = base + lane < T && *slot != id;
-                    const unsigned bal = __ballot_sync(FULL, keep);
-                    if (keep) {
-                        *slot = id;
-                        S.q[qn + __popc(bal & lt)] = make_uint2(r, id);
-                    }
-                    qn += __popc(bal);
-                    __syncwarp();
-                    if (qn >= 32) {
-                        hitbits |= ao_test_batch(S, lane, 32u, uobj);
-                        __syncwarp();
-                        if ((unsigned)lane < qn - 32) S.q[lane] = S.q[32 + lane];
-                        qn -= 32;
-                        __syncwarp();
-                    }
-                } else {
-                    const AoRay<R> ray = S.ray[r];
-                    R t;
-                    const bool hit = hit_object<R>(ao_obj(S, r, uobj), id, ray.o, ray.d, R(0), ray.tmax, t);
-                    hitbits |= hit ? (1u << r) : 0u;  // OR-ed over the warp after the last chunk
-                    __syncwarp();
-                }
+                const AoRay ray = S.ray[r];
+                float t;
+                const bool hit = hit_object<float>(ao_obj(S, r, uobj), id, ray.o, ray.d, 0.0f, ray.tmax, t);
+                hitbits |= hit ? (1u << r) : 0u;  // OR-ed over the warp after the last chunk
+                __syncwarp();
             }
-            if constexpr (AoCfg<R>::queue) {
-                if (qn > 0) hitbits |= ao_test_batch(S, lane, qn, uobj);
-            } else {
-                hitbits = __reduce_or_sync(FULL, hitbits);
-            }
+            hitbits = __reduce_or_sync(FULL, hitbits);
         }
         // 5. any hit occludes the ray; a ray whose walk ended escapes
         const bool occluded = (hitbits >> lane) & 1u;
@@ -919,6 +814,274 @@ __global__ void __launch_bounds__(256) k_ao_walk(const __grid_constant__ BatchDe
             has = false;
         }
         __syncwarp();
+    }
+    if (overflow) atomicOr(b.err, ERR_DDA_STEPS);
+}
+
+// ---- FP64 frames
+
+// The object filter. Every candidate of a cell is first tested, in FP32, as a
+// ball: a sphere itself, or the sphere around a tube (SceneDev::bs, tubes
+// marked by a negative radius). With b = w.d / d.d the ray's parameter at the
+// ball's centre (w = o - centre), m = w - b d the ray's offset there and
+// x = |m|^2 + max(b, 0)^2 - r^2, a ray that starts outside or inside the ball
+// meets it ahead exactly when x <= 0 (b > 0: the centre lies behind, and
+// |m|^2 + b^2 = |w|^2). FILTER_EPS r (|b| + r) bounds the rounding of x ten
+// times over: |m| is wrong by at most ~4e-7 (|b| + r) -- w is one rounding of
+// exact floats, b's error only moves m along the ray -- and so is the
+// reference test's own |m|. So x > margin is a miss and, for a sphere,
+// x < -margin a hit that the reference test (hit_prim, or any_hit_prim in
+// FP64) decides the same way; what lies between is left to that test. A miss,
+// nine candidates in ten, costs ~20 instructions instead of ~45, and in the
+// FP64 path no FP64 instruction.
+constexpr float FILTER_EPS = 1e-5f;
+
+// The ray a lane walks, and what settles it.
+//   o        origin relative to the grid's lower corner (formed in FP64,
+//            rounded once)
+//   idd      -1 / d.d
+//   tlim     a hit whose roots lie within tlim is within tmax
+struct AoRay64 {
+    V3<float> o, d;
+    float idd, tlim;
+    uint32_t lbit;
+    int64_t vslot;
+    int f;         // frame and sample: the exact ray is formed again where a
+    uint32_t smp;  // test needs it
+};
+
+// A tube in FP32, with error bounds: 0 it is missed, 1 it is
+// hit, 2 too close to tell. The arithmetic is hit_prim's; em bounds the error
+// of the offset m (as FILTER_EPS does, four times over), et that of a root's t.
+__device__ __forceinline__ int tube_filter(V3<float> o, V3<float> d, V3<float> p0, V3<float> a, float L, float r,
+                                           float tlim, float tmax, float om) {
+    const V3<float> w = o - p0;
+    const float wa = dot(w, a), da = dot(d, a);
+    const V3<float> wp = madd(w, -wa, a), dp = madd(d, -da, a);
+    const float A = dot(dp, dp);
+    if (!(A > 1e-3f)) return 2;
+    const float inv = 1.0f / A;
+    const float tc = -dot(wp, dp) * inv;
+    const V3<float> m = madd(wp, tc, dp);
+    const float em = 4e-6f * (fabsf(tc) + L + r + om);
+    const float disc = r * r - dot(m, m), md = 2.0f * (r + em) * em;
+    if (disc < -md) return 0;
+    if (!(disc > md)) return 2;
+    const float half = sqrtf(disc * inv);
+    const float et = em * inv + md * inv / half, es = et + em;
+    bool maybe = false;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const float t = k ? tc + half : tc - half, s = wa + t * da;
+        if (t > et && t < tlim - et && s > es && s < L - es) return 1;
+        maybe |= t > -et && t < tmax + et && s > -es && s < L + es;
+    }
+    return maybe ? 2 : 0;
+}
+
+// The FP64 path's reference test of one (ray, object) pair, from the hit's
+// FP64 record: any_hit_prim on the ray that the sample defines.
+__device__ __noinline__ bool ao_exact64(const BatchDev& b, int f, int64_t vslot, uint32_t smp, uint32_t id) {
+    const FrameDev& F = b.frames[f];
+    V3<double> o, n, d;
+    uint32_t q, own, lbit;
+    double tmax;
+    HitIO<double>::load(b.hits, vslot, o, n, q, own);
+    ao_direction<double>(F, q, smp, n, d, tmax, lbit);
+    return any_hit_object<double>(F.scene.obj64, id, o, d, tmax);
+}
+
+// What the filter left open: one pair through the reference test.
+__device__ __forceinline__ bool ao_settle(const BatchDev& b, const SceneDev& sc, const AoRay64& R, float tmax,
+                                          V3<float> lo, float om, uint32_t id) {
+    V3<float> p0, a;
+    float L, r;
+    Obj<float>::load(sc.obj, id, p0, a, L, r);
+    if (L > 0.0f) {
+        const int c = tube_filter(R.o, R.d, p0 - lo, a, L, r, R.tlim, tmax, om);
+        if (c != 2) return c == 1;
+    }
+    return ao_exact64(b, R.f, R.vslot, R.smp, id);
+}
+
+// AO walk of FP64 frames, one ray per lane, persistent. A lane holds its walk, the rest of
+// its current cell's item range [k, e), the record of the cell after it
+// (already loaded) and the id of its next candidate (already loaded), so that
+// an iteration -- one candidate through the filter, or one step into the next
+// cell -- waits for one load. Candidates the filter leaves open wait in
+// `pend`, one a lane, and are settled together: when a lane needs the slot
+// again, when half the warp has one, and before lanes are refilled. A lane
+// whose walk ended with an open candidate waits for that.
+// Refill: once fewer than `refill` lanes walk, the idle lanes take the next
+// rays from the warp's pool, which claims AO_CLAIM jobs at a time. The rays in
+// flight belong to one scene and grid (warp-uniform pointers); a warp whose
+// pool moves on to another scene lets its lanes drain first.
+// With every test and step in FP64 (1/64 of the FP32 rate) the FP64 pipe was
+// 87% busy and the walk took 15.5 of a 965 x 1137 frame's 17.9 ms; the filter
+// leaves FP64 to one pair in some ten thousand (frame 17.9 -> 4.4 ms, a
+// 256 x 256 frame at 8 samples 1.09 -> 0.63 ms). One ray a lane rather than
+// the FP32 frames' pair expansion: with a filter this cheap the expansion
+// costs more than the idle lanes (frame 6.4 ms with pairs queued in shared
+// memory). Bound now by instruction issue.
+__global__ void __launch_bounds__(256, 3) k_ao_walk64(const __grid_constant__ BatchDev b) {
+    grid_dependency_wait();
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    const unsigned long long total = b.job_off[b.nframes];
+    const int refill = b.refill;
+    const float inf = Num<float>::inf();
+    bool active = false, exhausted = false, overflow = false;
+    AoRay64 ray;
+    Walk<float> w;
+    uint32_t k = 0, e = 0;       // items left of the lane's cell
+    uint2 nxt = make_uint2(0, 0);  // the next cell's record, when more
+    bool more = false;
+    uint32_t id = 0;             // the candidate at k, when k < e
+    uint32_t pend = GBRT_MISS;   // a candidate the filter left open
+    bool waiting = false;        // walk over, pend not settled yet
+    float tmax = inf;
+    // the warp's pool of claimed jobs and the frame they belong to (uniform)
+    unsigned long long pool = 0, pool_end = 0, f_lo = 0, f_hi = 0;
+    int f = 0;
+    const FrameDev* F = b.frames;
+    SceneDev sc = F->scene;
+    const uint2* cells = nullptr;
+    const uint32_t* items = nullptr;
+    [[maybe_unused]] int64_t nitems = 0;
+    V3<float> lo = v3(0.0f, 0.0f, 0.0f);
+    float om = 0.0f;
+    while (true) {
+        unsigned act = __ballot_sync(FULL, active);
+        if (exhausted ? act == 0u : __popc(act) < refill) {
+            // settle what is open, finish the lanes that waited for it
+            if (__any_sync(FULL, pend != GBRT_MISS)) {
+                bool hit = false;
+                if (pend != GBRT_MISS) hit = ao_settle(b, sc, ray, tmax, lo, om, GBRT_INDEX(pend, sc.S + sc.C));
+                pend = GBRT_MISS;
+                if (waiting && !hit) ao_escape(b, ray.vslot, ray.lbit);
+                waiting = false;
+                active = active && !hit;
+                act = __ballot_sync(FULL, active);
+            }
+            if (exhausted) {
+                if (act == 0u) break;
+                continue;
+            }
+            if (pool == pool_end) {
+                unsigned long long c = 0;
+                if (lane == 0) c = atomicAdd(b.queue + 1, (unsigned long long)AO_CLAIM);
+                pool = __shfl_sync(FULL, c, 0);
+                pool_end = pool + AO_CLAIM < total ? pool + AO_CLAIM : total;
+                if (pool >= total) {
+                    exhausted = true;
+                    continue;
+                }
+            }
+            bool go = true;
+            if (pool >= f_hi) {
+                const int nf = b.nframes == 1 ? 0 : find_frame(b.job_off, b.nframes, pool);
+                const FrameDev* N = b.frames + nf;
+                const bool same = N->scene.bs == sc.bs && N->grid.cells == cells;
+                if (same || act == 0u) {
+                    f = nf;
+                    F = N;
+                    f_lo = b.job_off[f];
+                    f_hi = b.job_off[f + 1];
+                    if (!same) {
+                        sc = F->scene;
+                        cells = F->grid.cells;
+                        items = F->grid.items;
+                        nitems = F->grid.nitems;
+                        lo = v3(F->grid.lo[0], F->grid.lo[1], F->grid.lo[2]);
+                        om = 0.1f * fmaxf(F->grid.hi[0] - lo.x, fmaxf(F->grid.hi[1] - lo.y, F->grid.hi[2] - lo.z));
+                    }
+                } else {
+                    go = false;  // another scene: the lanes in flight drain first
+                }
+            }
+            if (go) {
+                const unsigned idle = ~act;
+                const unsigned long long stop = pool_end < f_hi ? pool_end : f_hi;
+                const unsigned i = __popc(idle & lt);
+                const unsigned long long left = stop - pool;
+                const unsigned n = left < (unsigned long long)__popc(idle) ? (unsigned)left : __popc(idle);
+                if (!active && i < n) {
+                    uint32_t h, q, own;
+                    V3<float> nrm;
+                    ao_split(*F, pool + i - f_lo, h, ray.smp);
+                    ray.vslot = GBRT_INDEX(F->hit_base + (int64_t)h, b.hit_cap);
+                    ray.f = f;
+                    HitIO<float>::load(b.hits32, ray.vslot, ray.o, nrm, q, own);
+                    if (ao_direction<float>(*F, q, ray.smp, nrm, ray.d, tmax, ray.lbit, true)) {
+                        if (walk_start_rel(F->grid, ray.o, ray.d, tmax, w)) {
+                            ray.idd = __fdividef(-1.0f, dot(ray.d, ray.d));
+                            ray.tlim = tmax * (1.0f - 1e-5f);
+                            k = e = 0;
+                            nxt = __ldg(cells + GBRT_INDEX(w.cell, w.ncells));
+                            more = true;
+                            active = true;
+                        } else {
+                            ao_escape(b, ray.vslot, ray.lbit);  // misses the objects' bounds
+                        }
+                    }
+                }
+                pool += n;
+                if (n < __popc(idle) && pool < total) continue;  // the rest from the next claim or frame
+            }
+        }
+        // one candidate, or one cell
+        bool ask = false;
+        const uint32_t cur = id;
+        const bool test = active && k < e;
+        float4 s = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (test) {
+            s = __ldg(sc.bs + GBRT_INDEX(cur, sc.S + sc.C));
+            ++k;
+        }
+        if (active && k >= e) {
+            if (more) {
+                k = nxt.x;
+                e = nxt.x + nxt.y;
+                more = walk_next(w, overflow);
+                if (more) nxt = __ldg(cells + GBRT_INDEX(w.cell, w.ncells));
+            } else if (!test) {
+                // walk over: nothing left to test
+                active = false;
+                waiting = pend != GBRT_MISS;
+                if (!waiting) ao_escape(b, ray.vslot, ray.lbit);
+            }
+        }
+        if (active && k < e) id = __ldg(items + GBRT_INDEX(k, nitems));
+        if (test) {
+            const V3<float> wv = ray.o - v3(s.x - lo.x, s.y - lo.y, s.z - lo.z);
+            const float bb = dot(wv, ray.d) * ray.idd;  // -b
+            const V3<float> m = madd(wv, bb, ray.d);
+            const float r = fabsf(s.w), bp = fminf(bb, 0.0f);
+            const float x = fmaf(-r, r, fmaf(bp, bp, dot(m, m)));
+            const float mg = FILTER_EPS * r * (fabsf(bb) + r + om);
+            if (x <= mg) {
+                if (s.w > 0.0f && x < -mg && fabsf(bb) + r <= ray.tlim) {
+                    active = false;  // occluded
+                    pend = GBRT_MISS;
+                } else {
+                    ask = true;
+                }
+            }
+        }
+        const unsigned asks = __ballot_sync(FULL, ask);
+        if (asks) {
+            const unsigned full = __ballot_sync(FULL, pend != GBRT_MISS);
+            if ((asks & full) != 0u || __popc(full) >= 16) {
+                bool hit = false;
+                if (pend != GBRT_MISS) hit = ao_settle(b, sc, ray, tmax, lo, om, GBRT_INDEX(pend, sc.S + sc.C));
+                pend = GBRT_MISS;
+                if (waiting && !hit) ao_escape(b, ray.vslot, ray.lbit);
+                waiting = false;
+                active = active && !hit;
+                ask = ask && !hit;
+            }
+            if (ask) pend = cur;
+        }
     }
     if (overflow) atomicOr(b.err, ERR_DDA_STEPS);
 }
@@ -937,7 +1100,7 @@ __global__ void __launch_bounds__(256) k_shade(const __grid_constant__ BatchDev 
         V3<R> o, n;
         uint32_t q, id;
         HitIO<R>::load(b.hits, slot, o, n, q, id);
-        q = GBRT_INDEX(q & ~HIT_INSIDE, (uint32_t)F.W * (uint32_t)F.H);
+        q = GBRT_INDEX(q, (uint32_t)F.W * (uint32_t)F.H);
         id = GBRT_INDEX(id, F.scene.S + F.scene.C);
         const uint32_t vis = b.vis[slot];
         V3<R> d;
@@ -1095,19 +1258,17 @@ static cudaError_t launch_dependent(void (*kernel)(BatchDev), dim3 grid, dim3 bl
     return cudaLaunchKernelEx(&cfg, kernel, bd);
 }
 
-// The AO walk of one precision and scene layout (UNI: one scene and grid for
-// the whole batch) with its dynamic shared memory; launched with an explicit
-// grid, or with one sized for the current device (grid <= 0).
-template <class R, bool UNI>
+template <bool UNI>
 static size_t ao_smem(int block) {
-    return (size_t)(block / 32) * sizeof(AoWarp<R, UNI>);
+    return (size_t)(block / 32) * sizeof(AoWarp<UNI>);
 }
 
 // Shared-memory share of the SM asked for the FP32 walk: just enough for four
 // resident CTAs of 256 threads (and the driver's per-CTA reservation), so the
 // rest of the SM's 256 KB serves as L1 for the walk's cell, item and object
 // loads (the 100 KB configuration instead of the 132 KB one the driver picks
-// by default: AO walk 1.185 -> 1.176 ms on the paper frame).
+// by default: AO walk 1.185 -> 1.176 ms on the paper frame). The FP64 walk
+// keeps no shared memory.
 template <bool UNI>
 static cudaError_t prefer_small_carveout() {
     int dev = 0, per_sm = 0, reserved = 0;
@@ -1115,40 +1276,24 @@ static cudaError_t prefer_small_carveout() {
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
     if (e != cudaSuccess || per_sm <= 0) return e;
-    const long long need = 4ll * ((long long)ao_smem<float, UNI>(256) + reserved);
+    const long long need = 4ll * ((long long)ao_smem<UNI>(256) + reserved);
     const int pct = (int)std::min<long long>(100, (need * 100 + per_sm - 1) / per_sm);
-    return cudaFuncSetAttribute(k_ao_walk<float, UNI>, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
+    return cudaFuncSetAttribute(k_ao_walk<UNI>, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
 }
 
-static cudaError_t set_ao_smem_limits() {
-    // a refused preference leaves the driver's choice (and its error is
-    // cleared here, so it is not taken for a later launch's)
-    if (prefer_small_carveout<true>() != cudaSuccess || prefer_small_carveout<false>() != cudaSuccess)
+// A refused preference leaves the driver's choice (and its error is cleared
+// here, so it is not taken for a later launch's).
+static void configure_ao() {
+    if (prefer_small_carveout<true>() != cudaSuccess || prefer_small_carveout<false>() != cudaSuccess ||
+        cudaFuncSetAttribute(k_ao_walk64, cudaFuncAttributePreferredSharedMemoryCarveout, 0) != cudaSuccess)
         (void)cudaGetLastError();
-    // the AO kernels' per-warp staging can exceed the 48 KB default
-    cudaError_t e = cudaFuncSetAttribute(k_ao_walk<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)ao_smem<float, false>(256));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_ao_walk<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)ao_smem<float, true>(256));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_ao_walk<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)ao_smem<double, false>(256));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_ao_walk<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)ao_smem<double, true>(256));
-    return e;
-}
-
-template <class R, bool UNI>
-static int ao_grid(Ctx* ctx, int block) {
-    return persistent_grid(ctx, k_ao_walk<R, UNI>, block, ao_smem<R, UNI>(block));
 }
 
 template <class R>
 static void launch_ao(const BatchDev& bd, bool uni, int grid, int block, cudaStream_t stream) {
-    if (uni) launch_dependent(k_ao_walk<R, true>, grid, block, ao_smem<R, true>(block), stream, bd);
-    else launch_dependent(k_ao_walk<R, false>, grid, block, ao_smem<R, false>(block), stream, bd);
+    if (std::is_same<R, double>::value) launch_dependent(k_ao_walk64, grid, block, 0, stream, bd);
+    else if (uni) launch_dependent(k_ao_walk<true>, grid, block, ao_smem<true>(block), stream, bd);
+    else launch_dependent(k_ao_walk<false>, grid, block, ao_smem<false>(block), stream, bd);
 }
 
 // The passes after the primary one: AO walk, shading, and the box filter of
@@ -1166,16 +1311,17 @@ static void launch_after_primary(const BatchDev& bd, bool uni, int ao_grid, int 
 static Grids grids_for(Ctx* ctx, int precision, bool uni) {
     const int block = ctx->tuning.block;
     if (!ctx->smem_configured) {
-        set_ao_smem_limits();
+        configure_ao();
         ctx->smem_configured = true;
     }
     Grids g;
     if (precision == GBRT_FP32) {
         g.primary = persistent_grid(ctx, k_primary<GBRT_FP32>, block);
-        g.ao = uni ? ao_grid<float, true>(ctx, block) : ao_grid<float, false>(ctx, block);
+        g.ao = uni ? persistent_grid(ctx, k_ao_walk<true>, block, ao_smem<true>(block))
+                   : persistent_grid(ctx, k_ao_walk<false>, block, ao_smem<false>(block));
     } else {
         g.primary = persistent_grid(ctx, k_primary<GBRT_FP64>, block);
-        g.ao = uni ? ao_grid<double, true>(ctx, block) : ao_grid<double, false>(ctx, block);
+        g.ao = persistent_grid(ctx, k_ao_walk64, block);
     }
     g.shade = ctx->num_sms * 8;
     g.resolve = ctx->num_sms * 4;
@@ -1241,7 +1387,9 @@ int render_frames(Ctx* ctx, FrameDev* frames, int n, bool use_graph) {
     for (int f = 1; f < n; ++f)
         if (frames[f].precision != precision) return GBRT_EINVAL;
     const int tw = ctx->tuning.tile_w, th = ctx->tuning.tile_h;
-    const size_t rec = precision == GBRT_FP32 ? 2 * sizeof(float4) : 4 * sizeof(double2);
+    // hit records: FP32, or FP64 and the AO walk's FP32 ones behind them
+    const size_t rec64 = precision == GBRT_FP32 ? 0 : 4 * sizeof(double2);
+    const size_t rec = rec64 + 2 * sizeof(float4);
     // descriptors: frames, then tile_off (n + 1)
     const size_t frames_bytes = ((size_t)n * sizeof(FrameDev) + 255) & ~(size_t)255;
     const size_t desc_bytes = frames_bytes + (size_t)(n + 1) * sizeof(long long);
@@ -1309,6 +1457,7 @@ int render_frames(Ctx* ctx, FrameDev* frames, int n, bool use_graph) {
     bd.hit_off = bd.job_off + (n + 1);
     bd.hit_count = (unsigned*)(bd.hit_off + (n + 1));
     bd.hits = ctx->d_hits;
+    bd.hits32 = (char*)ctx->d_hits + (size_t)px * rec64;
     bd.vis = ctx->d_vis;
     bd.lmask = ctx->d_lmask;
     bd.err = ctx->d_err;
@@ -1362,10 +1511,13 @@ int render_frames(Ctx* ctx, FrameDev* frames, int n, bool use_graph) {
     return GBRT_OK;
 }
 
-int configure_render_kernels() { return err_of(set_ao_smem_limits()); }
+int configure_render_kernels() {
+    configure_ao();
+    return GBRT_OK;
+}
 
 int enqueue_prepared(const BatchDev& bd, int precision, cudaStream_t stream, int block, int num_sms, bool patch) {
-    auto grid_of = [&](auto kernel, size_t smem) {
+    auto grid_of = [&](auto kernel, size_t smem = 0) {
         int per_sm = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, smem) != cudaSuccess || per_sm < 1)
             per_sm = 1;
@@ -1375,13 +1527,11 @@ int enqueue_prepared(const BatchDev& bd, int precision, cudaStream_t stream, int
     if (patch) k_patch_grids<<<1, 128, 0, stream>>>(bd);
     const auto none = [](int) {};
     if (precision == GBRT_FP32) {
-        k_primary<GBRT_FP32><<<grid_of(k_primary<GBRT_FP32>, 0), block, 0, stream>>>(bd);
-        launch_after_primary<float>(bd, true, grid_of(k_ao_walk<float, true>, ao_smem<float, true>(block)), block,
-                                    num_sms * 8, 0, false, stream, none);
+        k_primary<GBRT_FP32><<<grid_of(k_primary<GBRT_FP32>), block, 0, stream>>>(bd);
+        launch_after_primary<float>(bd, true, grid_of(k_ao_walk<true>, ao_smem<true>(block)), block, num_sms * 8, 0, false, stream, none);
     } else {
-        k_primary<GBRT_FP64><<<grid_of(k_primary<GBRT_FP64>, 0), block, 0, stream>>>(bd);
-        launch_after_primary<double>(bd, true, grid_of(k_ao_walk<double, true>, ao_smem<double, true>(block)), block,
-                                     num_sms * 8, 0, false, stream, none);
+        k_primary<GBRT_FP64><<<grid_of(k_primary<GBRT_FP64>), block, 0, stream>>>(bd);
+        launch_after_primary<double>(bd, true, grid_of(k_ao_walk64), block, num_sms * 8, 0, false, stream, none);
     }
     return err_of(cudaGetLastError());
 }

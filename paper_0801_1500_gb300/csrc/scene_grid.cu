@@ -32,7 +32,7 @@ static float float_of_ord(uint32_t o) {
 // when any object is invalid.
 __global__ void __launch_bounds__(256) k_scene_prep(const float* sph_in, int64_t S, const float* cyl_in, int64_t C,
                                                      const uint32_t* color, int32_t K, float4* obj, double2* obj64,
-                                                     float4* aabb, uint32_t* box, uint32_t* err) {
+                                                     float4* bs, float4* aabb, uint32_t* box, uint32_t* err) {
     const int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const float big = 3.0e38f;
     float lo[3] = {big, big, big}, hi[3] = {-big, -big, -big};
@@ -43,6 +43,7 @@ __global__ void __launch_bounds__(256) k_scene_prep(const float* sph_in, int64_t
         bad = !(isfinite(c[0]) && isfinite(c[1]) && isfinite(c[2]) && isfinite(r) && r > 0.0f);
         obj[2 * id] = make_float4(c[0], c[1], c[2], r);
         obj[2 * id + 1] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        bs[id] = make_float4(c[0], c[1], c[2], r);
         obj64[4 * id] = make_double2(c[0], c[1]);
         obj64[4 * id + 1] = make_double2(c[2], r);
         obj64[4 * id + 2] = make_double2(0.0, 0.0);
@@ -72,6 +73,12 @@ __global__ void __launch_bounds__(256) k_scene_prep(const float* sph_in, int64_t
         }
         obj[2 * id] = make_float4(p0[0], p0[1], p0[2], r);
         obj[2 * id + 1] = make_float4(a[0], a[1], a[2], L);
+        // the tube's points lie within sqrt((L/2)^2 + r^2) of its middle; the
+        // additions cover the rounding of the middle and of the radius
+        const float cmax = fmaxf(fmaxf(fabsf(p0[0]) + fabsf(p1[0]), fabsf(p0[1]) + fabsf(p1[1])),
+                                 fabsf(p0[2]) + fabsf(p1[2]));
+        bs[id] = make_float4(0.5f * p0[0] + 0.5f * p1[0], 0.5f * p0[1] + 0.5f * p1[1], 0.5f * p0[2] + 0.5f * p1[2],
+                             -(1.00001f * sqrtf(0.25f * L * L + r * r) + 4e-7f * cmax));
         obj64[4 * id] = make_double2(p0[0], p0[1]);
         obj64[4 * id + 1] = make_double2(p0[2], r);
         obj64[4 * id + 2] = make_double2(a64[0], a64[1]);
@@ -386,6 +393,7 @@ static bool host_scene_valid(const float* sph, int64_t S, const float* cyl, int6
 void scene_release(Scene* s) {
     cudaFree(s->obj);
     cudaFree(s->obj64);
+    cudaFree(s->bs);
     cudaFree(s->color);
     cudaFree(s->palette);
     cudaFree(s->aabb);
@@ -413,11 +421,12 @@ int scene_upload(Ctx* ctx, const float* spheres, int64_t S, const float* cyl, in
         const size_t nN = (size_t)std::max<int64_t>(N, 1);
         GB_TRY(cudaMalloc(&s->obj, 2 * nN * sizeof(float4)));
         GB_TRY(cudaMalloc(&s->obj64, 4 * nN * sizeof(double2)));
+        GB_TRY(cudaMalloc(&s->bs, nN * sizeof(float4)));
         GB_TRY(cudaMalloc(&s->color, nN * sizeof(uint32_t)));
         GB_TRY(cudaMalloc(&s->palette, (size_t)std::max(K, 1) * 3 * sizeof(float)));
         GB_TRY(cudaMalloc(&s->aabb, 2 * nN * sizeof(float4)));
         GB_TRY(cudaMalloc(&d_box, 8 * sizeof(uint32_t)));
-        s->bytes = nN * (2 * sizeof(float4) + 4 * sizeof(double2) + sizeof(uint32_t) + 2 * sizeof(float4)) +
+        s->bytes = nN * (3 * sizeof(float4) + 4 * sizeof(double2) + sizeof(uint32_t) + 2 * sizeof(float4)) +
                    (size_t)std::max(K, 1) * 3 * sizeof(float);
         if (host) {
             if (S > 0) {
@@ -458,7 +467,7 @@ int scene_upload(Ctx* ctx, const float* spheres, int64_t S, const float* cyl, in
         if (N > 0) {
             int blocks = (int)((N + 255) / 256);
             k_scene_prep<<<blocks, 256, 0, ctx->stream>>>(d_sph_in, S, d_cyl_in, C, s->color, K, s->obj, s->obj64,
-                                                          s->aabb, d_box, nullptr);
+                                                          s->bs, s->aabb, d_box, nullptr);
             ctx->launches++;
             GB_TRY(cudaGetLastError());
         }
@@ -760,7 +769,7 @@ int scene_update(Ctx* ctx, Scene* s, const float* spheres, const float* cyl, int
         cudaMemsetAsync(s->d_box + 3, 0, 5 * sizeof(uint32_t), ctx->stream) != cudaSuccess)
         return GBRT_EDEVICE;
     k_scene_prep<<<(int)((N + 255) / 256), 256, 0, ctx->stream>>>(sph_in, S, cyl_in, C, s->color, s->K, s->obj,
-                                                                  s->obj64, s->aabb, s->d_box, ctx->d_err);
+                                                                  s->obj64, s->bs, s->aabb, s->d_box, ctx->d_err);
     ctx->launches++;
     s->box_stale = true;
     return cudaGetLastError() == cudaSuccess ? GBRT_OK : GBRT_EDEVICE;
