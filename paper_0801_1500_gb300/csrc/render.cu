@@ -292,6 +292,154 @@ __device__ __forceinline__ bool nearest_fp32_refined(const FrameDev& f, int i, i
     return true;
 }
 
+// ---------------------------------------------------------------- FP32 filters of FP64 decisions
+
+// The object filter. Every candidate of a cell is first tested, in FP32, as a
+// ball: a sphere itself, or the sphere around a tube (SceneDev::bs, tubes
+// marked by a negative radius). With b = w.d / d.d the ray's parameter at the
+// ball's centre (w = o - centre), m = w - b d the ray's offset there and
+// x = |m|^2 + max(b, 0)^2 - r^2, a ray that starts outside or inside the ball
+// meets it ahead exactly when x <= 0 (b > 0: the centre lies behind, and
+// |m|^2 + b^2 = |w|^2). FILTER_EPS r (|b| + r) bounds the rounding of x ten
+// times over: |m| is wrong by at most ~4e-7 (|b| + r) -- w is one rounding of
+// exact floats, b's error only moves m along the ray -- and so is the
+// reference test's own |m|. So x > margin is a miss and, for a sphere,
+// x < -margin a hit that the reference test (hit_prim, or any_hit_prim in
+// FP64) decides the same way; what lies between is left to that test. A miss,
+// nine candidates in ten, costs ~20 instructions instead of ~45, and in the
+// FP64 path no FP64 instruction.
+constexpr float FILTER_EPS = 1e-5f;
+
+// What a filter says of one (ray, object) pair.
+enum : int { PAIR_MISS = 0, PAIR_HIT = 1, PAIR_OPEN = 2 };
+
+// A tube in FP32, with error bounds. The arithmetic is hit_prim's; em bounds
+// the error of the offset m (as FILTER_EPS does, four times over), et that of
+// a root's t. On PAIR_HIT t is the nearest root in (0, tmax] and et its error.
+// tlim: a root up to tlim - et is surely within tmax.
+__device__ __forceinline__ int tube_root32(V3<float> o, V3<float> d, V3<float> p0, V3<float> a, float L, float r,
+                                           float tlim, float tmax, float om, float& t, float& et) {
+    const V3<float> w = o - p0;
+    const float wa = dot(w, a), da = dot(d, a);
+    const V3<float> wp = madd(w, -wa, a), dp = madd(d, -da, a);
+    const float A = dot(dp, dp);
+    if (!(A > 1e-3f)) return PAIR_OPEN;
+    const float inv = 1.0f / A;
+    const float tc = -dot(wp, dp) * inv;
+    const V3<float> m = madd(wp, tc, dp);
+    const float em = 4e-6f * (fabsf(tc) + L + r + om);
+    const float disc = r * r - dot(m, m), md = 2.0f * (r + em) * em;
+    if (disc < -md) return PAIR_MISS;
+    if (!(disc > md)) return PAIR_OPEN;
+    const float half = sqrtf(disc * inv);
+    et = em * inv + md * inv / half;
+    const float es = et + em;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        t = k ? tc + half : tc - half;
+        const float s = wa + t * da;
+        if (t > et && t < tlim - et && s > es && s < L - es) return PAIR_HIT;
+        // a root that may count leaves the pair open, one that cannot is passed
+        if (t > -et && t < tmax + et && s > -es && s < L + es) return PAIR_OPEN;
+    }
+    return PAIR_MISS;
+}
+
+// A sphere's nearest root ahead, from the filter's values: the ray's parameter
+// tc at the centre, |m|^2 - r^2 and the margin of the latter.
+__device__ __forceinline__ int sphere_root32(float tc, float x, float mg, float r, float om, float& t, float& et) {
+    if (!(-x > mg)) return PAIR_OPEN;
+    const float half = sqrtf(-x);
+    et = 1e-6f * (fabsf(tc) + r + om) + mg / half;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        t = k ? tc + half : tc - half;
+        if (t > et) return PAIR_HIT;
+        if (t > -et) return PAIR_OPEN;
+    }
+    return PAIR_MISS;
+}
+
+// The exact root of pixel (i, j)'s FP64 ray with object id (infinity: none).
+__device__ __noinline__ double exact_root64(const FrameDev& f, int i, int j, uint32_t id) {
+    V3<double> o, d;
+    double t;
+    primary_ray64(f, i, j, o, d);
+    return hit_object<double>(f.scene, id, o, d, 0.0, Num<double>::inf(), t) ? t : Num<double>::inf();
+}
+
+// FP64 path: the nearest object of pixel (i, j)'s ray. The walk and the roots
+// are FP32, relative to the grid's lower corner, along the float-float ray from
+// just before it enters the objects' bounds; each root carries its error, and
+// FP64 roots (exact_root64) decide where the bounds do not: a pair too close
+// to grazing, to the tube's end or to the ray's start, and two roots closer
+// than their errors. The object is the one an FP64 walk finds; its FP64 root
+// is formed by the caller, once per hit pixel instead of once per candidate
+// (965 x 1137 frame, this kernel: 2.40 -> 0.215 ms; 256 x 256: 0.39 ->
+// 0.057 ms. The FP64 pipe was the bound; now the walk's load latency and the
+// winners' ~200 FP64 instructions are).
+__device__ __forceinline__ bool nearest_filtered64(const FrameDev& f, int i, int j, uint32_t& id, bool& overflow) {
+    const GridDev& g = f.grid;
+    const float inf = Num<float>::inf();
+    Ff3 o, d, x;
+    primary_ray_ff(f, i, j, o, d);
+    // start the walk short of the bounding sphere (its own clip is then exact
+    // enough however far the camera is)
+    const V3<float> c = o.hi - v3(g.bs[0], g.bs[1], g.bs[2]);
+    const float te0 = fmaxf(0.0f, -dot(c, d.hi) * (1.0f - 1e-6f) - 1.1f * g.bs[3]);
+    entry_point(o, d, te0, x);
+    const V3<float> lo = v3(g.lo[0], g.lo[1], g.lo[2]);
+    const V3<float> xr = (x.hi - lo) + x.lo;
+    const V3<float> df = d.hi;
+    Walk<float> w;
+    if (!walk_start_rel(g, xr, df, inf, w)) return false;
+    const float om = 0.1f * fmaxf(g.hi[0] - lo.x, fmaxf(g.hi[1] - lo.y, g.hi[2] - lo.z));
+    const float idd = __fdividef(-1.0f, dot(df, df));
+    id = GBRT_MISS;
+    float t1 = inf, e1 = 0.0f;
+    do {
+        const uint2 cr = __ldg(g.cells + GBRT_INDEX(w.cell, g.ncells));
+        for (uint32_t k = cr.x, e = cr.x + cr.y; k < e; ++k) {
+            const uint32_t cand = GBRT_INDEX(__ldg(g.items + GBRT_INDEX(k, g.nitems)), f.scene.S + f.scene.C);
+            if (cand == id) continue;
+            const float4 s = __ldg(f.scene.bs + cand);
+            const V3<float> wv = xr - v3(s.x - lo.x, s.y - lo.y, s.z - lo.z);
+            const float tc = dot(wv, df) * idd;
+            const V3<float> m = madd(wv, tc, df);
+            const float r = fabsf(s.w), bp = fminf(tc, 0.0f), x2 = fmaf(-r, r, dot(m, m));
+            const float mg = FILTER_EPS * r * (fabsf(tc) + r + om);
+            if (!(fmaf(bp, bp, x2) <= mg)) continue;
+            float t, et;
+            int what;
+            if (s.w > 0.0f) {
+                what = sphere_root32(tc, x2, mg, r, om, t, et);
+            } else {
+                V3<float> p0, a;
+                float L, rr;
+                Obj<float>::load(f.scene.obj, cand, p0, a, L, rr);
+                what = tube_root32(xr, df, p0 - lo, a, L, rr, inf, inf, om, t, et);
+            }
+            if (what == PAIR_MISS) continue;
+            bool nearer = t + et < t1 - e1;
+            if (what == PAIR_OPEN || !(nearer || t - et > t1 + e1)) {
+                const double t64 = exact_root64(f, i, j, cand);
+                if (t64 == Num<double>::inf()) continue;
+                const double b64 = id == GBRT_MISS ? Num<double>::inf() : exact_root64(f, i, j, id);
+                nearer = t64 < b64 || (t64 == b64 && cand < id);
+                t = (float)(t64 - (double)te0);
+                et = 2e-7f * fabsf(t);
+            }
+            if (nearer) {
+                id = cand;
+                t1 = t;
+                e1 = et;
+            }
+        }
+        if (id != GBRT_MISS && t1 <= walk_cell_exit(w)) break;
+    } while (walk_next(w, overflow));
+    return id != GBRT_MISS;
+}
+
 // Hit records: (AO origin xyz, pixel) and (normal xyz, object id).
 template <class R>
 struct HitIO;
@@ -381,20 +529,14 @@ __global__ void __launch_bounds__(256) k_primary(const __grid_constant__ BatchDe
         const int i = tx * b.tile_w + lane % b.tile_w;
         const int j = F.row0 + ty * b.tile_h + lane / b.tile_w;
         const bool inside = i < F.W && j < F.row0 + F.rows;
-        V3<double> o64, d64;
         uint32_t id = GBRT_MISS;
-        double t64 = 0.0;
         LocalHit lh;
         bool hit = false;
         if (inside) {
             if (MODE == GBRT_FP32) {
                 hit = nearest_fp32_refined(F, i, j, id, lh, overflow);
             } else {
-                primary_ray64(F, i, j, o64, d64);
-                Nearest<double> h;
-                hit = trace_nearest<double>(F.grid, F.scene, o64, d64, 0.0, Num<double>::inf(), h, overflow);
-                id = h.id1;
-                t64 = h.t1;
+                hit = nearest_filtered64(F, i, j, id, overflow);
             }
         }
         // warp-aggregated append to this frame's hit list
@@ -429,7 +571,10 @@ __global__ void __launch_bounds__(256) k_primary(const __grid_constant__ BatchDe
                 if (flip) nf = v3(-nf.x, -nf.y, -nf.z);
                 HitIO<float>::store_f(b.hits, slot, ao_o, nf, q, id);
             } else {
-                V3<double> p, n;
+                V3<double> o64, d64, p, n;
+                double t64;
+                primary_ray64(F, i, j, o64, d64);
+                hit_object<double>(F.scene, id, o64, d64, 0.0, Num<double>::inf(), t64);
                 reproject64(F.scene, id, o64, d64, t64, p, n);
                 const V3<double> ao_o = madd(p, F.eps, n);
                 HitIO<double>::store(b.hits, slot, ao_o, n, q, id);
@@ -820,22 +965,6 @@ __global__ void __launch_bounds__(256) k_ao_walk(const __grid_constant__ BatchDe
 
 // ---- FP64 frames
 
-// The object filter. Every candidate of a cell is first tested, in FP32, as a
-// ball: a sphere itself, or the sphere around a tube (SceneDev::bs, tubes
-// marked by a negative radius). With b = w.d / d.d the ray's parameter at the
-// ball's centre (w = o - centre), m = w - b d the ray's offset there and
-// x = |m|^2 + max(b, 0)^2 - r^2, a ray that starts outside or inside the ball
-// meets it ahead exactly when x <= 0 (b > 0: the centre lies behind, and
-// |m|^2 + b^2 = |w|^2). FILTER_EPS r (|b| + r) bounds the rounding of x ten
-// times over: |m| is wrong by at most ~4e-7 (|b| + r) -- w is one rounding of
-// exact floats, b's error only moves m along the ray -- and so is the
-// reference test's own |m|. So x > margin is a miss and, for a sphere,
-// x < -margin a hit that the reference test (hit_prim, or any_hit_prim in
-// FP64) decides the same way; what lies between is left to that test. A miss,
-// nine candidates in ten, costs ~20 instructions instead of ~45, and in the
-// FP64 path no FP64 instruction.
-constexpr float FILTER_EPS = 1e-5f;
-
 // The ray a lane walks, and what settles it.
 //   o        origin relative to the grid's lower corner (formed in FP64,
 //            rounded once)
@@ -849,35 +978,6 @@ struct AoRay64 {
     int f;         // frame and sample: the exact ray is formed again where a
     uint32_t smp;  // test needs it
 };
-
-// A tube in FP32, with error bounds: 0 it is missed, 1 it is
-// hit, 2 too close to tell. The arithmetic is hit_prim's; em bounds the error
-// of the offset m (as FILTER_EPS does, four times over), et that of a root's t.
-__device__ __forceinline__ int tube_filter(V3<float> o, V3<float> d, V3<float> p0, V3<float> a, float L, float r,
-                                           float tlim, float tmax, float om) {
-    const V3<float> w = o - p0;
-    const float wa = dot(w, a), da = dot(d, a);
-    const V3<float> wp = madd(w, -wa, a), dp = madd(d, -da, a);
-    const float A = dot(dp, dp);
-    if (!(A > 1e-3f)) return 2;
-    const float inv = 1.0f / A;
-    const float tc = -dot(wp, dp) * inv;
-    const V3<float> m = madd(wp, tc, dp);
-    const float em = 4e-6f * (fabsf(tc) + L + r + om);
-    const float disc = r * r - dot(m, m), md = 2.0f * (r + em) * em;
-    if (disc < -md) return 0;
-    if (!(disc > md)) return 2;
-    const float half = sqrtf(disc * inv);
-    const float et = em * inv + md * inv / half, es = et + em;
-    bool maybe = false;
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        const float t = k ? tc + half : tc - half, s = wa + t * da;
-        if (t > et && t < tlim - et && s > es && s < L - es) return 1;
-        maybe |= t > -et && t < tmax + et && s > -es && s < L + es;
-    }
-    return maybe ? 2 : 0;
-}
 
 // The FP64 path's reference test of one (ray, object) pair, from the hit's
 // FP64 record: any_hit_prim on the ray that the sample defines.
@@ -898,8 +998,9 @@ __device__ __forceinline__ bool ao_settle(const BatchDev& b, const SceneDev& sc,
     float L, r;
     Obj<float>::load(sc.obj, id, p0, a, L, r);
     if (L > 0.0f) {
-        const int c = tube_filter(R.o, R.d, p0 - lo, a, L, r, R.tlim, tmax, om);
-        if (c != 2) return c == 1;
+        float t, et;
+        const int c = tube_root32(R.o, R.d, p0 - lo, a, L, r, R.tlim, tmax, om, t, et);
+        if (c != PAIR_OPEN) return c == PAIR_HIT;
     }
     return ao_exact64(b, R.f, R.vslot, R.smp, id);
 }
