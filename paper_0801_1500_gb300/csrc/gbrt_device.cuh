@@ -475,21 +475,6 @@ __device__ bool trace_nearest(const GridDev& g, const SceneDev& s, V3<R> o, V3<R
     return h.id1 != GBRT_MISS;
 }
 
-// Any hit with 0 < t <= tmax (AO shadow ray): the first hit ends the walk.
-template <class R>
-__device__ bool trace_any(const GridDev& g, const SceneDev& s, V3<R> o, V3<R> d, R tmax, bool& overflow) {
-    Walk<R> w;
-    if (!walk_start(g, o, d, R(0), tmax, w)) return false;
-    do {
-        uint2 cr = __ldg(g.cells + GBRT_INDEX(w.cell, g.ncells));
-        for (uint32_t k = cr.x, e = cr.x + cr.y; k < e; ++k) {
-            uint32_t id = GBRT_INDEX(__ldg(g.items + GBRT_INDEX(k, g.nitems)), s.S + s.C);
-            if (any_hit_object<R>(Obj<R>::base(s), id, o, d, tmax)) return true;
-        }
-    } while (walk_next(w, overflow));
-    return false;
-}
-
 // ---------------------------------------------------------------- sampling
 
 // Philox4x32-10 (Salmon, Moraes, Dror, Shaw; SC'11): 10 rounds of two 32x32
@@ -540,19 +525,6 @@ __device__ __forceinline__ V3<R> cosine_dir(V3<R> n, uint32_t b1, uint32_t b2) {
     sincos_2pi<R>(u2, sp, cp);
     R x = r * cp, y = r * sp, z = sqrt_pos(R(1) - u1);
     return v3(x * e1.x + y * e2.x + z * n.x, x * e1.y + y * e2.y + z * n.y, x * e1.z + y * e2.z + z * n.z);
-}
-
-// Number of AO samples of (index q) that escape, from origin o about normal n.
-template <class R>
-__device__ __forceinline__ int ao_visible(const FrameDev& f, uint32_t q, V3<R> o, V3<R> n, R maxdist, bool& overflow) {
-    int vis = 0;
-    for (int s = 0; s < f.spp; ++s) {
-        uint32_t b1, b2;
-        ao_uniforms(q, (uint32_t)s, f.frame, f.seed_lo, f.seed_hi, b1, b2);
-        V3<R> d = cosine_dir(n, b1, b2);
-        if (!trace_any(f.grid, f.scene, o, d, maxdist, overflow)) ++vis;
-    }
-    return vis;
 }
 
 // ---------------------------------------------------------------- refinement
