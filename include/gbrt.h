@@ -252,8 +252,8 @@ GBRT_API int gbrt_scene_free(gbrt_ctx* ctx, gbrt_scene* scene);
 
 /* Build the uniform grid (Table 5 "Preprocess"): about lambda * (S + C) cells
  * over the scene box (lambda <= 0 selects 2.0); each object is listed in every
- * cell its padded bounding box overlaps, ids ascending within a cell
- * (counting sort: count, exclusive scan, scatter, per-cell sort). Synchronises
+ * cell its padded bounding box overlaps (counting sort: count, exclusive scan,
+ * scatter; the order within a cell is free: no result depends on it). Synchronises
  * (the reference count sizes the item array). */
 GBRT_API int gbrt_grid_build(gbrt_ctx* ctx, const gbrt_scene* scene, float lambda, gbrt_grid** out);
 
@@ -290,8 +290,7 @@ GBRT_API int gbrt_scene_update(gbrt_ctx* ctx, gbrt_scene* scene, const float* sp
  * GBRT_EINVAL) with the grid's own cells-per-object density: scene box ->
  * cells per axis -> count -> exclusive scan -> scatter -> bounding sphere,
  * all on the context's stream; renders enqueued after it use the new grid.
- * The ids of a cell stay in scatter order (a host build sorts them; no
- * render result depends on the order). The first call allocates buffers with headroom (cells
+ * The first call allocates buffers with headroom (cells
  * for 1.5x the target count, items for 1.5x the current references) and
  * waits for the stream once; later calls neither allocate nor wait, except
  * that a call which finds, from an earlier finished rebuild, that the items
@@ -395,7 +394,7 @@ GBRT_API int gbrt_get_tuning(const gbrt_ctx* ctx, gbrt_tuning* tuning);
 /* Per-kernel timing (phase timers). mode 0: off. GBRT_PROFILE_ALL (or any
  * other non-zero value): renders record CUDA events between all their kernels
  * on the context's stream. GBRT_PROFILE_AO_WALK: events only just before and
- * after the AO shadow-ray walk -- each event between two kernels costs a few
+ * after the AO shadow rays' kernels -- each event between two kernels costs a few
  * microseconds and the overlap of the dependent launch, so this mode times
  * the dominant kernel with the least disturbance. Renders replayed from a
  * CUDA graph are not timed. */
@@ -405,7 +404,7 @@ GBRT_API int gbrt_set_profiling(gbrt_ctx* ctx, int mode);
 
 /* Device time in ms of the last timed render's kernels: [0] primary walk and
  * refinement (its last CTA also lays out the AO pass), [1] 0 (the AO plan has
- * no kernel of its own), [2] AO shadow-ray walk, [3] shading; under
+ * no kernel of its own), [2] AO shadow rays (near pass and walk), [3] shading; under
  * GBRT_PROFILE_AO_WALK only [2] is measured and the others are -1. Waits for
  * that render. GBRT_EINVAL if no render was timed. */
 GBRT_API int gbrt_phase_times(gbrt_ctx* ctx, float ms[4]);

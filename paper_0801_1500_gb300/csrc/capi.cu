@@ -288,6 +288,7 @@ GBRT_API int gbrt_create(gbrt_ctx** out, int device, void* cuda_stream) {
         delete c;
         return GBRT_ENOMEM;
     }
+    pool_create(c);
     *out = c;
     return GBRT_OK;
 }
@@ -331,6 +332,9 @@ GBRT_API int gbrt_destroy(gbrt_ctx* ctx) {
     cudaFree(ctx->d_hits);
     cudaFree(ctx->d_vis);
     cudaFree(ctx->d_lmask);
+    cudaFree(ctx->d_near);
+    cudaFree(ctx->d_build);
+    if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
     cudaFree(ctx->d_fine);
     cudaFree(ctx->d_desc);
     cudaFreeHost(ctx->h_desc);
@@ -377,7 +381,7 @@ GBRT_API int gbrt_scene_free(gbrt_ctx* ctx, gbrt_scene* scene) {
     if (!ctx) return GBRT_EINVAL;
     DeviceGuard g(ctx->device);
     cudaStreamSynchronize(ctx->stream);
-    scene_release(scene);
+    scene_release(ctx, scene);
     delete scene;
     return GBRT_OK;
 }
@@ -449,7 +453,7 @@ GBRT_API int gbrt_grid_free(gbrt_ctx* ctx, gbrt_grid* grid) {
     if (!ctx) return GBRT_EINVAL;
     DeviceGuard g(ctx->device);
     cudaStreamSynchronize(ctx->stream);
-    grid_release(grid);
+    grid_release(ctx, grid);
     delete grid;
     return GBRT_OK;
 }

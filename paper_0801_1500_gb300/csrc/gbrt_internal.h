@@ -36,6 +36,14 @@ struct Ctx {
     size_t vis_cap = 0;
     unsigned int* d_lmask = nullptr;
     size_t lmask_cap = 0;
+    // memory of scenes and grids: freed blocks (64 MB of them at most) stay here
+    // for the next upload until the context is destroyed -- mapping fresh
+    // memory costs 100-200 us a block. Null: plain cudaMalloc.
+    cudaMemPool_t pool = nullptr;
+    void* d_build = nullptr;  // temporary arrays of a scene upload or a grid build
+    size_t build_cap = 0;
+    void* d_near = nullptr;  // near pass: tile records, units, job masks
+    size_t near_cap = 0;
     void* d_fine = nullptr;  // finer-raster colours of supersampled frames
     size_t fine_cap = 0;
     void* d_desc = nullptr;
@@ -61,10 +69,25 @@ struct Ctx {
     cudaEvent_t ev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
 };
 
+// One device allocation cut into 256-byte aligned arrays (each cudaMalloc and
+// cudaFree costs tens of microseconds): take() the arrays in the same order
+// once with a null base, for the size, and once with the allocation.
+struct Carve {
+    char* base = nullptr;
+    size_t size = 0;
+    template <class T>
+    T* take(int64_t n) {
+        T* p = base ? reinterpret_cast<T*>(base + size) : nullptr;
+        size += ((size_t)(n > 0 ? n : 1) * sizeof(T) + 255) & ~(size_t)255;
+        return p;
+    }
+};
+
 struct Scene {
     int device = 0;
     int64_t S = 0, C = 0;
     int32_t K = 0;
+    void* mem = nullptr;  // the one allocation that the arrays below (but d_in) lie in
     float4* obj = nullptr;
     double2* obj64 = nullptr;
     float4* bs = nullptr;
@@ -72,9 +95,10 @@ struct Scene {
     float* palette = nullptr;
     float4* aabb = nullptr;  // [2 (S + C)]: lo (xyz), hi (xyz) per object
     float lo[3] = {0, 0, 0}, hi[3] = {0, 0, 0};
+    float rmax = 0;  // largest radius of an object's ball
     size_t bytes = 0;
     // scene box on the device (order-preserving words: min xyz, max xyz,
-    // invalid flag); kept so device-side rebuilds read the current box
+    // invalid flag, largest ball radius); kept so device-side rebuilds read the current box
     uint32_t* d_box = nullptr;
     float* d_in = nullptr;  // staging of host geometry for gbrt_scene_update
     bool box_stale = false;  // lo/hi above predate a device-side update
@@ -118,8 +142,11 @@ struct BuildAux {
 
 struct Grid {
     GridDev dev{};
+    void* mem = nullptr;  // holds cells, balls, bstart and, of a rebuilt grid, d_counts and d_sums
     uint2* cells = nullptr;
     uint32_t* items = nullptr;
+    float4* balls = nullptr;  // [2 N]: sorted by cell, then by object id
+    uint32_t* bstart = nullptr;
     int64_t refs = 0;
     size_t bytes = 0;
     float lambda = 0.f;
@@ -141,13 +168,24 @@ struct Grid {
     cudaStream_t stream = nullptr;  // stream of the last rebuild
 };
 
+// scene_grid.cu: the context's pool (none if the device has no pools); memory
+// of a scene or grid from it, and back
+// (like cudaFree, after the device is idle: other streams may still read it)
+void pool_create(Ctx* ctx);
+cudaError_t block_alloc(Ctx* ctx, void** p, size_t bytes);
+void block_free(Ctx* ctx, void* p);
+
+// render.cu: grow a context buffer (drains the stream first: old work may still
+// read it)
+int grow(Ctx* ctx, void** p, size_t* cap, size_t need);
+
 // scene_grid.cu: fill a caller-allocated object; on failure it frees what it
 // allocated and leaves the object empty.
 int scene_upload(Ctx* ctx, const float* spheres, int64_t S, const float* cyl, int64_t C, const uint32_t* color,
                  const float* palette, int32_t K, int flags, Scene* out);
-void scene_release(Scene* s);
+void scene_release(Ctx* ctx, Scene* s);
 int grid_build(Ctx* ctx, const Scene* s, float lambda, Grid* out);
-void grid_release(Grid* g);
+void grid_release(Ctx* ctx, Grid* g);
 // device-side animation path: new geometry for a resident scene, and a grid
 // rebuild that neither allocates (after its first call) nor waits for the GPU
 int scene_update(Ctx* ctx, Scene* s, const float* spheres, const float* cyl, int flags);

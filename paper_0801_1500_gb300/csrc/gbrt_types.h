@@ -36,10 +36,16 @@ struct SceneDev {
     const float* palette;
 };
 
-// Uniform grid. cells[c] = (first item, item count) of cell
-// c = (z * ny + y) * nx + x; items are global object ids, ascending per cell
-// after a host build, in scatter order after a device-side rebuild (no result
-// depends on the order).
+// Uniform grid. balls are the scene's objects sorted by the cell of a grid with
+// half as many cells an axis (bn = ceil(n / 2), same corner, h doubled) that
+// holds their centre, x fastest: those of cells (x0..x1, y, z) are
+// [bstart[(z bny + y) bnx + x0], bstart[(z bny + y) bnx + x1 + 1]). A tube's
+// ball holds only the part outside its spheres (radius negated; 0: no such
+// part). rho is the reach of the AO rays' near pass (0: not used), rmax the
+// largest distance of an object's point from the centre it was sorted by.
+// cells[c] = (first item, item count) of cell
+// c = (z * ny + y) * nx + x; items are global object ids, in the order the
+// scatter pass left them (no result depends on the order).
 struct GridDev {
     float lo[3], hi[3], h[3], inv_h[3];
     double lo64[3], hi64[3], h64[3], inv_h64[3];
@@ -53,6 +59,13 @@ struct GridDev {
     int64_t nitems;  // length of the item buffer
     const uint2* cells;
     const uint32_t* items;
+    const float4* balls;
+    const uint32_t* bstart;
+    const float4* cut;  // the same balls by object id
+    int32_t bn[3];
+    int32_t nballs;
+    float rho, rmax;
+    float density;  // objects per volume of the grid box
 };
 
 // Everything one frame needs, in the precision each path reads.
@@ -112,6 +125,23 @@ struct FrameDev {
     int32_t row0, rows;
     int32_t tiles_x, tiles_y;
     int64_t hit_base;  // first slot of this frame's region of the hit buffers
+    // near pass: 1 when it looks for this frame's near occluders; the frame's
+    // words in the job masks (mask_words a hit, 16 jobs a word)
+    int32_t near_pass;
+    int32_t mask_words;
+    int32_t rec_words;  // words of one tile record
+    int64_t mask_base;
+};
+
+// Up to rec_words words of 16 jobs of the hits of one primary work item (tile),
+// as the near pass and the AO walk see them: the hits' first slot and number,
+// their frame, the first job word, and how far the near pass looked.
+struct TileRec {
+    int64_t slot;
+    int32_t n;
+    int32_t frame;
+    int32_t word;
+    float rho;
 };
 
 // One batch of frames as the render kernels see it (a kernel parameter).
@@ -127,7 +157,15 @@ struct FrameDev {
 //             to the grid's lower corner
 //   vis       escaped AO samples per hit slot
 //   lmask     per hit slot, bit l set when the shadow ray toward light l escaped
-//   queue     [0] next primary work item, [1] next AO ray, [2] next shading item
+//   queue     [0] next primary work item, [1] next AO ray (or unit), [2] next
+//             tile of the near pass
+// With a near pass (tiles not null):
+//   tiles     records of the work items with hits
+//   ntiles    their number
+//   masks     per hit and 16 jobs: low half the jobs whose ray still has to
+//             walk, high half those of them that walk from the start
+//   units     (record << 8 | group of 4 of the frame's jobs) with a ray left to walk
+//   nunits    their number
 struct BatchDev {
     const FrameDev* frames;
     const long long* tile_off;
@@ -140,6 +178,11 @@ struct BatchDev {
     unsigned int* lmask;
     unsigned long long* queue;
     unsigned int* err;
+    TileRec* tiles;
+    unsigned int* masks;
+    unsigned long long* units;
+    unsigned long long* nunits;
+    unsigned long long* ntiles;
     int64_t hit_cap;  // hit slots (records, vis, lmask) of the batch
     int32_t nframes;
     int32_t tile_w, tile_h;

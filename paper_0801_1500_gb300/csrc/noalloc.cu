@@ -120,6 +120,11 @@ extern "C" GBRT_API int gbrt_render_noalloc(const gbrt_scene* scene, const gbrt_
         bd.hits32 = params->precision == GBRT_FP64 ? base + OFF_HITS + (size_t)width * height * 64 : base + OFF_HITS;
         bd.vis = (unsigned int*)(base + OFF_VIS);
         bd.lmask = (unsigned int*)(base + OFF_LMASK);
+        bd.tiles = nullptr;  // no near pass: its buffers are not in the scratch
+        bd.masks = nullptr;
+        bd.units = nullptr;
+        bd.nunits = nullptr;
+        bd.ntiles = nullptr;
         bd.hit_cap = (int64_t)width * height;
         bd.nframes = 1;
         bd.tile_w = tw;

@@ -7,6 +7,8 @@
 //              origin, normal) to its frame's hit list; the last CTA to
 //              finish lays out the AO pass (prefix sums of hits and AO rays
 //              per frame);
+//   k_ao_near  (FP32 frames with rays enough) tests the AO rays of a tile
+//              against the balls around it before they walk;
 //   k_ao_walk  persistent; each lane holds one AO (or direct-light shadow)
 //              ray; a warp refills its idle lanes together from its ray pool
 //              once fewer than `refill` lanes still hold a ray, walks all of
@@ -20,6 +22,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <cmath>
 #include <functional>
 #include <type_traits>
 #include <vector>
@@ -547,6 +550,16 @@ __global__ void __launch_bounds__(256) k_primary(const __grid_constant__ BatchDe
             if (lane == leader) base = atomicAdd(b.hit_count + f, (unsigned)__popc(hm));
             base = __shfl_sync(FULL, base, leader);
         }
+        if (b.tiles && hm && lane == 0) {
+            unsigned long long at =
+                atomicAdd(b.ntiles, (unsigned long long)((F.mask_words + F.rec_words - 1) / F.rec_words));
+            for (int w = 0; w < F.mask_words; w += F.rec_words, ++at) {
+                b.tiles[at].slot = F.hit_base + (int64_t)base;
+                b.tiles[at].n = __popc(hm);
+                b.tiles[at].frame = f;
+                b.tiles[at].word = w;
+            }
+        }
         if (!inside) continue;
         const uint32_t q = (uint32_t)j * (uint32_t)F.W + (uint32_t)i;
         if (hit) {
@@ -668,6 +681,339 @@ __device__ __forceinline__ void ao_escape(const BatchDev& b, int64_t vslot, uint
 // AO rays a warp claims from the global queue at once (its local pool)
 constexpr unsigned AO_CLAIM = 64;
 
+// ---- near pass
+
+__device__ __forceinline__ float max3(float a, float b, float c) {
+    float m;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(m) : "f"(a), "f"(b), "f"(c));
+    return m;
+}
+// floats as integers of the same order, for the warp's integer reductions
+__device__ __forceinline__ int ord_i(float x) {
+    const int i = __float_as_int(x);
+    return i ^ ((i >> 31) & 0x7fffffff);
+}
+__device__ __forceinline__ float warp_min(float x) {
+    const int m = __reduce_min_sync(FULL, ord_i(x));
+    return __int_as_float(m ^ ((m >> 31) & 0x7fffffff));
+}
+__device__ __forceinline__ float warp_max(float x) { return -warp_min(-x); }
+__device__ __forceinline__ float warp_sum(float x) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(FULL, x, o);
+    return x;
+}
+
+// Candidates of a work item (balls); the directions of eight samples on their
+// way into registers; during the gather, where each row's balls lie.
+constexpr int NEAR_SPHERES = 160, NEAR_TUBES = 128;
+struct NearWarp {
+    float4 sph[NEAR_SPHERES], tub[NEAR_TUBES];
+    union {
+        float dir[8][3][32];
+        struct {
+            uint32_t off[32];    // ball of position p: p + off[row]
+            uint32_t owner[32];  // row whose balls start at this position of the chunk
+        } rows;
+    };
+};
+// Largest number of jobs a hit may have for its frame to have a near pass
+// (bounds the masks to 64 bytes a hit).
+constexpr int NEAR_MAX_JOBS = 256;
+constexpr int NEAR_MIN_JOBS = 8;
+// A record takes a warp some 40 us, most of it latency, and the walk's units are
+// coarser than its own claims: the pass pays when every resident warp gets
+// several (1.1 MP, 21,000 records: frame 1.12 -> 0.93 ms; 5,900
+// records: 0.416 -> 0.437 ms).
+constexpr double NEAR_MIN_RECS = 12288;
+
+// Largest b - q over the n candidates at c, for each of the NS directions: b =
+// w.d with w = centre - o, q = sqrt(|w|^2 - r^2). The ray meets a ball ahead of
+// an outside origin exactly when b >= q. w and q are per (hit, ball), so a
+// (ray, ball) pair costs three FMAs and half a three-input maximum. An origin
+// inside or within 5e-5 r of a ball sets bad (q would be too rough there),
+// unless it is the ball of the tube that the hit lies on (skip, its centre):
+// rays from a tube's outer side do not meet it again.
+struct NearSkip {
+    bool on;
+    V3<float> c;
+};
+__device__ __forceinline__ float near_q(float4 A, float q2, const NearSkip& skip, bool& bad) {
+    if (q2 < 1e-4f * A.w * A.w) {
+        if (skip.on && A.x == skip.c.x && A.y == skip.c.y && A.z == skip.c.z) return Num<float>::inf();
+        bad = true;
+    }
+    return sqrt_pos(q2);
+}
+template <int NS>
+__device__ __forceinline__ void near_scan(const float4* c, int n, V3<float> o, const float (&d)[NS][3], float (&m)[NS],
+                                          const NearSkip& skip, bool& bad) {
+    for (int k = 0; k < n; k += 2) {
+        const float4 A = c[k], B = c[k + 1 < n ? k + 1 : k];
+        const float ax = A.x - o.x, ay = A.y - o.y, az = A.z - o.z;
+        const float bx = B.x - o.x, by = B.y - o.y, bz = B.z - o.z;
+        const float qa = fmaf(ax, ax, fmaf(ay, ay, fmaf(az, az, -A.w * A.w)));
+        const float qb = fmaf(bx, bx, fmaf(by, by, fmaf(bz, bz, -B.w * B.w)));
+        const float na = -near_q(A, qa, skip, bad), nb = -near_q(B, qb, skip, bad);
+#pragma unroll
+        for (int s = 0; s < NS; ++s)
+            m[s] = max3(m[s], fmaf(ax, d[s][0], fmaf(ay, d[s][1], fmaf(az, d[s][2], na))),
+                        fmaf(bx, d[s][0], fmaf(by, d[s][1], fmaf(bz, d[s][2], nb))));
+    }
+}
+
+// NS jobs (from j0) of a work item's hits, one hit a lane: which are occluded
+// by a near sphere, which have to walk, which of those from the start, which
+// leave the objects' bounds before the near pass's reach.
+template <int NS>
+__device__ __forceinline__ void near_jobs(const FrameDev& F, NearWarp& S, int lane, int j0, V3<float> o, V3<float> nrm,
+                                          uint32_t q, const NearSkip& skip, int ns, int nt, float rho, float delta,
+                                          uint32_t& todo,
+                                          uint32_t& start, uint32_t& escaped) {
+    float d[NS][3], m[NS];
+    uint32_t valid = 0u;
+    for (int h = 0; h < NS; h += 8) {
+        const int cnt = NS - h < 8 ? NS - h : 8;
+        for (int s = 0; s < cnt; ++s) {
+            V3<float> dir = nrm;
+            if (j0 + h + s < F.jobs_per_hit) {
+                float tmax;
+                uint32_t lbit;
+                if (ao_direction<float>(F, q, (uint32_t)(j0 + h + s), nrm, dir, tmax, lbit)) valid |= 1u << (h + s);
+            }
+            S.dir[s][0][lane] = dir.x;
+            S.dir[s][1][lane] = dir.y;
+            S.dir[s][2][lane] = dir.z;
+        }
+#pragma unroll
+        for (int s = 0; s < NS; ++s)
+            if (s >= h && s < h + 8)
+#pragma unroll
+                for (int k = 0; k < 3; ++k) d[s][k] = S.dir[s - h][k][lane];
+    }
+    // spheres, then tubes, through the same code (it has to stay in the
+    // instruction cache): what a sphere's ball surely stops is hit, what comes
+    // close to one or meets a tube's stays open
+    bool bad = false;
+    uint32_t hit = 0u, open = 0u;
+    const float4* list = S.sph;
+    int n = ns;
+#pragma unroll 1
+    for (int kind = 0; kind < 2; ++kind) {
+#pragma unroll
+        for (int s = 0; s < NS; ++s) m[s] = -Num<float>::inf();
+        near_scan<NS>(list, n, o, d, m, skip, bad);
+        const float sure = kind == 0 ? delta : Num<float>::inf();
+#pragma unroll
+        for (int s = 0; s < NS; ++s) {
+            hit |= m[s] > sure ? 1u << s : 0u;
+            open |= m[s] >= -delta ? 1u << s : 0u;
+        }
+        list = S.tub;
+        n = nt;
+    }
+    const V3<float> f = v3(o.x - F.grid.bs[0], o.y - F.grid.bs[1], o.z - F.grid.bs[2]);
+    const float ff = dot(f, f) - F.grid.bs[3] * F.grid.bs[3];
+    escaped = 0u;
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+        // f.f + 2 t f.d + t^2 - r^2 > 0 at t = reach, from inside: the ray left
+        const float fd = f.x * d[s][0] + f.y * d[s][1] + f.z * d[s][2];
+        escaped |= fmaf(rho, fmaf(2.0f, fd, rho), ff) > 0.0f ? 1u << s : 0u;
+    }
+    todo = valid & ~hit;
+    start = todo & open;
+    if (bad) todo = start = valid;
+    escaped = ff < 0.0f ? escaped & todo & ~start : 0u;
+    todo &= ~escaped;
+}
+
+// The near pass of an AO batch, one warp per tile (the <= 32 hits of a primary
+// work item, one a lane). The hits of a tile lie close together, so their
+// rays share the objects that they can meet within rho of the hits: the warp
+// gathers those balls once, from the objects sorted by cell, drops the ones
+// behind all of the hits, and tests every ray of the tile against every ball
+// in registers (near_scan) instead of walking each ray through its first
+// cells. Rays a sphere surely stops are done; the others go on to the walk, at
+// distance rho. A ray too close to a silhouette to tell (delta), or that meets
+// a tube's ball, walks from its start: tubes are cut to what sticks out of
+// their atoms, so that is one ray in a hundred. The decisions are those of the
+// walk's own test (delta is ten times the rounding of both).
+// Measured (965 x 1137, 16 samples, 9.0 M AO rays): 148 balls a tile; 37% of the
+// rays hit, 13% left the bounds, 1% open; 243 M warp instructions (gather 39 M,
+// directions 48 M, scan 155 M) in 0.35 ms, and the walk 1.00 -> 0.44 ms. 3860 x
+// 4548: frame 15.9 -> 11.1 ms. Instruction issue (0.6 a cycle: 16 warps an SM,
+// for the directions in registers) bounds it. Tried: the scan as f16-pair
+// m16n8k16 mma.sync (13.7 cycles a 128 pairs, no faster than the FMAs), packed
+// f32x2 FMAs (20% fewer instructions, 10% slower), a row of cells per lane in
+// the gather (55 dependent rounds of loads instead of 16: 0.44 ms).
+__global__ void __launch_bounds__(128, 4) k_ao_near(const __grid_constant__ BatchDev b) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    NearWarp& S = reinterpret_cast<NearWarp*>(smem_raw)[threadIdx.x >> 5];
+    grid_dependency_wait();
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    const unsigned long long total = *b.ntiles;
+    while (true) {
+        unsigned long long tile = 0;
+        if (lane == 0) tile = atomicAdd(b.queue + 2, 1ull);
+        tile = __shfl_sync(FULL, tile, 0);
+        if (tile >= total) break;
+        const int n = b.tiles[tile].n;
+        const FrameDev& F = b.frames[b.tiles[tile].frame];
+        const int64_t slot = GBRT_INDEX(b.tiles[tile].slot + (lane < n ? lane : 0), b.hit_cap);
+        V3<float> o, nrm;
+        uint32_t q, own;
+        HitIO<float>::load(b.hits32, slot, o, nrm, q, own);
+        float rho = F.near_pass ? F.grid.rho : 0.0f, delta = 0.0f;
+        int ns = 0, nt = 0;
+        NearSkip skip;
+        skip.on = false;
+        if (rho > 0.0f) {
+            // a hit on a tube's outer side: its origin may lie inside the tube's ball
+            V3<float> p0, a;
+            float L, r;
+            own = GBRT_INDEX(own, F.scene.S + F.scene.C);
+            Obj<float>::load(F.scene.obj, own, p0, a, L, r);
+            if (L > 0.0f) {
+                const V3<float> w = o - p0, wp = madd(w, -dot(w, a), a);
+                const float4 c = __ldg(F.grid.cut + own);
+                skip.on = dot(wp, wp) > 1.0002f * r * r;  // surely outside
+                skip.c = v3(c.x, c.y, c.z);
+            }
+            // the hits' box, its centre, and the cone of their normals
+            const V3<float> mn = v3(warp_min(o.x), warp_min(o.y), warp_min(o.z));
+            const V3<float> mx = v3(warp_max(o.x), warp_max(o.y), warp_max(o.z));
+            const V3<float> ctr = 0.5f * (mn + mx), ext = 0.5f * (mx - mn);
+            const float spread = sqrtf(dot(ext, ext));
+            V3<float> ax = v3(warp_sum(nrm.x), warp_sum(nrm.y), warp_sum(nrm.z));
+            ax = rsqrtf(fmaxf(dot(ax, ax), 1e-20f)) * ax;
+            const float ca = warp_min(dot(ax, nrm)), sa = sqrtf(fmaxf(0.0f, 1.0f - ca * ca));
+            const float rmax = F.grid.rmax * 1.001f;
+            delta = 2.5e-4f * F.grid.rmax + 4e-6f * (rho + 2.0f * spread);
+            // look less far, or not at all, where the hits' box with that
+            // reach around it would hold more balls than pay (a pass of a
+            // job word costs 70 instructions a ball, a walk about 95 a ray)
+            const float most = 9.0f * (float)min(F.jobs_per_hit, 16);
+            for (int t = 0;; ++t) {
+                const float v = (ext.x + rho) * (ext.y + rho) * (ext.z + rho);
+                if (8.0f * v * F.grid.density <= most) break;
+                rho *= 0.75f;
+                if (t == 2) {
+                    rho = 0.0f;
+                    break;
+                }
+            }
+            for (int t = 0; t < 2 && rho > 0.0f; ++t) {
+                ns = nt = 0;
+                const float R = rho + rmax;
+                int c0[3], c1[3];
+                const float l[3] = {mn.x - R, mn.y - R, mn.z - R}, h[3] = {mx.x + R, mx.y + R, mx.z + R};
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    c0[k] = cell_of(F.grid, k, l[k]) >> 1;
+                    c1[k] = cell_of(F.grid, k, h[k]) >> 1;
+                }
+                const int ny = c1[1] - c0[1] + 1, rows = ny * (c1[2] - c0[2] + 1);
+                for (int r0 = 0; r0 < rows; r0 += 32) {
+                    // one row of cells a lane: a run of balls; the runs are
+                    // laid end to end and read 32 balls at a time
+                    uint32_t k = 0, cnt = 0;
+                    if (r0 + lane < rows) {
+                        const int y = c0[1] + (r0 + lane) % ny, z = c0[2] + (r0 + lane) / ny;
+                        const int64_t row = ((int64_t)z * F.grid.bn[1] + y) * F.grid.bn[0];
+                        k = __ldg(F.grid.bstart + row + c0[0]);
+                        cnt = __ldg(F.grid.bstart + row + c1[0] + 1) - k;
+                    }
+                    uint32_t incl = cnt;
+#pragma unroll
+                    for (int off = 1; off < 32; off <<= 1) {
+                        const uint32_t y = __shfl_up_sync(FULL, incl, off);
+                        if (lane >= off) incl += y;
+                    }
+                    const uint32_t T = __shfl_sync(FULL, incl, 31), ex = incl - cnt;
+                    S.rows.off[lane] = k - ex;
+                    for (uint32_t base = 0; base < T; base += 32) {
+                        const uint32_t u = ex > base ? ex : base, pos = u - base;
+                        const bool mine = pos < 32u && incl > u;
+                        __syncwarp();
+                        if (mine) S.rows.owner[pos] = (uint32_t)lane;
+                        const unsigned starts = __reduce_or_sync(FULL, mine ? 1u << pos : 0u);
+                        __syncwarp();
+                        const uint32_t p = base + lane;
+                        bool sph = false, tub = false;
+                        float4 s = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                        if (p < T) {
+                            const unsigned r = S.rows.owner[31 - __clz(starts & (0xFFFFFFFFu >> (31 - lane)))];
+                            s = __ldg(F.grid.balls + GBRT_INDEX(p + S.rows.off[r], (uint32_t)F.grid.nballs));
+                            const float rad = fabsf(s.w);
+                            const V3<float> v = v3(s.x, s.y, s.z) - ctr;
+                            const float ex2 = fmaxf(fabsf(v.x) - ext.x, 0.0f), ey2 = fmaxf(fabsf(v.y) - ext.y, 0.0f),
+                                        ez2 = fmaxf(fabsf(v.z) - ext.z, 0.0f), far = 1.001f * (rho + rad);
+                            // behind every hit's tangent plane: the normals
+                            // lie within the cone (ca) about ax
+                            const float along = dot(v, ax), off = sqrt_pos(dot(v, v) - along * along);
+                            const bool in = ex2 * ex2 + ey2 * ey2 + ez2 * ez2 <= far * far && s.w != 0.0f &&
+                                            !(ca > 0.0f && along * ca + off * sa + spread <
+                                                               -1.001f * rad - 1e-5f * (fabsf(along) + off));
+                            sph = in && s.w > 0.0f;
+                            tub = in && s.w < 0.0f;
+                        }
+                        const unsigned ms = __ballot_sync(FULL, sph), mt = __ballot_sync(FULL, tub);
+                        const int is = ns + __popc(ms & lt), it = nt + __popc(mt & lt);
+                        if (sph && is < NEAR_SPHERES) S.sph[is] = s;
+                        if (tub && it < NEAR_TUBES) S.tub[it] = make_float4(s.x, s.y, s.z, -s.w);
+                        ns += __popc(ms);
+                        nt += __popc(mt);
+                    }
+                    __syncwarp();
+                }
+                if (ns <= NEAR_SPHERES && nt <= NEAR_TUBES) break;
+                rho = t == 0 ? 0.6f * rho : 0.0f;  // the lists overflowed
+            }
+            __syncwarp();
+        }
+        if (lane == 0) b.tiles[tile].rho = rho;
+        const int w0 = b.tiles[tile].word, w1 = min(w0 + F.rec_words, F.mask_words);
+        for (int w = w0; w < w1; ++w) {
+            const int j0 = 16 * w, cnt = F.jobs_per_hit - j0 < 16 ? F.jobs_per_hit - j0 : 16;
+            uint32_t todo, start, esc = 0u;
+            if (rho > 0.0f) {
+                if (cnt > 8) {
+                    near_jobs<16>(F, S, lane, j0, o, nrm, q, skip, ns, nt, rho, delta, todo, start, esc);
+                } else {
+                    todo = start = 0u;
+                    for (int k = 0; k < cnt; k += 4) {
+                        uint32_t t4, s4, e4;
+                        near_jobs<4>(F, S, lane, j0 + k, o, nrm, q, skip, ns, nt, rho, delta, t4, s4, e4);
+                        todo |= t4 << k;
+                        start |= s4 << k;
+                        esc |= e4 << k;
+                    }
+                }
+            } else {
+                todo = start = (1u << cnt) - 1u;
+            }
+            if (lane >= n) todo = start = esc = 0u;
+            // escaped jobs: AO samples come first, then the lights
+            const int sp = F.spp - j0 > 0 ? (F.spp - j0 < 16 ? F.spp - j0 : 16) : 0;
+            const uint32_t vis = __popc(esc & ((1u << sp) - 1u));
+            if (vis) atomicAdd(b.vis + slot, vis);
+            if (esc >> sp) atomicOr(b.lmask + slot, (esc >> sp) << (j0 + sp - F.spp));
+            if (lane < n) b.masks[F.mask_base + (slot - F.hit_base) * F.mask_words + w] = todo | start << 16;
+            const uint32_t any = __reduce_or_sync(FULL, todo);
+            const uint32_t groups = ((any & 0xFu) != 0u) | ((any & 0xF0u) != 0u) << 1 | ((any & 0xF00u) != 0u) << 2 |
+                                    ((any & 0xF000u) != 0u) << 3;
+            if (groups && lane == 0) {
+                unsigned long long at = atomicAdd(b.nunits, (unsigned long long)__popc(groups));
+                for (int g = 0; g < 4; ++g)
+                    if ((groups >> g) & 1u) b.units[at++] = tile << 8 | (unsigned)(4 * w + g);
+            }
+        }
+        __syncwarp();
+    }
+}
+
 // ---- FP32 frames
 
 // Ray record in shared memory: (origin, tmax) and (direction, -) -- two
@@ -716,8 +1062,105 @@ struct AoPtrs<true> {};
 // warp (60 KB of L1) 2.5% slower, 5 KB (92 KB of L1, with an 8-slot mailbox
 // and a test queue) 1% slower.
 static_assert(AO_CELLS == 4, "the pair segments of a ray are kept as one uint4 of starts and one of offsets");
-template <bool UNI>
-struct AoWarp : AoPtrs<UNI> {
+// The unit of the near pass that a warp is taking rays from: 4 jobs of a work
+// item's hits. b[s], z[s]: hits whose job s has to walk, has to walk from its
+// start; used, rem: rays taken and left.
+struct AoUnit {
+    uint32_t b[4], z[4];
+    int64_t slot;
+    const FrameDev* F;
+    int job;
+    float tmin;
+    uint32_t used, rem;
+};
+template <bool NEAR>
+struct AoUnits {
+    AoUnit unit;
+};
+template <>
+struct AoUnits<false> {};
+
+// Position of the n-th (from 0) set bit of m.
+__device__ __forceinline__ int nth_bit(uint32_t m, unsigned n) {
+    int at = 0;
+#pragma unroll
+    for (int w = 16; w > 0; w >>= 1) {
+        const unsigned c = __popc((m >> at) & ((1u << w) - 1u));
+        const bool up = n >= c;
+        n -= up ? c : 0u;
+        at += up ? w : 0;
+    }
+    return at;
+}
+
+// Hands `need` rays of the near pass's units to the idle lanes (free; i: a
+// lane's rank among them): the hit slot, job, frame and start of each. The
+// warp's unit is kept in U; sets exhausted when no unit is left.
+__device__ __forceinline__ void unit_take(const BatchDev& b, AoUnit& U, int lane, unsigned long long total,
+                                          unsigned need, unsigned i, bool free, bool& exhausted, int64_t& vslot,
+                                          uint32_t& smp, float& tmin, const FrameDev*& Fp) {
+    for (unsigned done = 0; done < need;) {
+        unsigned rem = U.rem;
+        if (rem == 0u) {
+            unsigned long long at = 0;
+            if (lane == 0) at = atomicAdd(b.queue + 1, 1ull);
+            at = __shfl_sync(FULL, at, 0);
+            if (at >= total) {
+                exhausted = true;
+                break;
+            }
+            const unsigned long long unit = b.units[at];
+                        const int g = (int)(unit & 0xFFu), sh = 4 * (g & 3);
+            const TileRec T = b.tiles[unit >> 8];
+            const FrameDev& N = b.frames[T.frame];
+            uint32_t m = 0u;
+            if (lane < T.n)
+                m = b.masks[N.mask_base + (T.slot - N.hit_base + lane) * N.mask_words + (g >> 2)] >> sh;
+            __syncwarp();
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+                const unsigned todo = __ballot_sync(FULL, (m >> s) & 1u);
+                const unsigned start = __ballot_sync(FULL, (m >> (16 + s)) & 1u);
+                U.b[s] = todo;
+                U.z[s] = start;
+                rem += __popc(todo);
+            }
+            U.slot = T.slot;
+            U.F = &N;
+            U.job = 4 * g;
+            U.tmin = T.rho * (1.0f - 1e-4f);
+            U.used = 0u;
+            __syncwarp();
+        }
+        const unsigned take = rem < need - done ? rem : need - done;
+        if (free && i >= done && i < done + take) {
+            unsigned k = U.used + (i - done);
+            int s = 0;
+#pragma unroll
+            for (int t = 0; t < 3; ++t) {
+                const unsigned c = __popc(U.b[t]);
+                const bool up = s == t && k >= c;
+                k -= up ? c : 0u;
+                s += up ? 1 : 0;
+            }
+            const int hit = nth_bit(U.b[s], k);
+            vslot = GBRT_INDEX(U.slot + hit, b.hit_cap);
+            smp = (uint32_t)(U.job + s);
+            tmin = (U.z[s] >> hit) & 1u ? 0.0f : U.tmin;
+            Fp = U.F;
+        }
+        __syncwarp();
+        if (lane == 0) {
+            U.used += take;
+            U.rem = rem - take;
+        }
+        __syncwarp();
+        done += take;
+    }
+}
+
+template <bool UNI, bool NEAR>
+struct AoWarp : AoPtrs<UNI>, AoUnits<NEAR> {
     AoRay ray[32];
     // item index of pair p of ray r: p + sdo[r][g] for the last cell g whose
     // pairs start at or before p (sds[r][g])
@@ -728,27 +1171,27 @@ struct AoWarp : AoPtrs<UNI> {
     // at least one of its at most AO_CELLS cells, so AO_CELLS - 1 wait at most
     uint2 fifo[32][AO_CELLS - 1];
 };
-static_assert(sizeof(AoWarp<false>) <= 4096, "the FP32 AO walk's per-warp state outgrew its 4 KB");
+static_assert(sizeof(AoWarp<false, true>) <= 4096, "the FP32 AO walk's per-warp state outgrew its 4 KB");
 
-template <bool UNI>
-__device__ __forceinline__ const float4* ao_obj(const AoWarp<UNI>& S, unsigned r, const float4* uni) {
+template <bool UNI, bool NEAR>
+__device__ __forceinline__ const float4* ao_obj(const AoWarp<UNI, NEAR>& S, unsigned r, const float4* uni) {
     if constexpr (UNI) return uni;
     else return S.obj[r];
 }
-template <bool UNI>
-__device__ __forceinline__ const uint32_t* ao_items(const AoWarp<UNI>& S, unsigned r, const uint32_t* uni) {
+template <bool UNI, bool NEAR>
+__device__ __forceinline__ const uint32_t* ao_items(const AoWarp<UNI, NEAR>& S, unsigned r, const uint32_t* uni) {
     if constexpr (UNI) return uni;
     else return S.items[r];
 }
 #ifdef GBRT_CHECKED
 // ray r's item-buffer length and object count (the checked build's bounds)
-template <bool UNI>
-__device__ __forceinline__ int64_t ao_nitems(const AoWarp<UNI>& S, unsigned r, int64_t uni) {
+template <bool UNI, bool NEAR>
+__device__ __forceinline__ int64_t ao_nitems(const AoWarp<UNI, NEAR>& S, unsigned r, int64_t uni) {
     if constexpr (UNI) return uni;
     else return S.nitems[r];
 }
-template <bool UNI>
-__device__ __forceinline__ int64_t ao_nobj(const AoWarp<UNI>& S, unsigned r, int64_t uni) {
+template <bool UNI, bool NEAR>
+__device__ __forceinline__ int64_t ao_nobj(const AoWarp<UNI, NEAR>& S, unsigned r, int64_t uni) {
     if constexpr (UNI) return uni;
     else return S.nobj[r];
 }
@@ -763,11 +1206,16 @@ __device__ __forceinline__ int64_t ao_nobj(const AoWarp<UNI>& S, unsigned r, int
 // one to AO_CELLS cells (all lanes run the same step code); the warp lays the
 // (ray, item) pairs of those cells out densely with a scan and tests them 32
 // at a time, one pair per lane. UNI: every frame of the batch has the same scene and grid.
-template <bool UNI>
+// NEAR: the rays are those the near pass left, from its units.
+template <bool UNI, bool NEAR>
 __global__ void __launch_bounds__(256) k_ao_walk(const __grid_constant__ BatchDev b) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    AoWarp<UNI>& S = reinterpret_cast<AoWarp<UNI>*>(smem_raw)[threadIdx.x >> 5];
+    AoWarp<UNI, NEAR>& S = reinterpret_cast<AoWarp<UNI, NEAR>*>(smem_raw)[threadIdx.x >> 5];
     grid_dependency_wait();
+    if constexpr (NEAR) {
+        S.unit.rem = 0u;
+        __syncwarp();
+    }
     const float4* uobj = nullptr;
     const uint32_t* uitems = nullptr;
     const uint2* ucells = nullptr;
@@ -782,7 +1230,7 @@ __global__ void __launch_bounds__(256) k_ao_walk(const __grid_constant__ BatchDe
 #endif
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
-    const unsigned long long total = b.job_off[b.nframes];
+    const unsigned long long total = NEAR ? *b.nunits : b.job_off[b.nframes];
     const int refill = b.refill;
     bool has = false, exhausted = false, overflow = false;
     Walk<float> w;
@@ -801,61 +1249,74 @@ __global__ void __launch_bounds__(256) k_ao_walk(const __grid_constant__ BatchDe
         if (!exhausted && __popc(act) < refill) {
             const unsigned idle = ~act;
             const unsigned need = __popc(idle);
-            const unsigned long long rem = pool_end - pool;
-            unsigned long long fresh_base = 0;
-            if (rem < need) {
-                if (lane == 0) fresh_base = atomicAdd(b.queue + 1, (unsigned long long)AO_CLAIM);
-                fresh_base = __shfl_sync(FULL, fresh_base, 0);
-                if (fresh_base >= total) exhausted = true;
-            }
-            if (!has) {
-                const unsigned i = __popc(idle & lt);
-                const unsigned long long jj = i < rem ? pool + i : fresh_base + (i - rem);
-                if (jj < total) {
-                    const int f = b.nframes == 1 ? 0 : find_frame(b.job_off, b.nframes, jj);
-                    const FrameDev& F = b.frames[f];
-                    uint32_t h, smp, q, own;
-                    V3<float> o, n, d;
-                    float tmax;
-                    ao_split(F, jj - b.job_off[f], h, smp);
-                    vslot = GBRT_INDEX(F.hit_base + (int64_t)h, b.hit_cap);
-                    HitIO<float>::load(b.hits32, vslot, o, n, q, own);
-                    if (!ao_direction<float>(F, q, smp, n, d, tmax, lbit)) {
-                        // the light cannot reach this side: its bit stays clear
-                    } else if (walk_start(F.grid, o, d, 0.0f, tmax, w)) {
-                        if constexpr (UNI) {
-                            cells = ucells;
-                        } else {
-                            cells = F.grid.cells;
-                            S.obj[lane] = F.scene.obj;
-                            S.items[lane] = F.grid.items;
-#ifdef GBRT_CHECKED
-                            S.nitems[lane] = F.grid.nitems;
-                            S.nobj[lane] = (int64_t)F.scene.S + F.scene.C;
-#endif
-                        }
-                        AoRay ray;
-                        ray.o = o;
-                        ray.tmax = tmax;
-                        ray.d = d;
-                        ray.pad = 0.0f;
-                        S.ray[lane] = ray;
-                        // the walk stands on its first cell: its record waits in
-                        // the fifo, so every later cell comes from a step
-                        S.fifo[lane][0] = __ldg(cells + GBRT_INDEX(w.cell, w.ncells));
-                        nf = 1;
-                        wend = false;
-                        has = true;
+            // sets the lane up on job smp of hit vslot, from distance tmin on
+            auto set_up = [&](const FrameDev& F, uint32_t smp, float tmin) {
+                uint32_t q, own;
+                V3<float> o, n, d;
+                float tmax;
+                HitIO<float>::load(b.hits32, vslot, o, n, q, own);
+                if (!ao_direction<float>(F, q, smp, n, d, tmax, lbit)) {
+                    // the light cannot reach this side: its bit stays clear
+                } else if (walk_start(F.grid, o, d, tmin, tmax, w)) {
+                    if constexpr (UNI) {
+                        cells = ucells;
                     } else {
-                        ao_escape(b, vslot, lbit);  // misses the objects' bounds: escapes
+                        cells = F.grid.cells;
+                        S.obj[lane] = F.scene.obj;
+                        S.items[lane] = F.grid.items;
+#ifdef GBRT_CHECKED
+                        S.nitems[lane] = F.grid.nitems;
+                        S.nobj[lane] = (int64_t)F.scene.S + F.scene.C;
+#endif
+                    }
+                    AoRay ray;
+                    ray.o = o;
+                    ray.tmax = tmax;
+                    ray.d = d;
+                    ray.pad = 0.0f;
+                    S.ray[lane] = ray;
+                    // the walk stands on its first cell: its record waits in
+                    // the fifo, so every later cell comes from a step
+                    S.fifo[lane][0] = __ldg(cells + GBRT_INDEX(w.cell, w.ncells));
+                    nf = 1;
+                    wend = false;
+                    has = true;
+                } else {
+                    ao_escape(b, vslot, lbit);  // misses the objects' bounds: escapes
+                }
+            };
+            if constexpr (NEAR) {
+                const FrameDev* Fp = nullptr;  // the frame of the ray this lane takes
+                uint32_t smp = 0;
+                float tmin = 0.0f;
+                unit_take(b, S.unit, lane, total, need, __popc(idle & lt), !has, exhausted, vslot, smp, tmin, Fp);
+                if (Fp) set_up(*Fp, smp, tmin);
+            } else {
+                const unsigned long long rem = pool_end - pool;
+                unsigned long long fresh_base = 0;
+                if (rem < need) {
+                    if (lane == 0) fresh_base = atomicAdd(b.queue + 1, (unsigned long long)AO_CLAIM);
+                    fresh_base = __shfl_sync(FULL, fresh_base, 0);
+                    if (fresh_base >= total) exhausted = true;
+                }
+                if (!has) {
+                    const unsigned i = __popc(idle & lt);
+                    const unsigned long long jj = i < rem ? pool + i : fresh_base + (i - rem);
+                    if (jj < total) {
+                        const int f = b.nframes == 1 ? 0 : find_frame(b.job_off, b.nframes, jj);
+                        const FrameDev& F = b.frames[f];
+                        uint32_t h, smp;
+                        ao_split(F, jj - b.job_off[f], h, smp);
+                        vslot = GBRT_INDEX(F.hit_base + (int64_t)h, b.hit_cap);
+                        set_up(F, smp, 0.0f);
                     }
                 }
-            }
-            if (rem >= need) {
-                pool += need;
-            } else {
-                pool = fresh_base + (need - rem);
-                pool_end = fresh_base + AO_CLAIM;
+                if (rem >= need) {
+                    pool += need;
+                } else {
+                    pool = fresh_base + (need - rem);
+                    pool_end = fresh_base + AO_CLAIM;
+                }
             }
         }
         if (exhausted && __ballot_sync(FULL, has) == 0) break;
@@ -995,8 +1456,12 @@ struct LaneScene {
     int32_t nobj;
     V3<float> lo;
     float om;
+    bool cut;
     __device__ __forceinline__ void set(const FrameDev& F) {
-        bs = F.scene.bs;
+        // tubes cut to what sticks out of their spheres: a ray without a limit
+        // that meets the rest meets the sphere as well
+        cut = isinf(F.ao_maxdist_f);
+        bs = cut ? F.grid.cut : F.scene.bs;
         nobj = F.scene.S + F.scene.C;
         cells = F.grid.cells;
         items = F.grid.items;
@@ -1179,7 +1644,7 @@ struct FrameRays {
         if (next >= f_hi) {
             const int nf = b.nframes == 1 ? 0 : find_frame(b.job_off, b.nframes, next);
             const FrameDev& N = b.frames[nf];
-            const bool same = N.scene.bs == A.bs && N.grid.cells == A.cells;
+            const bool same = N.grid.cells == A.cells && isinf(N.ao_maxdist_f) == A.cut;
             if (!same && act != 0u) return LANES_GO;  // another scene: the lanes in flight drain first
             f = nf;
             f_lo = b.job_off[f];
@@ -1218,8 +1683,8 @@ __global__ void __launch_bounds__(256, 3) k_ao_walk64(const __grid_constant__ Ba
     grid_dependency_wait();
     FrameRays src(b);
     LaneScene A;
-    A.bs = nullptr;
     A.cells = nullptr;
+    A.cut = false;
     lane_walk(src, A, b.refill, b.err);
 }
 
@@ -1419,7 +1884,17 @@ int err_of(cudaError_t e) {
     return e == cudaErrorMemoryAllocation ? GBRT_ENOMEM : GBRT_EDEVICE;
 }
 
-// Grow a device buffer (the stream is drained first: old work may still read it).
+template <class K>
+int persistent_grid(Ctx* ctx, K kernel, int block, size_t smem = 0) {
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, smem) != cudaSuccess || per_sm < 1)
+        per_sm = 1;
+    if (ctx->tuning.ctas_per_sm > 0) per_sm = std::min(per_sm, ctx->tuning.ctas_per_sm);
+    return per_sm * ctx->num_sms;
+}
+
+}  // namespace
+
 int grow(Ctx* ctx, void** p, size_t* cap, size_t need) {
     if (*cap >= need) return GBRT_OK;
     cudaStreamSynchronize(ctx->stream);
@@ -1433,21 +1908,10 @@ int grow(Ctx* ctx, void** p, size_t* cap, size_t need) {
     return rc;
 }
 
-template <class K>
-int persistent_grid(Ctx* ctx, K kernel, int block, size_t smem = 0) {
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, smem) != cudaSuccess || per_sm < 1)
-        per_sm = 1;
-    if (ctx->tuning.ctas_per_sm > 0) per_sm = std::min(per_sm, ctx->tuning.ctas_per_sm);
-    return per_sm * ctx->num_sms;
-}
-
-}  // namespace
-
 // Lay out one batch (all frames of one precision), upload its descriptors and
 // enqueue memsets + the four kernels on `stream`.
 struct Grids {
-    int primary, ao, shade, resolve;
+    int primary, near, ao, shade, resolve;  // near: 0 without a near pass
 };
 
 // Launch `kernel` as a programmatic dependent of the kernel before it in
@@ -1468,10 +1932,12 @@ static cudaError_t launch_dependent(void (*kernel)(BatchDev), dim3 grid, dim3 bl
     return cudaLaunchKernelEx(&cfg, kernel, bd);
 }
 
-template <bool UNI>
+template <bool UNI, bool NEAR>
 static size_t ao_smem(int block) {
-    return (size_t)(block / 32) * sizeof(AoWarp<UNI>);
+    return (size_t)(block / 32) * sizeof(AoWarp<UNI, NEAR>);
 }
+constexpr int NEAR_BLOCK = 128;
+constexpr size_t NEAR_SMEM = NEAR_BLOCK / 32 * sizeof(NearWarp);
 
 // Shared-memory share of the SM asked for an AO walk whose CTAs of 256 threads
 // use `smem` bytes: just enough for four of them (and the driver's per-CTA
@@ -1493,50 +1959,67 @@ static cudaError_t prefer_small_carveout(K kernel, size_t smem) {
 
 // A refused preference leaves the driver's choice (and its error is cleared
 // here, so it is not taken for a later launch's).
-static void configure_ao() {
-    if (prefer_small_carveout(k_ao_walk<true>, ao_smem<true>(256)) != cudaSuccess ||
-        prefer_small_carveout(k_ao_walk<false>, ao_smem<false>(256)) != cudaSuccess ||
+static cudaError_t configure_ao() {
+    if (prefer_small_carveout(k_ao_walk<true, false>, ao_smem<true, false>(256)) != cudaSuccess ||
+        prefer_small_carveout(k_ao_walk<false, false>, ao_smem<false, false>(256)) != cudaSuccess ||
+        prefer_small_carveout(k_ao_walk<true, true>, ao_smem<true, true>(256)) != cudaSuccess ||
+        prefer_small_carveout(k_ao_walk<false, true>, ao_smem<false, true>(256)) != cudaSuccess ||
         prefer_small_carveout(k_ao_walk64, 0) != cudaSuccess)
         (void)cudaGetLastError();
+    // the near pass's candidate lists exceed the 48 KB default
+    return cudaFuncSetAttribute(k_ao_near, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)NEAR_SMEM);
 }
 
+// uni: one scene and grid for the whole batch; near > 0: with a near pass of
+// that many CTAs
 template <class R>
-static void launch_ao(const BatchDev& bd, bool uni, int grid, int block, cudaStream_t stream) {
-    if (std::is_same<R, double>::value) launch_dependent(k_ao_walk64, grid, block, 0, stream, bd);
-    else if (uni) launch_dependent(k_ao_walk<true>, grid, block, ao_smem<true>(block), stream, bd);
-    else launch_dependent(k_ao_walk<false>, grid, block, ao_smem<false>(block), stream, bd);
+static void launch_ao(const BatchDev& bd, bool uni, int near, int grid, int block, cudaStream_t stream) {
+    if (std::is_same<R, double>::value) {
+        launch_dependent(k_ao_walk64, grid, block, 0, stream, bd);
+    } else if (near > 0) {
+        launch_dependent(k_ao_near, near, NEAR_BLOCK, NEAR_SMEM, stream, bd);
+        if (uni) launch_dependent(k_ao_walk<true, true>, grid, block, ao_smem<true, true>(block), stream, bd);
+        else launch_dependent(k_ao_walk<false, true>, grid, block, ao_smem<false, true>(block), stream, bd);
+    } else {
+        if (uni) launch_dependent(k_ao_walk<true, false>, grid, block, ao_smem<true, false>(block), stream, bd);
+        else launch_dependent(k_ao_walk<false, false>, grid, block, ao_smem<false, false>(block), stream, bd);
+    }
 }
 
 // The passes after the primary one: AO walk, shading, and the box filter of
 // supersampled frames (the AO plan runs in the primary kernel's last CTA).
 template <class R>
-static void launch_after_primary(const BatchDev& bd, bool uni, int ao_grid, int block, int shade_grid,
+static void launch_after_primary(const BatchDev& bd, bool uni, int near, int ao_grid, int block, int shade_grid,
                                  int resolve_grid, bool resolve, cudaStream_t stream,
                                  const std::function<void(int)>& mark) {
-    launch_ao<R>(bd, uni, ao_grid, block, stream);
+    launch_ao<R>(bd, uni, near, ao_grid, block, stream);
     mark(3);
     launch_dependent(k_shade<R>, shade_grid, 256, 0, stream, bd);
     if (resolve) launch_dependent(k_resolve<R>, dim3(resolve_grid, std::min(bd.nframes, 65535)), 256, 0, stream, bd);
 }
 
-static Grids grids_for(Ctx* ctx, int precision, bool uni) {
+static int grids_for(Ctx* ctx, int precision, bool uni, bool near, Grids& g) {
     const int block = ctx->tuning.block;
     if (!ctx->smem_configured) {
-        configure_ao();
+        if (configure_ao() != cudaSuccess) return GBRT_EDEVICE;
         ctx->smem_configured = true;
     }
-    Grids g;
+    g.near = near ? persistent_grid(ctx, k_ao_near, NEAR_BLOCK, NEAR_SMEM) : 0;
     if (precision == GBRT_FP32) {
         g.primary = persistent_grid(ctx, k_primary<GBRT_FP32>, block);
-        g.ao = uni ? persistent_grid(ctx, k_ao_walk<true>, block, ao_smem<true>(block))
-                   : persistent_grid(ctx, k_ao_walk<false>, block, ao_smem<false>(block));
+        if (near)
+            g.ao = uni ? persistent_grid(ctx, k_ao_walk<true, true>, block, ao_smem<true, true>(block))
+                       : persistent_grid(ctx, k_ao_walk<false, true>, block, ao_smem<false, true>(block));
+        else
+            g.ao = uni ? persistent_grid(ctx, k_ao_walk<true, false>, block, ao_smem<true, false>(block))
+                       : persistent_grid(ctx, k_ao_walk<false, false>, block, ao_smem<false, false>(block));
     } else {
         g.primary = persistent_grid(ctx, k_primary<GBRT_FP64>, block);
         g.ao = persistent_grid(ctx, k_ao_walk64, block);
     }
     g.shade = ctx->num_sms * 8;
     g.resolve = ctx->num_sms * 4;
-    return g;
+    return GBRT_OK;
 }
 
 // Every frame of the batch reads the same scene and grid (device-side rebuilt
@@ -1550,6 +2033,26 @@ static bool one_scene(const FrameDev* frames, int n) {
             return false;
     }
     return true;
+}
+
+// Whether a near pass suits a frame's AO rays: enough of them a hit to share its
+// per-hit work, no limit on their length (the pass takes a hit at any distance
+// for one), and objects small enough (grid.rho).
+static bool near_pass_suits(const FrameDev& f) {
+    return f.precision == GBRT_FP32 && f.grid.rho > 0.0f && std::isinf(f.ao_maxdist_f) &&
+           f.jobs_per_hit >= NEAR_MIN_JOBS && f.jobs_per_hit <= NEAR_MAX_JOBS;
+}
+
+// Share of a frame's pixels that the objects' bounding sphere covers, roughly
+// (a disc against the window; 1 from inside).
+static double hit_share(const FrameDev& f) {
+    double along = 0.0, r = f.grid.bs64[3], scale = 1.0;
+    for (int k = 0; k < 3; ++k) along += (f.grid.bs64[k] - f.eye[k]) * f.dir_unit[k];
+    if (f.cam_kind == GBRT_CAMERA_PINHOLE) {
+        if (along <= r) return 1.0;
+        scale = along;
+    }
+    return 0.785 * std::min(1.0, r / (f.half_w * scale)) * std::min(1.0, r / (f.half_h * scale));
 }
 
 // optional passes of a batch, and its scene layout
@@ -1579,16 +2082,16 @@ static int enqueue_batch(Ctx* ctx, cudaStream_t stream, int precision, const Bat
         k_primary<GBRT_FP32><<<gr.primary, block, 0, stream>>>(bd);
         mark(1);
         mark(2);
-        launch_after_primary<float>(bd, uni, gr.ao, block, gr.shade, gr.resolve, resolve, stream, mark);
+        launch_after_primary<float>(bd, uni, gr.near, gr.ao, block, gr.shade, gr.resolve, resolve, stream, mark);
     } else {
         k_primary<GBRT_FP64><<<gr.primary, block, 0, stream>>>(bd);
         mark(1);
         mark(2);
-        launch_after_primary<double>(bd, uni, gr.ao, block, gr.shade, gr.resolve, resolve, stream, mark);
+        launch_after_primary<double>(bd, uni, gr.near, gr.ao, block, gr.shade, gr.resolve, resolve, stream, mark);
     }
     mark(4);
     if (tm) ctx->timed = tm;
-    ctx->launches += resolve ? 4 : 3;
+    ctx->launches += 3 + (resolve ? 1 : 0) + (gr.near ? 1 : 0);
     return err_of(cudaGetLastError());
 }
 
@@ -1604,11 +2107,16 @@ int render_frames(Ctx* ctx, FrameDev* frames, int n, bool use_graph) {
     // descriptors: frames, then tile_off (n + 1)
     const size_t frames_bytes = ((size_t)n * sizeof(FrameDev) + 255) & ~(size_t)255;
     const size_t desc_bytes = frames_bytes + (size_t)(n + 1) * sizeof(long long);
-    // counters: queue [4], hit_count [n], job_off [n + 1], hit_off [n + 1]
-    const size_t counters_bytes = 4 * sizeof(unsigned long long) + (size_t)n * sizeof(unsigned) +
+    // counters: queue [4], near units, near tiles, hit_count [n], job_off [n + 1],
+    // hit_off [n + 1]
+    const size_t counters_bytes = 6 * sizeof(unsigned long long) + (size_t)n * sizeof(unsigned) +
                                   2 * (size_t)(n + 1) * sizeof(unsigned long long) + 64;
     int64_t px = 0;
     long long tiles = 0;
+    int64_t near_rays = 0;  // rays of the frames that a near pass suits, if every pixel hits
+    bool many = false;      // a frame with too many jobs a hit for masks
+    double near_recs = 0;   // and their expected tile records
+    int64_t mask_words = 0, recs = 0, all_rays = 0;
     size_t fine_bytes = 0;  // finer-raster colours of the supersampled frames' bands
     bool resolve = false;
     int extra = 0;
@@ -1617,8 +2125,27 @@ int render_frames(Ctx* ctx, FrameDev* frames, int n, bool use_graph) {
         frames[f].tiles_x = (frames[f].W + tw - 1) / tw;
         frames[f].tiles_y = (frames[f].rows + th - 1) / th;
         frames[f].hit_base = px;
-        px += (int64_t)frames[f].W * frames[f].rows;
-        tiles += (long long)frames[f].tiles_x * frames[f].tiles_y;
+        const int64_t fpx = (int64_t)frames[f].W * frames[f].rows;
+        const long long ftiles = (long long)frames[f].tiles_x * frames[f].tiles_y;
+        px += fpx;
+        tiles += ftiles;
+        frames[f].near_pass = near_pass_suits(frames[f]) ? 1 : 0;
+        frames[f].mask_words = std::min((frames[f].jobs_per_hit + 15) / 16, (NEAR_MAX_JOBS + 15) / 16);
+        frames[f].mask_base = mask_words;
+        // a record takes all of its tile's words (they share the gather) unless
+        // that leaves too few records
+        const double hit_tiles = std::max(1.0, (double)ftiles * hit_share(frames[f]));
+        const int per_tile = (int)std::min<double>(std::ceil(NEAR_MIN_RECS / hit_tiles),
+                                                   (double)std::max(frames[f].mask_words, 1));
+        frames[f].rec_words = std::max(1, (frames[f].mask_words + per_tile - 1) / per_tile);
+        if (frames[f].near_pass) {
+            near_rays += fpx * frames[f].jobs_per_hit;
+            near_recs += hit_tiles * frames[f].mask_words;
+        }
+        all_rays += fpx * frames[f].jobs_per_hit;
+        many = many || frames[f].jobs_per_hit > NEAR_MAX_JOBS;
+        mask_words += fpx * frames[f].mask_words;
+        recs += ftiles * frames[f].mask_words;
         if (frames[f].grid_src) extra |= EXTRA_PATCH;
         if (frames[f].aa > 1) {
             resolve = true;
@@ -1640,6 +2167,14 @@ int render_frames(Ctx* ctx, FrameDev* frames, int n, bool use_graph) {
     if ((rc = grow(ctx, &ctx->d_hits, &ctx->hits_cap, (size_t)px * rec)) != GBRT_OK) return rc;
     if ((rc = grow(ctx, (void**)&ctx->d_vis, &ctx->vis_cap, (size_t)px * sizeof(unsigned))) != GBRT_OK) return rc;
     if ((rc = grow(ctx, (void**)&ctx->d_lmask, &ctx->lmask_cap, (size_t)px * sizeof(unsigned))) != GBRT_OK)
+        return rc;
+    // enough of them to keep every warp of one more kernel busy, and at least
+    // half of the batch's rays
+    const bool near = near_recs >= NEAR_MIN_RECS && 2 * near_rays >= all_rays && !many;
+    const size_t units_at = (size_t)recs * sizeof(TileRec);
+    const size_t masks_at = units_at + 4 * (size_t)recs * sizeof(unsigned long long);
+    if (near &&
+        (rc = grow(ctx, &ctx->d_near, &ctx->near_cap, masks_at + (size_t)mask_words * sizeof(unsigned))) != GBRT_OK)
         return rc;
     if ((rc = grow(ctx, &ctx->d_desc, &ctx->desc_cap, desc_bytes)) != GBRT_OK) return rc;
     if ((rc = grow(ctx, &ctx->d_counters, &ctx->counters_cap, counters_bytes)) != GBRT_OK) return rc;
@@ -1664,7 +2199,9 @@ int render_frames(Ctx* ctx, FrameDev* frames, int n, bool use_graph) {
     bd.tile_off = (const long long*)((char*)ctx->d_desc + frames_bytes);
     char* cb = (char*)ctx->d_counters;
     bd.queue = (unsigned long long*)cb;
-    bd.job_off = (unsigned long long*)(cb + 4 * sizeof(unsigned long long));
+    bd.nunits = bd.queue + 4;
+    bd.ntiles = bd.queue + 5;
+    bd.job_off = bd.queue + 6;
     bd.hit_off = bd.job_off + (n + 1);
     bd.hit_count = (unsigned*)(bd.hit_off + (n + 1));
     bd.hits = ctx->d_hits;
@@ -1672,6 +2209,9 @@ int render_frames(Ctx* ctx, FrameDev* frames, int n, bool use_graph) {
     bd.vis = ctx->d_vis;
     bd.lmask = ctx->d_lmask;
     bd.err = ctx->d_err;
+    bd.tiles = near ? (TileRec*)ctx->d_near : nullptr;
+    bd.units = near ? (unsigned long long*)((char*)ctx->d_near + units_at) : nullptr;
+    bd.masks = near ? (unsigned*)((char*)ctx->d_near + masks_at) : nullptr;
     bd.hit_cap = (int64_t)px;
     bd.nframes = n;
     bd.tile_w = tw;
@@ -1681,7 +2221,8 @@ int render_frames(Ctx* ctx, FrameDev* frames, int n, bool use_graph) {
 
     const bool uni = one_scene(frames, n);
     if (uni) extra |= EXTRA_UNI;
-    const Grids gr = grids_for(ctx, precision, uni);
+    Grids gr;
+    if ((rc = grids_for(ctx, precision, uni, near, gr)) != GBRT_OK) return rc;
     if (!use_graph) {
         rc = enqueue_batch(ctx, ctx->stream, precision, bd, desc_bytes, gr, extra);
     } else {
@@ -1714,7 +2255,7 @@ int render_frames(Ctx* ctx, FrameDev* frames, int n, bool use_graph) {
             ctx->graph_bd = bd;
         }
         rc = err_of(cudaGraphLaunch(ctx->graph_exec, ctx->stream));
-        ctx->launches += 3 + (resolve ? 1 : 0) + ((extra & EXTRA_PATCH) ? 1 : 0);
+        ctx->launches += 3 + (resolve ? 1 : 0) + (gr.near ? 1 : 0) + ((extra & EXTRA_PATCH) ? 1 : 0);
     }
     if (rc != GBRT_OK) return rc;
     cudaEventRecord(ctx->staging_done, ctx->stream);
@@ -1722,10 +2263,7 @@ int render_frames(Ctx* ctx, FrameDev* frames, int n, bool use_graph) {
     return GBRT_OK;
 }
 
-int configure_render_kernels() {
-    configure_ao();
-    return GBRT_OK;
-}
+int configure_render_kernels() { return err_of(configure_ao()); }
 
 int enqueue_prepared(const BatchDev& bd, int precision, cudaStream_t stream, int block, int num_sms, bool patch) {
     auto grid_of = [&](auto kernel, size_t smem = 0) {
@@ -1739,10 +2277,10 @@ int enqueue_prepared(const BatchDev& bd, int precision, cudaStream_t stream, int
     const auto none = [](int) {};
     if (precision == GBRT_FP32) {
         k_primary<GBRT_FP32><<<grid_of(k_primary<GBRT_FP32>), block, 0, stream>>>(bd);
-        launch_after_primary<float>(bd, true, grid_of(k_ao_walk<true>, ao_smem<true>(block)), block, num_sms * 8, 0, false, stream, none);
+        launch_after_primary<float>(bd, true, 0, grid_of(k_ao_walk<true, false>, ao_smem<true, false>(block)), block, num_sms * 8, 0, false, stream, none);
     } else {
         k_primary<GBRT_FP64><<<grid_of(k_primary<GBRT_FP64>), block, 0, stream>>>(bd);
-        launch_after_primary<double>(bd, true, grid_of(k_ao_walk64), block, num_sms * 8, 0, false, stream, none);
+        launch_after_primary<double>(bd, true, 0, grid_of(k_ao_walk64), block, num_sms * 8, 0, false, stream, none);
     }
     return err_of(cudaGetLastError());
 }

@@ -1,5 +1,5 @@
 // Scene upload (input arrays -> device records + FP64 copies + scene box) and
-// the uniform-grid build: count -> exclusive scan -> scatter -> per-cell sort.
+// the uniform-grid build: count -> exclusive scan -> scatter -> balls.
 // The grid is the acceleration structure of the tracer; its build is the
 // paper's preprocessing phase (Table 5). For animated scenes the geometry can
 // be replaced in place (scene_update) and the grid rebuilt on the device with
@@ -36,6 +36,7 @@ __global__ void __launch_bounds__(256) k_scene_prep(const float* sph_in, int64_t
     const int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const float big = 3.0e38f;
     float lo[3] = {big, big, big}, hi[3] = {-big, -big, -big};
+    float rb = 0.0f;  // radius of the object's ball
     bool bad = false;
     if (id < S) {
         const float* p = sph_in + 4 * id;
@@ -44,6 +45,7 @@ __global__ void __launch_bounds__(256) k_scene_prep(const float* sph_in, int64_t
         obj[2 * id] = make_float4(c[0], c[1], c[2], r);
         obj[2 * id + 1] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         bs[id] = make_float4(c[0], c[1], c[2], r);
+        rb = r;
         obj64[4 * id] = make_double2(c[0], c[1]);
         obj64[4 * id + 1] = make_double2(c[2], r);
         obj64[4 * id + 2] = make_double2(0.0, 0.0);
@@ -77,8 +79,9 @@ __global__ void __launch_bounds__(256) k_scene_prep(const float* sph_in, int64_t
         // additions cover the rounding of the middle and of the radius
         const float cmax = fmaxf(fmaxf(fabsf(p0[0]) + fabsf(p1[0]), fabsf(p0[1]) + fabsf(p1[1])),
                                  fabsf(p0[2]) + fabsf(p1[2]));
+        rb = 1.00001f * sqrtf(0.25f * L * L + r * r) + 4e-7f * cmax;
         bs[id] = make_float4(0.5f * p0[0] + 0.5f * p1[0], 0.5f * p0[1] + 0.5f * p1[1], 0.5f * p0[2] + 0.5f * p1[2],
-                             -(1.00001f * sqrtf(0.25f * L * L + r * r) + 4e-7f * cmax));
+                             -rb);
         obj64[4 * id] = make_double2(p0[0], p0[1]);
         obj64[4 * id + 1] = make_double2(p0[2], r);
         obj64[4 * id + 2] = make_double2(a64[0], a64[1]);
@@ -103,6 +106,8 @@ __global__ void __launch_bounds__(256) k_scene_prep(const float* sph_in, int64_t
         }
     }
     // warp reduction, then one atomic per warp and component
+    const uint32_t rbits = __reduce_max_sync(0xffffffffu, bad ? 0u : __float_as_uint(rb));
+    if ((threadIdx.x & 31) == 0) atomicMax(box + 7, rbits);  // non-negative floats order as ints
     for (int k = 0; k < 3; ++k) {
         float l = lo[k], h = hi[k];
         for (int off = 16; off > 0; off >>= 1) {
@@ -181,19 +186,59 @@ __device__ __forceinline__ void span_cell(const int c0[3], int nx, int ny, int k
     z = c0[2] + k / (nx * ny);
 }
 
+// Cell of the halved grid that holds a ball's centre.
+__device__ __forceinline__ int64_t ball_cell(const BuildP& p, float4 s) {
+    const int bx = (p.n[0] + 1) >> 1, by = (p.n[1] + 1) >> 1;
+    const int x = build_cell(p, 0, s.x) >> 1, y = build_cell(p, 1, s.y) >> 1, z = build_cell(p, 2, s.z) >> 1;
+    return ((int64_t)z * by + y) * bx + x;
+}
+
 // Blocks of 256 threads for one warp per object over N objects.
 inline int object_warp_blocks(int64_t N) {
     return (int)std::min<int64_t>((std::max<int64_t>(N, 1) + 7) / 8, 1 << 20);
 }
 
+// Blocks of k_ball_sort for S spheres (a thread each) and C tubes (a warp each).
+inline int ball_sort_blocks(int64_t S, int64_t C) { return object_warp_blocks((S + 31) / 32 + C); }
+
+// CTAs of 256 threads that find the bounding radius of N objects.
+inline unsigned int radius_blocks(int64_t N) { return (unsigned int)((N + 255) / 256); }
+
+// Radius of the sphere about aux->ctr that holds every object: sphere |c - ctr|
+// + r, cylinder max over both ends of |p - ctr| + r (FP64, rounded up to float).
+__device__ __forceinline__ void bound_radius(const double2* obj64, int64_t N, int64_t id, BuildAux* aux) {
+    float rr = 0.0f;
+    if (id < N) {
+        const double cx = aux->ctr[0], cy = aux->ctr[1], cz = aux->ctr[2];
+        const double2* q = obj64 + 4 * id;
+        double2 q0 = q[0], q1 = q[1], q2 = q[2], q3 = q[3];
+        double px = q0.x - cx, py = q0.y - cy, pz = q1.x - cz;
+        double r = q1.y, L = q3.y;
+        double ex = px + L * q2.x, ey = py + L * q2.y, ez = pz + L * q3.x;
+        double d = fmax(sqrt(px * px + py * py + pz * pz), sqrt(ex * ex + ey * ey + ez * ez)) + r;
+        rr = __double2float_ru(d);
+    }
+    for (int off = 16; off > 0; off >>= 1) rr = fmaxf(rr, __shfl_xor_sync(0xffffffffu, rr, off));
+    if ((threadIdx.x & 31) == 0) atomicMax(&aux->rbits, __float_as_uint(rr));  // non-negative floats order as ints
+}
+
 // Count pass. When an object's box spans at most 64 cells, the cells its shape
 // reaches are also recorded as bits k in reach[id], so the scatter pass need
 // not repeat the test; wider objects get all-ones and are tested again there.
-__global__ void __launch_bounds__(256) k_grid_count(const float4* aabb, const float4* obj, int64_t N,
-                                                     const BuildP* bp, uint32_t* counts,
-                                                     unsigned long long* reach) {
+// Objects per cell of the halved grid (see GridDev::balls) go to bcounts.
+// The last radius_blocks(N) CTAs find the bounding sphere's radius instead (its
+// own kernel before: 5 us and a launch in a chain of short ones).
+__global__ void __launch_bounds__(256) k_grid_count(const float4* aabb, const float4* obj, const double2* obj64,
+                                                     const float4* bs, int64_t N, BuildAux* aux, uint32_t* counts,
+                                                     uint32_t* bcounts, unsigned long long* reach,
+                                                     unsigned int count_blocks) {
+    if (blockIdx.x >= count_blocks) {
+        bound_radius(obj64, N, (int64_t)(blockIdx.x - count_blocks) * blockDim.x + threadIdx.x, aux);
+        return;
+    }
+    const BuildP* bp = &aux->p;
     const int lane = threadIdx.x & 31;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    const int64_t warps = (int64_t)count_blocks * (blockDim.x >> 5);
     const BuildP p = *bp;
     for (int64_t id = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; id < N; id += warps) {
         int c0[3], c1[3];
@@ -213,7 +258,10 @@ __global__ void __launch_bounds__(256) k_grid_count(const float4* aabb, const fl
             const unsigned got = __ballot_sync(0xffffffffu, hit);
             if (base < 64) bits |= (unsigned long long)got << base;
         }
-        if (lane == 0) reach[id] = span <= 64 ? bits : ~0ull;
+        if (lane == 0) {
+            reach[id] = span <= 64 ? bits : ~0ull;
+            atomicAdd(bcounts + ball_cell(p, bs[id]), 1u);
+        }
     }
 }
 
@@ -245,43 +293,68 @@ __global__ void __launch_bounds__(256) k_grid_scatter(const float4* aabb, const 
     }
 }
 
-// Radius of the sphere about `ctr` that holds every object: sphere |c - ctr| + r,
-// cylinder max over both ends of |p - ctr| + r (FP64, rounded up to float).
-__global__ void __launch_bounds__(256) k_bound_radius(const double2* obj64, int64_t N, const double* ctr,
-                                                       unsigned int* rbits) {
-    int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    float rr = 0.0f;
-    if (id < N) {
-        const double cx = ctr[0], cy = ctr[1], cz = ctr[2];
-        const double2* q = obj64 + 4 * id;
-        double2 q0 = q[0], q1 = q[1], q2 = q[2], q3 = q[3];
-        double px = q0.x - cx, py = q0.y - cy, pz = q1.x - cz;
-        double r = q1.y, L = q3.y;
-        double ex = px + L * q2.x, ey = py + L * q2.y, ez = pz + L * q3.x;
-        double d = fmax(sqrt(px * px + py * py + pz * pz), sqrt(ex * ex + ey * ey + ez * ez)) + r;
-        rr = __double2float_ru(d);
-    }
-    for (int off = 16; off > 0; off >>= 1) rr = fmaxf(rr, __shfl_xor_sync(0xffffffffu, rr, off));
-    if ((threadIdx.x & 31) == 0) atomicMax(rbits, __float_as_uint(rr));  // non-negative floats order as ints
-}
-
-// Atomic scatter order is arbitrary: sort each cell's ids ascending (spheres
-// first, then cylinders; deterministic lists).
-__global__ void __launch_bounds__(256) k_cell_sort(const uint2* cells, int64_t ncells, uint32_t* items,
-                                                    uint64_t items_cap) {
-    int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= ncells) return;
-    uint2 cr = cells[c];
-    if ((uint64_t)cr.x + cr.y > items_cap) return;  // overflowed rebuild: the grid is disabled
-    uint32_t* it = items + cr.x;
-    for (uint32_t a = 1; a < cr.y; ++a) {
-        uint32_t v = it[a];
-        uint32_t b = a;
-        while (b > 0 && it[b - 1] > v) {
-            it[b] = it[b - 1];
-            --b;
+// The objects' balls, tubes cut to the part outside their spheres, in the order
+// of the halved grid's cells and then again by object id (after the scatter).
+// A thread per sphere, then a warp per tube: the lanes take the spheres listed
+// in the cells of the tube's two ends (the first half-warp one end, the second
+// the other). A cross-section (radius r, at axial coordinate s) lies inside a
+// sphere of radius R whose centre is h from the axis at coordinate sc when
+// (s - sc)^2 + (h + r)^2 < R^2; R is taken 0.1% smaller, so what is cut off
+// lies well inside: a ray that meets the tube there meets that sphere too.
+// (One thread a tube, going through both cells twice: 36 us for 12,818 tubes,
+// all of it load latency; a warp a tube 12 us.)
+__global__ void __launch_bounds__(256) k_ball_sort(const float4* obj, const float4* bs, int64_t S, int64_t N,
+                                                    const BuildP* bp, const uint2* cells, const uint32_t* items,
+                                                    uint64_t items_cap, const uint32_t* bstart, uint32_t* bcursor,
+                                                    float4* balls) {
+    const int lane = threadIdx.x & 31;
+    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    const int64_t sphere_warps = (S + 31) >> 5;
+    const BuildP p = *bp;
+    for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < sphere_warps + (N - S); w += warps) {
+        const bool tube = w >= sphere_warps;
+        const int64_t id = tube ? S + (w - sphere_warps) : 32 * w + lane;
+        if (id >= N || (!tube && id >= S)) continue;
+        float4 s = bs[id];
+        const int64_t c = ball_cell(p, s);
+        if (tube) {
+            const float4 A = obj[2 * id], B = obj[2 * id + 1];
+            const float t = lane < 16 ? 0.0f : B.w;
+            const int x = build_cell(p, 0, A.x + t * B.x), y = build_cell(p, 1, A.y + t * B.y),
+                      z = build_cell(p, 2, A.z + t * B.z);
+            uint2 cr = cells[((int64_t)z * p.n[1] + y) * p.n[0] + x];
+            if ((uint64_t)cr.x + cr.y > items_cap) cr.y = 0u;  // an overflowed rebuild
+            // the axis part inside the lane's spheres: joined to one end of
+            // the tube (what reaches past both ends covers it)
+            float s0 = 0.0f, s1 = B.w;
+            for (uint32_t k = lane & 15; k < cr.y; k += 16) {
+                const uint32_t j = items[cr.x + k];
+                if (j >= S) continue;
+                const float4 Q = bs[j];
+                const float wx = Q.x - A.x, wy = Q.y - A.y, wz = Q.z - A.z;
+                const float sc = wx * B.x + wy * B.y + wz * B.z;
+                const float ex = wx - sc * B.x, ey = wy - sc * B.y, ez = wz - sc * B.z;
+                const float h = sqrtf(ex * ex + ey * ey + ez * ez) + A.w, R = 0.999f * Q.w;
+                if (h >= R) continue;
+                const float half = sqrtf(R * R - h * h);
+                if (sc - half <= 0.0f) s0 = fmaxf(s0, sc + half);
+                if (sc + half >= B.w) s1 = fminf(s1, sc - half);
+            }
+            s0 = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(s0)));  // non-negative: ordered
+            s1 = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(fmaxf(s1, 0.0f))));
+            if (s0 >= s1) {
+                s.w = 0.0f;
+            } else if (s0 > 0.0f || s1 < B.w) {
+                const float m = 0.5f * (s0 + s1), hl = 0.5f * (s1 - s0);
+                const float mag = fmaxf(fmaxf(fabsf(A.x), fabsf(A.y)), fabsf(A.z)) + B.w;
+                s = make_float4(A.x + m * B.x, A.y + m * B.y, A.z + m * B.z,
+                                -(1.0001f * sqrtf(hl * hl + A.w * A.w) + 1e-6f * mag));
+            }
         }
-        it[b] = v;
+        if (!tube || lane == 0) {
+            balls[bstart[c] + atomicAdd(bcursor + c, 1u)] = s;
+            balls[N + id] = s;
+        }
     }
 }
 
@@ -328,6 +401,7 @@ __global__ void __launch_bounds__(SCAN_T) k_scan_reduce(const uint32_t* in, int6
     if (threadIdx.x == 0) sums[blockIdx.x] = tot;
 }
 
+// Block sums -> exclusive prefixes (only when there are more than SCAN_T).
 __global__ void __launch_bounds__(SCAN_T) k_scan_sums(unsigned long long* sums, int64_t nb, unsigned long long* total) {
     int64_t per = (nb + SCAN_T - 1) / SCAN_T;
     int64_t b0 = (int64_t)threadIdx.x * per;
@@ -343,8 +417,43 @@ __global__ void __launch_bounds__(SCAN_T) k_scan_sums(unsigned long long* sums, 
     if (threadIdx.x == 0) *total = tot;
 }
 
-__global__ void __launch_bounds__(SCAN_T) k_scan_apply(const uint32_t* in, int64_t n, const unsigned long long* offs,
-                                                        uint2* cells) {
+// Last step of the scan. Words [0, nc) of `in` are the cells' counts; those
+// from nc on are the halved grid's (N objects in all, counted after the cells'
+// references) and become starts. The words are zeroed: they are the scatter
+// passes' cursors next. Up to SCAN_T block sums every CTA adds up for itself
+// (one kernel less in the chain); above that k_scan_sums has been run.
+// A device-side rebuild (geom not null) finishes here too: bounding sphere,
+// reference count; one that outgrew its item buffer disables the grid (renders
+// then see no objects) and flags the context's error word.
+struct ScanOut {
+    uint2* cells;
+    int64_t nc;
+    uint32_t* bstart;
+    unsigned long long* total;  // references + N
+    int64_t N;
+    GridDev* geom;
+    const BuildAux* aux;
+    unsigned long long items_cap;
+    GridStat* stat;
+    uint32_t* err;
+};
+__device__ void grid_finish(const ScanOut& o, unsigned long long refs);
+__global__ void __launch_bounds__(SCAN_T) k_scan_apply(uint32_t* in, int64_t n, const unsigned long long* sums,
+                                                        int64_t nb, ScanOut o) {
+    __shared__ unsigned long long before_s;
+    unsigned long long before, all;
+    if (nb <= SCAN_T) {
+        const unsigned long long mine = threadIdx.x < nb ? sums[threadIdx.x] : 0ull;
+        const unsigned long long ex = block_exclusive_scan(mine, all);
+        if (threadIdx.x == blockIdx.x) before_s = ex;
+        __syncthreads();
+        before = before_s;
+        if (blockIdx.x == 0 && threadIdx.x == 0) *o.total = all;
+    } else {
+        before = sums[blockIdx.x];
+        all = *o.total;
+    }
+    const unsigned long long refs = all - (unsigned long long)o.N;
     int64_t base = (int64_t)blockIdx.x * SCAN_TILE + (int64_t)threadIdx.x * SCAN_PER;
     uint32_t v[SCAN_PER];
     unsigned long long s = 0;
@@ -353,11 +462,14 @@ __global__ void __launch_bounds__(SCAN_T) k_scan_apply(const uint32_t* in, int64
         s += v[k];
     }
     unsigned long long tot;
-    unsigned long long run = offs[blockIdx.x] + block_exclusive_scan(s, tot);
+    unsigned long long run = before + block_exclusive_scan(s, tot);
     for (int k = 0; k < SCAN_PER; ++k) {
-        if (base + k < n) cells[base + k] = make_uint2((uint32_t)run, v[k]);
+        if (base + k < n) in[base + k] = 0u;
+        if (base + k < o.nc) o.cells[base + k] = make_uint2((uint32_t)run, v[k]);
+        else if (base + k < n) o.bstart[base + k - o.nc] = (uint32_t)(run - refs);
         run += v[k];
     }
+    if (o.geom && blockIdx.x == 0 && threadIdx.x == 0) grid_finish(o, refs);
 }
 
 // ---------------------------------------------------------------- host side
@@ -390,16 +502,55 @@ static bool host_scene_valid(const float* sph, int64_t S, const float* cyl, int6
     return true;
 }
 
-void scene_release(Scene* s) {
-    cudaFree(s->obj);
-    cudaFree(s->obj64);
-    cudaFree(s->bs);
-    cudaFree(s->color);
-    cudaFree(s->palette);
-    cudaFree(s->aabb);
-    cudaFree(s->d_box);
+void pool_create(Ctx* ctx) {
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = ctx->device;
+    unsigned long long keep = 64ull << 20;
+    if (cudaMemPoolCreate(&ctx->pool, &props) != cudaSuccess) {
+        ctx->pool = nullptr;
+        (void)cudaGetLastError();
+        return;
+    }
+    cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep);
+}
+
+cudaError_t block_alloc(Ctx* ctx, void** p, size_t bytes) {
+    if (!ctx->pool) return cudaMalloc(p, bytes);
+    return cudaMallocFromPoolAsync(p, bytes, ctx->pool, ctx->stream);
+}
+
+void block_free(Ctx* ctx, void* p) {
+    if (!p) return;
+    if (!ctx->pool) {
+        cudaFree(p);
+        return;
+    }
+    cudaDeviceSynchronize();
+    if (cudaFreeAsync(p, ctx->stream) != cudaSuccess) {
+        // not from a pool (another context's plain allocation)
+        (void)cudaGetLastError();
+        cudaFree(p);
+    }
+}
+
+void scene_release(Ctx* ctx, Scene* s) {
+    block_free(ctx, s->mem);
     cudaFree(s->d_in);
     *s = Scene();
+}
+
+// A scene's arrays, cut from one allocation.
+static void scene_arrays(Scene* s, Carve& c) {
+    const int64_t N = s->S + s->C;
+    s->obj = c.take<float4>(2 * N);
+    s->obj64 = c.take<double2>(4 * N);
+    s->bs = c.take<float4>(N);
+    s->aabb = c.take<float4>(2 * N);
+    s->color = c.take<uint32_t>(N);
+    s->palette = c.take<float>(3 * (int64_t)s->K);
+    s->d_box = c.take<uint32_t>(8);
 }
 
 int scene_upload(Ctx* ctx, const float* spheres, int64_t S, const float* cyl, int64_t C, const uint32_t* color,
@@ -419,23 +570,24 @@ int scene_upload(Ctx* ctx, const float* spheres, int64_t S, const float* cyl, in
     s->K = K;
     {
         const size_t nN = (size_t)std::max<int64_t>(N, 1);
-        GB_TRY(cudaMalloc(&s->obj, 2 * nN * sizeof(float4)));
-        GB_TRY(cudaMalloc(&s->obj64, 4 * nN * sizeof(double2)));
-        GB_TRY(cudaMalloc(&s->bs, nN * sizeof(float4)));
-        GB_TRY(cudaMalloc(&s->color, nN * sizeof(uint32_t)));
-        GB_TRY(cudaMalloc(&s->palette, (size_t)std::max(K, 1) * 3 * sizeof(float)));
-        GB_TRY(cudaMalloc(&s->aabb, 2 * nN * sizeof(float4)));
-        GB_TRY(cudaMalloc(&d_box, 8 * sizeof(uint32_t)));
+        Carve size, cut;
+        scene_arrays(s, size);
+        GB_TRY(block_alloc(ctx, &s->mem, size.size));
+        cut.base = (char*)s->mem;
+        scene_arrays(s, cut);
+        d_box = s->d_box;
         s->bytes = nN * (3 * sizeof(float4) + 4 * sizeof(double2) + sizeof(uint32_t) + 2 * sizeof(float4)) +
                    (size_t)std::max(K, 1) * 3 * sizeof(float);
         if (host) {
+            if ((rc = grow(ctx, &ctx->d_build, &ctx->build_cap, (size_t)(4 * S + 7 * C) * sizeof(float))) != GBRT_OK)
+                goto fail;
+            d_sph_in = (float*)ctx->d_build;
+            d_cyl_in = d_sph_in + 4 * S;
             if (S > 0) {
-                GB_TRY(cudaMalloc(&d_sph_in, (size_t)S * 4 * sizeof(float)));
                 GB_TRY(cudaMemcpyAsync(d_sph_in, spheres, (size_t)S * 4 * sizeof(float), cudaMemcpyHostToDevice,
                                        ctx->stream));
             }
             if (C > 0) {
-                GB_TRY(cudaMalloc(&d_cyl_in, (size_t)C * 7 * sizeof(float)));
                 GB_TRY(cudaMemcpyAsync(d_cyl_in, cyl, (size_t)C * 7 * sizeof(float), cudaMemcpyHostToDevice,
                                        ctx->stream));
             }
@@ -481,31 +633,20 @@ int scene_upload(Ctx* ctx, const float* spheres, int64_t S, const float* cyl, in
             s->lo[k] = N > 0 ? float_of_ord(h_box[k]) : 0.0f;
             s->hi[k] = N > 0 ? float_of_ord(h_box[3 + k]) : 0.0f;
         }
+        memcpy(&s->rmax, &h_box[7], 4);
     }
-    if (host) {
-        cudaFree(d_sph_in);
-        cudaFree(d_cyl_in);
-    }
-    s->d_box = d_box;  // kept: device-side rebuilds read the box from here
     return GBRT_OK;
 fail:
     cudaStreamSynchronize(ctx->stream);
-    if (host) {
-        cudaFree(d_sph_in);
-        cudaFree(d_cyl_in);
-    }
-    cudaFree(d_box);
-    scene_release(s);
+    scene_release(ctx, s);
     return rc;
 }
 
-void grid_release(Grid* g) {
-    cudaFree(g->cells);
-    cudaFree(g->items);
+void grid_release(Ctx* ctx, Grid* g) {
+    block_free(ctx, g->mem);
+    block_free(ctx, g->items);
     cudaFree(g->d_geom);
     cudaFree(g->d_aux);
-    cudaFree(g->d_counts);
-    cudaFree(g->d_sums);
     cudaFree(g->d_reach);
     cudaFree(g->d_stat);
     cudaFreeHost(g->h_stat);
@@ -537,10 +678,12 @@ __host__ __device__ inline int64_t grid_dims(const double E[3], double kk, int32
     return nc;
 }
 
+constexpr float NEAR_REACH = 2.0f;
+
 // Fill the grid geometry (GridDev fields, build parameters, bounding-sphere
 // centre) from the padded scene box; `cells_cap` > 0 caps the cell count.
-__host__ __device__ inline void grid_geometry(const float slo[3], const float shi[3], int64_t N, float lambda,
-                                              int64_t cells_cap, GridDev& d, BuildAux& a) {
+__host__ __device__ inline void grid_geometry(const float slo[3], const float shi[3], float rmax, int64_t N,
+                                              float lambda, int64_t cells_cap, GridDev& d, BuildAux& a) {
     float emax = fmaxf(shi[0] - slo[0], fmaxf(shi[1] - slo[1], shi[2] - slo[2]));
     float pad = 1e-5f * fmaxf(emax, 1.0f);
     double E[3], V = 1.0;
@@ -551,7 +694,8 @@ __host__ __device__ inline void grid_geometry(const float slo[3], const float sh
         V *= E[k];
     }
     double target = fmin(fmax((double)lambda * (double)N, 1.0), 67108864.0);
-    double kk = cbrt(target / V);
+    const double kk0 = cbrt(target / V);
+    double kk = kk0;
     d.ncells = grid_dims(E, kk, d.n);
     for (int it = 0; cells_cap > 0 && d.ncells > cells_cap && it < 64; ++it) {
         kk *= 0.98 * cbrt((double)cells_cap / (double)d.ncells);
@@ -579,6 +723,15 @@ __host__ __device__ inline void grid_geometry(const float slo[3], const float sh
     a.rbits = 0u;
     a.pad = 0u;
     d.empty = N == 0 ? 1 : 0;
+    for (int k = 0; k < 3; ++k) d.bn[k] = (d.n[k] + 1) / 2;
+    d.nballs = (int32_t)(N < 0x7fffffff ? N : 0);
+    // the near pass looks NEAR_REACH mean object distances far; scenes with
+    // objects larger than that reach (its candidate boxes would be mostly
+    // margin) do without it
+    d.rmax = rmax;
+    d.density = (float)((double)N / V);
+    d.rho = NEAR_REACH * cbrtf((float)(target / (double)(N > 0 ? N : 1))) / (float)kk0;
+    if (d.nballs == 0 || !(rmax <= d.rho)) d.rho = 0.0f;
 }
 
 // Bounding sphere from its centre and the reduced radius bits.
@@ -601,7 +754,8 @@ __device__ __forceinline__ float float_of_ord_dev(uint32_t o) {
 
 // Device-side rebuild, step 1 (one thread): geometry from the current scene box.
 __global__ void k_grid_geometry(const uint32_t* box, int64_t N, float lambda, int64_t cells_cap, const uint2* cells,
-                                const uint32_t* items, int64_t items_cap, GridDev* geom, BuildAux* aux) {
+                                const uint32_t* items, int64_t items_cap, const float4* balls,
+                                const uint32_t* bstart, GridDev* geom, BuildAux* aux) {
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     float lo[3], hi[3];
     for (int k = 0; k < 3; ++k) {
@@ -610,7 +764,10 @@ __global__ void k_grid_geometry(const uint32_t* box, int64_t N, float lambda, in
     }
     GridDev d = *geom;
     BuildAux a;
-    grid_geometry(lo, hi, N, lambda, cells_cap, d, a);
+    grid_geometry(lo, hi, __uint_as_float(box[7]), N, lambda, cells_cap, d, a);
+    d.balls = balls;
+    d.cut = balls + N;
+    d.bstart = bstart;
     d.cells = cells;
     d.items = items;
     d.nitems = items_cap;
@@ -618,25 +775,29 @@ __global__ void k_grid_geometry(const uint32_t* box, int64_t N, float lambda, in
     *aux = a;
 }
 
-// Device-side rebuild, last step (one thread): bounding sphere, reference
-// count; a rebuild that outgrew its item buffer disables the grid (renders
-// then see no objects) and flags the context's error word.
-__global__ void k_grid_finish(GridDev* geom, const BuildAux* aux, const unsigned long long* total,
-                              unsigned long long items_cap, GridStat* stat, uint32_t* err) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    GridDev d = *geom;
-    grid_bound_sphere(*aux, d);
-    const unsigned long long refs = *total;
-    const unsigned int over = refs > items_cap ? 1u : 0u;
+__device__ void grid_finish(const ScanOut& o, unsigned long long refs) {
+    GridDev d = *o.geom;
+    grid_bound_sphere(*o.aux, d);
+    const unsigned int over = refs > o.items_cap ? 1u : 0u;
     if (over) {
         d.empty = 1;
-        atomicOr(err, ERR_GRID_CAPACITY);
+        atomicOr(o.err, ERR_GRID_CAPACITY);
     }
-    *geom = d;
-    stat->refs = refs;
-    stat->ncells = (unsigned long long)d.ncells;
-    stat->overflow = over;
-    stat->pad = 0u;
+    *o.geom = d;
+    o.stat->refs = refs;
+    o.stat->ncells = (unsigned long long)d.ncells;
+    o.stat->overflow = over;
+    o.stat->pad = 0u;
+}
+
+// The scan passes on `st`: counts [0, n) -> o.cells, o.bstart; returns the
+// kernels launched.
+static int launch_scan(uint32_t* counts, int64_t n, unsigned long long* sums, const ScanOut& o, cudaStream_t st) {
+    const int64_t nb = (n + SCAN_TILE - 1) / SCAN_TILE;
+    k_scan_reduce<<<(int)nb, SCAN_T, 0, st>>>(counts, n, sums);
+    if (nb > SCAN_T) k_scan_sums<<<1, SCAN_T, 0, st>>>(sums, nb, o.total);
+    k_scan_apply<<<(int)nb, SCAN_T, 0, st>>>(counts, n, sums, nb, o);
+    return nb > SCAN_T ? 3 : 2;
 }
 
 int grid_build(Ctx* ctx, const Scene* s, float lambda, Grid* g) {
@@ -659,66 +820,88 @@ int grid_build(Ctx* ctx, const Scene* s, float lambda, Grid* g) {
     }
     {
         BuildAux a;
-        grid_geometry(s->lo, s->hi, N, lambda, 0, d, a);
+        grid_geometry(s->lo, s->hi, s->rmax, N, lambda, 0, d, a);
         const int64_t nc = d.ncells;
-        GB_TRY(cudaMalloc(&g->cells, (size_t)nc * sizeof(uint2)));
-        GB_TRY(cudaMalloc(&counts, (size_t)nc * sizeof(uint32_t)));
-        GB_TRY(cudaMalloc(&reach, (size_t)std::max<int64_t>(N, 1) * sizeof(unsigned long long)));
-        GB_TRY(cudaMemsetAsync(counts, 0, (size_t)nc * sizeof(uint32_t), ctx->stream));
-        const int64_t nb = (nc + SCAN_TILE - 1) / SCAN_TILE;
-        // sums: nb block sums, total, then the build parameters
-        GB_TRY(cudaMalloc(&sums, (size_t)(nb + 2) * sizeof(unsigned long long) + sizeof(BuildAux)));
-        BuildAux* d_aux = (BuildAux*)(sums + nb + 2);
+        // the counts of the cells, then of the halved grid's cells and one more
+        const int64_t nbc = (int64_t)d.bn[0] * d.bn[1] * d.bn[2] + 1, nall = nc + nbc;
+        const int64_t nb = (nall + SCAN_TILE - 1) / SCAN_TILE;
+        Carve size, cut;
+        auto arrays = [&](Carve& c) {
+            g->cells = c.take<uint2>(nc);
+            g->balls = c.take<float4>(2 * N);
+            g->bstart = c.take<uint32_t>(nbc);
+        };
+        arrays(size);
+        GB_TRY(block_alloc(ctx, &g->mem, size.size));
+        cut.base = (char*)g->mem;
+        arrays(cut);
+        // temporaries: counts (then fill cursors), reached cells, block sums
+        // and their total, build parameters
+        BuildAux* d_aux = nullptr;
+        auto temporaries = [&](Carve& c) {
+            counts = c.take<uint32_t>(nall);
+            reach = c.take<unsigned long long>(N);
+            sums = c.take<unsigned long long>(nb + 1);
+            d_aux = c.take<BuildAux>(1);
+        };
+        Carve tsize, tcut;
+        temporaries(tsize);
+        if ((rc = grow(ctx, &ctx->d_build, &ctx->build_cap, tsize.size)) != GBRT_OK) goto fail;
+        tcut.base = (char*)ctx->d_build;
+        temporaries(tcut);
+        GB_TRY(cudaMemsetAsync(counts, 0, (size_t)nall * sizeof(uint32_t), ctx->stream));
         GB_TRY(cudaMemcpyAsync(d_aux, &a, sizeof(a), cudaMemcpyHostToDevice, ctx->stream));
         if (N > 0) {
-            k_grid_count<<<object_warp_blocks(N), 256, 0, ctx->stream>>>(s->aabb, s->obj, N, &d_aux->p, counts,
-                                                                          reach);
-            k_bound_radius<<<(int)((N + 255) / 256), 256, 0, ctx->stream>>>(s->obj64, N, d_aux->ctr, &d_aux->rbits);
-            ctx->launches += 2;
+            const unsigned int cb = (unsigned int)object_warp_blocks(N);
+            k_grid_count<<<cb + radius_blocks(N), 256, 0, ctx->stream>>>(s->aabb, s->obj, s->obj64, s->bs, N, d_aux, counts,
+                                                                         counts + nc, reach, cb);
+            ctx->launches++;
             GB_TRY(cudaGetLastError());
         }
-        k_scan_reduce<<<(int)nb, SCAN_T, 0, ctx->stream>>>(counts, nc, sums);
-        k_scan_sums<<<1, SCAN_T, 0, ctx->stream>>>(sums, nb, sums + nb);
-        k_scan_apply<<<(int)nb, SCAN_T, 0, ctx->stream>>>(counts, nc, sums, g->cells);
-        ctx->launches += 3;
+        ScanOut so = {};
+        so.cells = g->cells;
+        so.nc = nc;
+        so.bstart = g->bstart;
+        so.total = sums + nb;
+        so.N = N;
+        ctx->launches += launch_scan(counts, nall, sums, so, ctx->stream);
         GB_TRY(cudaGetLastError());
         GB_TRY(cudaMemcpyAsync(&h_total, sums + nb, sizeof(h_total), cudaMemcpyDeviceToHost, ctx->stream));
         GB_TRY(cudaMemcpyAsync(&a.rbits, &d_aux->rbits, sizeof(a.rbits), cudaMemcpyDeviceToHost, ctx->stream));
         GB_TRY(cudaStreamSynchronize(ctx->stream));
         grid_bound_sphere(a, d);
+        h_total -= (unsigned long long)N;
         if (h_total >= 0xFFFFFFFFull) {
             rc = GBRT_ENOMEM;
             goto fail;
         }
         g->refs = (int64_t)h_total;
-        GB_TRY(cudaMalloc(&g->items, (size_t)std::max<int64_t>(g->refs, 1) * sizeof(uint32_t)));
+        GB_TRY(block_alloc(ctx, (void**)&g->items, (size_t)std::max<int64_t>(g->refs, 1) * sizeof(uint32_t)));
         if (N > 0) {
-            cursor = counts;  // reuse as per-cell fill cursor
-            GB_TRY(cudaMemsetAsync(cursor, 0, (size_t)nc * sizeof(uint32_t), ctx->stream));
+            cursor = counts;  // zeroed by the scan: the fill cursors
             k_grid_scatter<<<object_warp_blocks(N), 256, 0, ctx->stream>>>(s->aabb, s->obj, N, &d_aux->p, reach,
                                                                             g->cells,
                                                                             cursor, g->items, (uint64_t)g->refs);
-            k_cell_sort<<<(int)((nc + 255) / 256), 256, 0, ctx->stream>>>(g->cells, nc, g->items,
-                                                                          (uint64_t)g->refs);
+            k_ball_sort<<<ball_sort_blocks(s->S, s->C), 256, 0, ctx->stream>>>(s->obj, s->bs, s->S, N, &d_aux->p,
+                                                                               g->cells, g->items, (uint64_t)g->refs,
+                                                                               g->bstart, cursor + nc, g->balls);
             ctx->launches += 2;
             GB_TRY(cudaGetLastError());
         }
         GB_TRY(cudaStreamSynchronize(ctx->stream));
         d.cells = g->cells;
         d.items = g->items;
+        d.balls = g->balls;
+        d.cut = g->balls + N;
+        d.bstart = g->bstart;
         d.nitems = std::max<int64_t>(g->refs, 1);
-        g->bytes = (size_t)nc * sizeof(uint2) + (size_t)std::max<int64_t>(g->refs, 1) * sizeof(uint32_t);
+        g->bytes = (size_t)nc * sizeof(uint2) + (size_t)std::max<int64_t>(g->refs, 1) * sizeof(uint32_t) +
+                   (size_t)nbc * sizeof(uint32_t) + 2 * (size_t)std::max<int64_t>(N, 1) * sizeof(float4);
     }
-    cudaFree(counts);
-    cudaFree(reach);
-    cudaFree(sums);
     return GBRT_OK;
 fail:
     cudaStreamSynchronize(ctx->stream);
-    cudaFree(counts);
-    cudaFree(reach);
-    cudaFree(sums);
-    grid_release(g);
+    grid_release(ctx, g);
     return rc;
 }
 
@@ -735,6 +918,7 @@ int scene_refresh_host(Scene* s, cudaStream_t stream) {
         s->lo[k] = N > 0 ? float_of_ord(h_box[k]) : 0.0f;
         s->hi[k] = N > 0 ? float_of_ord(h_box[3 + k]) : 0.0f;
     }
+    memcpy(&s->rmax, &h_box[7], 4);
     s->box_stale = false;
     return h_box[6] ? GBRT_EINVAL : GBRT_OK;
 }
@@ -778,35 +962,50 @@ int scene_update(Ctx* ctx, Scene* s, const float* spheres, const float* cyl, int
 // Buffers of a device-side rebuild: cells, counts and scan sums for cells_cap,
 // items for items_cap. All or nothing: on failure the grid keeps its previous
 // buffers (and stays usable); the caller has drained the stream.
-static int dyn_alloc(Grid* g, int64_t cells_cap, int64_t items_cap) {
-    const int64_t nb = (cells_cap + SCAN_TILE - 1) / SCAN_TILE;
-    uint2* cells = nullptr;
+static int dyn_alloc(Ctx* ctx, Grid* g, int64_t cells_cap, int64_t items_cap) {
+    // counts and starts: the cells', then the halved grid's (never more cells
+    // than the grid itself) and one more
+    const int64_t nall = 2 * cells_cap + 1;
+    const int64_t nb = (nall + SCAN_TILE - 1) / SCAN_TILE;
+    void* mem = nullptr;
     uint32_t* items = nullptr;
-    uint32_t* counts = nullptr;
-    unsigned long long* sums = nullptr;
-    if (cudaMalloc(&cells, (size_t)cells_cap * sizeof(uint2)) != cudaSuccess ||
-        cudaMalloc(&items, (size_t)items_cap * sizeof(uint32_t)) != cudaSuccess ||
-        cudaMalloc(&counts, (size_t)cells_cap * sizeof(uint32_t)) != cudaSuccess ||
-        cudaMalloc(&sums, (size_t)(nb + 2) * sizeof(unsigned long long)) != cudaSuccess) {
-        cudaFree(cells);
-        cudaFree(items);
-        cudaFree(counts);
-        cudaFree(sums);
+    auto arrays = [&](Carve& c) {
+        uint2* cells = c.take<uint2>(cells_cap);
+        float4* balls = c.take<float4>(2 * g->N);
+        uint32_t* bstart = c.take<uint32_t>(cells_cap + 1);
+        uint32_t* counts = c.take<uint32_t>(nall);
+        unsigned long long* sums = c.take<unsigned long long>(nb + 1);
+        if (c.base) {
+            g->cells = cells;
+            g->balls = balls;
+            g->bstart = bstart;
+            g->d_counts = counts;
+            g->d_sums = sums;
+        }
+    };
+    Carve size, cut;
+    arrays(size);
+    if (block_alloc(ctx, &mem, size.size) != cudaSuccess ||
+        block_alloc(ctx, (void**)&items, (size_t)items_cap * sizeof(uint32_t)) != cudaSuccess) {
+        (void)cudaGetLastError();
+        block_free(ctx, mem);
         return GBRT_ENOMEM;
     }
-    cudaFree(g->cells);
-    cudaFree(g->items);
-    cudaFree(g->d_counts);
-    cudaFree(g->d_sums);
-    g->cells = cells;
+    block_free(ctx, g->mem);
+    block_free(ctx, g->items);
+    g->mem = mem;
     g->items = items;
-    g->d_counts = counts;
-    g->d_sums = sums;
+    cut.base = (char*)mem;
+    arrays(cut);
     g->cells_cap = cells_cap;
     g->items_cap = items_cap;
-    g->bytes = (size_t)cells_cap * (sizeof(uint2) + sizeof(uint32_t)) + (size_t)items_cap * sizeof(uint32_t);
+    g->bytes = (size_t)cells_cap * (sizeof(uint2) + 3 * sizeof(uint32_t)) + (size_t)items_cap * sizeof(uint32_t) +
+               2 * (size_t)g->N * sizeof(float4);
     g->dev.cells = g->cells;
     g->dev.items = g->items;
+    g->dev.balls = g->balls;
+    g->dev.cut = g->balls + g->N;
+    g->dev.bstart = g->bstart;
     g->dev.nitems = items_cap;
     return GBRT_OK;
 }
@@ -830,7 +1029,7 @@ int grid_rebuild(Ctx* ctx, const Scene* s, Grid* g) {
         const int64_t target = (int64_t)std::min(std::max((double)g->lambda * (double)N, 1.0), 67108864.0);
         const int64_t cells_cap = std::max<int64_t>(g->dev.ncells, target + target / 2) + 4096;
         const int64_t items_cap = std::max<int64_t>(g->refs + g->refs / 2, 4096);
-        if ((rc = dyn_alloc(g, cells_cap, items_cap)) != GBRT_OK) return rc;
+        if ((rc = dyn_alloc(ctx, g, cells_cap, items_cap)) != GBRT_OK) return rc;
         if (cudaMemcpy(g->d_geom, &g->dev, sizeof(GridDev), cudaMemcpyHostToDevice) != cudaSuccess) {
             // the new buffers hold no lists yet: leave the grid unusable (renders
             // reject it) until a rebuild succeeds
@@ -849,35 +1048,45 @@ int grid_rebuild(Ctx* ctx, const Scene* s, Grid* g) {
             cudaStreamSynchronize(ctx->stream);
             const int64_t items_cap = (int64_t)st.refs + (int64_t)st.refs / 2 + 4096;
             if (items_cap >= (int64_t)0xFFFFFFFFll) return GBRT_ENOMEM;
-            if ((rc = dyn_alloc(g, g->cells_cap, items_cap)) != GBRT_OK) return rc;
+            if ((rc = dyn_alloc(ctx, g, g->cells_cap, items_cap)) != GBRT_OK) return rc;
         }
     }
     g->stream = ctx->stream;
     cudaStream_t st = ctx->stream;
     const int64_t nc = g->cells_cap;
-    const int64_t nb = (nc + SCAN_TILE - 1) / SCAN_TILE;
-    const int blocksN = (int)((std::max<int64_t>(N, 1) + 255) / 256);
-    if (cudaMemsetAsync(g->d_counts, 0, (size_t)nc * sizeof(uint32_t), st) != cudaSuccess) return GBRT_EDEVICE;
-    k_grid_geometry<<<1, 32, 0, st>>>(s->d_box, N, g->lambda, nc, g->cells, g->items, g->items_cap, g->d_geom,
-                                      g->d_aux);
+    const int64_t nall = 2 * nc + 1;
+    const int64_t nb = (nall + SCAN_TILE - 1) / SCAN_TILE;
+    if (cudaMemsetAsync(g->d_counts, 0, (size_t)nall * sizeof(uint32_t), st) != cudaSuccess) return GBRT_EDEVICE;
+    k_grid_geometry<<<1, 32, 0, st>>>(s->d_box, N, g->lambda, nc, g->cells, g->items, g->items_cap, g->balls, g->bstart,
+                                      g->d_geom, g->d_aux);
     if (N > 0) {
-        k_grid_count<<<object_warp_blocks(N), 256, 0, st>>>(s->aabb, s->obj, N, &g->d_aux->p, g->d_counts, g->d_reach);
-        k_bound_radius<<<blocksN, 256, 0, st>>>(s->obj64, N, g->d_aux->ctr, &g->d_aux->rbits);
+        const unsigned int cb = (unsigned int)object_warp_blocks(N);
+        k_grid_count<<<cb + radius_blocks(N), 256, 0, st>>>(s->aabb, s->obj, s->obj64, s->bs, N, g->d_aux, g->d_counts,
+                                                            g->d_counts + nc, g->d_reach, cb);
     }
-    k_scan_reduce<<<(int)nb, SCAN_T, 0, st>>>(g->d_counts, nc, g->d_sums);
-    k_scan_sums<<<1, SCAN_T, 0, st>>>(g->d_sums, nb, g->d_sums + nb);
-    k_scan_apply<<<(int)nb, SCAN_T, 0, st>>>(g->d_counts, nc, g->d_sums, g->cells);
+    ScanOut so = {};
+    so.cells = g->cells;
+    so.nc = nc;
+    so.bstart = g->bstart;
+    so.total = g->d_sums + nb;
+    so.N = N;
+    so.geom = g->d_geom;
+    so.aux = g->d_aux;
+    so.items_cap = (unsigned long long)g->items_cap;
+    so.stat = g->d_stat;
+    so.err = ctx->d_err;
+    const int scans = launch_scan(g->d_counts, nall, g->d_sums, so, st);
     if (N > 0) {
-        if (cudaMemsetAsync(g->d_counts, 0, (size_t)nc * sizeof(uint32_t), st) != cudaSuccess) return GBRT_EDEVICE;
         k_grid_scatter<<<object_warp_blocks(N), 256, 0, st>>>(s->aabb, s->obj, N, &g->d_aux->p, g->d_reach, g->cells, g->d_counts,
                                                 g->items,
                                                 (uint64_t)g->items_cap);
+        k_ball_sort<<<ball_sort_blocks(s->S, s->C), 256, 0, st>>>(s->obj, s->bs, s->S, N, &g->d_aux->p, g->cells,
+                                                                  g->items, (uint64_t)g->items_cap, g->bstart,
+                                                                  g->d_counts + nc, g->balls);
         // no per-cell sort: no result depends on the order of a cell's ids
         // (nearest hits rank by (t, id), any-hit queries OR their tests)
     }
-    k_grid_finish<<<1, 32, 0, st>>>(g->d_geom, g->d_aux, g->d_sums + nb, (unsigned long long)g->items_cap, g->d_stat,
-                                    ctx->d_err);
-    ctx->launches += N > 0 ? 8 : 5;
+    ctx->launches += scans + (N > 0 ? 4 : 1);
     if (cudaGetLastError() != cudaSuccess) return GBRT_EDEVICE;
     if (cudaMemcpyAsync(g->h_stat, g->d_stat, sizeof(GridStat), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaEventRecord(g->stat_ev, st) != cudaSuccess)
