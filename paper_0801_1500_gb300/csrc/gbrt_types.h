@@ -158,7 +158,8 @@ struct TileRec {
 //   vis       escaped AO samples per hit slot
 //   lmask     per hit slot, bit l set when the shadow ray toward light l escaped
 //   queue     [0] next primary work item, [1] next AO ray (or unit), [2] next
-//             tile of the near pass
+//             tile of the near pass, [3] finished CTAs of the primary pass, then
+//             the number of rays an AO warp claims at once
 // With a near pass (tiles not null):
 //   tiles     records of the work items with hits
 //   ntiles    their number
@@ -187,6 +188,8 @@ struct BatchDev {
     int32_t nframes;
     int32_t tile_w, tile_h;
     int32_t refill;
+    int32_t ao_warps;  // warps of the AO walk
+    int32_t pad;
 };
 
 }  // namespace gbrt

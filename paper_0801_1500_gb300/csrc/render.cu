@@ -496,6 +496,16 @@ __device__ __forceinline__ double ao_maxdist<double>(const FrameDev& f) { return
 
 // ---------------------------------------------------------------- primary pass
 
+// AO rays a warp claims from the global queue at once (its local pool): 64, and
+// fewer, down to 8, where 64 would leave warps without any. A small frame's AO
+// pass is one round of such claims, bound by the latency of one warp's rays:
+// 41 -> 30 us at 256 x 256, 4 samples; 33 -> 21 us at 128 x 96; FP64, 256 x 256
+// at 8: 105 -> 88 us (64 at once against this).
+__device__ __forceinline__ unsigned ao_claim(unsigned long long rays, int warps) {
+    const unsigned long long share = rays / (unsigned)warps + 1ull;
+    return share >= 64ull ? 64u : share <= 8ull ? 8u : (unsigned)(share + 7ull) & ~7u;
+}
+
 // Prefix sums of hits and AO rays per frame; resets the AO and shading queues.
 // Run by one thread of the primary pass's last CTA once every CTA's hits are
 // counted (the counts are read through L2: other CTAs added them atomically).
@@ -512,6 +522,7 @@ __device__ __forceinline__ void ao_plan(const BatchDev& b) {
     }
     b.queue[1] = 0;
     b.queue[2] = 0;
+    b.queue[3] = ao_claim(jobs, b.ao_warps);
 }
 
 
@@ -677,9 +688,6 @@ __device__ __forceinline__ void ao_escape(const BatchDev& b, int64_t vslot, uint
     if (lbit) atomicOr(b.lmask + vslot, lbit);
     else atomicAdd(b.vis + vslot, 1u);
 }
-
-// AO rays a warp claims from the global queue at once (its local pool)
-constexpr unsigned AO_CLAIM = 64;
 
 // ---- near pass
 
@@ -1243,8 +1251,8 @@ __global__ void __launch_bounds__(256) k_ao_walk(const __grid_constant__ BatchDe
     unsigned long long pool = 0, pool_end = 0;
     while (true) {
         // 1. compaction of rays: idle lanes take the next rays together, from
-        //    the warp's pool, which claims AO_CLAIM more rays from the global
-        //    queue when it runs short (one atomic per AO_CLAIM rays)
+        //    the warp's pool, which claims ao_claim more rays from the global
+        //    queue when it runs short
         const unsigned act = __ballot_sync(FULL, has);
         if (!exhausted && __popc(act) < refill) {
             const unsigned idle = ~act;
@@ -1294,13 +1302,16 @@ __global__ void __launch_bounds__(256) k_ao_walk(const __grid_constant__ BatchDe
             } else {
                 const unsigned long long rem = pool_end - pool;
                 unsigned long long fresh_base = 0;
+                unsigned claim = 0;
                 if (rem < need) {
-                    if (lane == 0) fresh_base = atomicAdd(b.queue + 1, (unsigned long long)AO_CLAIM);
+                    claim = (unsigned)b.queue[3];
+                    if (lane == 0) fresh_base = atomicAdd(b.queue + 1, (unsigned long long)claim);
                     fresh_base = __shfl_sync(FULL, fresh_base, 0);
                     if (fresh_base >= total) exhausted = true;
                 }
-                if (!has) {
-                    const unsigned i = __popc(idle & lt);
+                const unsigned n = rem + claim < need ? (unsigned)rem + claim : need;
+                const unsigned i = __popc(idle & lt);
+                if (!has && i < n) {
                     const unsigned long long jj = i < rem ? pool + i : fresh_base + (i - rem);
                     if (jj < total) {
                         const int f = b.nframes == 1 ? 0 : find_frame(b.job_off, b.nframes, jj);
@@ -1314,8 +1325,8 @@ __global__ void __launch_bounds__(256) k_ao_walk(const __grid_constant__ BatchDe
                 if (rem >= need) {
                     pool += need;
                 } else {
-                    pool = fresh_base + (need - rem);
-                    pool_end = fresh_base + AO_CLAIM;
+                    pool = fresh_base + (n - rem);
+                    pool_end = fresh_base + claim;
                 }
             }
         }
@@ -1611,7 +1622,7 @@ __device__ __forceinline__ bool ao_exact64(const BatchDev& b, int f, int64_t vsl
     return any_hit_object<double>(F.scene.obj64, id, o, d, tmax);
 }
 
-// The rays of a batch's FP64 frames: the warp's pool claims AO_CLAIM jobs at a
+// The rays of a batch's FP64 frames: the warp's pool claims ao_claim jobs at a
 // time. The rays in flight belong to one scene and grid; a warp whose pool
 // moves on to another scene lets its lanes drain first.
 struct FrameRays {
@@ -1636,10 +1647,11 @@ struct FrameRays {
         const unsigned long long total = b.job_off[b.nframes];
         if (next == end) {
             unsigned long long c = 0;
-            if (lane == 0) c = atomicAdd(b.queue + 1, (unsigned long long)AO_CLAIM);
+            const unsigned claim = (unsigned)b.queue[3];
+            if (lane == 0) c = atomicAdd(b.queue + 1, (unsigned long long)claim);
             next = __shfl_sync(FULL, c, 0);
             if (next >= total) return LANES_END;
-            end = next + AO_CLAIM < total ? next + AO_CLAIM : total;
+            end = next + claim < total ? next + claim : total;
         }
         if (next >= f_hi) {
             const int nf = b.nframes == 1 ? 0 : find_frame(b.job_off, b.nframes, next);
@@ -2217,12 +2229,14 @@ int render_frames(Ctx* ctx, FrameDev* frames, int n, bool use_graph) {
     bd.tile_w = tw;
     bd.tile_h = th;
     bd.refill = ctx->tuning.refill;
+    bd.pad = 0;
     ctx->counters_bytes_used = counters_bytes;
 
     const bool uni = one_scene(frames, n);
     if (uni) extra |= EXTRA_UNI;
     Grids gr;
     if ((rc = grids_for(ctx, precision, uni, near, gr)) != GBRT_OK) return rc;
+    bd.ao_warps = gr.ao * (ctx->tuning.block / 32);
     if (!use_graph) {
         rc = enqueue_batch(ctx, ctx->stream, precision, bd, desc_bytes, gr, extra);
     } else {
@@ -2265,7 +2279,7 @@ int render_frames(Ctx* ctx, FrameDev* frames, int n, bool use_graph) {
 
 int configure_render_kernels() { return err_of(configure_ao()); }
 
-int enqueue_prepared(const BatchDev& bd, int precision, cudaStream_t stream, int block, int num_sms, bool patch) {
+int enqueue_prepared(BatchDev bd, int precision, cudaStream_t stream, int block, int num_sms, bool patch) {
     auto grid_of = [&](auto kernel, size_t smem = 0) {
         int per_sm = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, smem) != cudaSuccess || per_sm < 1)
@@ -2275,12 +2289,15 @@ int enqueue_prepared(const BatchDev& bd, int precision, cudaStream_t stream, int
     // one frame: one scene and grid
     if (patch) k_patch_grids<<<1, 128, 0, stream>>>(bd);
     const auto none = [](int) {};
+    const int ao = precision == GBRT_FP32 ? grid_of(k_ao_walk<true, false>, ao_smem<true, false>(block))
+                                          : grid_of(k_ao_walk64);
+    bd.ao_warps = ao * (block / 32);
     if (precision == GBRT_FP32) {
         k_primary<GBRT_FP32><<<grid_of(k_primary<GBRT_FP32>), block, 0, stream>>>(bd);
-        launch_after_primary<float>(bd, true, 0, grid_of(k_ao_walk<true, false>, ao_smem<true, false>(block)), block, num_sms * 8, 0, false, stream, none);
+        launch_after_primary<float>(bd, true, 0, ao, block, num_sms * 8, 0, false, stream, none);
     } else {
         k_primary<GBRT_FP64><<<grid_of(k_primary<GBRT_FP64>), block, 0, stream>>>(bd);
-        launch_after_primary<double>(bd, true, 0, grid_of(k_ao_walk64), block, num_sms * 8, 0, false, stream, none);
+        launch_after_primary<double>(bd, true, 0, ao, block, num_sms * 8, 0, false, stream, none);
     }
     return err_of(cudaGetLastError());
 }

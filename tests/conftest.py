@@ -1,3 +1,4 @@
+import gc
 import os
 import sys
 
@@ -17,3 +18,10 @@ def oracle():
     import oracle as O
     O.lib()
     return O
+
+
+def pytest_runtest_setup(item):
+    # an earlier test's traceback can hold device tensors in a cycle; collected
+    # in the middle of a test that counts allocations, they would show there
+    if item.get_closest_marker("gpu"):
+        gc.collect()
