@@ -83,6 +83,15 @@ __device__ __forceinline__ V3<double> ld3(const double* p) { return v3(p[0], p[1
 
 // ---------------------------------------------------------------- objects
 
+// Steps that are fused, or not, in every kernel alike (left to itself the
+// compiler chooses per kernel, and a pixel's bits would depend on which of the
+// primary kernels found its hit).
+__device__ __forceinline__ float square_less(float a, float b) { return __fsub_rn(__fmul_rn(a, a), b); }
+__device__ __forceinline__ double square_less(double a, double b) { return __dsub_rn(__dmul_rn(a, a), b); }
+__device__ __forceinline__ float dot_zyx(V3<float> a, V3<float> b) {
+    return __fmaf_rn(a.z, b.z, __fmaf_rn(a.y, b.y, __fmul_rn(a.x, b.x)));
+}
+
 // Reciprocal and square root used inside the primitive test: the FP32 path
 // takes the hardware approximations (about 2 ulp), the FP64 path IEEE ones.
 __device__ __forceinline__ float rcp_(float x) { return __fdividef(1.0f, x); }
@@ -145,7 +154,7 @@ __device__ __forceinline__ bool hit_prim(V3<R> o, V3<R> d, V3<R> p0, V3<R> a, R 
     R inv = rcp_(A);
     R tc = -dot(wp, dp) * inv;
     V3<R> m = madd(wp, tc, dp);
-    R disc = r * r - dot(m, m);
+    R disc = fma(r, r, -dot(m, m));
     R half = sqrt_pos(disc * inv);
     R t0 = tc - half, t1 = tc + half;
     R s0 = wa + t0 * da, s1 = wa + t1 * da;
@@ -261,7 +270,7 @@ __device__ __forceinline__ bool clip_grid(const GridDev& g, V3<R> o, V3<R> d, V3
     R bb = dot(f, d);
     V3<R> v = madd(f, -bb, d);
     R rb = GridP<R>::bs(g, 3);
-    R disc = rb * rb - dot(v, v);
+    R disc = square_less(rb, dot(v, v));
     if (disc < R(0)) return false;
     R sq = Num<R>::sqrt_(disc);
     a = (-bb - sq) > a ? (-bb - sq) : a;
@@ -453,26 +462,50 @@ __device__ __forceinline__ void nearest_consider(Nearest<R>& h, uint32_t id, R t
     }
 }
 
-// Nearest hit in (tmin, tmax]: walk cells in ray order and stop after the
-// first cell whose exit t is at or beyond the best hit (every object whose hit
-// point lies in a visited cell is listed there).
-template <class R>
-__device__ bool trace_nearest(const GridDev& g, const SceneDev& s, V3<R> o, V3<R> d, R tmin, R tmax, Nearest<R>& h,
-                              bool& overflow) {
-    h.t1 = h.t2 = Num<R>::inf();
-    h.id1 = h.id2 = GBRT_MISS;
-    Walk<R> w;
-    if (!walk_start(g, o, d, tmin, tmax, w)) return false;
-    do {
+// A primary ray's walk dealt over `parts` adjacent lanes (SPLIT; else the lane
+// has the ray to itself): lane `sub` visits the cells sub, sub + parts, ... in
+// ray order, and the lanes share their best hit after each of these rounds.
+// The whole warp calls split_walk together (lanes with nothing to walk pass
+// on = false); visit() tests the cell's objects and best() is the nearest hit
+// so far.
+template <class Visit, class Best>
+__device__ __forceinline__ void split_walk(Walk<float>& w, bool on, int sub, int parts, bool& overflow, Visit visit,
+                                           Best best) {
+    for (int q = 0; q < sub && on; ++q) on = walk_next(w, overflow);
+    while (__any_sync(0xffffffffu, on)) {
+        if (on) visit();
+        float m = best();
+        for (int x = 1; x < parts; x <<= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, x));
+        if (on && m < Num<float>::inf() && m <= walk_cell_exit(w)) on = false;
+        for (int q = 0; q < parts && on; ++q) on = walk_next(w, overflow);
+    }
+}
+
+// Nearest hit ahead: walk cells in ray order and stop after the first cell whose
+// exit t is at or beyond the best hit (every object whose hit point lies in a
+// visited cell is listed there).
+template <bool SPLIT>
+__device__ __forceinline__ void trace_nearest(const GridDev& g, const SceneDev& s, V3<float> o, V3<float> d, bool on,
+                                              int sub, int parts, Nearest<float>& h, bool& overflow) {
+    Walk<float> w;
+    on = on && walk_start(g, o, d, 0.0f, Num<float>::inf(), w);
+    auto visit = [&] {
         uint2 cr = __ldg(g.cells + GBRT_INDEX(w.cell, g.ncells));
         for (uint32_t k = cr.x, e = cr.x + cr.y; k < e; ++k) {
             uint32_t id = GBRT_INDEX(__ldg(g.items + GBRT_INDEX(k, g.nitems)), s.S + s.C);
-            R t;
-            if (hit_object(s, id, o, d, tmin, tmax, t)) nearest_consider(h, id, t);
+            float t;
+            if (hit_object(s, id, o, d, 0.0f, Num<float>::inf(), t)) nearest_consider(h, id, t);
         }
+    };
+    if (SPLIT) {
+        split_walk(w, on, sub, parts, overflow, visit, [&] { return h.t1; });
+        return;
+    }
+    if (!on) return;
+    do {
+        visit();
         if (h.id1 != GBRT_MISS && h.t1 <= walk_cell_exit(w)) break;
     } while (walk_next(w, overflow));
-    return h.id1 != GBRT_MISS;
 }
 
 // ---------------------------------------------------------------- sampling

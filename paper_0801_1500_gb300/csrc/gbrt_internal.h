@@ -211,7 +211,8 @@ int render_frames(Ctx* ctx, FrameDev* frames, int n, bool use_graph);
 // opt the AO kernels into their shared memory (once per device), then launch
 // the four wavefront kernels with grids sized for the current device.
 int configure_render_kernels();
-int enqueue_prepared(BatchDev bd, int precision, cudaStream_t stream, int block, int num_sms, bool patch);
+int enqueue_prepared(BatchDev bd, int precision, long long tiles, cudaStream_t stream, int block, int num_sms,
+                     bool patch);
 
 #ifdef GBRT_CHECKED
 // checked build: indices the render kernels found outside their buffers since

@@ -189,7 +189,7 @@ struct BatchDev {
     int32_t tile_w, tile_h;
     int32_t refill;
     int32_t ao_warps;  // warps of the AO walk
-    int32_t pad;
+    int32_t parts;     // lanes that share a primary ray (1, 2, 4 or 8)
 };
 
 }  // namespace gbrt

@@ -130,9 +130,8 @@ extern "C" GBRT_API int gbrt_render_noalloc(const gbrt_scene* scene, const gbrt_
         bd.tile_w = tw;
         bd.tile_h = th;
         bd.refill = refill;
-        bd.pad = 0;
         rc = cudaGetLastError() == cudaSuccess ? GBRT_OK : GBRT_EDEVICE;
-        if (rc == GBRT_OK) rc = enqueue_prepared(bd, params->precision, stream, block, sms, f.grid_src != nullptr);
+        if (rc == GBRT_OK) rc = enqueue_prepared(bd, params->precision, tiles, stream, block, sms, f.grid_src != nullptr);
     }
     if (prev != scene->device) cudaSetDevice(prev);
     return rc;

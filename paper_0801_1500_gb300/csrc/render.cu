@@ -229,7 +229,7 @@ __device__ __forceinline__ bool local_root(const SceneDev& sc, uint32_t id, cons
     float L, r;
     Obj<float>::load(sc.obj, id, p0f, a, L, r);
     const V3<float> w = ff_point3(x, t, d, p0f);
-    const float wa = dot(w, a), da = dot(df, a);
+    const float wa = dot_zyx(w, a), da = dot(df, a);
     const V3<float> wp = madd(w, -wa, a), dp = madd(df, -da, a);
     const float A = dot(dp, dp), B = dot(wp, dp), C = fmaf(-r, r, dot(wp, wp));
     float s = 0.0f, corr = 0.0f;
@@ -255,24 +255,41 @@ __device__ __forceinline__ void entry_point(const Ff3& o, const Ff3& d, float te
 }
 
 // FP32 path: nearest hit in FP32 from the float-float ray re-based at its
-// grid entry (one rounding, so coordinates stay small relative to the scene),
-// then the winner -- and a runner-up within a relative 1e-4 band -- refined in
-// its object's frame (local_root); the nearer refined root wins.
-__device__ __forceinline__ bool nearest_fp32_refined(const FrameDev& f, int i, int j, uint32_t& id, LocalHit& lh,
-                                                     bool& overflow) {
+// grid entry te0 (one rounding, so coordinates stay small relative to the
+// scene).
+template <bool SPLIT>
+__device__ __forceinline__ void nearest_fp32(const FrameDev& f, int i, int j, bool on, int sub, int parts, float& te0,
+                                             Nearest<float>& h, bool& overflow) {
+    if (!SPLIT && !on) return;
     const float inf = Num<float>::inf();
     Ff3 o, d, x;
     primary_ray_ff(f, i, j, o, d);
-    float te0, te1;
-    if (!clip_grid<float>(f.grid, o.hi, d.hi, 0.0f, inf, te0, te1)) return false;
+    float te1;
+    if (!clip_grid<float>(f.grid, o.hi, d.hi, 0.0f, inf, te0, te1)) {
+        if (!SPLIT) return;
+        on = false;
+    }
     // the walk starts at the entry point rounded once
     entry_point(o, d, te0, x);
-    Nearest<float> h;
-    if (!trace_nearest<float>(f.grid, f.scene, x.hi, d.hi, 0.0f, inf, h, overflow)) return false;
+    trace_nearest<SPLIT>(f.grid, f.scene, x.hi, d.hi, on, sub, parts, h, overflow);
+    // the lanes' hits, merged
+    for (int y = 1; SPLIT && y < parts; y <<= 1) {
+        const float t1 = __shfl_xor_sync(FULL, h.t1, y), t2 = __shfl_xor_sync(FULL, h.t2, y);
+        const uint32_t k1 = __shfl_xor_sync(FULL, h.id1, y), k2 = __shfl_xor_sync(FULL, h.id2, y);
+        if (k1 != GBRT_MISS) nearest_consider(h, k1, t1);
+        if (k2 != GBRT_MISS) nearest_consider(h, k2, t2);
+    }
+}
+
+// The winner -- and a runner-up within a relative 1e-4 band -- refined in its
+// object's frame (local_root); the nearer refined root wins.
+__device__ __forceinline__ void refine_fp32(const FrameDev& f, int i, int j, float te0, const Nearest<float>& h,
+                                            uint32_t& id, LocalHit& lh) {
     // the refinement needs what the rounding left out: the ray and its entry
     // point are formed again (the same steps give the same floats), which is
     // cheaper than holding their low parts in registers through the walk
     // (the copies of i and j keep the compiler from reusing the first ones)
+    Ff3 o, d, x;
     int i2, j2;
     asm volatile("mov.b32 %0, %1;" : "=r"(i2) : "r"(i));
     asm volatile("mov.b32 %0, %1;" : "=r"(j2) : "r"(j));
@@ -292,7 +309,6 @@ __device__ __forceinline__ bool nearest_fp32_refined(const FrameDev& f, int i, i
             lh = l2;
         }
     }
-    return true;
 }
 
 // ---------------------------------------------------------------- FP32 filters of FP64 decisions
@@ -381,7 +397,34 @@ __device__ __noinline__ double exact_root64(const FrameDev& f, int i, int j, uin
 // (965 x 1137 frame, this kernel: 2.40 -> 0.215 ms; 256 x 256: 0.39 ->
 // 0.057 ms. The FP64 pipe was the bound; now the walk's load latency and the
 // winners' ~200 FP64 instructions are).
-__device__ __forceinline__ bool nearest_filtered64(const FrameDev& f, int i, int j, uint32_t& id, bool& overflow) {
+struct Near64 {
+    uint32_t id;     // GBRT_MISS: none
+    float t, e;      // its root from the grid entry, and that root's error
+};
+
+// A candidate's root (or, open, a candidate that may have one) joins h.
+__device__ __forceinline__ void near64_consider(const FrameDev& f, int i, int j, float te0, Near64& h, uint32_t cand,
+                                                bool open, float t, float et) {
+    bool nearer = t + et < h.t - h.e;
+    if (open || !(nearer || t - et > h.t + h.e)) {
+        const double t64 = exact_root64(f, i, j, cand);
+        if (t64 == Num<double>::inf()) return;
+        const double b64 = h.id == GBRT_MISS ? Num<double>::inf() : exact_root64(f, i, j, h.id);
+        nearer = t64 < b64 || (t64 == b64 && cand < h.id);
+        t = (float)(t64 - (double)te0);
+        et = 2e-7f * fabsf(t);
+    }
+    if (nearer) {
+        h.id = cand;
+        h.t = t;
+        h.e = et;
+    }
+}
+
+template <bool SPLIT>
+__device__ __forceinline__ void nearest_filtered64(const FrameDev& f, int i, int j, bool on, int sub, int parts,
+                                                   Near64& h, bool& overflow) {
+    if (!SPLIT && !on) return;
     const GridDev& g = f.grid;
     const float inf = Num<float>::inf();
     Ff3 o, d, x;
@@ -395,16 +438,15 @@ __device__ __forceinline__ bool nearest_filtered64(const FrameDev& f, int i, int
     const V3<float> xr = (x.hi - lo) + x.lo;
     const V3<float> df = d.hi;
     Walk<float> w;
-    if (!walk_start_rel(g, xr, df, inf, w)) return false;
+    on = on && walk_start_rel(g, xr, df, inf, w);
+    if (!SPLIT && !on) return;
     const float om = 0.1f * fmaxf(g.hi[0] - lo.x, fmaxf(g.hi[1] - lo.y, g.hi[2] - lo.z));
     const float idd = __fdividef(-1.0f, dot(df, df));
-    id = GBRT_MISS;
-    float t1 = inf, e1 = 0.0f;
-    do {
+    auto visit = [&] {
         const uint2 cr = __ldg(g.cells + GBRT_INDEX(w.cell, g.ncells));
         for (uint32_t k = cr.x, e = cr.x + cr.y; k < e; ++k) {
             const uint32_t cand = GBRT_INDEX(__ldg(g.items + GBRT_INDEX(k, g.nitems)), f.scene.S + f.scene.C);
-            if (cand == id) continue;
+            if (cand == h.id) continue;
             const float4 s = __ldg(f.scene.bs + cand);
             const V3<float> wv = xr - v3(s.x - lo.x, s.y - lo.y, s.z - lo.z);
             const float tc = dot(wv, df) * idd;
@@ -422,25 +464,23 @@ __device__ __forceinline__ bool nearest_filtered64(const FrameDev& f, int i, int
                 Obj<float>::load(f.scene.obj, cand, p0, a, L, rr);
                 what = tube_root32(xr, df, p0 - lo, a, L, rr, inf, inf, om, t, et);
             }
-            if (what == PAIR_MISS) continue;
-            bool nearer = t + et < t1 - e1;
-            if (what == PAIR_OPEN || !(nearer || t - et > t1 + e1)) {
-                const double t64 = exact_root64(f, i, j, cand);
-                if (t64 == Num<double>::inf()) continue;
-                const double b64 = id == GBRT_MISS ? Num<double>::inf() : exact_root64(f, i, j, id);
-                nearer = t64 < b64 || (t64 == b64 && cand < id);
-                t = (float)(t64 - (double)te0);
-                et = 2e-7f * fabsf(t);
-            }
-            if (nearer) {
-                id = cand;
-                t1 = t;
-                e1 = et;
-            }
+            if (what != PAIR_MISS) near64_consider(f, i, j, te0, h, cand, what == PAIR_OPEN, t, et);
         }
-        if (id != GBRT_MISS && t1 <= walk_cell_exit(w)) break;
-    } while (walk_next(w, overflow));
-    return id != GBRT_MISS;
+    };
+    if (!SPLIT) {
+        do {
+            visit();
+            if (h.id != GBRT_MISS && h.t <= walk_cell_exit(w)) break;
+        } while (walk_next(w, overflow));
+        return;
+    }
+    split_walk(w, on, sub, parts, overflow, visit, [&] { return h.t; });
+    // the lanes' hits, merged
+    for (int x = 1; x < parts; x <<= 1) {
+        const uint32_t k = __shfl_xor_sync(FULL, h.id, x);
+        const float t = __shfl_xor_sync(FULL, h.t, x), e = __shfl_xor_sync(FULL, h.e, x);
+        if (k != GBRT_MISS && k != h.id) near64_consider(f, i, j, te0, h, k, false, t, e);
+    }
 }
 
 // Hit records: (AO origin xyz, pixel) and (normal xyz, object id).
@@ -525,33 +565,50 @@ __device__ __forceinline__ void ao_plan(const BatchDev& b) {
     b.queue[3] = ao_claim(jobs, b.ao_warps);
 }
 
-
-template <int MODE>
+// SPLIT: b.parts lanes share a primary ray (ray_parts).
+template <int MODE, bool SPLIT>
 __global__ void __launch_bounds__(256) k_primary(const __grid_constant__ BatchDev b) {
     const int lane = threadIdx.x & 31;
-    const long long total = b.tile_off[b.nframes];
+    const int parts = SPLIT ? b.parts : 1, sub = lane & (parts - 1);
+    const long long total = b.tile_off[b.nframes] * parts;
     bool overflow = false;
     while (true) {
         long long item = 0;
         if (lane == 0) item = (long long)atomicAdd(b.queue, 1ull);
         item = __shfl_sync(FULL, item, 0);
         if (item >= total) break;
+        int px = lane;  // the lane's pixel of the tile
+        if (SPLIT) {    // (an item is 32 / parts pixels)
+            px = ((int)(item & (parts - 1)) * 32 + lane) / parts;
+            item /= parts;
+        }
         const int f = find_frame(b.tile_off, b.nframes, item);
         const FrameDev& F = b.frames[f];
         const long long t = item - b.tile_off[f];
         const int tx = (int)(t % F.tiles_x), ty = (int)(t / F.tiles_x);
-        const int i = tx * b.tile_w + lane % b.tile_w;
-        const int j = F.row0 + ty * b.tile_h + lane / b.tile_w;
+        const int i = tx * b.tile_w + px % b.tile_w;
+        const int j = F.row0 + ty * b.tile_h + px / b.tile_w;
         const bool inside = i < F.W && j < F.row0 + F.rows;
+        const bool mine = inside && sub == 0;  // the lane that writes the pixel
         uint32_t id = GBRT_MISS;
         LocalHit lh;
         bool hit = false;
-        if (inside) {
-            if (MODE == GBRT_FP32) {
-                hit = nearest_fp32_refined(F, i, j, id, lh, overflow);
-            } else {
-                hit = nearest_filtered64(F, i, j, id, overflow);
-            }
+        if (MODE == GBRT_FP32) {
+            float te0 = 0.0f;
+            Nearest<float> h;
+            h.t1 = h.t2 = Num<float>::inf();
+            h.id1 = h.id2 = GBRT_MISS;
+            nearest_fp32<SPLIT>(F, i, j, inside, sub, parts, te0, h, overflow);
+            hit = mine && h.id1 != GBRT_MISS;
+            if (hit) refine_fp32(F, i, j, te0, h, id, lh);
+        } else {
+            Near64 h;
+            h.id = GBRT_MISS;
+            h.t = Num<float>::inf();
+            h.e = 0.0f;
+            nearest_filtered64<SPLIT>(F, i, j, inside, sub, parts, h, overflow);
+            id = h.id;
+            hit = mine && id != GBRT_MISS;
         }
         // warp-aggregated append to this frame's hit list
         const unsigned hm = __ballot_sync(FULL, hit);
@@ -561,7 +618,7 @@ __global__ void __launch_bounds__(256) k_primary(const __grid_constant__ BatchDe
             if (lane == leader) base = atomicAdd(b.hit_count + f, (unsigned)__popc(hm));
             base = __shfl_sync(FULL, base, leader);
         }
-        if (b.tiles && hm && lane == 0) {
+        if (b.tiles && hm && lane == 0) {  // (the near pass's frames are not split into parts)
             unsigned long long at =
                 atomicAdd(b.ntiles, (unsigned long long)((F.mask_words + F.rec_words - 1) / F.rec_words));
             for (int w = 0; w < F.mask_words; w += F.rec_words, ++at) {
@@ -571,7 +628,7 @@ __global__ void __launch_bounds__(256) k_primary(const __grid_constant__ BatchDe
                 b.tiles[at].word = w;
             }
         }
-        if (!inside) continue;
+        if (!mine) continue;
         const uint32_t q = (uint32_t)j * (uint32_t)F.W + (uint32_t)i;
         if (hit) {
             const int64_t slot = GBRT_INDEX(F.hit_base + base + __popc(hm & ((1u << lane) - 1u)), b.hit_cap);
@@ -1998,6 +2055,12 @@ static void launch_ao(const BatchDev& bd, bool uni, int near, int grid, int bloc
     }
 }
 
+template <int MODE>
+static void launch_primary(const BatchDev& bd, int grid, int block, cudaStream_t stream) {
+    if (bd.parts > 1) k_primary<MODE, true><<<grid, block, 0, stream>>>(bd);
+    else k_primary<MODE, false><<<grid, block, 0, stream>>>(bd);
+}
+
 // The passes after the primary one: AO walk, shading, and the box filter of
 // supersampled frames (the AO plan runs in the primary kernel's last CTA).
 template <class R>
@@ -2018,7 +2081,7 @@ static int grids_for(Ctx* ctx, int precision, bool uni, bool near, Grids& g) {
     }
     g.near = near ? persistent_grid(ctx, k_ao_near, NEAR_BLOCK, NEAR_SMEM) : 0;
     if (precision == GBRT_FP32) {
-        g.primary = persistent_grid(ctx, k_primary<GBRT_FP32>, block);
+        g.primary = persistent_grid(ctx, k_primary<GBRT_FP32, false>, block);
         if (near)
             g.ao = uni ? persistent_grid(ctx, k_ao_walk<true, true>, block, ao_smem<true, true>(block))
                        : persistent_grid(ctx, k_ao_walk<false, true>, block, ao_smem<false, true>(block));
@@ -2026,7 +2089,7 @@ static int grids_for(Ctx* ctx, int precision, bool uni, bool near, Grids& g) {
             g.ao = uni ? persistent_grid(ctx, k_ao_walk<true, false>, block, ao_smem<true, false>(block))
                        : persistent_grid(ctx, k_ao_walk<false, false>, block, ao_smem<false, false>(block));
     } else {
-        g.primary = persistent_grid(ctx, k_primary<GBRT_FP64>, block);
+        g.primary = persistent_grid(ctx, k_primary<GBRT_FP64, false>, block);
         g.ao = persistent_grid(ctx, k_ao_walk64, block);
     }
     g.shade = ctx->num_sms * 8;
@@ -2053,6 +2116,20 @@ static bool one_scene(const FrameDev* frames, int n) {
 static bool near_pass_suits(const FrameDev& f) {
     return f.precision == GBRT_FP32 && f.grid.rho > 0.0f && std::isinf(f.ao_maxdist_f) &&
            f.jobs_per_hit >= NEAR_MIN_JOBS && f.jobs_per_hit <= NEAR_MAX_JOBS;
+}
+
+// Lanes that share a primary ray (split_walk). A frame with fewer tiles than the
+// kernel has warps is bound by the latency of its slowest warp, a chain of
+// dependent loads and tests (cell, item, object): 128 x 96 pixels, 36 us of
+// which the mean warp is busy for 7. Then 2, 4 or 8 lanes walk a ray between
+// them: 29 us with 8 at 128 x 96 (a frame 66.7 -> 59.4), a 256 x 256 frame
+// 75.2 -> 72.8 with 2. With more lanes than keep every tile resident at once
+// the cells visited past the hit cost more than they hide (256 x 256: 4 lanes
+// 75.7, 8 lanes 88.6; FP64 195 us with one lane, 217 with 4).
+static int ray_parts(long long tiles, int warps) {
+    int parts = 1;
+    while (parts < 8 && 2 * parts * tiles <= warps) parts *= 2;
+    return parts;
 }
 
 // Share of a frame's pixels that the objects' bounding sphere covers, roughly
@@ -2091,12 +2168,12 @@ static int enqueue_batch(Ctx* ctx, cudaStream_t stream, int precision, const Bat
     mark(0);
     const bool uni = (extra & EXTRA_UNI) != 0;
     if (precision == GBRT_FP32) {
-        k_primary<GBRT_FP32><<<gr.primary, block, 0, stream>>>(bd);
+        launch_primary<GBRT_FP32>(bd, gr.primary, block, stream);
         mark(1);
         mark(2);
         launch_after_primary<float>(bd, uni, gr.near, gr.ao, block, gr.shade, gr.resolve, resolve, stream, mark);
     } else {
-        k_primary<GBRT_FP64><<<gr.primary, block, 0, stream>>>(bd);
+        launch_primary<GBRT_FP64>(bd, gr.primary, block, stream);
         mark(1);
         mark(2);
         launch_after_primary<double>(bd, uni, gr.near, gr.ao, block, gr.shade, gr.resolve, resolve, stream, mark);
@@ -2229,7 +2306,6 @@ int render_frames(Ctx* ctx, FrameDev* frames, int n, bool use_graph) {
     bd.tile_w = tw;
     bd.tile_h = th;
     bd.refill = ctx->tuning.refill;
-    bd.pad = 0;
     ctx->counters_bytes_used = counters_bytes;
 
     const bool uni = one_scene(frames, n);
@@ -2237,6 +2313,7 @@ int render_frames(Ctx* ctx, FrameDev* frames, int n, bool use_graph) {
     Grids gr;
     if ((rc = grids_for(ctx, precision, uni, near, gr)) != GBRT_OK) return rc;
     bd.ao_warps = gr.ao * (ctx->tuning.block / 32);
+    bd.parts = near ? 1 : ray_parts(tiles, gr.primary * (ctx->tuning.block / 32));
     if (!use_graph) {
         rc = enqueue_batch(ctx, ctx->stream, precision, bd, desc_bytes, gr, extra);
     } else {
@@ -2279,7 +2356,8 @@ int render_frames(Ctx* ctx, FrameDev* frames, int n, bool use_graph) {
 
 int configure_render_kernels() { return err_of(configure_ao()); }
 
-int enqueue_prepared(BatchDev bd, int precision, cudaStream_t stream, int block, int num_sms, bool patch) {
+int enqueue_prepared(BatchDev bd, int precision, long long tiles, cudaStream_t stream, int block, int num_sms,
+                     bool patch) {
     auto grid_of = [&](auto kernel, size_t smem = 0) {
         int per_sm = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, smem) != cudaSuccess || per_sm < 1)
@@ -2292,11 +2370,13 @@ int enqueue_prepared(BatchDev bd, int precision, cudaStream_t stream, int block,
     const int ao = precision == GBRT_FP32 ? grid_of(k_ao_walk<true, false>, ao_smem<true, false>(block))
                                           : grid_of(k_ao_walk64);
     bd.ao_warps = ao * (block / 32);
+    const int primary = precision == GBRT_FP32 ? grid_of(k_primary<GBRT_FP32, false>) : grid_of(k_primary<GBRT_FP64, false>);
+    bd.parts = ray_parts(tiles, primary * (block / 32));
     if (precision == GBRT_FP32) {
-        k_primary<GBRT_FP32><<<grid_of(k_primary<GBRT_FP32>), block, 0, stream>>>(bd);
+        launch_primary<GBRT_FP32>(bd, primary, block, stream);
         launch_after_primary<float>(bd, true, 0, ao, block, num_sms * 8, 0, false, stream, none);
     } else {
-        k_primary<GBRT_FP64><<<grid_of(k_primary<GBRT_FP64>), block, 0, stream>>>(bd);
+        launch_primary<GBRT_FP64>(bd, primary, block, stream);
         launch_after_primary<double>(bd, true, 0, ao, block, num_sms * 8, 0, false, stream, none);
     }
     return err_of(cudaGetLastError());
