@@ -133,6 +133,9 @@ FrameDev make_frame(const gbrt_scene* scene, const gbrt_grid* grid, const gbrt_c
     f.k_d = p->k_d;
     f.k_s = p->k_s;
     f.phong = p->phong_exp;
+    f.phong_n = p->phong_exp >= 1.0 && p->phong_exp <= 1024.0 && p->phong_exp == std::floor(p->phong_exp)
+                    ? (int32_t)p->phong_exp
+                    : 0;
     f.sky_kao_f = (float)f.sky_kao;
     f.k_d_f = (float)f.k_d;
     f.k_s_f = (float)f.k_s;

