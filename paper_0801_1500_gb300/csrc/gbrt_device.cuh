@@ -349,12 +349,12 @@ __device__ __forceinline__ bool walk_start(const GridDev& g, V3<R> o, V3<R> d, R
 // The same set-up for a ray whose origin is relative to the grid's lower
 // corner (FP64 rays: the difference is formed in FP64 and rounded once, so the
 // walk's error stays relative to the grid's extent).
-__device__ __forceinline__ bool walk_start_rel(const GridDev& g, V3<float> o, V3<float> d, float tmax,
+__device__ __forceinline__ bool walk_start_rel(const GridDev& g, V3<float> o, V3<float> d, float tmin, float tmax,
                                                Walk<float>& w) {
     if (g.empty) return false;
     const V3<float> inv = inv_dir(d);
     const float oo[3] = {o.x, o.y, o.z}, dd[3] = {d.x, d.y, d.z}, ii[3] = {inv.x, inv.y, inv.z};
-    float t0 = 0.0f, t1 = tmax;
+    float t0 = tmin, t1 = tmax;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         const float hi = g.hi[k] - g.lo[k];

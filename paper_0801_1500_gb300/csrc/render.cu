@@ -7,7 +7,7 @@
 //              origin, normal) to its frame's hit list; the last CTA to
 //              finish lays out the AO pass (prefix sums of hits and AO rays
 //              per frame);
-//   k_ao_near  (FP32 frames with rays enough) tests the AO rays of a tile
+//   k_ao_near  (frames with rays enough) tests the AO rays of a tile
 //              against the balls around it before they walk;
 //   k_ao_walk  persistent; each lane holds one AO (or direct-light shadow)
 //              ray; a warp refills its idle lanes together from its ray pool
@@ -438,7 +438,7 @@ __device__ __forceinline__ void nearest_filtered64(const FrameDev& f, int i, int
     const V3<float> xr = (x.hi - lo) + x.lo;
     const V3<float> df = d.hi;
     Walk<float> w;
-    on = on && walk_start_rel(g, xr, df, inf, w);
+    on = on && walk_start_rel(g, xr, df, 0.0f, inf, w);
     if (!SPLIT && !on) return;
     const float om = 0.1f * fmaxf(g.hi[0] - lo.x, fmaxf(g.hi[1] - lo.y, g.hi[2] - lo.z));
     const float idd = __fdividef(-1.0f, dot(df, df));
@@ -789,8 +789,10 @@ constexpr int NEAR_MIN_JOBS = 8;
 // A record takes a warp some 40 us, most of it latency, and the walk's units are
 // coarser than its own claims: the pass pays when every resident warp gets
 // several (1.1 MP, 21,000 records: frame 1.12 -> 0.93 ms; 5,900
-// records: 0.416 -> 0.437 ms).
-constexpr double NEAR_MIN_RECS = 12288;
+// records: 0.416 -> 0.437 ms). FP64 rays walk slower, and one a lane: there it
+// pays from 3,000 on (360 x 360 at 16 samples, 3,180 records: 0.392 -> 0.380 ms;
+// 640 x 640, 10,000: 0.940 -> 0.794 ms).
+constexpr double NEAR_MIN_RECS = 12288, NEAR_MIN_RECS64 = 3072;
 
 // Largest b - q over the n candidates at c, for each of the NS directions: b =
 // w.d with w = centre - o, q = sqrt(|w|^2 - r^2). The ray meets a ball ahead of
@@ -798,7 +800,8 @@ constexpr double NEAR_MIN_RECS = 12288;
 // (ray, ball) pair costs three FMAs and half a three-input maximum. An origin
 // inside or within 5e-5 r of a ball sets bad (q would be too rough there),
 // unless it is the ball of the tube that the hit lies on (skip, its centre):
-// rays from a tube's outer side do not meet it again.
+// rays from a tube's outer side do not meet it again. An FP64 origin is o + ol
+// (float pairs: w then has FP32's relative error however large the coordinates).
 struct NearSkip {
     bool on;
     V3<float> c;
@@ -810,13 +813,17 @@ __device__ __forceinline__ float near_q(float4 A, float q2, const NearSkip& skip
     }
     return sqrt_pos(q2);
 }
-template <int NS>
-__device__ __forceinline__ void near_scan(const float4* c, int n, V3<float> o, const float (&d)[NS][3], float (&m)[NS],
-                                          const NearSkip& skip, bool& bad) {
+template <int NS, bool F64>
+__device__ __forceinline__ void near_scan(const float4* c, int n, V3<float> o, V3<float> ol, const float (&d)[NS][3],
+                                          float (&m)[NS], const NearSkip& skip, bool& bad) {
     for (int k = 0; k < n; k += 2) {
         const float4 A = c[k], B = c[k + 1 < n ? k + 1 : k];
-        const float ax = A.x - o.x, ay = A.y - o.y, az = A.z - o.z;
-        const float bx = B.x - o.x, by = B.y - o.y, bz = B.z - o.z;
+        float ax = A.x - o.x, ay = A.y - o.y, az = A.z - o.z;
+        float bx = B.x - o.x, by = B.y - o.y, bz = B.z - o.z;
+        if (F64) {
+            ax -= ol.x, ay -= ol.y, az -= ol.z;
+            bx -= ol.x, by -= ol.y, bz -= ol.z;
+        }
         const float qa = fmaf(ax, ax, fmaf(ay, ay, fmaf(az, az, -A.w * A.w)));
         const float qb = fmaf(bx, bx, fmaf(by, by, fmaf(bz, bz, -B.w * B.w)));
         const float na = -near_q(A, qa, skip, bad), nb = -near_q(B, qb, skip, bad);
@@ -830,11 +837,10 @@ __device__ __forceinline__ void near_scan(const float4* c, int n, V3<float> o, c
 // NS jobs (from j0) of a work item's hits, one hit a lane: which are occluded
 // by a near sphere, which have to walk, which of those from the start, which
 // leave the objects' bounds before the near pass's reach.
-template <int NS>
-__device__ __forceinline__ void near_jobs(const FrameDev& F, NearWarp& S, int lane, int j0, V3<float> o, V3<float> nrm,
-                                          uint32_t q, const NearSkip& skip, int ns, int nt, float rho, float delta,
-                                          uint32_t& todo,
-                                          uint32_t& start, uint32_t& escaped) {
+template <int NS, bool F64>
+__device__ __forceinline__ void near_jobs(const FrameDev& F, NearWarp& S, int lane, int j0, V3<float> o, V3<float> ol,
+                                          V3<float> nrm, uint32_t q, const NearSkip& skip, int ns, int nt, float rho,
+                                          float delta, uint32_t& todo, uint32_t& start, uint32_t& escaped) {
     float d[NS][3], m[NS];
     uint32_t valid = 0u;
     for (int h = 0; h < NS; h += 8) {
@@ -844,7 +850,7 @@ __device__ __forceinline__ void near_jobs(const FrameDev& F, NearWarp& S, int la
             if (j0 + h + s < F.jobs_per_hit) {
                 float tmax;
                 uint32_t lbit;
-                if (ao_direction<float>(F, q, (uint32_t)(j0 + h + s), nrm, dir, tmax, lbit)) valid |= 1u << (h + s);
+                if (ao_direction<float>(F, q, (uint32_t)(j0 + h + s), nrm, dir, tmax, lbit, F64)) valid |= 1u << (h + s);
             }
             S.dir[s][0][lane] = dir.x;
             S.dir[s][1][lane] = dir.y;
@@ -867,7 +873,7 @@ __device__ __forceinline__ void near_jobs(const FrameDev& F, NearWarp& S, int la
     for (int kind = 0; kind < 2; ++kind) {
 #pragma unroll
         for (int s = 0; s < NS; ++s) m[s] = -Num<float>::inf();
-        near_scan<NS>(list, n, o, d, m, skip, bad);
+        near_scan<NS, F64>(list, n, o, ol, d, m, skip, bad);
         const float sure = kind == 0 ? delta : Num<float>::inf();
 #pragma unroll
         for (int s = 0; s < NS; ++s) {
@@ -912,6 +918,10 @@ __device__ __forceinline__ void near_jobs(const FrameDev& F, NearWarp& S, int la
 // m16n8k16 mma.sync (13.7 cycles a 128 pairs, no faster than the FMAs), packed
 // f32x2 FMAs (20% fewer instructions, 10% slower), a row of cells per lane in
 // the gather (55 dependent rounds of loads instead of 16: 0.44 ms).
+// F64: the same for FP64 frames, whose decisions delta covers as well (the
+// directions are the FP32 ones the walk filters with, the origins float pairs):
+// 0.38 ms, and the walk 1.53 -> 0.78 (965 x 1137, frame 1.87 -> 1.48 ms).
+template <bool F64>
 __global__ void __launch_bounds__(128, 4) k_ao_near(const __grid_constant__ BatchDev b) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     NearWarp& S = reinterpret_cast<NearWarp*>(smem_raw)[threadIdx.x >> 5];
@@ -927,9 +937,15 @@ __global__ void __launch_bounds__(128, 4) k_ao_near(const __grid_constant__ Batc
         const int n = b.tiles[tile].n;
         const FrameDev& F = b.frames[b.tiles[tile].frame];
         const int64_t slot = GBRT_INDEX(b.tiles[tile].slot + (lane < n ? lane : 0), b.hit_cap);
-        V3<float> o, nrm;
+        V3<float> o, nrm, ol = v3(0.0f, 0.0f, 0.0f);
         uint32_t q, own;
         HitIO<float>::load(b.hits32, slot, o, nrm, q, own);
+        if (F64) {  // hits32 holds the origin relative to the grid's corner
+            V3<double> o64, n64;
+            HitIO<double>::load(b.hits, slot, o64, n64, q, own);
+            o = to_f(o64);
+            ol = to_f(o64 - to_d(o));
+        }
         float rho = F.near_pass ? F.grid.rho : 0.0f, delta = 0.0f;
         int ns = 0, nt = 0;
         NearSkip skip;
@@ -941,7 +957,7 @@ __global__ void __launch_bounds__(128, 4) k_ao_near(const __grid_constant__ Batc
             own = GBRT_INDEX(own, F.scene.S + F.scene.C);
             Obj<float>::load(F.scene.obj, own, p0, a, L, r);
             if (L > 0.0f) {
-                const V3<float> w = o - p0, wp = madd(w, -dot(w, a), a);
+                const V3<float> w = (o - p0) + ol, wp = madd(w, -dot(w, a), a);
                 const float4 c = __ldg(F.grid.cut + own);
                 skip.on = dot(wp, wp) > 1.0002f * r * r;  // surely outside
                 skip.c = v3(c.x, c.y, c.z);
@@ -1045,12 +1061,12 @@ __global__ void __launch_bounds__(128, 4) k_ao_near(const __grid_constant__ Batc
             uint32_t todo, start, esc = 0u;
             if (rho > 0.0f) {
                 if (cnt > 8) {
-                    near_jobs<16>(F, S, lane, j0, o, nrm, q, skip, ns, nt, rho, delta, todo, start, esc);
+                    near_jobs<16, F64>(F, S, lane, j0, o, ol, nrm, q, skip, ns, nt, rho, delta, todo, start, esc);
                 } else {
                     todo = start = 0u;
                     for (int k = 0; k < cnt; k += 4) {
                         uint32_t t4, s4, e4;
-                        near_jobs<4>(F, S, lane, j0 + k, o, nrm, q, skip, ns, nt, rho, delta, t4, s4, e4);
+                        near_jobs<4, F64>(F, S, lane, j0 + k, o, ol, nrm, q, skip, ns, nt, rho, delta, t4, s4, e4);
                         todo |= t4 << k;
                         start |= s4 << k;
                         esc |= e4 << k;
@@ -1175,7 +1191,7 @@ __device__ __forceinline__ void unit_take(const BatchDev& b, AoUnit& U, int lane
                 break;
             }
             const unsigned long long unit = b.units[at];
-                        const int g = (int)(unit & 0xFFu), sh = 4 * (g & 3);
+            const int g = (int)(unit & 0xFFu), sh = 4 * (g & 3);
             const TileRec T = b.tiles[unit >> 8];
             const FrameDev& N = b.frames[T.frame];
             uint32_t m = 0u;
@@ -1681,15 +1697,19 @@ __device__ __forceinline__ bool ao_exact64(const BatchDev& b, int f, int64_t vsl
 
 // The rays of a batch's FP64 frames: the warp's pool claims ao_claim jobs at a
 // time. The rays in flight belong to one scene and grid; a warp whose pool
-// moves on to another scene lets its lanes drain first.
+// moves on to another scene lets its lanes drain first. NEAR: the rays that the
+// near pass left instead, from its units (every frame has the same scene and
+// grid, and no AO limit).
+template <bool NEAR>
 struct FrameRays {
     static constexpr bool F64 = true;
     const BatchDev& b;
+    AoUnit* const U;
     // the warp's claimed jobs [next, end) and the frame they belong to (uniform)
     unsigned long long next = 0, end = 0, f_lo = 0, f_hi = 0;
     int f = 0;
 
-    __device__ __forceinline__ explicit FrameRays(const BatchDev& batch) : b(batch) {}
+    __device__ __forceinline__ FrameRays(const BatchDev& batch, AoUnit* unit) : b(batch), U(unit) {}
 
     __device__ __forceinline__ void escape(const LaneRay& ray) const { ao_escape(b, ray.slot, ray.lbit); }
 
@@ -1699,8 +1719,36 @@ struct FrameRays {
         return ao_exact64(b, ray.f, ray.slot, ray.smp, id);
     }
 
+    // Job smp of the hit in `slot`, from distance tmin on.
+    __device__ __forceinline__ void set_up(const FrameDev& F, int fi, int64_t slot, uint32_t smp, float tmin,
+                                           LaneRay& ray, Walk<float>& w, bool& fresh) {
+        uint32_t q, own;
+        V3<float> nrm;
+        ray.slot = slot;
+        ray.smp = smp;
+        ray.f = fi;
+        HitIO<float>::load(b.hits32, slot, ray.o, nrm, q, own);
+        if (ao_direction<float>(F, q, smp, nrm, ray.d, ray.tmax, ray.lbit, true)) {
+            fresh = walk_start_rel(F.grid, ray.o, ray.d, tmin, ray.tmax, w);
+            if (!fresh) ao_escape(b, slot, ray.lbit);  // misses the objects' bounds
+        }
+    }
+
     __device__ __forceinline__ int refill(LaneScene& A, int lane, unsigned act, bool free, LaneRay& ray, Walk<float>& w,
                                           bool& fresh) {
+        if constexpr (NEAR) {
+            if (!A.cells) A.set(b.frames[0]);
+            const unsigned idle = ~act;
+            const FrameDev* Fp = nullptr;
+            int64_t slot = 0;
+            uint32_t smp = 0;
+            float tmin = 0.0f;
+            bool done = false;
+            unit_take(b, *U, lane, *b.nunits, __popc(idle), __popc(idle & ((1u << lane) - 1u)), free, done, slot, smp,
+                      tmin, Fp);
+            if (Fp) set_up(*Fp, (int)(Fp - b.frames), slot, smp, tmin, ray, w, fresh);
+            return done ? LANES_END : LANES_GO;
+        }
         const unsigned long long total = b.job_off[b.nframes];
         if (next == end) {
             unsigned long long c = 0;
@@ -1725,16 +1773,9 @@ struct FrameRays {
         const unsigned long long left = (end < f_hi ? end : f_hi) - next;
         const unsigned n = left < (unsigned long long)__popc(idle) ? (unsigned)left : __popc(idle);
         if (free && i < n) {
-            uint32_t h, q, own;
-            V3<float> nrm;
-            ao_split(F, next + i - f_lo, h, ray.smp);
-            ray.slot = GBRT_INDEX(F.hit_base + (int64_t)h, b.hit_cap);
-            ray.f = f;
-            HitIO<float>::load(b.hits32, ray.slot, ray.o, nrm, q, own);
-            if (ao_direction<float>(F, q, ray.smp, nrm, ray.d, ray.tmax, ray.lbit, true)) {
-                fresh = walk_start_rel(F.grid, ray.o, ray.d, ray.tmax, w);
-                if (!fresh) ao_escape(b, ray.slot, ray.lbit);  // misses the objects' bounds
-            }
+            uint32_t h, smp;
+            ao_split(F, next + i - f_lo, h, smp);
+            set_up(F, f, GBRT_INDEX(F.hit_base + (int64_t)h, b.hit_cap), smp, 0.0f, ray, w, fresh);
         }
         next += n;
         return n < __popc(idle) && next < total ? LANES_AGAIN : LANES_GO;  // the rest from the next claim or frame
@@ -1747,10 +1788,18 @@ struct FrameRays {
 // thousand (walk 1.7 ms; 256 x 256 frame at 8 samples 0.57 -> 0.11 ms). One
 // ray a lane rather than the FP32 frames' pair expansion: with a filter this
 // cheap the expansion costs more than the idle lanes (walk 3.8 ms with pairs
-// queued in shared memory). Bound now by instruction issue.
+// queued in shared memory). Bound now by instruction issue. NEAR: after a near
+// pass, over the rays it left (0.78 ms).
+template <bool NEAR>
 __global__ void __launch_bounds__(256, 3) k_ao_walk64(const __grid_constant__ BatchDev b) {
+    __shared__ AoUnit units[NEAR ? 8 : 1];
+    AoUnit* const unit = units + (NEAR ? threadIdx.x >> 5 : 0);
     grid_dependency_wait();
-    FrameRays src(b);
+    if (NEAR) {
+        unit->rem = 0u;
+        __syncwarp();
+    }
+    FrameRays<NEAR> src(b, unit);
     LaneScene A;
     A.cells = nullptr;
     A.cut = false;
@@ -1904,7 +1953,7 @@ struct ProbeRays {
             float tmax;
             uint32_t lbit;
             ao_direction<float>(F, (uint32_t)pt, smp, n0, ray.d, tmax, lbit);
-            if constexpr (FP64) fresh = walk_start_rel(F.grid, ray.o, ray.d, tmax, w);
+            if constexpr (FP64) fresh = walk_start_rel(F.grid, ray.o, ray.d, 0.0f, tmax, w);
             else fresh = walk_start(F.grid, ray.o, ray.d, 0.0f, tmax, w);
             ray.slot = (int64_t)pt;
             ray.tmax = tmax;
@@ -2033,10 +2082,14 @@ static cudaError_t configure_ao() {
         prefer_small_carveout(k_ao_walk<false, false>, ao_smem<false, false>(256)) != cudaSuccess ||
         prefer_small_carveout(k_ao_walk<true, true>, ao_smem<true, true>(256)) != cudaSuccess ||
         prefer_small_carveout(k_ao_walk<false, true>, ao_smem<false, true>(256)) != cudaSuccess ||
-        prefer_small_carveout(k_ao_walk64, 0) != cudaSuccess)
+        prefer_small_carveout(k_ao_walk64<false>, 0) != cudaSuccess ||
+        prefer_small_carveout(k_ao_walk64<true>, 8 * sizeof(AoUnit)) != cudaSuccess)
         (void)cudaGetLastError();
     // the near pass's candidate lists exceed the 48 KB default
-    return cudaFuncSetAttribute(k_ao_near, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)NEAR_SMEM);
+    cudaError_t e = cudaFuncSetAttribute(k_ao_near<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)NEAR_SMEM);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_ao_near<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)NEAR_SMEM);
+    return e;
 }
 
 // uni: one scene and grid for the whole batch; near > 0: with a near pass of
@@ -2044,9 +2097,14 @@ static cudaError_t configure_ao() {
 template <class R>
 static void launch_ao(const BatchDev& bd, bool uni, int near, int grid, int block, cudaStream_t stream) {
     if (std::is_same<R, double>::value) {
-        launch_dependent(k_ao_walk64, grid, block, 0, stream, bd);
+        if (near > 0) {
+            launch_dependent(k_ao_near<true>, near, NEAR_BLOCK, NEAR_SMEM, stream, bd);
+            launch_dependent(k_ao_walk64<true>, grid, block, 0, stream, bd);
+        } else {
+            launch_dependent(k_ao_walk64<false>, grid, block, 0, stream, bd);
+        }
     } else if (near > 0) {
-        launch_dependent(k_ao_near, near, NEAR_BLOCK, NEAR_SMEM, stream, bd);
+        launch_dependent(k_ao_near<false>, near, NEAR_BLOCK, NEAR_SMEM, stream, bd);
         if (uni) launch_dependent(k_ao_walk<true, true>, grid, block, ao_smem<true, true>(block), stream, bd);
         else launch_dependent(k_ao_walk<false, true>, grid, block, ao_smem<false, true>(block), stream, bd);
     } else {
@@ -2079,7 +2137,9 @@ static int grids_for(Ctx* ctx, int precision, bool uni, bool near, Grids& g) {
         if (configure_ao() != cudaSuccess) return GBRT_EDEVICE;
         ctx->smem_configured = true;
     }
-    g.near = near ? persistent_grid(ctx, k_ao_near, NEAR_BLOCK, NEAR_SMEM) : 0;
+    g.near = !near ? 0
+             : precision == GBRT_FP32 ? persistent_grid(ctx, k_ao_near<false>, NEAR_BLOCK, NEAR_SMEM)
+                                      : persistent_grid(ctx, k_ao_near<true>, NEAR_BLOCK, NEAR_SMEM);
     if (precision == GBRT_FP32) {
         g.primary = persistent_grid(ctx, k_primary<GBRT_FP32, false>, block);
         if (near)
@@ -2090,7 +2150,7 @@ static int grids_for(Ctx* ctx, int precision, bool uni, bool near, Grids& g) {
                        : persistent_grid(ctx, k_ao_walk<false, false>, block, ao_smem<false, false>(block));
     } else {
         g.primary = persistent_grid(ctx, k_primary<GBRT_FP64, false>, block);
-        g.ao = persistent_grid(ctx, k_ao_walk64, block);
+        g.ao = near ? persistent_grid(ctx, k_ao_walk64<true>, block) : persistent_grid(ctx, k_ao_walk64<false>, block);
     }
     g.shade = ctx->num_sms * 8;
     g.resolve = ctx->num_sms * 4;
@@ -2114,7 +2174,7 @@ static bool one_scene(const FrameDev* frames, int n) {
 // per-hit work, no limit on their length (the pass takes a hit at any distance
 // for one), and objects small enough (grid.rho).
 static bool near_pass_suits(const FrameDev& f) {
-    return f.precision == GBRT_FP32 && f.grid.rho > 0.0f && std::isinf(f.ao_maxdist_f) &&
+    return f.grid.rho > 0.0f && std::isinf(f.ao_maxdist_f) &&
            f.jobs_per_hit >= NEAR_MIN_JOBS && f.jobs_per_hit <= NEAR_MAX_JOBS;
 }
 
@@ -2259,7 +2319,10 @@ int render_frames(Ctx* ctx, FrameDev* frames, int n, bool use_graph) {
         return rc;
     // enough of them to keep every warp of one more kernel busy, and at least
     // half of the batch's rays
-    const bool near = near_recs >= NEAR_MIN_RECS && 2 * near_rays >= all_rays && !many;
+    const bool uni = one_scene(frames, n);
+    const bool near = precision == GBRT_FP32
+                          ? near_recs >= NEAR_MIN_RECS && 2 * near_rays >= all_rays && !many
+                          : near_recs >= NEAR_MIN_RECS64 && near_rays == all_rays && !many && uni;
     const size_t units_at = (size_t)recs * sizeof(TileRec);
     const size_t masks_at = units_at + 4 * (size_t)recs * sizeof(unsigned long long);
     if (near &&
@@ -2308,7 +2371,6 @@ int render_frames(Ctx* ctx, FrameDev* frames, int n, bool use_graph) {
     bd.refill = ctx->tuning.refill;
     ctx->counters_bytes_used = counters_bytes;
 
-    const bool uni = one_scene(frames, n);
     if (uni) extra |= EXTRA_UNI;
     Grids gr;
     if ((rc = grids_for(ctx, precision, uni, near, gr)) != GBRT_OK) return rc;
@@ -2368,7 +2430,7 @@ int enqueue_prepared(BatchDev bd, int precision, long long tiles, cudaStream_t s
     if (patch) k_patch_grids<<<1, 128, 0, stream>>>(bd);
     const auto none = [](int) {};
     const int ao = precision == GBRT_FP32 ? grid_of(k_ao_walk<true, false>, ao_smem<true, false>(block))
-                                          : grid_of(k_ao_walk64);
+                                          : grid_of(k_ao_walk64<false>);
     bd.ao_warps = ao * (block / 32);
     const int primary = precision == GBRT_FP32 ? grid_of(k_primary<GBRT_FP32, false>) : grid_of(k_primary<GBRT_FP64, false>);
     bd.parts = ray_parts(tiles, primary * (block / 32));

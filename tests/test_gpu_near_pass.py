@@ -119,3 +119,39 @@ def test_rebuilt_grid_and_mixed_batch(G):
         G.gbrt_sync(R.ctx)
         for a, b in zip(got, ref):
             assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("kind,spp,shadows,eps,far", [
+    ("globule", 16, False, 1e-3, 0.0), ("globule", 9, True, 1e-3, 0.0), ("globule", 17, False, 0.0, 0.0),
+    ("globule", 16, False, 1e-3, 3000.0), ("inside", 8, False, 1e-3, 0.0), ("tubes", 16, True, 1e-3, 0.0),
+    ("crowded", 16, False, 1e-3, 0.0)])
+def test_fp64_frame_with_and_without_the_near_pass(G, kind, spp, shadows, eps, far):
+    # far: the molecule stands away from the origin, where an FP32 coordinate
+    # is 2e-4 wide
+    import torch
+    sc = _scene(kind)
+    if far:
+        shift = np.array([far, -far, 0.5 * far])
+        sph, cyl = sc.spheres.copy(), sc.cylinders.copy()
+        sph[:, :3] += shift
+        cyl[:, :3] += shift
+        cyl[:, 3:6] += shift
+        sc = S.make_scene(sph, cyl)
+    cam, lights = _camera(sc, kind, 1), S.default_lights()
+    p = S.Params(ao_samples=spp, seed=5, eps=eps, shadows=shadows, precision=S.PRECISION_FP64)
+
+    def outputs():
+        return (torch.full((H, W, 3), -1.0, device="cuda", dtype=torch.float64),) + _outputs(torch, W, H, 1)[1:]
+
+    with G.Renderer(0) as R:
+        scene, grid = R.upload(sc, lam=8.0)
+        got, ref = outputs(), outputs()
+        n0 = G.gbrt_launch_count(R.ctx)
+        G.gbrt_render(R.ctx, scene, grid, cam, W, H, spp, lights, p, *got)
+        n1 = G.gbrt_launch_count(R.ctx)
+        _in_bands(G, R.ctx, scene, grid, cam, W, H, lights, p, ref)
+        n2 = G.gbrt_launch_count(R.ctx)
+        G.gbrt_sync(R.ctx)
+        assert n1 - n0 == 4 and n2 - n1 == BANDS * 3
+        for a, b in zip(got, ref):
+            assert torch.equal(a, b)
