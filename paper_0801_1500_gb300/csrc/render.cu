@@ -787,12 +787,14 @@ struct NearWarp {
 constexpr int NEAR_MAX_JOBS = 256;
 constexpr int NEAR_MIN_JOBS = 8;
 // A record takes a warp some 40 us, most of it latency, and the walk's units are
-// coarser than its own claims: the pass pays when every resident warp gets
-// several (1.1 MP, 21,000 records: frame 1.12 -> 0.93 ms; 5,900
-// records: 0.416 -> 0.437 ms). FP64 rays walk slower, and one a lane: there it
-// pays from 3,000 on (360 x 360 at 16 samples, 3,180 records: 0.392 -> 0.380 ms;
-// 640 x 640, 10,000: 0.940 -> 0.794 ms).
-constexpr double NEAR_MIN_RECS = 12288, NEAR_MIN_RECS64 = 3072;
+// coarser than its own claims: the pass pays when most resident warps get one or
+// two. Frame with and without it, 16 samples: 360 x 360 (3,200 records) 0.247 and
+// 0.242 ms, 480 x 480 (5,600) 0.330 and 0.348, 640 x 640 (10,000) 0.474 and
+// 0.545. FP64 rays walk slower, and one a lane: 360 x 360 0.380 and 0.392 ms,
+// 640 x 640 0.794 and 0.940.
+// NEAR_FULL_RECS: with fewer records than this a tile's job words, which share
+// its gather, are dealt to several records.
+constexpr double NEAR_MIN_RECS = 4608, NEAR_MIN_RECS64 = 3072, NEAR_FULL_RECS = 12288;
 
 // Largest b - q over the n candidates at c, for each of the NS directions: b =
 // w.d with w = centre - o, q = sqrt(|w|^2 - r^2). The ray meets a ball ahead of
@@ -816,6 +818,7 @@ __device__ __forceinline__ float near_q(float4 A, float q2, const NearSkip& skip
 template <int NS, bool F64>
 __device__ __forceinline__ void near_scan(const float4* c, int n, V3<float> o, V3<float> ol, const float (&d)[NS][3],
                                           float (&m)[NS], const NearSkip& skip, bool& bad) {
+#pragma unroll 1
     for (int k = 0; k < n; k += 2) {
         const float4 A = c[k], B = c[k + 1 < n ? k + 1 : k];
         float ax = A.x - o.x, ay = A.y - o.y, az = A.z - o.z;
@@ -834,6 +837,30 @@ __device__ __forceinline__ void near_scan(const float4* c, int n, V3<float> o, V
     }
 }
 
+// Directions of cnt <= 8 jobs from j0 on, one hit a lane; which of them are rays.
+// One copy of this code for both widths of near_jobs, and not unrolled: the
+// kernel was short of instruction cache (0.35 -> 0.31 ms at 965 x 1137, with the
+// scan's loop not unrolled either; figure with lights, which alternates the
+// widths, 1.62 -> 1.17).
+template <bool F64>
+__device__ __forceinline__ uint32_t near_dirs(const FrameDev& F, NearWarp& S, int lane, int j0, int cnt, V3<float> nrm,
+                                           uint32_t q) {
+    uint32_t valid = 0u;
+#pragma unroll 1
+    for (int s = 0; s < cnt; ++s) {
+        V3<float> dir = nrm;
+        if (j0 + s < F.jobs_per_hit) {
+            float tmax;
+            uint32_t lbit;
+            if (ao_direction<float>(F, q, (uint32_t)(j0 + s), nrm, dir, tmax, lbit, F64)) valid |= 1u << s;
+        }
+        S.dir[s][0][lane] = dir.x;
+        S.dir[s][1][lane] = dir.y;
+        S.dir[s][2][lane] = dir.z;
+    }
+    return valid;
+}
+
 // NS jobs (from j0) of a work item's hits, one hit a lane: which are occluded
 // by a near sphere, which have to walk, which of those from the start, which
 // leave the objects' bounds before the near pass's reach.
@@ -843,24 +870,14 @@ __device__ __forceinline__ void near_jobs(const FrameDev& F, NearWarp& S, int la
                                           float delta, uint32_t& todo, uint32_t& start, uint32_t& escaped) {
     float d[NS][3], m[NS];
     uint32_t valid = 0u;
-    for (int h = 0; h < NS; h += 8) {
-        const int cnt = NS - h < 8 ? NS - h : 8;
-        for (int s = 0; s < cnt; ++s) {
-            V3<float> dir = nrm;
-            if (j0 + h + s < F.jobs_per_hit) {
-                float tmax;
-                uint32_t lbit;
-                if (ao_direction<float>(F, q, (uint32_t)(j0 + h + s), nrm, dir, tmax, lbit, F64)) valid |= 1u << (h + s);
-            }
-            S.dir[s][0][lane] = dir.x;
-            S.dir[s][1][lane] = dir.y;
-            S.dir[s][2][lane] = dir.z;
-        }
+    constexpr int W = NS < 8 ? NS : 8;
 #pragma unroll
-        for (int s = 0; s < NS; ++s)
-            if (s >= h && s < h + 8)
+    for (int h = 0; h < NS; h += W) {
+        valid |= near_dirs<F64>(F, S, lane, j0 + h, W, nrm, q) << h;
 #pragma unroll
-                for (int k = 0; k < 3; ++k) d[s][k] = S.dir[s - h][k][lane];
+        for (int s = 0; s < W; ++s)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) d[h + s][k] = S.dir[s][k][lane];
     }
     // spheres, then tubes, through the same code (it has to stay in the
     // instruction cache): what a sphere's ball surely stops is hit, what comes
@@ -975,7 +992,7 @@ __global__ void __launch_bounds__(128, 4) k_ao_near(const __grid_constant__ Batc
             // look less far, or not at all, where the hits' box with that
             // reach around it would hold more balls than pay (a pass of a
             // job word costs 70 instructions a ball, a walk about 95 a ray)
-            const float most = 9.0f * (float)min(F.jobs_per_hit, 16);
+            const float most = 8.0f * (float)min(F.jobs_per_hit, 16);
             for (int t = 0;; ++t) {
                 const float v = (ext.x + rho) * (ext.y + rho) * (ext.z + rho);
                 if (8.0f * v * F.grid.density <= most) break;
@@ -2284,7 +2301,7 @@ int render_frames(Ctx* ctx, FrameDev* frames, int n, bool use_graph) {
         // a record takes all of its tile's words (they share the gather) unless
         // that leaves too few records
         const double hit_tiles = std::max(1.0, (double)ftiles * hit_share(frames[f]));
-        const int per_tile = (int)std::min<double>(std::ceil(NEAR_MIN_RECS / hit_tiles),
+        const int per_tile = (int)std::min<double>(std::ceil(NEAR_FULL_RECS / hit_tiles),
                                                    (double)std::max(frames[f].mask_words, 1));
         frames[f].rec_words = std::max(1, (frames[f].mask_words + per_tile - 1) / per_tile);
         if (frames[f].near_pass) {
