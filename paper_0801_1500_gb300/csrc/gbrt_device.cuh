@@ -87,7 +87,6 @@ __device__ __forceinline__ V3<double> ld3(const double* p) { return v3(p[0], p[1
 // compiler chooses per kernel, and a pixel's bits would depend on which of the
 // primary kernels found its hit).
 __device__ __forceinline__ float square_less(float a, float b) { return __fsub_rn(__fmul_rn(a, a), b); }
-__device__ __forceinline__ double square_less(double a, double b) { return __dsub_rn(__dmul_rn(a, a), b); }
 __device__ __forceinline__ float dot_zyx(V3<float> a, V3<float> b) {
     return __fmaf_rn(a.z, b.z, __fmaf_rn(a.y, b.y, __fmul_rn(a.x, b.x)));
 }
@@ -220,59 +219,35 @@ __device__ __forceinline__ bool any_hit_object(ObjPtr<R> obj, uint32_t id, V3<R>
 
 // ---------------------------------------------------------------- grid walk
 
-template <class R>
-struct GridP;
-
-template <>
-struct GridP<float> {
-    static __device__ __forceinline__ float bs(const GridDev& g, int k) { return g.bs[k]; }
-    static __device__ __forceinline__ float rcp(float x) { return __fdividef(1.0f, x); }
-    static __device__ __forceinline__ float lo(const GridDev& g, int k) { return g.lo[k]; }
-    static __device__ __forceinline__ float hi(const GridDev& g, int k) { return g.hi[k]; }
-    static __device__ __forceinline__ float h(const GridDev& g, int k) { return g.h[k]; }
-    static __device__ __forceinline__ float inv_h(const GridDev& g, int k) { return g.inv_h[k]; }
-};
-
-template <>
-struct GridP<double> {
-    static __device__ __forceinline__ double bs(const GridDev& g, int k) { return g.bs64[k]; }
-    static __device__ __forceinline__ double rcp(double x) { return 1.0 / x; }
-    static __device__ __forceinline__ double lo(const GridDev& g, int k) { return g.lo64[k]; }
-    static __device__ __forceinline__ double hi(const GridDev& g, int k) { return g.hi64[k]; }
-    static __device__ __forceinline__ double h(const GridDev& g, int k) { return g.h64[k]; }
-    static __device__ __forceinline__ double inv_h(const GridDev& g, int k) { return g.inv_h64[k]; }
-};
-
 // Clip o + t d, t in [tmin, tmax], to the grid box and to the bounding sphere
 // of the objects (nothing can be hit outside either). inv = 1/d per axis
 // (unused where d is 0).
-template <class R>
-__device__ __forceinline__ bool clip_grid(const GridDev& g, V3<R> o, V3<R> d, V3<R> inv, R tmin, R tmax, R& t0,
-                                          R& t1) {
-    R a = tmin, b = tmax;
-    const R oo[3] = {o.x, o.y, o.z};
-    const R dd[3] = {d.x, d.y, d.z};
-    const R ii[3] = {inv.x, inv.y, inv.z};
+__device__ __forceinline__ bool clip_grid(const GridDev& g, V3<float> o, V3<float> d, V3<float> inv, float tmin,
+                                          float tmax, float& t0, float& t1) {
+    float a = tmin, b = tmax;
+    const float oo[3] = {o.x, o.y, o.z};
+    const float dd[3] = {d.x, d.y, d.z};
+    const float ii[3] = {inv.x, inv.y, inv.z};
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        R lo = GridP<R>::lo(g, k), hi = GridP<R>::hi(g, k);
-        if (dd[k] == R(0)) {
+        float lo = g.lo[k], hi = g.hi[k];
+        if (dd[k] == 0.0f) {
             if (oo[k] < lo || oo[k] > hi) return false;
         } else {
-            R ta = (lo - oo[k]) * ii[k], tb = (hi - oo[k]) * ii[k];
-            R mn = ta < tb ? ta : tb, mx = ta < tb ? tb : ta;
+            float ta = (lo - oo[k]) * ii[k], tb = (hi - oo[k]) * ii[k];
+            float mn = ta < tb ? ta : tb, mx = ta < tb ? tb : ta;
             a = mn > a ? mn : a;
             b = mx < b ? mx : b;
         }
     }
     // bounding sphere: |o + t d - c| <= rb (|d| = 1)
-    V3<R> f = v3(o.x - GridP<R>::bs(g, 0), o.y - GridP<R>::bs(g, 1), o.z - GridP<R>::bs(g, 2));
-    R bb = dot(f, d);
-    V3<R> v = madd(f, -bb, d);
-    R rb = GridP<R>::bs(g, 3);
-    R disc = square_less(rb, dot(v, v));
-    if (disc < R(0)) return false;
-    R sq = Num<R>::sqrt_(disc);
+    V3<float> f = v3(o.x - g.bs[0], o.y - g.bs[1], o.z - g.bs[2]);
+    float bb = dot(f, d);
+    V3<float> v = madd(f, -bb, d);
+    float rb = g.bs[3];
+    float disc = square_less(rb, dot(v, v));
+    if (disc < 0.0f) return false;
+    float sq = Num<float>::sqrt_(disc);
     a = (-bb - sq) > a ? (-bb - sq) : a;
     b = (-bb + sq) < b ? (-bb + sq) : b;
     t0 = a;
@@ -280,13 +255,12 @@ __device__ __forceinline__ bool clip_grid(const GridDev& g, V3<R> o, V3<R> d, V3
     return a <= b;
 }
 
-template <class R>
-__device__ __forceinline__ V3<R> inv_dir(V3<R> d) {
-    return v3(GridP<R>::rcp(d.x), GridP<R>::rcp(d.y), GridP<R>::rcp(d.z));
+__device__ __forceinline__ V3<float> inv_dir(V3<float> d) {
+    return v3(rcp_(d.x), rcp_(d.y), rcp_(d.z));
 }
 
-template <class R>
-__device__ __forceinline__ bool clip_grid(const GridDev& g, V3<R> o, V3<R> d, R tmin, R tmax, R& t0, R& t1) {
+__device__ __forceinline__ bool clip_grid(const GridDev& g, V3<float> o, V3<float> d, float tmin, float tmax,
+                                          float& t0, float& t1) {
     return clip_grid(g, o, d, inv_dir(d), tmin, tmax, t0, t1);
 }
 
@@ -295,12 +269,11 @@ __device__ __forceinline__ bool clip_grid(const GridDev& g, V3<R> o, V3<R> d, R 
 // the t between crossings; the end of the clipped interval and the number of
 // cells (the walk's bounds); `left` counts down the steps (or, in the AO walk,
 // the lockstep iterations) a walk may take: nx + ny + nz + 3.
-template <class R>
 struct Walk {
     int stx, sty, stz;
-    R tnx, tny, tnz;
-    R tdx, tdy, tdz;
-    R t1;
+    float tnx, tny, tnz;
+    float tdx, tdy, tdz;
+    float t1;
     int cell;
     int left;
     unsigned ncells;
@@ -309,31 +282,29 @@ struct Walk {
 // One axis of the walk's set-up (selects, not branches: lanes differ in the
 // signs of their directions). Moving up the axis the next boundary is the
 // cell's upper face, moving down its lower face; a zero component never steps.
-template <class R>
-__device__ __forceinline__ void axis_setup(const GridDev& g, int k, R o, R d, R inv, int c, int stride, int& st,
-                                           R& tn, R& td) {
-    const bool up = d > R(0), down = d < R(0);
-    const R h = GridP<R>::h(g, k);
+__device__ __forceinline__ void axis_setup(const GridDev& g, int k, float o, float d, float inv, int c, int stride,
+                                           int& st, float& tn, float& td) {
+    const bool up = d > 0.0f, down = d < 0.0f;
+    const float h = g.h[k];
     st = up ? stride : (down ? -stride : 0);
-    const R face = GridP<R>::lo(g, k) + R(up ? c + 1 : c) * h;
-    tn = (up || down) ? (face - o) * inv : Num<R>::inf();
-    td = (up || down) ? (up ? h : -h) * inv : Num<R>::inf();
+    const float face = g.lo[k] + float(up ? c + 1 : c) * h;
+    tn = (up || down) ? (face - o) * inv : Num<float>::inf();
+    td = (up || down) ? (up ? h : -h) * inv : Num<float>::inf();
 }
 
-template <class R>
-__device__ __forceinline__ int cell_of(const GridDev& g, int k, R x) {
-    R f = floor((x - GridP<R>::lo(g, k)) * GridP<R>::inv_h(g, k));
+__device__ __forceinline__ int cell_of(const GridDev& g, int k, float x) {
+    float f = floor((x - g.lo[k]) * g.inv_h[k]);
     int c = (int)f;
     c = c < 0 ? 0 : c;
     return c > g.n[k] - 1 ? g.n[k] - 1 : c;
 }
 
-template <class R>
-__device__ __forceinline__ bool walk_start(const GridDev& g, V3<R> o, V3<R> d, R tmin, R tmax, Walk<R>& w) {
-    R t0, t1;
-    const V3<R> inv = inv_dir(d);
+__device__ __forceinline__ bool walk_start(const GridDev& g, V3<float> o, V3<float> d, float tmin, float tmax,
+                                           Walk& w) {
+    float t0, t1;
+    const V3<float> inv = inv_dir(d);
     if (g.empty || !clip_grid(g, o, d, inv, tmin, tmax, t0, t1)) return false;
-    V3<R> p = madd(o, t0, d);
+    V3<float> p = madd(o, t0, d);
     const int cx = cell_of(g, 0, p.x), cy = cell_of(g, 1, p.y), cz = cell_of(g, 2, p.z);
     const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
     axis_setup(g, 0, o.x, d.x, inv.x, cx, 1, w.stx, w.tnx, w.tdx);
@@ -350,7 +321,7 @@ __device__ __forceinline__ bool walk_start(const GridDev& g, V3<R> o, V3<R> d, R
 // corner (FP64 rays: the difference is formed in FP64 and rounded once, so the
 // walk's error stays relative to the grid's extent).
 __device__ __forceinline__ bool walk_start_rel(const GridDev& g, V3<float> o, V3<float> d, float tmin, float tmax,
-                                               Walk<float>& w) {
+                                               Walk& w) {
     if (g.empty) return false;
     const V3<float> inv = inv_dir(d);
     const float oo[3] = {o.x, o.y, o.z}, dd[3] = {d.x, d.y, d.z}, ii[3] = {inv.x, inv.y, inv.z};
@@ -398,9 +369,8 @@ __device__ __forceinline__ bool walk_start_rel(const GridDev& g, V3<float> o, V3
     return true;
 }
 
-template <class R>
-__device__ __forceinline__ R walk_cell_exit(const Walk<R>& w) {
-    R m = w.tnx < w.tny ? w.tnx : w.tny;
+__device__ __forceinline__ float walk_cell_exit(const Walk& w) {
+    float m = w.tnx < w.tny ? w.tnx : w.tny;
     return m < w.tnz ? m : w.tnz;
 }
 
@@ -415,12 +385,11 @@ __device__ __forceinline__ R walk_cell_exit(const Walk<R>& w) {
 // cost tests but change no result: every object the ray meets has its hit
 // point inside the grid, in a cell the walk visits before, and a test of any
 // other object finds only true intersections.
-template <class R>
-__device__ __forceinline__ bool walk_step(Walk<R>& w) {
+__device__ __forceinline__ bool walk_step(Walk& w) {
     const bool bx = w.tnx <= w.tny && w.tnx <= w.tnz;
     const bool by = !bx && w.tny <= w.tnz;
     const bool bz = !bx && !by;
-    const R tn = bx ? w.tnx : (by ? w.tny : w.tnz);
+    const float tn = bx ? w.tnx : (by ? w.tny : w.tnz);
     if (tn > w.t1) return false;
     w.tnx = bx ? w.tnx + w.tdx : w.tnx;
     w.tny = by ? w.tny + w.tdy : w.tny;
@@ -431,8 +400,7 @@ __device__ __forceinline__ bool walk_step(Walk<R>& w) {
 
 // walk_step within the walk's step bound: past it (only a walk whose crossing
 // times are not numbers can get there) the walk ends and *overflow is set.
-template <class R>
-__device__ __forceinline__ bool walk_next(Walk<R>& w, bool& overflow) {
+__device__ __forceinline__ bool walk_next(Walk& w, bool& overflow) {
     if (--w.left <= 0) {
         overflow = true;
         return false;
@@ -442,14 +410,12 @@ __device__ __forceinline__ bool walk_next(Walk<R>& w, bool& overflow) {
 
 // ---------------------------------------------------------------- traversal
 
-template <class R>
 struct Nearest {
-    R t1, t2;
+    float t1, t2;
     uint32_t id1, id2;
 };
 
-template <class R>
-__device__ __forceinline__ void nearest_consider(Nearest<R>& h, uint32_t id, R t) {
+__device__ __forceinline__ void nearest_consider(Nearest& h, uint32_t id, float t) {
     if (id == h.id1) return;  // the same object listed in another cell
     if (t < h.t1 || (t == h.t1 && id < h.id1)) {
         h.t2 = h.t1;
@@ -469,7 +435,7 @@ __device__ __forceinline__ void nearest_consider(Nearest<R>& h, uint32_t id, R t
 // on = false); visit() tests the cell's objects and best() is the nearest hit
 // so far.
 template <class Visit, class Best>
-__device__ __forceinline__ void split_walk(Walk<float>& w, bool on, int sub, int parts, bool& overflow, Visit visit,
+__device__ __forceinline__ void split_walk(Walk& w, bool on, int sub, int parts, bool& overflow, Visit visit,
                                            Best best) {
     for (int q = 0; q < sub && on; ++q) on = walk_next(w, overflow);
     while (__any_sync(0xffffffffu, on)) {
@@ -486,8 +452,8 @@ __device__ __forceinline__ void split_walk(Walk<float>& w, bool on, int sub, int
 // visited cell is listed there).
 template <bool SPLIT>
 __device__ __forceinline__ void trace_nearest(const GridDev& g, const SceneDev& s, V3<float> o, V3<float> d, bool on,
-                                              int sub, int parts, Nearest<float>& h, bool& overflow) {
-    Walk<float> w;
+                                              int sub, int parts, Nearest& h, bool& overflow) {
+    Walk w;
     on = on && walk_start(g, o, d, 0.0f, Num<float>::inf(), w);
     auto visit = [&] {
         uint2 cr = __ldg(g.cells + GBRT_INDEX(w.cell, g.ncells));

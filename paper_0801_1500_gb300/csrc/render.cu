@@ -259,13 +259,13 @@ __device__ __forceinline__ void entry_point(const Ff3& o, const Ff3& d, float te
 // scene).
 template <bool SPLIT>
 __device__ __forceinline__ void nearest_fp32(const FrameDev& f, int i, int j, bool on, int sub, int parts, float& te0,
-                                             Nearest<float>& h, bool& overflow) {
+                                             Nearest& h, bool& overflow) {
     if (!SPLIT && !on) return;
     const float inf = Num<float>::inf();
     Ff3 o, d, x;
     primary_ray_ff(f, i, j, o, d);
     float te1;
-    if (!clip_grid<float>(f.grid, o.hi, d.hi, 0.0f, inf, te0, te1)) {
+    if (!clip_grid(f.grid, o.hi, d.hi, 0.0f, inf, te0, te1)) {
         if (!SPLIT) return;
         on = false;
     }
@@ -283,7 +283,7 @@ __device__ __forceinline__ void nearest_fp32(const FrameDev& f, int i, int j, bo
 
 // The winner -- and a runner-up within a relative 1e-4 band -- refined in its
 // object's frame (local_root); the nearer refined root wins.
-__device__ __forceinline__ void refine_fp32(const FrameDev& f, int i, int j, float te0, const Nearest<float>& h,
+__device__ __forceinline__ void refine_fp32(const FrameDev& f, int i, int j, float te0, const Nearest& h,
                                             uint32_t& id, LocalHit& lh) {
     // the refinement needs what the rounding left out: the ray and its entry
     // point are formed again (the same steps give the same floats), which is
@@ -437,7 +437,7 @@ __device__ __forceinline__ void nearest_filtered64(const FrameDev& f, int i, int
     const V3<float> lo = v3(g.lo[0], g.lo[1], g.lo[2]);
     const V3<float> xr = (x.hi - lo) + x.lo;
     const V3<float> df = d.hi;
-    Walk<float> w;
+    Walk w;
     on = on && walk_start_rel(g, xr, df, 0.0f, inf, w);
     if (!SPLIT && !on) return;
     const float om = 0.1f * fmaxf(g.hi[0] - lo.x, fmaxf(g.hi[1] - lo.y, g.hi[2] - lo.z));
@@ -595,7 +595,7 @@ __global__ void __launch_bounds__(256) k_primary(const __grid_constant__ BatchDe
         bool hit = false;
         if (MODE == GBRT_FP32) {
             float te0 = 0.0f;
-            Nearest<float> h;
+            Nearest h;
             h.t1 = h.t2 = Num<float>::inf();
             h.id1 = h.id2 = GBRT_MISS;
             nearest_fp32<SPLIT>(F, i, j, inside, sub, parts, te0, h, overflow);
@@ -838,10 +838,9 @@ __device__ __forceinline__ void near_scan(const float4* c, int n, V3<float> o, V
 }
 
 // Directions of cnt <= 8 jobs from j0 on, one hit a lane; which of them are rays.
-// One copy of this code for both widths of near_jobs, and not unrolled: the
-// kernel was short of instruction cache (0.35 -> 0.31 ms at 965 x 1137, with the
-// scan's loop not unrolled either; figure with lights, which alternates the
-// widths, 1.62 -> 1.17).
+// Not unrolled, like the scan's loop: the kernel was short of instruction cache
+// (0.35 -> 0.31 ms at 965 x 1137; the figure with two lights, 16 + 2 jobs a hit,
+// which goes from one width of near_jobs to the other, 1.62 -> 1.16 ms).
 template <bool F64>
 __device__ __forceinline__ uint32_t near_dirs(const FrameDev& F, NearWarp& S, int lane, int j0, int cnt, V3<float> nrm,
                                            uint32_t q) {
@@ -871,6 +870,7 @@ __device__ __forceinline__ void near_jobs(const FrameDev& F, NearWarp& S, int la
     float d[NS][3], m[NS];
     uint32_t valid = 0u;
     constexpr int W = NS < 8 ? NS : 8;
+    // (unrolled by order: rolled, nvcc 13.0 loses the first eight directions)
 #pragma unroll
     for (int h = 0; h < NS; h += W) {
         valid |= near_dirs<F64>(F, S, lane, j0 + h, W, nrm, q) << h;
@@ -927,17 +927,17 @@ __device__ __forceinline__ void near_jobs(const FrameDev& F, NearWarp& S, int la
 // a tube's ball, walks from its start: tubes are cut to what sticks out of
 // their atoms, so that is one ray in a hundred. The decisions are those of the
 // walk's own test (delta is ten times the rounding of both).
-// Measured (965 x 1137, 16 samples, 9.0 M AO rays): 148 balls a tile; 37% of the
-// rays hit, 13% left the bounds, 1% open; 243 M warp instructions (gather 39 M,
-// directions 48 M, scan 155 M) in 0.35 ms, and the walk 1.00 -> 0.44 ms. 3860 x
-// 4548: frame 15.9 -> 11.1 ms. Instruction issue (0.6 a cycle: 16 warps an SM,
-// for the directions in registers) bounds it. Tried: the scan as f16-pair
+// Measured (965 x 1137, 16 samples, 9.0 M AO rays): 140 balls a tile; 37% of the
+// rays hit, 13% left the bounds, 1% open; some 240 M warp instructions (gather 39
+// M, directions 48 M, scan 150 M) in 0.31 ms, and the walk 1.00 -> 0.45 ms. 3860 x
+// 4548: frame 15.8 -> 10.3 ms. Instruction issue (16 warps an SM, for the
+// directions in registers) and the instruction cache bound it. Tried: the scan as f16-pair
 // m16n8k16 mma.sync (13.7 cycles a 128 pairs, no faster than the FMAs), packed
 // f32x2 FMAs (20% fewer instructions, 10% slower), a row of cells per lane in
 // the gather (55 dependent rounds of loads instead of 16: 0.44 ms).
 // F64: the same for FP64 frames, whose decisions delta covers as well (the
 // directions are the FP32 ones the walk filters with, the origins float pairs):
-// 0.38 ms, and the walk 1.53 -> 0.78 (965 x 1137, frame 1.87 -> 1.48 ms).
+// 0.32 ms, and the walk 1.53 -> 0.79 (965 x 1137, frame 1.87 -> 1.46 ms).
 template <bool F64>
 __global__ void __launch_bounds__(128, 4) k_ao_near(const __grid_constant__ BatchDev b) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1331,7 +1331,7 @@ __global__ void __launch_bounds__(256) k_ao_walk(const __grid_constant__ BatchDe
     const unsigned long long total = NEAR ? *b.nunits : b.job_off[b.nframes];
     const int refill = b.refill;
     bool has = false, exhausted = false, overflow = false;
-    Walk<float> w;
+    Walk w;
     unsigned nf = 0;      // cells waiting in this lane's fifo
     bool wend = false;    // the walk has no further cells
     uint32_t lbit = 0;  // 0: an AO sample; 1 << l: the shadow ray toward light l
@@ -1606,7 +1606,7 @@ __device__ __forceinline__ void lane_walk(Src& src, LaneScene& A, int refill, ui
     const int lane = threadIdx.x & 31;
     bool active = false, exhausted = false, overflow = false;
     LaneRay ray;
-    Walk<float> w;
+    Walk w;
     uint32_t k = 0, e = 0;         // items left of the lane's cell
     uint2 nxt = make_uint2(0, 0);  // the next cell's record, when more
     bool more = false;
@@ -1738,7 +1738,7 @@ struct FrameRays {
 
     // Job smp of the hit in `slot`, from distance tmin on.
     __device__ __forceinline__ void set_up(const FrameDev& F, int fi, int64_t slot, uint32_t smp, float tmin,
-                                           LaneRay& ray, Walk<float>& w, bool& fresh) {
+                                           LaneRay& ray, Walk& w, bool& fresh) {
         uint32_t q, own;
         V3<float> nrm;
         ray.slot = slot;
@@ -1751,7 +1751,7 @@ struct FrameRays {
         }
     }
 
-    __device__ __forceinline__ int refill(LaneScene& A, int lane, unsigned act, bool free, LaneRay& ray, Walk<float>& w,
+    __device__ __forceinline__ int refill(LaneScene& A, int lane, unsigned act, bool free, LaneRay& ray, Walk& w,
                                           bool& fresh) {
         if constexpr (NEAR) {
             if (!A.cells) A.set(b.frames[0]);
@@ -1802,11 +1802,11 @@ struct FrameRays {
 // AO walk of FP64 frames, persistent. With every test and step in FP64 (1/64
 // of the FP32 rate) the FP64 pipe was 87% busy and the walk took 15.5 of a
 // 965 x 1137 frame's 17.9 ms; the filter leaves FP64 to one pair in some ten
-// thousand (walk 1.7 ms; 256 x 256 frame at 8 samples 0.57 -> 0.11 ms). One
+// thousand (walk 1.53 ms; 256 x 256 frame at 8 samples 0.57 -> 0.09 ms). One
 // ray a lane rather than the FP32 frames' pair expansion: with a filter this
 // cheap the expansion costs more than the idle lanes (walk 3.8 ms with pairs
-// queued in shared memory). Bound now by instruction issue. NEAR: after a near
-// pass, over the rays it left (0.78 ms).
+// queued in shared memory). Bound now by instruction issue and load
+// latency. NEAR: after a near pass, over the rays it left (0.79 ms).
 template <bool NEAR>
 __global__ void __launch_bounds__(256, 3) k_ao_walk64(const __grid_constant__ BatchDev b) {
     __shared__ AoUnit units[NEAR ? 8 : 1];
@@ -1943,7 +1943,7 @@ struct ProbeRays {
         return any_hit_object<double>(F.scene.obj64, id, o, d, tmax);
     }
 
-    __device__ __forceinline__ int refill(LaneScene&, int lane, unsigned act, bool free, LaneRay& ray, Walk<float>& w,
+    __device__ __forceinline__ int refill(LaneScene&, int lane, unsigned act, bool free, LaneRay& ray, Walk& w,
                                           bool& fresh) {
         if (pool == pool_end) return LANES_END;
         const unsigned idle = ~act, i = __popc(idle & ((1u << lane) - 1u));
@@ -2199,10 +2199,11 @@ static bool near_pass_suits(const FrameDev& f) {
 // kernel has warps is bound by the latency of its slowest warp, a chain of
 // dependent loads and tests (cell, item, object): 128 x 96 pixels, 36 us of
 // which the mean warp is busy for 7. Then 2, 4 or 8 lanes walk a ray between
-// them: 29 us with 8 at 128 x 96 (a frame 66.7 -> 59.4), a 256 x 256 frame
-// 75.2 -> 72.8 with 2. With more lanes than keep every tile resident at once
-// the cells visited past the hit cost more than they hide (256 x 256: 4 lanes
-// 75.7, 8 lanes 88.6; FP64 195 us with one lane, 217 with 4).
+// them: 29 us with 8 at 128 x 96 (a frame of 520 atoms 66.7 -> 59.4, of 128,200
+// atoms 127 -> 87), a 256 x 256 frame 75.2 -> 72.8 and 145 -> 134 with 2. With
+// more lanes than keep every tile resident at once the cells visited past the
+// hit cost more than they hide (256 x 256: 4 lanes 75.7, 8 lanes 88.6; FP64 195
+// us with one lane, 217 with 4).
 static int ray_parts(long long tiles, int warps) {
     int parts = 1;
     while (parts < 8 && 2 * parts * tiles <= warps) parts *= 2;
@@ -2449,7 +2450,8 @@ int enqueue_prepared(BatchDev bd, int precision, long long tiles, cudaStream_t s
     const int ao = precision == GBRT_FP32 ? grid_of(k_ao_walk<true, false>, ao_smem<true, false>(block))
                                           : grid_of(k_ao_walk64<false>);
     bd.ao_warps = ao * (block / 32);
-    const int primary = precision == GBRT_FP32 ? grid_of(k_primary<GBRT_FP32, false>) : grid_of(k_primary<GBRT_FP64, false>);
+    const int primary = precision == GBRT_FP32 ? grid_of(k_primary<GBRT_FP32, false>)
+                                               : grid_of(k_primary<GBRT_FP64, false>);
     bd.parts = ray_parts(tiles, primary * (block / 32));
     if (precision == GBRT_FP32) {
         launch_primary<GBRT_FP32>(bd, primary, block, stream);
