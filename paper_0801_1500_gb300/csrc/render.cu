@@ -394,31 +394,55 @@ __device__ __noinline__ double exact_root64(const FrameDev& f, int i, int j, uin
 // to grazing, to the tube's end or to the ray's start, and two roots closer
 // than their errors. The object is the one an FP64 walk finds; its FP64 root
 // is formed by the caller, once per hit pixel instead of once per candidate
-// (965 x 1137 frame, this kernel: 2.40 -> 0.215 ms; 256 x 256: 0.39 ->
-// 0.057 ms. The FP64 pipe was the bound; now the walk's load latency and the
-// winners' ~200 FP64 instructions are).
+// (965 x 1137 frame, this kernel: 2.40 -> 0.205 ms; 256 x 256: 0.39 ->
+// 0.048 ms. The FP64 pipe was the bound; now the walk's load latency and the
+// winners' ~140 FP64 instructions are).
 struct Near64 {
-    uint32_t id;     // GBRT_MISS: none
-    float t, e;      // its root from the grid entry, and that root's error
+    uint32_t id;    // GBRT_MISS: none
+    float t, e;     // its root from the grid entry, and that root's error
+    uint32_t pend;  // a candidate that only FP64 can place (GBRT_MISS: none)
+    float lo;       // which has no root before this
 };
 
-// A candidate's root (or, open, a candidate that may have one) joins h.
-__device__ __forceinline__ void near64_consider(const FrameDev& f, int i, int j, float te0, Near64& h, uint32_t cand,
-                                                bool open, float t, float et) {
-    bool nearer = t + et < h.t - h.e;
-    if (open || !(nearer || t - et > h.t + h.e)) {
-        const double t64 = exact_root64(f, i, j, cand);
-        if (t64 == Num<double>::inf()) return;
-        const double b64 = h.id == GBRT_MISS ? Num<double>::inf() : exact_root64(f, i, j, h.id);
-        nearer = t64 < b64 || (t64 == b64 && cand < h.id);
-        t = (float)(t64 - (double)te0);
-        et = 2e-7f * fabsf(t);
-    }
-    if (nearer) {
+__device__ __forceinline__ void near64_settle(const FrameDev& f, int i, int j, float te0, Near64& h, uint32_t cand) {
+    const double t64 = exact_root64(f, i, j, cand);
+    if (t64 == Num<double>::inf()) return;
+    const double b64 = h.id == GBRT_MISS ? Num<double>::inf() : exact_root64(f, i, j, h.id);
+    if (t64 < b64 || (t64 == b64 && cand < h.id)) {
         h.id = cand;
-        h.t = t;
-        h.e = et;
+        h.t = (float)(t64 - (double)te0);
+        h.e = 2e-7f * fabsf(h.t);
     }
+}
+
+// A candidate's root (or, open, a candidate that may have one from lo on) joins
+// h. What FP64 has to decide waits, one candidate a lane, for the end of the walk:
+// most are behind the hit by then, and the warp's lanes settle theirs together (an
+// FP64 instruction occupies the SM's pipe as long for one lane as for 32).
+// Settled at once instead: 0.213 and 0.057 ms.
+__device__ __forceinline__ void near64_consider(const FrameDev& f, int i, int j, float te0, Near64& h, uint32_t cand,
+                                                bool open, float t, float et, float lo) {
+    if (!open) {
+        if (t + et < h.t - h.e) {
+            h.id = cand;
+            h.t = t;
+            h.e = et;
+            return;
+        }
+        lo = t - et;
+    }
+    if (lo > h.t + h.e || cand == h.pend) return;
+    if (h.pend == GBRT_MISS || h.lo > h.t + h.e) {
+        h.pend = cand;
+        h.lo = lo;
+    } else {
+        near64_settle(f, i, j, te0, h, cand);
+    }
+}
+
+__device__ __forceinline__ void near64_finish(const FrameDev& f, int i, int j, float te0, Near64& h) {
+    if (h.pend != GBRT_MISS && !(h.lo > h.t + h.e)) near64_settle(f, i, j, te0, h, h.pend);
+    h.pend = GBRT_MISS;
 }
 
 template <bool SPLIT>
@@ -464,7 +488,9 @@ __device__ __forceinline__ void nearest_filtered64(const FrameDev& f, int i, int
                 Obj<float>::load(f.scene.obj, cand, p0, a, L, rr);
                 what = tube_root32(xr, df, p0 - lo, a, L, rr, inf, inf, om, t, et);
             }
-            if (what != PAIR_MISS) near64_consider(f, i, j, te0, h, cand, what == PAIR_OPEN, t, et);
+            // (no root of what lies in the ball comes before the ball)
+            const float front = tc - 1.001f * sqrt_pos(mg - x2) - 1e-5f * (fabsf(tc) + r + om);
+            if (what != PAIR_MISS) near64_consider(f, i, j, te0, h, cand, what == PAIR_OPEN, t, et, front);
         }
     };
     if (!SPLIT) {
@@ -472,14 +498,17 @@ __device__ __forceinline__ void nearest_filtered64(const FrameDev& f, int i, int
             visit();
             if (h.id != GBRT_MISS && h.t <= walk_cell_exit(w)) break;
         } while (walk_next(w, overflow));
+        near64_finish(f, i, j, te0, h);
         return;
     }
     split_walk(w, on, sub, parts, overflow, visit, [&] { return h.t; });
+    near64_finish(f, i, j, te0, h);
     // the lanes' hits, merged
     for (int x = 1; x < parts; x <<= 1) {
         const uint32_t k = __shfl_xor_sync(FULL, h.id, x);
         const float t = __shfl_xor_sync(FULL, h.t, x), e = __shfl_xor_sync(FULL, h.e, x);
-        if (k != GBRT_MISS && k != h.id) near64_consider(f, i, j, te0, h, k, false, t, e);
+        if (k != GBRT_MISS && k != h.id) near64_consider(f, i, j, te0, h, k, false, t, e, t);
+        near64_finish(f, i, j, te0, h);
     }
 }
 
@@ -539,8 +568,8 @@ __device__ __forceinline__ double ao_maxdist<double>(const FrameDev& f) { return
 // AO rays a warp claims from the global queue at once (its local pool): 64, and
 // fewer, down to 8, where 64 would leave warps without any. A small frame's AO
 // pass is one round of such claims, bound by the latency of one warp's rays:
-// 41 -> 30 us at 256 x 256, 4 samples; 33 -> 21 us at 128 x 96; FP64, 256 x 256
-// at 8: 105 -> 88 us (64 at once against this).
+// 41 -> 30 us at 256 x 256, 4 samples; 33 -> 21 us at 128 x 96 (64 at once
+// against this; shares of a half or a quarter: 34 us at 256 x 256).
 __device__ __forceinline__ unsigned ao_claim(unsigned long long rays, int warps) {
     const unsigned long long share = rays / (unsigned)warps + 1ull;
     return share >= 64ull ? 64u : share <= 8ull ? 8u : (unsigned)(share + 7ull) & ~7u;
@@ -603,9 +632,9 @@ __global__ void __launch_bounds__(256) k_primary(const __grid_constant__ BatchDe
             if (hit) refine_fp32(F, i, j, te0, h, id, lh);
         } else {
             Near64 h;
-            h.id = GBRT_MISS;
+            h.id = h.pend = GBRT_MISS;
             h.t = Num<float>::inf();
-            h.e = 0.0f;
+            h.e = h.lo = 0.0f;
             nearest_filtered64<SPLIT>(F, i, j, inside, sub, parts, h, overflow);
             id = h.id;
             hit = mine && id != GBRT_MISS;
