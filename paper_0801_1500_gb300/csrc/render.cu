@@ -830,23 +830,33 @@ constexpr double NEAR_MIN_RECS = 4608, NEAR_MIN_RECS64 = 3072, NEAR_FULL_RECS = 
 // an outside origin exactly when b >= q. w and q are per (hit, ball), so a
 // (ray, ball) pair costs three FMAs and half a three-input maximum. An origin
 // inside or within 5e-5 r of a ball sets bad (q would be too rough there),
-// unless it is the ball of the tube that the hit lies on (skip, its centre):
-// rays from a tube's outer side do not meet it again. An FP64 origin is o + ol
+// unless it is the ball of the tube that the hit lies on (skip): rays from a
+// tube's outer side do not meet it again. An FP64 origin is o + ol
 // (float pairs: w then has FP32's relative error however large the coordinates).
+//
+// The tube is known by its ball, of which it is one of the candidates: the ball
+// holds the origin, so neither the reach nor the tangent planes drop it. A ball
+// with the same centre and radius may still be another tube's (the arms of a
+// cross, a tube drawn twice); it holds the origin as well, so of several such
+// candidates one is passed over and the next sets bad.
 struct NearSkip {
     bool on;
     V3<float> c;
+    float r;
 };
-__device__ __forceinline__ float near_q(float4 A, float q2, const NearSkip& skip, bool& bad) {
+__device__ __forceinline__ float near_q(float4 A, float q2, const NearSkip& skip, bool& left, bool& bad) {
     if (q2 < 1e-4f * A.w * A.w) {
-        if (skip.on && A.x == skip.c.x && A.y == skip.c.y && A.z == skip.c.z) return Num<float>::inf();
+        if (left && A.x == skip.c.x && A.y == skip.c.y && A.z == skip.c.z && A.w == skip.r) {
+            left = false;
+            return Num<float>::inf();
+        }
         bad = true;
     }
     return sqrt_pos(q2);
 }
 template <int NS, bool F64>
 __device__ __forceinline__ void near_scan(const float4* c, int n, V3<float> o, V3<float> ol, const float (&d)[NS][3],
-                                          float (&m)[NS], const NearSkip& skip, bool& bad) {
+                                          float (&m)[NS], const NearSkip& skip, bool left, bool& bad) {
 #pragma unroll 1
     for (int k = 0; k < n; k += 2) {
         const float4 A = c[k], B = c[k + 1 < n ? k + 1 : k];
@@ -858,7 +868,11 @@ __device__ __forceinline__ void near_scan(const float4* c, int n, V3<float> o, V
         }
         const float qa = fmaf(ax, ax, fmaf(ay, ay, fmaf(az, az, -A.w * A.w)));
         const float qb = fmaf(bx, bx, fmaf(by, by, fmaf(bz, bz, -B.w * B.w)));
-        const float na = -near_q(A, qa, skip, bad), nb = -near_q(B, qb, skip, bad);
+        const float na = -near_q(A, qa, skip, left, bad);
+        const bool more = k + 1 < n;  // else B is A again, not one more candidate (an own tube there only walks)
+        bool twin = false;
+        const float nb = -near_q(B, qb, skip, left, twin);
+        bad |= twin && more;
 #pragma unroll
         for (int s = 0; s < NS; ++s)
             m[s] = max3(m[s], fmaf(ax, d[s][0], fmaf(ay, d[s][1], fmaf(az, d[s][2], na))),
@@ -919,7 +933,7 @@ __device__ __forceinline__ void near_jobs(const FrameDev& F, NearWarp& S, int la
     for (int kind = 0; kind < 2; ++kind) {
 #pragma unroll
         for (int s = 0; s < NS; ++s) m[s] = -Num<float>::inf();
-        near_scan<NS, F64>(list, n, o, ol, d, m, skip, bad);
+        near_scan<NS, F64>(list, n, o, ol, d, m, skip, skip.on && kind == 1, bad);
         const float sure = kind == 0 ? delta : Num<float>::inf();
 #pragma unroll
         for (int s = 0; s < NS; ++s) {
@@ -996,6 +1010,7 @@ __global__ void __launch_bounds__(128, 4) k_ao_near(const __grid_constant__ Batc
         int ns = 0, nt = 0;
         NearSkip skip;
         skip.on = false;
+        skip.r = 0.0f;
         if (rho > 0.0f) {
             // a hit on a tube's outer side: its origin may lie inside the tube's ball
             V3<float> p0, a;
@@ -1005,8 +1020,9 @@ __global__ void __launch_bounds__(128, 4) k_ao_near(const __grid_constant__ Batc
             if (L > 0.0f) {
                 const V3<float> w = (o - p0) + ol, wp = madd(w, -dot(w, a), a);
                 const float4 c = __ldg(F.grid.cut + own);
-                skip.on = dot(wp, wp) > 1.0002f * r * r;  // surely outside
+                skip.on = c.w < 0.0f && dot(wp, wp) > 1.0002f * r * r;  // surely outside
                 skip.c = v3(c.x, c.y, c.z);
+                skip.r = -c.w;
             }
             // the hits' box, its centre, and the cone of their normals
             const V3<float> mn = v3(warp_min(o.x), warp_min(o.y), warp_min(o.z));
