@@ -392,7 +392,8 @@ __device__ __noinline__ double exact_root64(const FrameDev& f, int i, int j, uin
 // just before it enters the objects' bounds; each root carries its error, and
 // FP64 roots (exact_root64) decide where the bounds do not: a pair too close
 // to grazing, to the tube's end or to the ray's start, and two roots closer
-// than their errors. The object is the one an FP64 walk finds; its FP64 root
+// than their errors; the walk ends where the nearest root, with its error, lies
+// before the cell's exit. The object is the one an FP64 walk finds; its FP64 root
 // is formed by the caller, once per hit pixel instead of once per candidate
 // (965 x 1137 frame, this kernel: 2.40 -> 0.205 ms; 256 x 256: 0.39 ->
 // 0.048 ms. The FP64 pipe was the bound; now the walk's load latency and the
@@ -496,12 +497,12 @@ __device__ __forceinline__ void nearest_filtered64(const FrameDev& f, int i, int
     if (!SPLIT) {
         do {
             visit();
-            if (h.id != GBRT_MISS && h.t <= walk_cell_exit(w)) break;
+            if (h.id != GBRT_MISS && h.t + h.e <= walk_cell_exit(w)) break;
         } while (walk_next(w, overflow));
         near64_finish(f, i, j, te0, h);
         return;
     }
-    split_walk(w, on, sub, parts, overflow, visit, [&] { return h.t; });
+    split_walk(w, on, sub, parts, overflow, visit, [&] { return h.t + h.e; });
     near64_finish(f, i, j, te0, h);
     // the lanes' hits, merged
     for (int x = 1; x < parts; x <<= 1) {
