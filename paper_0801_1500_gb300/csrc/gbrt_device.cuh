@@ -317,6 +317,9 @@ __device__ __forceinline__ bool walk_start(const GridDev& g, V3<float> o, V3<flo
     return true;
 }
 
+// Steps after which an FP64 ray's walk forms its crossings anew (walk_next_rel).
+constexpr int WALK_RENEW = 32;
+
 // The same set-up for a ray whose origin is relative to the grid's lower
 // corner (FP64 rays: the difference is formed in FP64 and rounded once, so the
 // walk's error stays relative to the grid's extent).
@@ -365,7 +368,7 @@ __device__ __forceinline__ bool walk_start_rel(const GridDev& g, V3<float> o, V3
     w.ncells = (unsigned)g.ncells;
     w.t1 = t1;
     w.cell = (c[2] * g.n[1] + c[1]) * g.n[0] + c[0];
-    w.left = g.n[0] + g.n[1] + g.n[2] + 3;
+    w.left = (g.n[0] + g.n[1] + g.n[2] + 3 + WALK_RENEW) & ~(WALK_RENEW - 1);  // walk_next_rel counts in periods
     return true;
 }
 
@@ -408,6 +411,29 @@ __device__ __forceinline__ bool walk_next(Walk& w, bool& overflow) {
     return walk_step(w);
 }
 
+// walk_next for the walk of an FP64 ray (walk_start_rel). The cells' lists are
+// padded by 1e-5 of the grid's extent, and a walk of n steps adds up crossings
+// that are each wrong by up to 2^-24 of the path or twice that: 2000 steps
+// through a grid of 1000 cells a side were off by 2e-5 and missed objects. So
+// every WALK_RENEW steps the crossings are formed anew from the cell (wrong by
+// less than 4e-6 of the extent in between). A cell in another row, past the grid's edge,
+// is off by a whole cell and changes nothing.
+__device__ __forceinline__ float axis_renew(float tn, float o, float inv, int st, int c, float h, float t1) {
+    const float t = ((float)(st > 0 ? c + 1 : c) * h - o) * inv;
+    return st != 0 && fabsf(t - tn) <= 2e-5f * t1 ? t : tn;
+}
+__device__ __forceinline__ bool walk_next_rel(Walk& w, const GridDev& g, V3<float> o, V3<float> d, bool& overflow) {
+    if (!walk_next(w, overflow)) return false;
+    if ((w.left & (WALK_RENEW - 1)) == 0) {
+        const V3<float> inv = inv_dir(d);
+        const int nx = g.n[0], ny = g.n[1], row = w.cell / nx;
+        w.tnx = axis_renew(w.tnx, o.x, inv.x, w.stx, w.cell - row * nx, g.h[0], w.t1);
+        w.tny = axis_renew(w.tny, o.y, inv.y, w.sty, row % ny, g.h[1], w.t1);
+        w.tnz = axis_renew(w.tnz, o.z, inv.z, w.stz, row / ny, g.h[2], w.t1);
+    }
+    return true;
+}
+
 // ---------------------------------------------------------------- traversal
 
 struct Nearest {
@@ -432,18 +458,18 @@ __device__ __forceinline__ void nearest_consider(Nearest& h, uint32_t id, float 
 // has the ray to itself): lane `sub` visits the cells sub, sub + parts, ... in
 // ray order, and the lanes share their best hit after each of these rounds.
 // The whole warp calls split_walk together (lanes with nothing to walk pass
-// on = false); visit() tests the cell's objects and best() is the nearest hit
-// so far.
-template <class Visit, class Best>
-__device__ __forceinline__ void split_walk(Walk& w, bool on, int sub, int parts, bool& overflow, Visit visit,
+// on = false); next() steps to the next cell, visit() tests the cell's objects
+// and best() is the nearest hit so far.
+template <class Next, class Visit, class Best>
+__device__ __forceinline__ void split_walk(const Walk& w, bool on, int sub, int parts, Next next, Visit visit,
                                            Best best) {
-    for (int q = 0; q < sub && on; ++q) on = walk_next(w, overflow);
+    for (int q = 0; q < sub && on; ++q) on = next();
     while (__any_sync(0xffffffffu, on)) {
         if (on) visit();
         float m = best();
         for (int x = 1; x < parts; x <<= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, x));
         if (on && m < Num<float>::inf() && m <= walk_cell_exit(w)) on = false;
-        for (int q = 0; q < parts && on; ++q) on = walk_next(w, overflow);
+        for (int q = 0; q < parts && on; ++q) on = next();
     }
 }
 
@@ -464,7 +490,7 @@ __device__ __forceinline__ void trace_nearest(const GridDev& g, const SceneDev& 
         }
     };
     if (SPLIT) {
-        split_walk(w, on, sub, parts, overflow, visit, [&] { return h.t1; });
+        split_walk(w, on, sub, parts, [&] { return walk_next(w, overflow); }, visit, [&] { return h.t1; });
         return;
     }
     if (!on) return;

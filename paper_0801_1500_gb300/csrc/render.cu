@@ -494,15 +494,16 @@ __device__ __forceinline__ void nearest_filtered64(const FrameDev& f, int i, int
             if (what != PAIR_MISS) near64_consider(f, i, j, te0, h, cand, what == PAIR_OPEN, t, et, front);
         }
     };
+    auto next = [&] { return walk_next_rel(w, g, xr, df, overflow); };
     if (!SPLIT) {
         do {
             visit();
             if (h.id != GBRT_MISS && h.t + h.e <= walk_cell_exit(w)) break;
-        } while (walk_next(w, overflow));
+        } while (next());
         near64_finish(f, i, j, te0, h);
         return;
     }
-    split_walk(w, on, sub, parts, overflow, visit, [&] { return h.t + h.e; });
+    split_walk(w, on, sub, parts, next, visit, [&] { return h.t + h.e; });
     near64_finish(f, i, j, te0, h);
     // the lanes' hits, merged
     for (int x = 1; x < parts; x <<= 1) {
@@ -1707,7 +1708,8 @@ __device__ __forceinline__ void lane_walk(Src& src, LaneScene& A, int refill, ui
             if (more) {
                 k = nxt.x;
                 e = nxt.x + nxt.y;
-                more = walk_next(w, overflow);
+                if constexpr (Src::F64) more = walk_next_rel(w, src.frame(ray).grid, ray.o, ray.d, overflow);
+                else more = walk_next(w, overflow);
                 if (more) nxt = __ldg(A.cells + GBRT_INDEX(w.cell, w.ncells));
             } else if (!test) {
                 // walk over: nothing left to test
