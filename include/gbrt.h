@@ -281,7 +281,9 @@ GBRT_API int gbrt_grid_free(gbrt_ctx* ctx, gbrt_grid* grid);
  * checked on the device: a bad value makes the next gbrt_sync return
  * GBRT_EINVAL, and the scene's geometry is then unspecified until the next
  * good update. Grids built on the scene keep their contents until
- * gbrt_grid_rebuild. */
+ * gbrt_grid_rebuild: until then a render or probe through such a grid tests
+ * the new geometry, but only in the cells that the old one was listed in (right
+ * where objects have only shrunk), and without the AO near pass. */
 GBRT_API int gbrt_scene_update(gbrt_ctx* ctx, gbrt_scene* scene, const float* spheres, const float* cylinders,
                                int flags);
 

@@ -149,6 +149,7 @@ FrameDev make_frame(const gbrt_scene* scene, const gbrt_grid* grid, const gbrt_c
         f.bg_f[k] = (float)p->background[k];
     }
     f.grid_src = grid->dynamic ? grid->d_geom : nullptr;
+    f.stale = grid->geometry != scene->geometry ? 1 : 0;
     f.out_rgb = out_rgb;
     f.out_final = out_rgb;
     f.rgb_q0 = 0;

@@ -102,6 +102,7 @@ struct Scene {
     uint32_t* d_box = nullptr;
     float* d_in = nullptr;  // staging of host geometry for gbrt_scene_update
     bool box_stale = false;  // lo/hi above predate a device-side update
+    uint64_t geometry = 0;   // names the geometry in the arrays (new_geometry): no other scene or update has it
 
     SceneDev view() const {
         SceneDev v;
@@ -151,6 +152,7 @@ struct Grid {
     size_t bytes = 0;
     float lambda = 0.f;
     int64_t N = 0;  // objects of the scene it was built for
+    uint64_t geometry = 0;  // the geometry that balls holds (Scene::geometry; 0: none)
     int device = 0;  // the scene's device
     // device-side rebuilds (gbrt_grid_rebuild): the authoritative geometry is
     // d_geom on the device; renders copy it into their frame descriptors
@@ -178,6 +180,9 @@ void block_free(Ctx* ctx, void* p);
 // render.cu: grow a context buffer (drains the stream first: old work may still
 // read it)
 int grow(Ctx* ctx, void** p, size_t* cap, size_t need);
+
+// scene_grid.cu: a value that no call returned before (never 0)
+uint64_t new_geometry();
 
 // scene_grid.cu: fill a caller-allocated object; on failure it frees what it
 // allocated and leaves the object empty.

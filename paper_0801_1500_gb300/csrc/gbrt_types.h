@@ -41,7 +41,8 @@ struct SceneDev {
 // holds their centre, x fastest: those of cells (x0..x1, y, z) are
 // [bstart[(z bny + y) bnx + x0], bstart[(z bny + y) bnx + x1 + 1]). A tube's
 // ball holds only the part outside its spheres (radius negated; 0: no such
-// part). rho is the reach of the AO rays' near pass (0: not used), rmax the
+// part). They are copies: a scene that was updated since, or another one of as
+// many objects, is rendered without them (FrameDev::stale). rho is the reach of the AO rays' near pass (0: not used), rmax the
 // largest distance of an object's point from the centre it was sorted by.
 // cells[c] = (first item, item count) of cell
 // c = (z * ny + y) * nx + x; items are global object ids, in the order the
@@ -126,6 +127,7 @@ struct FrameDev {
     int32_t row0, rows;
     int32_t tiles_x, tiles_y;
     int64_t hit_base;  // first slot of this frame's region of the hit buffers
+    int32_t stale;     // 1: the grid's balls are of another geometry than the scene's
     // near pass: 1 when it looks for this frame's near occluders; the frame's
     // words in the job masks (mask_words a hit, 16 jobs a word)
     int32_t near_pass;

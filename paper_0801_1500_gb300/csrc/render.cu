@@ -1604,12 +1604,15 @@ struct LaneScene {
     int32_t nobj;
     V3<float> lo;
     float om;
-    bool cut;
+    // The balls a frame's rays are tested with: tubes cut to what sticks out of
+    // their spheres (a ray without a limit that meets the rest meets the sphere
+    // as well), unless the cut is of another geometry.
+    static __device__ __forceinline__ const float4* balls(const FrameDev& F) {
+        return isinf(F.ao_maxdist_f) && !F.stale ? F.grid.cut : F.scene.bs;
+    }
+    __device__ __forceinline__ bool is(const FrameDev& F) const { return F.grid.cells == cells && balls(F) == bs; }
     __device__ __forceinline__ void set(const FrameDev& F) {
-        // tubes cut to what sticks out of their spheres: a ray without a limit
-        // that meets the rest meets the sphere as well
-        cut = isinf(F.ao_maxdist_f);
-        bs = cut ? F.grid.cut : F.scene.bs;
+        bs = balls(F);
         nobj = F.scene.S + F.scene.C;
         cells = F.grid.cells;
         items = F.grid.items;
@@ -1826,7 +1829,7 @@ struct FrameRays {
         if (next >= f_hi) {
             const int nf = b.nframes == 1 ? 0 : find_frame(b.job_off, b.nframes, next);
             const FrameDev& N = b.frames[nf];
-            const bool same = N.grid.cells == A.cells && isinf(N.ao_maxdist_f) == A.cut;
+            const bool same = A.is(N);
             if (!same && act != 0u) return LANES_GO;  // another scene: the lanes in flight drain first
             f = nf;
             f_lo = b.job_off[f];
@@ -1867,7 +1870,7 @@ __global__ void __launch_bounds__(256, 3) k_ao_walk64(const __grid_constant__ Ba
     FrameRays<NEAR> src(b, unit);
     LaneScene A;
     A.cells = nullptr;
-    A.cut = false;
+    A.bs = nullptr;
     lane_walk(src, A, b.refill, b.err);
 }
 
@@ -2237,9 +2240,10 @@ static bool one_scene(const FrameDev* frames, int n) {
 
 // Whether a near pass suits a frame's AO rays: enough of them a hit to share its
 // per-hit work, no limit on their length (the pass takes a hit at any distance
-// for one), and objects small enough (grid.rho).
+// for one), and objects small enough (grid.rho); the grid's balls have to be the
+// scene's.
 static bool near_pass_suits(const FrameDev& f) {
-    return f.grid.rho > 0.0f && std::isinf(f.ao_maxdist_f) &&
+    return f.grid.rho > 0.0f && !f.stale && std::isinf(f.ao_maxdist_f) &&
            f.jobs_per_hit >= NEAR_MIN_JOBS && f.jobs_per_hit <= NEAR_MAX_JOBS;
 }
 

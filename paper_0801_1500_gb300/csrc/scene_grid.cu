@@ -9,6 +9,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 
 #include "gbrt_internal.h"
@@ -635,6 +636,7 @@ int scene_upload(Ctx* ctx, const float* spheres, int64_t S, const float* cyl, in
         }
         memcpy(&s->rmax, &h_box[7], 4);
     }
+    s->geometry = new_geometry();
     return GBRT_OK;
 fail:
     cudaStreamSynchronize(ctx->stream);
@@ -895,6 +897,7 @@ int grid_build(Ctx* ctx, const Scene* s, float lambda, Grid* g) {
         d.cut = g->balls + N;
         d.bstart = g->bstart;
         d.nitems = std::max<int64_t>(g->refs, 1);
+        g->geometry = s->geometry;
         g->bytes = (size_t)nc * sizeof(uint2) + (size_t)std::max<int64_t>(g->refs, 1) * sizeof(uint32_t) +
                    (size_t)nbc * sizeof(uint32_t) + 2 * (size_t)std::max<int64_t>(N, 1) * sizeof(float4);
     }
@@ -923,6 +926,11 @@ int scene_refresh_host(Scene* s, cudaStream_t stream) {
     return h_box[6] ? GBRT_EINVAL : GBRT_OK;
 }
 
+uint64_t new_geometry() {
+    static std::atomic<uint64_t> last{0};
+    return ++last;
+}
+
 int scene_update(Ctx* ctx, Scene* s, const float* spheres, const float* cyl, int flags) {
     const bool host = (flags & GBRT_HOST_PTRS) != 0;
     const int64_t S = s->S, C = s->C, N = S + C;
@@ -948,6 +956,7 @@ int scene_update(Ctx* ctx, Scene* s, const float* spheres, const float* cyl, int
         sph_in = dsph;
         cyl_in = dcyl;
     }
+    s->geometry = new_geometry();
     // box words: min <- all ones (above every ordered float), max <- 0, flag <- 0
     if (cudaMemsetAsync(s->d_box, 0xFF, 3 * sizeof(uint32_t), ctx->stream) != cudaSuccess ||
         cudaMemsetAsync(s->d_box + 3, 0, 5 * sizeof(uint32_t), ctx->stream) != cudaSuccess)
@@ -1052,6 +1061,7 @@ int grid_rebuild(Ctx* ctx, const Scene* s, Grid* g) {
         }
     }
     g->stream = ctx->stream;
+    g->geometry = 0;
     cudaStream_t st = ctx->stream;
     const int64_t nc = g->cells_cap;
     const int64_t nall = 2 * nc + 1;
@@ -1088,6 +1098,7 @@ int grid_rebuild(Ctx* ctx, const Scene* s, Grid* g) {
     }
     ctx->launches += scans + (N > 0 ? 4 : 1);
     if (cudaGetLastError() != cudaSuccess) return GBRT_EDEVICE;
+    g->geometry = s->geometry;
     if (cudaMemcpyAsync(g->h_stat, g->d_stat, sizeof(GridStat), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaEventRecord(g->stat_ev, st) != cudaSuccess)
         return GBRT_EDEVICE;
