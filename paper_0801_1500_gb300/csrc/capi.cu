@@ -48,9 +48,11 @@ int check_frame_args(const gbrt_scene* scene, const gbrt_grid* grid, const gbrt_
     return GBRT_OK;
 }
 
-FrameDev make_frame(const gbrt_scene* scene, const gbrt_grid* grid, const gbrt_camera* cam, int32_t W, int32_t H,
-                    int32_t spp, const gbrt_lights* lights, const gbrt_params* p, void* out_rgb, uint32_t* out_ids,
-                    uint32_t* out_vis) {
+FrameDev make_frame(const Ctx* ctx, const gbrt_scene* scene, const gbrt_grid* grid, const gbrt_camera* cam, int32_t W,
+                    int32_t H, int32_t spp, const gbrt_lights* lights, const gbrt_params* p, void* out_rgb,
+                    uint32_t* out_ids, uint32_t* out_vis) {
+    scene->users.add(ctx);
+    grid->users.add(ctx);
     FrameDev f;
     memset(&f, 0, sizeof(f));
     // supersampling renders the m-times finer raster (its pixel centres are
@@ -501,7 +503,7 @@ GBRT_API int gbrt_render(gbrt_ctx* ctx, const gbrt_scene* scene, const gbrt_grid
         }
         if (out_ao_visible) d_vis = (uint32_t*)(base + off);
     }
-    FrameDev f = make_frame(scene, grid, camera, width, height, ao_samples, lights, params, d_rgb, d_ids, d_vis);
+    FrameDev f = make_frame(ctx, scene, grid, camera, width, height, ao_samples, lights, params, d_rgb, d_ids, d_vis);
     rc = render_frames(ctx, &f, 1, false);
     if (rc != GBRT_OK) return rc;
     if (host) {
@@ -546,7 +548,7 @@ GBRT_API int gbrt_render_batch(gbrt_ctx* ctx, const gbrt_render_item* items, int
         for (int32_t k = 0; k < n; ++k) {
             const gbrt_render_item& it = items[k];
             if (it.params.precision != prec) continue;
-            frames.push_back(make_frame(it.scene, it.grid, &it.camera, it.width, it.height, it.ao_samples,
+            frames.push_back(make_frame(ctx, it.scene, it.grid, &it.camera, it.width, it.height, it.ao_samples,
                                         &it.lights, &it.params, it.out_rgb, it.out_hit_ids, it.out_ao_visible));
             if (it.row_end > 0) {
                 const int32_t m = frames.back().aa;
@@ -584,7 +586,7 @@ GBRT_API int gbrt_ao_probe(gbrt_ctx* ctx, const gbrt_scene* scene, const gbrt_gr
         if (rc != GBRT_OK) return rc;
     }
     if (grid->dev.cells == nullptr) return GBRT_EINVAL;  // a grid left unusable by a failed rebuild
-    FrameDev f = make_frame(scene, grid, &cam, 1, 1, ao_samples, &lights, params, nullptr, nullptr, nullptr);
+    FrameDev f = make_frame(ctx, scene, grid, &cam, 1, 1, ao_samples, &lights, params, nullptr, nullptr, nullptr);
     return launch_ao_probe(ctx, f, pts, nrm, n, out_visibility);
 }
 

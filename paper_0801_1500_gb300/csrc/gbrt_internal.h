@@ -3,6 +3,8 @@
 #pragma once
 
 #include <cuda_runtime.h>
+
+#include <atomic>
 #include <stdint.h>
 
 #include "gbrt.h"
@@ -83,7 +85,28 @@ struct Carve {
     }
 };
 
+// Whose work may still read an object's memory when it is freed: the context
+// that made it (its stream is in hand), or, once another one or
+// gbrt_render_noalloc has used it, any stream.
+struct Users {
+    const Ctx* owner = nullptr;
+    Users() = default;
+    Users& operator=(const Users& o) {
+        owner = o.owner;
+        others.store(o.others.load(std::memory_order_relaxed), std::memory_order_relaxed);
+        return *this;
+    }
+    void add(const Ctx* c) const {
+        if (c != owner) others.store(true, std::memory_order_relaxed);
+    }
+    bool only(const Ctx* c) const { return c == owner && !others.load(std::memory_order_relaxed); }
+
+  private:
+    mutable std::atomic<bool> others{false};
+};
+
 struct Scene {
+    Users users;
     int device = 0;
     int64_t S = 0, C = 0;
     int32_t K = 0;
@@ -142,6 +165,7 @@ struct BuildAux {
 };
 
 struct Grid {
+    Users users;
     GridDev dev{};
     void* mem = nullptr;  // holds cells, balls, bstart and, of a rebuilt grid, d_counts and d_sums
     uint2* cells = nullptr;
@@ -171,11 +195,11 @@ struct Grid {
 };
 
 // scene_grid.cu: the context's pool (none if the device has no pools); memory
-// of a scene or grid from it, and back
-// (like cudaFree, after the device is idle: other streams may still read it)
+// of a scene or grid from it, and back: after blocks_idle, with the context's
+// stream drained
 void pool_create(Ctx* ctx);
 cudaError_t block_alloc(Ctx* ctx, void** p, size_t bytes);
-void block_free(Ctx* ctx, void* p);
+void blocks_idle(const Ctx* ctx, const Users& users);
 
 // render.cu: grow a context buffer (drains the stream first: old work may still
 // read it)
@@ -205,9 +229,10 @@ int run_microbench(Ctx* ctx, int kind, double* value);
 // capi.cu: argument checks and the frame descriptor of one render
 int check_frame_args(const gbrt_scene* scene, const gbrt_grid* grid, const gbrt_camera* cam, int32_t W, int32_t H,
                      int32_t spp, const gbrt_lights* lights, const gbrt_params* params, const void* out_rgb);
-FrameDev make_frame(const gbrt_scene* scene, const gbrt_grid* grid, const gbrt_camera* cam, int32_t W, int32_t H,
-                    int32_t spp, const gbrt_lights* lights, const gbrt_params* p, void* out_rgb, uint32_t* out_ids,
-                    uint32_t* out_vis);
+// (ctx: whose stream reads the scene and grid; null: a stream of the caller's)
+FrameDev make_frame(const Ctx* ctx, const gbrt_scene* scene, const gbrt_grid* grid, const gbrt_camera* cam, int32_t W,
+                    int32_t H, int32_t spp, const gbrt_lights* lights, const gbrt_params* p, void* out_rgb,
+                    uint32_t* out_ids, uint32_t* out_vis);
 
 // render.cu: render n frames of one precision (descriptors filled by the
 // caller; tiling and hit-buffer fields are set here).

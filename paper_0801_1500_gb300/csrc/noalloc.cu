@@ -99,7 +99,7 @@ extern "C" GBRT_API int gbrt_render_noalloc(const gbrt_scene* scene, const gbrt_
     rc = setup_device(scene->device, &base, &sms);
     if (rc == GBRT_OK) {
         const int tw = 8, th = 4, block = 256, refill = 16;
-        FrameDev f = make_frame(scene, grid, camera, width, height, ao_samples, lights, params, out_rgb,
+        FrameDev f = make_frame(nullptr, scene, grid, camera, width, height, ao_samples, lights, params, out_rgb,
                                 out_hit_ids, out_ao_visible);
         f.tiles_x = (width + tw - 1) / tw;
         f.tiles_y = (height + th - 1) / th;

@@ -522,22 +522,26 @@ cudaError_t block_alloc(Ctx* ctx, void** p, size_t bytes) {
     return cudaMallocFromPoolAsync(p, bytes, ctx->pool, ctx->stream);
 }
 
-void block_free(Ctx* ctx, void* p) {
-    if (!p) return;
-    if (!ctx->pool) {
+// Waits for whatever may read the memory of an object with these users, beside
+// the context's own stream. Freed pool memory goes back at once (cudaFree waits
+// only for memory that cudaMalloc gave), so where other streams may read it a
+// plain block is freed first: that waits for all of them, also while another
+// thread captures a stream, which cudaDeviceSynchronize would refuse and break
+// off. 57 us, against nothing for an object that its own context used alone.
+void blocks_idle(const Ctx* ctx, const Users& users) {
+    if (users.only(ctx)) return;
+    void* p = nullptr;
+    if (cudaMalloc(&p, 256) == cudaSuccess) {
         cudaFree(p);
         return;
     }
+    (void)cudaGetLastError();
     cudaDeviceSynchronize();
-    if (cudaFreeAsync(p, ctx->stream) != cudaSuccess) {
-        // not from a pool (another context's plain allocation)
-        (void)cudaGetLastError();
-        cudaFree(p);
-    }
 }
 
 void scene_release(Ctx* ctx, Scene* s) {
-    block_free(ctx, s->mem);
+    if (s->mem) blocks_idle(ctx, s->users);
+    cudaFree(s->mem);
     cudaFree(s->d_in);
     *s = Scene();
 }
@@ -565,6 +569,7 @@ int scene_upload(Ctx* ctx, const float* spheres, int64_t S, const float* cyl, in
     uint32_t h_box[8];
     if (host && N > 0 && !host_scene_valid(spheres, S, cyl, C, color, K)) return GBRT_EINVAL;
     *s = Scene();
+    s->users.owner = ctx;
     s->device = ctx->device;
     s->S = S;
     s->C = C;
@@ -645,8 +650,9 @@ fail:
 }
 
 void grid_release(Ctx* ctx, Grid* g) {
-    block_free(ctx, g->mem);
-    block_free(ctx, g->items);
+    if (g->mem) blocks_idle(ctx, g->users);
+    cudaFree(g->mem);
+    cudaFree(g->items);
     cudaFree(g->d_geom);
     cudaFree(g->d_aux);
     cudaFree(g->d_reach);
@@ -810,6 +816,8 @@ int grid_build(Ctx* ctx, const Scene* s, float lambda, Grid* g) {
     unsigned long long* sums = nullptr;
     unsigned long long h_total = 0;
     *g = Grid();
+    g->users.owner = ctx;
+    s->users.add(ctx);
     if (!(lambda > 0.0f)) lambda = 2.0f;
     g->lambda = lambda;
     const int64_t N = s->S + s->C;
@@ -957,6 +965,7 @@ int scene_update(Ctx* ctx, Scene* s, const float* spheres, const float* cyl, int
         cyl_in = dcyl;
     }
     s->geometry = new_geometry();
+    s->users.add(ctx);
     // box words: min <- all ones (above every ordered float), max <- 0, flag <- 0
     if (cudaMemsetAsync(s->d_box, 0xFF, 3 * sizeof(uint32_t), ctx->stream) != cudaSuccess ||
         cudaMemsetAsync(s->d_box + 3, 0, 5 * sizeof(uint32_t), ctx->stream) != cudaSuccess)
@@ -997,11 +1006,12 @@ static int dyn_alloc(Ctx* ctx, Grid* g, int64_t cells_cap, int64_t items_cap) {
     if (block_alloc(ctx, &mem, size.size) != cudaSuccess ||
         block_alloc(ctx, (void**)&items, (size_t)items_cap * sizeof(uint32_t)) != cudaSuccess) {
         (void)cudaGetLastError();
-        block_free(ctx, mem);
+        cudaFree(mem);
         return GBRT_ENOMEM;
     }
-    block_free(ctx, g->mem);
-    block_free(ctx, g->items);
+    blocks_idle(ctx, g->users);
+    cudaFree(g->mem);
+    cudaFree(g->items);
     g->mem = mem;
     g->items = items;
     cut.base = (char*)mem;
@@ -1062,6 +1072,8 @@ int grid_rebuild(Ctx* ctx, const Scene* s, Grid* g) {
     }
     g->stream = ctx->stream;
     g->geometry = 0;
+    g->users.add(ctx);
+    s->users.add(ctx);
     cudaStream_t st = ctx->stream;
     const int64_t nc = g->cells_cap;
     const int64_t nall = 2 * nc + 1;
