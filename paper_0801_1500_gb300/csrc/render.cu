@@ -832,17 +832,16 @@ constexpr double NEAR_MIN_RECS = 4608, NEAR_MIN_RECS64 = 3072, NEAR_FULL_RECS = 
 // an outside origin exactly when b >= q. w and q are per (hit, ball), so a
 // (ray, ball) pair costs three FMAs and half a three-input maximum. An origin
 // inside or within 5e-5 r of a ball sets bad (q would be too rough there),
-// unless it is the ball of the tube that the hit lies on (skip): rays from a
-// tube's outer side do not meet it again. An FP64 origin is o + ol
+// unless it is the ball of the object that the hit lies on (skip): rays from the
+// outer side of a sphere or a tube do not meet it again. An FP64 origin is o + ol
 // (float pairs: w then has FP32's relative error however large the coordinates).
 //
-// The tube is known by its ball, of which it is one of the candidates: the ball
-// holds the origin, so neither the reach nor the tangent planes drop it. A ball
-// with the same centre and radius may still be another tube's (the arms of a
-// cross, a tube drawn twice); it holds the origin as well, so of several such
-// candidates one is passed over and the next sets bad.
+// The object is known by its ball. A ball with the same centre and radius may
+// still be another object's (the arms of a cross, a tube drawn twice), but the
+// gather takes equal balls together or not at all: of several such candidates
+// one is passed over and the next sets bad.
 struct NearSkip {
-    bool on;
+    int kind;  // 0: a sphere, 1: a tube, -1: nothing is passed over
     V3<float> c;
     float r;
 };
@@ -935,7 +934,7 @@ __device__ __forceinline__ void near_jobs(const FrameDev& F, NearWarp& S, int la
     for (int kind = 0; kind < 2; ++kind) {
 #pragma unroll
         for (int s = 0; s < NS; ++s) m[s] = -Num<float>::inf();
-        near_scan<NS, F64>(list, n, o, ol, d, m, skip, skip.on && kind == 1, bad);
+        near_scan<NS, F64>(list, n, o, ol, d, m, skip, skip.kind == kind, bad);
         const float sure = kind == 0 ? delta : Num<float>::inf();
 #pragma unroll
         for (int s = 0; s < NS; ++s) {
@@ -1011,21 +1010,29 @@ __global__ void __launch_bounds__(128, 4) k_ao_near(const __grid_constant__ Batc
         float rho = F.near_pass ? F.grid.rho : 0.0f, delta = 0.0f;
         int ns = 0, nt = 0;
         NearSkip skip;
-        skip.on = false;
+        skip.kind = -1;
         skip.r = 0.0f;
         if (rho > 0.0f) {
-            // a hit on a tube's outer side: its origin may lie inside the tube's ball
+            // The hit's own ball, passed over where the origin is surely outside
+            // the object: a tube's ball may hold it, and with a small eps it is
+            // closer to a sphere than bad allows (1e-6 r keeps clear of the
+            // rounding of |w|^2 and of the walk's own test).
             V3<float> p0, a;
             float L, r;
             own = GBRT_INDEX(own, F.scene.S + F.scene.C);
             Obj<float>::load(F.scene.obj, own, p0, a, L, r);
-            if (L > 0.0f) {
-                const V3<float> w = (o - p0) + ol, wp = madd(w, -dot(w, a), a);
-                const float4 c = __ldg(F.grid.cut + own);
-                skip.on = c.w < 0.0f && dot(wp, wp) > 1.0002f * r * r;  // surely outside
-                skip.c = v3(c.x, c.y, c.z);
-                skip.r = -c.w;
-            }
+            const float4 c = __ldg(F.grid.cut + own);
+            const V3<float> w = (o - p0) + ol, v = (o - v3(c.x, c.y, c.z)) + ol;
+            const V3<float> wp = madd(w, -dot(w, a), a);  // (a sphere's axis is 0)
+            skip.c = v3(c.x, c.y, c.z);
+            skip.r = fabsf(c.w);
+            if (c.w != 0.0f && dot(wp, wp) > (L > 0.0f ? 1.0002f : 1.000002f) * r * r) skip.kind = L > 0.0f ? 1 : 0;
+            // where the own ball keeps most of the hits from being looked at (an
+            // eps of next to nothing, a view from inside) the pass is left out
+            const bool kept = skip.kind < 0 && dot(v, v) - c.w * c.w < 1e-4f * c.w * c.w;
+            if (2 * __popc(__ballot_sync(FULL, lane < n && kept)) > n) rho = 0.0f;
+        }
+        if (rho > 0.0f) {
             // the hits' box, its centre, and the cone of their normals
             const V3<float> mn = v3(warp_min(o.x), warp_min(o.y), warp_min(o.z));
             const V3<float> mx = v3(warp_max(o.x), warp_max(o.y), warp_max(o.z));

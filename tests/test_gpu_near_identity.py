@@ -85,3 +85,38 @@ def test_objects_with_one_centre(G, kind, eps, half, fp64):
         assert n1 - n0 == 4 and n2 - n1 == 3 * BANDS
         for a, b in zip(got, ref):
             assert torch.equal(a, b), int((a != b).sum())
+
+
+@pytest.mark.parametrize("fp64", [False, True])
+def test_small_offsets(G, fp64):
+    """Offsets eps from 1e-4 of a radius down to 0: an origin so close to its own
+    atom must not send its rays through the whole walk after the near pass. Same
+    bits as the bands, and no frame takes twice the time of the one at eps 1e-3
+    (FP64 frames took seven times as long)."""
+    import torch
+    sc = S.globule(1500, 1425, 27.0, seed=3)
+    cam, lights = S.ortho_camera(sc, W, H, angle_deg=20.0), S.default_lights()
+    times = {}
+    with G.Renderer(0) as R:
+        scene, grid = R.upload(sc, lam=8.0)
+        for eps in (1e-3, 1e-4, 5e-5, 1e-5, 4e-6, 2e-6, 0.0):
+            p = S.Params(ao_samples=16, seed=9, eps=eps, shadows=True,
+                         precision=S.PRECISION_FP64 if fp64 else S.PRECISION_FP32)
+            got, ref = [[torch.full((H, W, 3), -1.0, device="cuda", dtype=torch.float64 if fp64 else torch.float32)] +
+                        [torch.full((H, W), -7, dtype=torch.int32, device="cuda") for _ in range(2)] for _ in range(2)]
+            took = []
+            for _ in range(5):
+                a, b = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+                a.record()
+                G.gbrt_render(R.ctx, scene, grid, cam, W, H, p.ao_samples, lights, p, *got)
+                b.record()
+                b.synchronize()
+                took.append(a.elapsed_time(b))
+            times[eps] = min(took)
+            for k in range(BANDS):
+                rows = (k * H // BANDS, (k + 1) * H // BANDS)
+                G.gbrt_render_batch(R.ctx, [G.make_item(scene, grid, cam, W, H, p.ao_samples, lights, p, *ref, rows=rows)])
+            G.gbrt_sync(R.ctx)
+            for a, b in zip(got, ref):
+                assert torch.equal(a, b), (eps, int((a != b).sum()))
+    assert all(times[e] < 2.0 * times[1e-3] for e in times if e >= 4e-6), times
