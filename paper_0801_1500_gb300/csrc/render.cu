@@ -2342,7 +2342,7 @@ int render_frames(Ctx* ctx, FrameDev* frames, int n, bool use_graph) {
     int64_t near_rays = 0;  // rays of the frames that a near pass suits, if every pixel hits
     bool many = false;      // a frame with too many jobs a hit for masks
     double near_recs = 0;   // and their expected tile records
-    int64_t mask_words = 0, recs = 0, all_rays = 0;
+    int64_t mask_words = 0, recs = 0, words = 0, all_rays = 0;  // recs, words: tile records, and their job words
     size_t fine_bytes = 0;  // finer-raster colours of the supersampled frames' bands
     bool resolve = false;
     int extra = 0;
@@ -2371,7 +2371,8 @@ int render_frames(Ctx* ctx, FrameDev* frames, int n, bool use_graph) {
         all_rays += fpx * frames[f].jobs_per_hit;
         many = many || frames[f].jobs_per_hit > NEAR_MAX_JOBS;
         mask_words += fpx * frames[f].mask_words;
-        recs += ftiles * frames[f].mask_words;
+        recs += ftiles * ((frames[f].mask_words + frames[f].rec_words - 1) / frames[f].rec_words);
+        words += ftiles * frames[f].mask_words;
         if (frames[f].grid_src) extra |= EXTRA_PATCH;
         if (frames[f].aa > 1) {
             resolve = true;
@@ -2397,14 +2398,20 @@ int render_frames(Ctx* ctx, FrameDev* frames, int n, bool use_graph) {
     // enough of them to keep every warp of one more kernel busy, and at least
     // half of the batch's rays
     const bool uni = one_scene(frames, n);
-    const bool near = precision == GBRT_FP32
-                          ? near_recs >= NEAR_MIN_RECS && 2 * near_rays >= all_rays && !many
-                          : near_recs >= NEAR_MIN_RECS64 && near_rays == all_rays && !many && uni;
+    bool near = precision == GBRT_FP32
+                    ? near_recs >= NEAR_MIN_RECS && 2 * near_rays >= all_rays && !many
+                    : near_recs >= NEAR_MIN_RECS64 && near_rays == all_rays && !many && uni;
     const size_t units_at = (size_t)recs * sizeof(TileRec);
-    const size_t masks_at = units_at + 4 * (size_t)recs * sizeof(unsigned long long);
-    if (near &&
-        (rc = grow(ctx, &ctx->d_near, &ctx->near_cap, masks_at + (size_t)mask_words * sizeof(unsigned))) != GBRT_OK)
-        return rc;
+    const size_t masks_at = units_at + 4 * (size_t)words * sizeof(unsigned long long);
+    if (near) {
+        rc = grow(ctx, &ctx->d_near, &ctx->near_cap, masks_at + (size_t)mask_words * sizeof(unsigned));
+        if (rc == GBRT_ENOMEM) {  // without memory for it, the frame does without the pass
+            (void)cudaGetLastError();
+            near = false;
+        } else if (rc != GBRT_OK) {
+            return rc;
+        }
+    }
     if ((rc = grow(ctx, &ctx->d_desc, &ctx->desc_cap, desc_bytes)) != GBRT_OK) return rc;
     if ((rc = grow(ctx, &ctx->d_counters, &ctx->counters_cap, counters_bytes)) != GBRT_OK) return rc;
     if (ctx->h_desc_cap < desc_bytes) {
