@@ -118,10 +118,9 @@ struct Scene {
     float* palette = nullptr;
     float4* aabb = nullptr;  // [2 (S + C)]: lo (xyz), hi (xyz) per object
     float lo[3] = {0, 0, 0}, hi[3] = {0, 0, 0};
-    float rmax = 0;  // largest radius of an object's ball
     size_t bytes = 0;
     // scene box on the device (order-preserving words: min xyz, max xyz,
-    // invalid flag, largest ball radius); kept so device-side rebuilds read the current box
+    // invalid flag); kept so device-side rebuilds read the current box
     uint32_t* d_box = nullptr;
     float* d_in = nullptr;  // staging of host geometry for gbrt_scene_update
     bool box_stale = false;  // lo/hi above predate a device-side update
@@ -161,7 +160,7 @@ struct BuildAux {
     BuildP p;
     double ctr[3];        // centre of the bounding sphere
     unsigned int rbits;   // its radius (float bits, atomicMax)
-    unsigned int pad;
+    unsigned int ballbits;  // largest radius of an object's ball (the same)
 };
 
 struct Grid {

@@ -37,7 +37,6 @@ __global__ void __launch_bounds__(256) k_scene_prep(const float* sph_in, int64_t
     const int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const float big = 3.0e38f;
     float lo[3] = {big, big, big}, hi[3] = {-big, -big, -big};
-    float rb = 0.0f;  // radius of the object's ball
     bool bad = false;
     if (id < S) {
         const float* p = sph_in + 4 * id;
@@ -46,7 +45,6 @@ __global__ void __launch_bounds__(256) k_scene_prep(const float* sph_in, int64_t
         obj[2 * id] = make_float4(c[0], c[1], c[2], r);
         obj[2 * id + 1] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         bs[id] = make_float4(c[0], c[1], c[2], r);
-        rb = r;
         obj64[4 * id] = make_double2(c[0], c[1]);
         obj64[4 * id + 1] = make_double2(c[2], r);
         obj64[4 * id + 2] = make_double2(0.0, 0.0);
@@ -80,7 +78,7 @@ __global__ void __launch_bounds__(256) k_scene_prep(const float* sph_in, int64_t
         // additions cover the rounding of the middle and of the radius
         const float cmax = fmaxf(fmaxf(fabsf(p0[0]) + fabsf(p1[0]), fabsf(p0[1]) + fabsf(p1[1])),
                                  fabsf(p0[2]) + fabsf(p1[2]));
-        rb = 1.00001f * sqrtf(0.25f * L * L + r * r) + 4e-7f * cmax;
+        const float rb = 1.00001f * sqrtf(0.25f * L * L + r * r) + 4e-7f * cmax;
         bs[id] = make_float4(0.5f * p0[0] + 0.5f * p1[0], 0.5f * p0[1] + 0.5f * p1[1], 0.5f * p0[2] + 0.5f * p1[2],
                              -rb);
         obj64[4 * id] = make_double2(p0[0], p0[1]);
@@ -107,8 +105,6 @@ __global__ void __launch_bounds__(256) k_scene_prep(const float* sph_in, int64_t
         }
     }
     // warp reduction, then one atomic per warp and component
-    const uint32_t rbits = __reduce_max_sync(0xffffffffu, bad ? 0u : __float_as_uint(rb));
-    if ((threadIdx.x & 31) == 0) atomicMax(box + 7, rbits);  // non-negative floats order as ints
     for (int k = 0; k < 3; ++k) {
         float l = lo[k], h = hi[k];
         for (int off = 16; off > 0; off >>= 1) {
@@ -199,18 +195,45 @@ inline int object_warp_blocks(int64_t N) {
     return (int)std::min<int64_t>((std::max<int64_t>(N, 1) + 7) / 8, 1 << 20);
 }
 
-// Blocks of k_ball_sort for S spheres (a thread each) and C tubes (a warp each).
-inline int ball_sort_blocks(int64_t S, int64_t C) { return object_warp_blocks((S + 31) / 32 + C); }
+// Cells of the grid, and of the halved grid.
+__device__ __forceinline__ int64_t build_cells(const BuildP& p) { return (int64_t)p.n[0] * p.n[1] * p.n[2]; }
+__device__ __forceinline__ int64_t ball_cells(const BuildP& p) {
+    return (int64_t)((p.n[0] + 1) >> 1) * ((p.n[1] + 1) >> 1) * ((p.n[2] + 1) >> 1);
+}
 
-// CTAs of 256 threads that find the bounding radius of N objects.
-inline unsigned int radius_blocks(int64_t N) { return (unsigned int)((N + 255) / 256); }
+// CTAs of 256 threads, a thread per object.
+inline unsigned int object_blocks(int64_t N) { return (unsigned int)((N + 255) / 256); }
 
-// Radius of the sphere about aux->ctr that holds every object: sphere |c - ctr|
-// + r, cylinder max over both ends of |p - ctr| + r (FP64, rounded up to float).
-__device__ __forceinline__ void bound_radius(const double2* obj64, int64_t N, int64_t id, BuildAux* aux) {
-    float rr = 0.0f;
+// A CTA's 256 objects, a thread each: the radius of the sphere about aux->ctr
+// that holds them -- sphere |c - ctr| + r, cylinder max over both ends of
+// |p - ctr| + r, in FP64, rounded up to float -- and the largest radius of their
+// balls, both joined to aux. Few objects need the FP64 evaluation (it had kept
+// the FP64 units busy for 18 us of 250,000 objects): those whose ball, in FP32,
+// reaches as far as the CTA's farthest sphere does for sure.
+__device__ __forceinline__ void bound_radius(const double2* obj64, const float4* bs, int64_t N, int64_t id,
+                                             BuildAux* aux) {
+    __shared__ uint32_t far_s;
+    if (threadIdx.x == 0) far_s = 0u;
+    __syncthreads();
+    const double cx = aux->ctr[0], cy = aux->ctr[1], cz = aux->ctr[2];
+    float up = -1.0f, low = 0.0f, rb = 0.0f;  // the object's reach lies between low and up (up < 0: no object)
     if (id < N) {
-        const double cx = aux->ctr[0], cy = aux->ctr[1], cz = aux->ctr[2];
+        const float4 s = bs[id];
+        const float x = s.x - (float)cx, y = s.y - (float)cy, z = s.z - (float)cz;
+        rb = fabsf(s.w);
+        // (half a tube's length and its radius add up to sqrt(2) of its ball's radius at most)
+        const float u = sqrtf(x * x + y * y + z * z) + (s.w < 0.0f ? 1.4143f * rb : rb);
+        const float e = 4e-6f * u + 1e-6f * (fabsf(s.x) + fabsf(s.y) + fabsf(s.z) + fabsf((float)cx) +
+                                             fabsf((float)cy) + fabsf((float)cz));
+        up = u + e;
+        if (s.w > 0.0f && u - e > 0.0f && up < 3.0e38f) low = u - e;
+        if (!(up < 3.0e38f)) up = 3.4e38f;  // no number: left to FP64
+    }
+    const uint32_t far = __reduce_max_sync(0xffffffffu, __float_as_uint(low));  // non-negative floats order as ints
+    if ((threadIdx.x & 31) == 0) atomicMax(&far_s, far);
+    __syncthreads();
+    float rr = 0.0f;
+    if (id < N && up >= __uint_as_float(far_s)) {
         const double2* q = obj64 + 4 * id;
         double2 q0 = q[0], q1 = q[1], q2 = q[2], q3 = q[3];
         double px = q0.x - cx, py = q0.y - cy, pz = q1.x - cz;
@@ -219,29 +242,37 @@ __device__ __forceinline__ void bound_radius(const double2* obj64, int64_t N, in
         double d = fmax(sqrt(px * px + py * py + pz * pz), sqrt(ex * ex + ey * ey + ez * ez)) + r;
         rr = __double2float_ru(d);
     }
-    for (int off = 16; off > 0; off >>= 1) rr = fmaxf(rr, __shfl_xor_sync(0xffffffffu, rr, off));
-    if ((threadIdx.x & 31) == 0) atomicMax(&aux->rbits, __float_as_uint(rr));  // non-negative floats order as ints
+    const uint32_t wr = __reduce_max_sync(0xffffffffu, __float_as_uint(rr));
+    const uint32_t wb = __reduce_max_sync(0xffffffffu, __float_as_uint(rb));
+    if ((threadIdx.x & 31) == 0) {
+        if (wr > __ldcg(&aux->rbits)) atomicMax(&aux->rbits, wr);
+        if (wb > __ldcg(&aux->ballbits)) atomicMax(&aux->ballbits, wb);
+    }
 }
 
 // Count pass. When an object's box spans at most 64 cells, the cells its shape
 // reaches are also recorded as bits k in reach[id], so the scatter pass need
 // not repeat the test; wider objects get all-ones and are tested again there.
-// Objects per cell of the halved grid (see GridDev::balls) go to bcounts.
-// The last radius_blocks(N) CTAs find the bounding sphere's radius instead (its
-// own kernel before: 5 us and a launch in a chain of short ones).
+// The first object_blocks(N) CTAs, a thread per object, find the bounding sphere's
+// radius instead (its own kernel before: 5 us and a launch in a chain of short
+// ones) and count the objects per cell of the halved grid (see GridDev::balls)
+// behind the grid's own cells (counted by the warps that have the object, 12 us
+// more of 174 for 250,000 objects).
 __global__ void __launch_bounds__(256) k_grid_count(const float4* aabb, const float4* obj, const double2* obj64,
                                                      const float4* bs, int64_t N, BuildAux* aux, uint32_t* counts,
-                                                     uint32_t* bcounts, unsigned long long* reach,
-                                                     unsigned int count_blocks) {
-    if (blockIdx.x >= count_blocks) {
-        bound_radius(obj64, N, (int64_t)(blockIdx.x - count_blocks) * blockDim.x + threadIdx.x, aux);
+                                                     unsigned long long* reach, unsigned int count_blocks) {
+    const unsigned int first = gridDim.x - count_blocks;
+    if (blockIdx.x < first) {
+        const int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+        if (id < N) atomicAdd(counts + build_cells(aux->p) + ball_cell(aux->p, bs[id]), 1u);
+        bound_radius(obj64, bs, N, id, aux);
         return;
     }
     const BuildP* bp = &aux->p;
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)count_blocks * (blockDim.x >> 5);
     const BuildP p = *bp;
-    for (int64_t id = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; id < N; id += warps) {
+    for (int64_t id = ((int64_t)(blockIdx.x - first) * blockDim.x + threadIdx.x) >> 5; id < N; id += warps) {
         int c0[3], c1[3];
         cell_range(aabb, id, p, c0, c1);
         const int nx = c1[0] - c0[0] + 1, ny = c1[1] - c0[1] + 1;
@@ -259,21 +290,35 @@ __global__ void __launch_bounds__(256) k_grid_count(const float4* aabb, const fl
             const unsigned got = __ballot_sync(0xffffffffu, hit);
             if (base < 64) bits |= (unsigned long long)got << base;
         }
-        if (lane == 0) {
-            reach[id] = span <= 64 ? bits : ~0ull;
-            atomicAdd(bcounts + ball_cell(p, bs[id]), 1u);
-        }
+        if (lane == 0) reach[id] = span <= 64 ? bits : ~0ull;
     }
 }
 
+// A ball's two places: by cell of the halved grid, and by object id.
+__device__ __forceinline__ void ball_store(float4 s, int64_t id, int64_t N, int64_t cell, const uint32_t* bstart,
+                                           uint32_t* bcursor, float4* balls) {
+    balls[bstart[cell] + atomicAdd(bcursor + cell, 1u)] = s;
+    balls[N + id] = s;
+}
+
 // Items past `items_cap` are dropped (a device-side rebuild that outgrew its
-// buffer; its finish step then disables the grid and flags the error).
-__global__ void __launch_bounds__(256) k_grid_scatter(const float4* aabb, const float4* obj, int64_t N,
-                                                       const BuildP* bp, const unsigned long long* reach,
-                                                       const uint2* cells, uint32_t* cursor, uint32_t* items,
-                                                       uint64_t items_cap) {
+// buffer; its finish step then disables the grid and flags the error). The CTAs
+// from scatter_blocks on, a thread per sphere, place the spheres' balls.
+__global__ void __launch_bounds__(256) k_grid_scatter(const float4* aabb, const float4* obj, const float4* bs,
+                                                       int64_t S, int64_t N, const BuildP* bp,
+                                                       const unsigned long long* reach, const uint2* cells,
+                                                       uint32_t* cursor, uint32_t* items, uint64_t items_cap,
+                                                       const uint32_t* bstart, float4* balls,
+                                                       unsigned int scatter_blocks) {
+    if (blockIdx.x >= scatter_blocks) {
+        const int64_t id = (int64_t)(blockIdx.x - scatter_blocks) * blockDim.x + threadIdx.x;
+        if (id >= S) return;
+        const float4 s = bs[id];
+        ball_store(s, id, N, ball_cell(*bp, s), bstart, cursor + build_cells(*bp), balls);
+        return;
+    }
     const int lane = threadIdx.x & 31;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    const int64_t warps = (int64_t)scatter_blocks * (blockDim.x >> 5);
     const BuildP p = *bp;
     for (int64_t id = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; id < N; id += warps) {
         int c0[3], c1[3];
@@ -294,68 +339,64 @@ __global__ void __launch_bounds__(256) k_grid_scatter(const float4* aabb, const 
     }
 }
 
-// The objects' balls, tubes cut to the part outside their spheres, in the order
-// of the halved grid's cells and then again by object id (after the scatter).
-// A thread per sphere, then a warp per tube: the lanes take the spheres listed
-// in the cells of the tube's two ends (the first half-warp one end, the second
-// the other). A cross-section (radius r, at axial coordinate s) lies inside a
+// The tubes' balls, cut to the part outside their spheres, in the order of the
+// halved grid's cells and then again by object id (after the scatter, which
+// places the spheres'). 8 lanes per tube: they take the spheres listed
+// in the cells of the tube's two ends (the first four one end, the others the
+// other). A cross-section (radius r, at axial coordinate s) lies inside a
 // sphere of radius R whose centre is h from the axis at coordinate sc when
 // (s - sc)^2 + (h + r)^2 < R^2; R is taken 0.1% smaller, so what is cut off
 // lies well inside: a ray that meets the tube there meets that sphere too.
 // (One thread a tube, going through both cells twice: 36 us for 12,818 tubes,
-// all of it load latency; a warp a tube 12 us.)
+// all of it load latency; a warp a tube 12 us, but 70 us for 121,790.)
 __global__ void __launch_bounds__(256) k_ball_sort(const float4* obj, const float4* bs, int64_t S, int64_t N,
                                                     const BuildP* bp, const uint2* cells, const uint32_t* items,
-                                                    uint64_t items_cap, const uint32_t* bstart, uint32_t* bcursor,
+                                                    uint64_t items_cap, const uint32_t* bstart, uint32_t* cursor,
                                                     float4* balls) {
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    const int64_t sphere_warps = (S + 31) >> 5;
     const BuildP p = *bp;
-    for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < sphere_warps + (N - S); w += warps) {
-        const bool tube = w >= sphere_warps;
-        const int64_t id = tube ? S + (w - sphere_warps) : 32 * w + lane;
-        if (id >= N || (!tube && id >= S)) continue;
-        float4 s = bs[id];
+    for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; 4 * w < N - S; w += warps) {
+        const int64_t id = S + 4 * w + (lane >> 3);
+        const bool on = id < N;
+        float4 s = on ? bs[id] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         const int64_t c = ball_cell(p, s);
-        if (tube) {
-            const float4 A = obj[2 * id], B = obj[2 * id + 1];
-            const float t = lane < 16 ? 0.0f : B.w;
-            const int x = build_cell(p, 0, A.x + t * B.x), y = build_cell(p, 1, A.y + t * B.y),
-                      z = build_cell(p, 2, A.z + t * B.z);
-            uint2 cr = cells[((int64_t)z * p.n[1] + y) * p.n[0] + x];
-            if ((uint64_t)cr.x + cr.y > items_cap) cr.y = 0u;  // an overflowed rebuild
-            // the axis part inside the lane's spheres: joined to one end of
-            // the tube (what reaches past both ends covers it)
-            float s0 = 0.0f, s1 = B.w;
-            for (uint32_t k = lane & 15; k < cr.y; k += 16) {
-                const uint32_t j = items[cr.x + k];
-                if (j >= S) continue;
-                const float4 Q = bs[j];
-                const float wx = Q.x - A.x, wy = Q.y - A.y, wz = Q.z - A.z;
-                const float sc = wx * B.x + wy * B.y + wz * B.z;
-                const float ex = wx - sc * B.x, ey = wy - sc * B.y, ez = wz - sc * B.z;
-                const float h = sqrtf(ex * ex + ey * ey + ez * ez) + A.w, R = 0.999f * Q.w;
-                if (h >= R) continue;
-                const float half = sqrtf(R * R - h * h);
-                if (sc - half <= 0.0f) s0 = fmaxf(s0, sc + half);
-                if (sc + half >= B.w) s1 = fminf(s1, sc - half);
-            }
-            s0 = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(s0)));  // non-negative: ordered
-            s1 = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(fmaxf(s1, 0.0f))));
-            if (s0 >= s1) {
-                s.w = 0.0f;
-            } else if (s0 > 0.0f || s1 < B.w) {
-                const float m = 0.5f * (s0 + s1), hl = 0.5f * (s1 - s0);
-                const float mag = fmaxf(fmaxf(fabsf(A.x), fabsf(A.y)), fabsf(A.z)) + B.w;
-                s = make_float4(A.x + m * B.x, A.y + m * B.y, A.z + m * B.z,
-                                -(1.0001f * sqrtf(hl * hl + A.w * A.w) + 1e-6f * mag));
-            }
+        const float4 A = on ? obj[2 * id] : s, B = on ? obj[2 * id + 1] : s;
+        const float t = (lane & 7) < 4 ? 0.0f : B.w;
+        const int x = build_cell(p, 0, A.x + t * B.x), y = build_cell(p, 1, A.y + t * B.y),
+                  z = build_cell(p, 2, A.z + t * B.z);
+        uint2 cr = cells[((int64_t)z * p.n[1] + y) * p.n[0] + x];
+        if (!on || (uint64_t)cr.x + cr.y > items_cap) cr.y = 0u;  // (an overflowed rebuild)
+        // the axis part inside the lane's spheres: joined to one end of
+        // the tube (what reaches past both ends covers it)
+        float s0 = 0.0f, s1 = B.w;
+        for (uint32_t k = lane & 3; k < cr.y; k += 4) {
+            const uint32_t j = items[cr.x + k];
+            if (j >= S) continue;
+            const float4 Q = bs[j];
+            const float wx = Q.x - A.x, wy = Q.y - A.y, wz = Q.z - A.z;
+            const float sc = wx * B.x + wy * B.y + wz * B.z;
+            const float ex = wx - sc * B.x, ey = wy - sc * B.y, ez = wz - sc * B.z;
+            const float h = sqrtf(ex * ex + ey * ey + ez * ez) + A.w, R = 0.999f * Q.w;
+            if (h >= R) continue;
+            const float half = sqrtf(R * R - h * h);
+            if (sc - half <= 0.0f) s0 = fmaxf(s0, sc + half);
+            if (sc + half >= B.w) s1 = fminf(s1, sc - half);
         }
-        if (!tube || lane == 0) {
-            balls[bstart[c] + atomicAdd(bcursor + c, 1u)] = s;
-            balls[N + id] = s;
+        s1 = fmaxf(s1, 0.0f);
+        for (int off = 1; off < 8; off <<= 1) {
+            s0 = fmaxf(s0, __shfl_xor_sync(0xffffffffu, s0, off));
+            s1 = fminf(s1, __shfl_xor_sync(0xffffffffu, s1, off));
         }
+        if (s0 >= s1) {
+            s.w = 0.0f;
+        } else if (s0 > 0.0f || s1 < B.w) {
+            const float m = 0.5f * (s0 + s1), hl = 0.5f * (s1 - s0);
+            const float mag = fmaxf(fmaxf(fabsf(A.x), fabsf(A.y)), fabsf(A.z)) + B.w;
+            s = make_float4(A.x + m * B.x, A.y + m * B.y, A.z + m * B.z,
+                            -(1.0001f * sqrtf(hl * hl + A.w * A.w) + 1e-6f * mag));
+        }
+        if (on && (lane & 7) == 0) ball_store(s, id, N, c, bstart, cursor + build_cells(p), balls);
     }
 }
 
@@ -364,6 +405,7 @@ __global__ void __launch_bounds__(256) k_ball_sort(const float4* obj, const floa
 constexpr int SCAN_T = 1024;
 constexpr int SCAN_PER = 4;
 constexpr int SCAN_TILE = SCAN_T * SCAN_PER;
+static_assert(SCAN_PER == 4, "a thread's words are one uint4");
 
 // Exclusive block scan of one value per thread; returns the block total.
 __device__ __forceinline__ unsigned long long block_exclusive_scan(unsigned long long v, unsigned long long& total) {
@@ -392,8 +434,18 @@ __device__ __forceinline__ unsigned long long block_exclusive_scan(unsigned long
     return before + x - v;
 }
 
-__global__ void __launch_bounds__(SCAN_T) k_scan_reduce(const uint32_t* in, int64_t n, unsigned long long* sums) {
+// The words scanned: the counts of the grid's cells, then those of the halved
+// grid's and one more. A rebuild launches for the most cells its buffers hold;
+// the CTAs past the words there are leave at once.
+__device__ __forceinline__ int64_t scan_words(const BuildP& p) { return build_cells(p) + ball_cells(p) + 1; }
+
+__global__ void __launch_bounds__(SCAN_T) k_scan_reduce(const uint32_t* in, const BuildP* bp, unsigned long long* sums) {
+    const int64_t n = scan_words(*bp);
     int64_t base = (int64_t)blockIdx.x * SCAN_TILE + (int64_t)threadIdx.x * SCAN_PER;
+    if ((int64_t)blockIdx.x * SCAN_TILE >= n) {
+        if (threadIdx.x == 0) sums[blockIdx.x] = 0ull;
+        return;
+    }
     unsigned long long s = 0;
     for (int k = 0; k < SCAN_PER; ++k)
         if (base + k < n) s += in[base + k];
@@ -418,8 +470,8 @@ __global__ void __launch_bounds__(SCAN_T) k_scan_sums(unsigned long long* sums, 
     if (threadIdx.x == 0) *total = tot;
 }
 
-// Last step of the scan. Words [0, nc) of `in` are the cells' counts; those
-// from nc on are the halved grid's (N objects in all, counted after the cells'
+// Last step of the scan. The first words of `in` are the cells' counts; those
+// behind them are the halved grid's (N objects in all, counted after the cells'
 // references) and become starts. The words are zeroed: they are the scatter
 // passes' cursors next. Up to SCAN_T block sums every CTA adds up for itself
 // (one kernel less in the chain); above that k_scan_sums has been run.
@@ -428,20 +480,21 @@ __global__ void __launch_bounds__(SCAN_T) k_scan_sums(unsigned long long* sums, 
 // then see no objects) and flags the context's error word.
 struct ScanOut {
     uint2* cells;
-    int64_t nc;
     uint32_t* bstart;
     unsigned long long* total;  // references + N
     int64_t N;
-    GridDev* geom;
     const BuildAux* aux;
+    GridDev* geom;
     unsigned long long items_cap;
     GridStat* stat;
     uint32_t* err;
 };
-__device__ void grid_finish(const ScanOut& o, unsigned long long refs);
-__global__ void __launch_bounds__(SCAN_T) k_scan_apply(uint32_t* in, int64_t n, const unsigned long long* sums,
-                                                        int64_t nb, ScanOut o) {
+__device__ __forceinline__ void grid_finish(const ScanOut& o, unsigned long long refs);
+__global__ void __launch_bounds__(SCAN_T) k_scan_apply(uint32_t* in, const unsigned long long* sums, int64_t nb,
+                                                        ScanOut o) {
     __shared__ unsigned long long before_s;
+    const int64_t n = scan_words(o.aux->p), nc = build_cells(o.aux->p);
+    if ((int64_t)blockIdx.x * SCAN_TILE >= n) return;
     unsigned long long before, all;
     if (nb <= SCAN_T) {
         const unsigned long long mine = threadIdx.x < nb ? sums[threadIdx.x] : 0ull;
@@ -458,16 +511,22 @@ __global__ void __launch_bounds__(SCAN_T) k_scan_apply(uint32_t* in, int64_t n, 
     int64_t base = (int64_t)blockIdx.x * SCAN_TILE + (int64_t)threadIdx.x * SCAN_PER;
     uint32_t v[SCAN_PER];
     unsigned long long s = 0;
-    for (int k = 0; k < SCAN_PER; ++k) {
-        v[k] = base + k < n ? in[base + k] : 0u;
-        s += v[k];
+    if (base + SCAN_PER <= n) {  // (base is a multiple of 4, `in` of 256 bytes)
+        const uint4 q = *reinterpret_cast<const uint4*>(in + base);
+        v[0] = q.x, v[1] = q.y, v[2] = q.z, v[3] = q.w;
+        *reinterpret_cast<uint4*>(in + base) = make_uint4(0u, 0u, 0u, 0u);
+    } else {
+        for (int k = 0; k < SCAN_PER; ++k) {
+            v[k] = base + k < n ? in[base + k] : 0u;
+            if (base + k < n) in[base + k] = 0u;
+        }
     }
+    for (int k = 0; k < SCAN_PER; ++k) s += v[k];
     unsigned long long tot;
     unsigned long long run = before + block_exclusive_scan(s, tot);
     for (int k = 0; k < SCAN_PER; ++k) {
-        if (base + k < n) in[base + k] = 0u;
-        if (base + k < o.nc) o.cells[base + k] = make_uint2((uint32_t)run, v[k]);
-        else if (base + k < n) o.bstart[base + k - o.nc] = (uint32_t)(run - refs);
+        if (base + k < nc) o.cells[base + k] = make_uint2((uint32_t)run, v[k]);
+        else if (base + k < n) o.bstart[base + k - nc] = (uint32_t)(run - refs);
         run += v[k];
     }
     if (o.geom && blockIdx.x == 0 && threadIdx.x == 0) grid_finish(o, refs);
@@ -639,7 +698,6 @@ int scene_upload(Ctx* ctx, const float* spheres, int64_t S, const float* cyl, in
             s->lo[k] = N > 0 ? float_of_ord(h_box[k]) : 0.0f;
             s->hi[k] = N > 0 ? float_of_ord(h_box[3 + k]) : 0.0f;
         }
-        memcpy(&s->rmax, &h_box[7], 4);
     }
     s->geometry = new_geometry();
     return GBRT_OK;
@@ -690,8 +748,8 @@ constexpr float NEAR_REACH = 2.0f;
 
 // Fill the grid geometry (GridDev fields, build parameters, bounding-sphere
 // centre) from the padded scene box; `cells_cap` > 0 caps the cell count.
-__host__ __device__ inline void grid_geometry(const float slo[3], const float shi[3], float rmax, int64_t N,
-                                              float lambda, int64_t cells_cap, GridDev& d, BuildAux& a) {
+__host__ __device__ inline void grid_geometry(const float slo[3], const float shi[3], int64_t N, float lambda,
+                                              int64_t cells_cap, GridDev& d, BuildAux& a) {
     float emax = fmaxf(shi[0] - slo[0], fmaxf(shi[1] - slo[1], shi[2] - slo[2]));
     float pad = 1e-5f * fmaxf(emax, 1.0f);
     double E[3], V = 1.0;
@@ -729,22 +787,22 @@ __host__ __device__ inline void grid_geometry(const float slo[3], const float sh
     }
     a.p.pad = pad;
     a.rbits = 0u;
-    a.pad = 0u;
+    a.ballbits = 0u;
     d.empty = N == 0 ? 1 : 0;
     for (int k = 0; k < 3; ++k) d.bn[k] = (d.n[k] + 1) / 2;
     d.nballs = (int32_t)(N < 0x7fffffff ? N : 0);
-    // the near pass looks NEAR_REACH mean object distances far; scenes with
-    // objects larger than that reach (its candidate boxes would be mostly
-    // margin) do without it
-    d.rmax = rmax;
+    // the near pass looks NEAR_REACH mean object distances far
     d.density = (float)((double)N / V);
-    d.rho = NEAR_REACH * cbrtf((float)(target / (double)(N > 0 ? N : 1))) / (float)kk0;
-    if (d.nballs == 0 || !(rmax <= d.rho)) d.rho = 0.0f;
+    d.rho = d.nballs == 0 ? 0.0f : NEAR_REACH * cbrtf((float)(target / (double)(N > 0 ? N : 1))) / (float)kk0;
 }
 
-// Bounding sphere from its centre and the reduced radius bits.
+// Bounding sphere from its centre and the reduced radius bits; the largest ball.
 __host__ __device__ inline void grid_bound_sphere(const BuildAux& a, GridDev& d) {
     float rb;
+    // scenes with objects larger than the near pass's reach (its candidate boxes
+    // would be mostly margin) do without it
+    memcpy(&d.rmax, &a.ballbits, 4);
+    if (!(d.rmax <= d.rho)) d.rho = 0.0f;
     memcpy(&rb, &a.rbits, 4);
     const double rpad = mul_add_rn((double)rb, 1.0 + 1e-5, (double)a.p.pad);
     for (int k = 0; k < 3; ++k) {
@@ -772,7 +830,7 @@ __global__ void k_grid_geometry(const uint32_t* box, int64_t N, float lambda, in
     }
     GridDev d = *geom;
     BuildAux a;
-    grid_geometry(lo, hi, __uint_as_float(box[7]), N, lambda, cells_cap, d, a);
+    grid_geometry(lo, hi, N, lambda, cells_cap, d, a);
     d.balls = balls;
     d.cut = balls + N;
     d.bstart = bstart;
@@ -783,29 +841,43 @@ __global__ void k_grid_geometry(const uint32_t* box, int64_t N, float lambda, in
     *aux = a;
 }
 
-__device__ void grid_finish(const ScanOut& o, unsigned long long refs) {
-    GridDev d = *o.geom;
-    grid_bound_sphere(*o.aux, d);
+// (in place, one value after another: a copy of the geometry costs every thread of
+// the scan its registers)
+__device__ __forceinline__ void grid_finish(const ScanOut& o, unsigned long long refs) {
+    grid_bound_sphere(*o.aux, *o.geom);
     const unsigned int over = refs > o.items_cap ? 1u : 0u;
     if (over) {
-        d.empty = 1;
+        o.geom->empty = 1;
         atomicOr(o.err, ERR_GRID_CAPACITY);
     }
-    *o.geom = d;
     o.stat->refs = refs;
-    o.stat->ncells = (unsigned long long)d.ncells;
+    o.stat->ncells = (unsigned long long)o.geom->ncells;
     o.stat->overflow = over;
     o.stat->pad = 0u;
 }
 
-// The scan passes on `st`: counts [0, n) -> o.cells, o.bstart; returns the
-// kernels launched.
+// The scan passes on `st`: counts (n words at most) -> o.cells, o.bstart; returns
+// the kernels launched.
 static int launch_scan(uint32_t* counts, int64_t n, unsigned long long* sums, const ScanOut& o, cudaStream_t st) {
     const int64_t nb = (n + SCAN_TILE - 1) / SCAN_TILE;
-    k_scan_reduce<<<(int)nb, SCAN_T, 0, st>>>(counts, n, sums);
+    k_scan_reduce<<<(int)nb, SCAN_T, 0, st>>>(counts, &o.aux->p, sums);
     if (nb > SCAN_T) k_scan_sums<<<1, SCAN_T, 0, st>>>(sums, nb, o.total);
-    k_scan_apply<<<(int)nb, SCAN_T, 0, st>>>(counts, n, sums, nb, o);
+    k_scan_apply<<<(int)nb, SCAN_T, 0, st>>>(counts, sums, nb, o);
     return nb > SCAN_T ? 3 : 2;
+}
+
+// The item lists and the balls of a grid whose cells are scanned; returns the
+// kernels launched.
+static int launch_lists(const Scene* s, const BuildP* p, const unsigned long long* reach, uint32_t* cursor,
+                        const Grid& g, uint64_t items_cap, cudaStream_t st) {
+    const int64_t N = s->S + s->C;
+    const unsigned int sb = (unsigned int)object_warp_blocks(N);
+    k_grid_scatter<<<sb + object_blocks(s->S), 256, 0, st>>>(s->aabb, s->obj, s->bs, s->S, N, p, reach, g.cells, cursor,
+                                                             g.items, items_cap, g.bstart, g.balls, sb);
+    if (s->C == 0) return 1;
+    k_ball_sort<<<object_warp_blocks((s->C + 3) / 4), 256, 0, st>>>(s->obj, s->bs, s->S, N, p, g.cells, g.items,
+                                                                    items_cap, g.bstart, cursor, g.balls);
+    return 2;
 }
 
 int grid_build(Ctx* ctx, const Scene* s, float lambda, Grid* g) {
@@ -830,7 +902,7 @@ int grid_build(Ctx* ctx, const Scene* s, float lambda, Grid* g) {
     }
     {
         BuildAux a;
-        grid_geometry(s->lo, s->hi, s->rmax, N, lambda, 0, d, a);
+        grid_geometry(s->lo, s->hi, N, lambda, 0, d, a);
         const int64_t nc = d.ncells;
         // the counts of the cells, then of the halved grid's cells and one more
         const int64_t nbc = (int64_t)d.bn[0] * d.bn[1] * d.bn[2] + 1, nall = nc + nbc;
@@ -863,21 +935,22 @@ int grid_build(Ctx* ctx, const Scene* s, float lambda, Grid* g) {
         GB_TRY(cudaMemcpyAsync(d_aux, &a, sizeof(a), cudaMemcpyHostToDevice, ctx->stream));
         if (N > 0) {
             const unsigned int cb = (unsigned int)object_warp_blocks(N);
-            k_grid_count<<<cb + radius_blocks(N), 256, 0, ctx->stream>>>(s->aabb, s->obj, s->obj64, s->bs, N, d_aux, counts,
-                                                                         counts + nc, reach, cb);
+            k_grid_count<<<cb + object_blocks(N), 256, 0, ctx->stream>>>(s->aabb, s->obj, s->obj64, s->bs, N, d_aux,
+                                                                         counts, reach, cb);
             ctx->launches++;
             GB_TRY(cudaGetLastError());
         }
         ScanOut so = {};
         so.cells = g->cells;
-        so.nc = nc;
         so.bstart = g->bstart;
         so.total = sums + nb;
         so.N = N;
+        so.aux = d_aux;
         ctx->launches += launch_scan(counts, nall, sums, so, ctx->stream);
         GB_TRY(cudaGetLastError());
         GB_TRY(cudaMemcpyAsync(&h_total, sums + nb, sizeof(h_total), cudaMemcpyDeviceToHost, ctx->stream));
-        GB_TRY(cudaMemcpyAsync(&a.rbits, &d_aux->rbits, sizeof(a.rbits), cudaMemcpyDeviceToHost, ctx->stream));
+        GB_TRY(cudaMemcpyAsync(&a.rbits, &d_aux->rbits, sizeof(a.rbits) + sizeof(a.ballbits), cudaMemcpyDeviceToHost,
+                               ctx->stream));
         GB_TRY(cudaStreamSynchronize(ctx->stream));
         grid_bound_sphere(a, d);
         h_total -= (unsigned long long)N;
@@ -889,13 +962,7 @@ int grid_build(Ctx* ctx, const Scene* s, float lambda, Grid* g) {
         GB_TRY(block_alloc(ctx, (void**)&g->items, (size_t)std::max<int64_t>(g->refs, 1) * sizeof(uint32_t)));
         if (N > 0) {
             cursor = counts;  // zeroed by the scan: the fill cursors
-            k_grid_scatter<<<object_warp_blocks(N), 256, 0, ctx->stream>>>(s->aabb, s->obj, N, &d_aux->p, reach,
-                                                                            g->cells,
-                                                                            cursor, g->items, (uint64_t)g->refs);
-            k_ball_sort<<<ball_sort_blocks(s->S, s->C), 256, 0, ctx->stream>>>(s->obj, s->bs, s->S, N, &d_aux->p,
-                                                                               g->cells, g->items, (uint64_t)g->refs,
-                                                                               g->bstart, cursor + nc, g->balls);
-            ctx->launches += 2;
+            ctx->launches += launch_lists(s, &d_aux->p, reach, cursor, *g, (uint64_t)g->refs, ctx->stream);
             GB_TRY(cudaGetLastError());
         }
         GB_TRY(cudaStreamSynchronize(ctx->stream));
@@ -929,7 +996,6 @@ int scene_refresh_host(Scene* s, cudaStream_t stream) {
         s->lo[k] = N > 0 ? float_of_ord(h_box[k]) : 0.0f;
         s->hi[k] = N > 0 ? float_of_ord(h_box[3 + k]) : 0.0f;
     }
-    memcpy(&s->rmax, &h_box[7], 4);
     s->box_stale = false;
     return h_box[6] ? GBRT_EINVAL : GBRT_OK;
 }
@@ -1083,12 +1149,11 @@ int grid_rebuild(Ctx* ctx, const Scene* s, Grid* g) {
                                       g->d_geom, g->d_aux);
     if (N > 0) {
         const unsigned int cb = (unsigned int)object_warp_blocks(N);
-        k_grid_count<<<cb + radius_blocks(N), 256, 0, st>>>(s->aabb, s->obj, s->obj64, s->bs, N, g->d_aux, g->d_counts,
-                                                            g->d_counts + nc, g->d_reach, cb);
+        k_grid_count<<<cb + object_blocks(N), 256, 0, st>>>(s->aabb, s->obj, s->obj64, s->bs, N, g->d_aux, g->d_counts,
+                                                            g->d_reach, cb);
     }
     ScanOut so = {};
     so.cells = g->cells;
-    so.nc = nc;
     so.bstart = g->bstart;
     so.total = g->d_sums + nb;
     so.N = N;
@@ -1098,17 +1163,13 @@ int grid_rebuild(Ctx* ctx, const Scene* s, Grid* g) {
     so.stat = g->d_stat;
     so.err = ctx->d_err;
     const int scans = launch_scan(g->d_counts, nall, g->d_sums, so, st);
+    int lists = 0;
     if (N > 0) {
-        k_grid_scatter<<<object_warp_blocks(N), 256, 0, st>>>(s->aabb, s->obj, N, &g->d_aux->p, g->d_reach, g->cells, g->d_counts,
-                                                g->items,
-                                                (uint64_t)g->items_cap);
-        k_ball_sort<<<ball_sort_blocks(s->S, s->C), 256, 0, st>>>(s->obj, s->bs, s->S, N, &g->d_aux->p, g->cells,
-                                                                  g->items, (uint64_t)g->items_cap, g->bstart,
-                                                                  g->d_counts + nc, g->balls);
+        lists = launch_lists(s, &g->d_aux->p, g->d_reach, g->d_counts, *g, (uint64_t)g->items_cap, st);
         // no per-cell sort: no result depends on the order of a cell's ids
         // (nearest hits rank by (t, id), any-hit queries OR their tests)
     }
-    ctx->launches += scans + (N > 0 ? 4 : 1);
+    ctx->launches += scans + lists + (N > 0 ? 2 : 1);
     if (cudaGetLastError() != cudaSuccess) return GBRT_EDEVICE;
     g->geometry = s->geometry;
     if (cudaMemcpyAsync(g->h_stat, g->d_stat, sizeof(GridStat), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
