@@ -817,15 +817,13 @@ struct NearWarp {
 // (bounds the masks to 64 bytes a hit).
 constexpr int NEAR_MAX_JOBS = 256;
 constexpr int NEAR_MIN_JOBS = 8;
-// A record takes a warp some 40 us, most of it latency, and the walk's units are
-// coarser than its own claims: the pass pays when most resident warps get one or
-// two. Frame with and without it, 16 samples: 360 x 360 (3,200 records) 0.247 and
-// 0.242 ms, 480 x 480 (5,600) 0.330 and 0.348, 640 x 640 (10,000) 0.474 and
-// 0.545. FP64 rays walk slower, and one a lane: 360 x 360 0.380 and 0.392 ms,
-// 640 x 640 0.794 and 0.940.
-// NEAR_FULL_RECS: with fewer records than this a tile's job words, which share
-// its gather, are dealt to several records.
-constexpr double NEAR_MIN_RECS = 4608, NEAR_MIN_RECS64 = 3072, NEAR_FULL_RECS = 12288;
+// The pass pays where what it saves (near_work) is above these: its launch, the
+// latency of its records (some 40 us a warp) and the walk's coarser units cost a
+// frame the same however little that is. FP64 rays walk slower, and one a lane.
+constexpr double NEAR_MIN_WORK = 28500, NEAR_MIN_WORK64 = 16000;
+// With fewer records than this a tile's job words, which share its gather, are
+// dealt to several records.
+constexpr double NEAR_FULL_RECS = 12288;
 
 // Largest b - q over the n candidates at c, for each of the NS directions: b =
 // w.d with w = centre - o, q = sqrt(|w|^2 - r^2). The ray meets a ball ahead of
@@ -2281,6 +2279,39 @@ static double hit_share(const FrameDev& f) {
     return 0.785 * std::min(1.0, r / (f.half_w * scale)) * std::min(1.0, r / (f.half_h * scale));
 }
 
+// What the near pass saves a frame with that many tiles that are hit, in rays of a
+// tile. A word of 16 jobs pays for its gather and scan with some 5 of them; a
+// later word of 8 or fewer, scanned in fours, with all. The larger a tile is
+// against the objects' distance, the more balls stand around it and the less far
+// the pass looks, sooner with few jobs a hit. Fitted to 1,600 pairs of frames
+// with and without the pass (orthographic; 1,014 to 249,990 objects; 200 to 1,300
+// pixels a side; 8 to 64 jobs; the whole molecule or a third of it; FP32 and
+// FP64): of the frames that get the pass, three lose by it, 2% at most; of those
+// that do not, none would gain more than 11%. A line at a number of records (4,608
+// and 3,072), as before, let frames of 8 jobs lose up to 16%: 26,318 objects at
+// 560 x 560, 0.293 ms without and 0.318 with the pass; 250,000 objects at 330 x
+// 330 and 48 samples, 0.547 and 0.599.
+static double near_work(const FrameDev& f, double hit_tiles) {
+    const int words = (f.jobs_per_hit + 15) / 16;
+    double jobs = 0.0;
+    for (int w = 0; w < words; ++w) {
+        const int n = std::min(16, f.jobs_per_hit - 16 * w);
+        if (w == 0 || n > 8) jobs += std::max(0, n - 5);
+    }
+    // a tile's linear size in mean distances of the objects, where they are
+    double scale = 1.0;
+    if (f.cam_kind == GBRT_CAMERA_PINHOLE) {
+        double along = 0.0;
+        for (int k = 0; k < 3; ++k) along += (f.grid.bs64[k] - f.eye[k]) * f.dir_unit[k];
+        scale = std::max(along, 0.5 * f.grid.bs64[3]);
+    }
+    const double pixel = 2.0 * scale * std::sqrt(f.half_w * f.half_h * f.inv_w * f.inv_h);
+    const double tile = std::sqrt(32.0) * pixel * std::cbrt((double)f.grid.density);
+    const double full = std::min(f.jobs_per_hit, 16) / 16.0;
+    const double reach = tile / (f.precision == GBRT_FP64 ? 0.2 + 0.2 * full : 0.3 * full);
+    return hit_tiles * jobs / (1.0 + reach * reach);
+}
+
 // optional passes of a batch, and its scene layout
 enum : int { EXTRA_RESOLVE = 1, EXTRA_PATCH = 2, EXTRA_UNI = 4 };
 
@@ -2341,7 +2372,7 @@ int render_frames(Ctx* ctx, FrameDev* frames, int n, bool use_graph) {
     long long tiles = 0;
     int64_t near_rays = 0;  // rays of the frames that a near pass suits, if every pixel hits
     bool many = false;      // a frame with too many jobs a hit for masks
-    double near_recs = 0;   // and their expected tile records
+    double near_gain = 0;   // and what the pass saves them (near_work)
     int64_t mask_words = 0, recs = 0, words = 0, all_rays = 0;  // recs, words: tile records, and their job words
     size_t fine_bytes = 0;  // finer-raster colours of the supersampled frames' bands
     bool resolve = false;
@@ -2366,7 +2397,7 @@ int render_frames(Ctx* ctx, FrameDev* frames, int n, bool use_graph) {
         frames[f].rec_words = std::max(1, (frames[f].mask_words + per_tile - 1) / per_tile);
         if (frames[f].near_pass) {
             near_rays += fpx * frames[f].jobs_per_hit;
-            near_recs += hit_tiles * frames[f].mask_words;
+            near_gain += near_work(frames[f], hit_tiles);
         }
         all_rays += fpx * frames[f].jobs_per_hit;
         many = many || frames[f].jobs_per_hit > NEAR_MAX_JOBS;
@@ -2395,12 +2426,12 @@ int render_frames(Ctx* ctx, FrameDev* frames, int n, bool use_graph) {
     if ((rc = grow(ctx, (void**)&ctx->d_vis, &ctx->vis_cap, (size_t)px * sizeof(unsigned))) != GBRT_OK) return rc;
     if ((rc = grow(ctx, (void**)&ctx->d_lmask, &ctx->lmask_cap, (size_t)px * sizeof(unsigned))) != GBRT_OK)
         return rc;
-    // enough of them to keep every warp of one more kernel busy, and at least
-    // half of the batch's rays
+    // enough of them to pay for one more kernel, and at least half of the batch's
+    // rays
     const bool uni = one_scene(frames, n);
     bool near = precision == GBRT_FP32
-                    ? near_recs >= NEAR_MIN_RECS && 2 * near_rays >= all_rays && !many
-                    : near_recs >= NEAR_MIN_RECS64 && near_rays == all_rays && !many && uni;
+                    ? near_gain >= NEAR_MIN_WORK && 2 * near_rays >= all_rays && !many
+                    : near_gain >= NEAR_MIN_WORK64 && near_rays == all_rays && !many && uni;
     const size_t units_at = (size_t)recs * sizeof(TileRec);
     const size_t masks_at = units_at + 4 * (size_t)words * sizeof(unsigned long long);
     if (near) {
