@@ -1971,6 +1971,42 @@ __global__ void __launch_bounds__(256) k_resolve(const __grid_constant__ BatchDe
 
 // ---------------------------------------------------------------- probe, Philox
 
+// The FP64 ray of sample smp of a probe's point pt. From far outside the objects
+// it starts shortly before them instead (true): FP32 coordinates and crossings
+// that grow with the distance would miss the cells, and an FP64 test loses its
+// digits.
+__device__ __forceinline__ bool probe_ray64(const FrameDev& F, const double* pts, const double* nrm, int64_t pt,
+                                            uint32_t smp, V3<double>& o, V3<double>& d, double& tmax) {
+    const V3<double> n = ld3(nrm + 3 * pt);
+    o = madd(ld3(pts + 3 * pt), F.eps, n);
+    uint32_t lbit;
+    ao_direction<double>(F, (uint32_t)pt, smp, n, d, tmax, lbit);
+    const double rb = F.grid.bs64[3], te = dot(ld3(F.grid.bs64) - o, d) - 1.1 * rb;
+    if (!(te > rb)) return false;
+    o = madd(o, te, d);
+    tmax -= te;
+    return true;
+}
+
+// That ray in FP32 where it is one from far outside (out of line: it is rare, and
+// the probe's registers are the walk's).
+struct FarRay {
+    V3<float> o, d;
+    float tmax;
+    bool on;
+};
+__device__ __noinline__ FarRay probe_far_ray(const FrameDev& F, const double* pts, const double* nrm, int64_t pt,
+                                             uint32_t smp) {
+    V3<double> o, d;
+    double tmax;
+    FarRay r;
+    r.on = probe_ray64(F, pts, nrm, pt, smp, o, d, tmax);
+    r.o = to_f(o - ld3(F.grid.lo64));
+    r.d = to_f(d);
+    r.tmax = (float)tmax;
+    return r;
+}
+
 // The rays of a probe's points: each warp takes a run of jobs (point, sample)
 // of its own, so nothing is shared but the counts. A count is a float that
 // escaped samples add 1 to: exact up to 2^24, the sample bound is 2^20.
@@ -1991,11 +2027,9 @@ struct ProbeRays {
     __device__ __forceinline__ const FrameDev& frame(const LaneRay&) const { return F; }
 
     __device__ __forceinline__ bool exact(const LaneRay& ray, uint32_t id) const {
-        const V3<double> n = ld3(nrm + 3 * ray.slot), o = madd(ld3(pts + 3 * ray.slot), F.eps, n);
-        V3<double> d;
+        V3<double> o, d;
         double tmax;
-        uint32_t lbit;
-        ao_direction<double>(F, (uint32_t)ray.slot, ray.smp, n, d, tmax, lbit);
+        probe_ray64(F, pts, nrm, ray.slot, ray.smp, o, d, tmax);
         return any_hit_object<double>(F.scene.obj64, id, o, d, tmax);
     }
 
@@ -2026,8 +2060,21 @@ struct ProbeRays {
             float tmax;
             uint32_t lbit;
             ao_direction<float>(F, (uint32_t)pt, smp, n0, ray.d, tmax, lbit);
-            if constexpr (FP64) fresh = walk_start_rel(F.grid, ray.o, ray.d, 0.0f, tmax, w);
-            else fresh = walk_start(F.grid, ray.o, ray.d, 0.0f, tmax, w);
+            if constexpr (FP64) {
+                const GridDev& g = F.grid;
+                const V3<float> q = ray.o - v3(g.bs[0] - g.lo[0], g.bs[1] - g.lo[1], g.bs[2] - g.lo[2]);
+                if (dot(q, q) > 4.0f * g.bs[3] * g.bs[3]) {
+                    const FarRay far = probe_far_ray(F, pts, nrm, (int64_t)pt, smp);
+                    if (far.on) {
+                        ray.o = far.o;
+                        ray.d = far.d;
+                        tmax = far.tmax;
+                    }
+                }
+                fresh = walk_start_rel(g, ray.o, ray.d, 0.0f, tmax, w);
+            } else {
+                fresh = walk_start(F.grid, ray.o, ray.d, 0.0f, tmax, w);
+            }
             ray.slot = (int64_t)pt;
             ray.tmax = tmax;
             ray.smp = smp;
