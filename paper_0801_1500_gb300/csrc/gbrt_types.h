@@ -188,6 +188,7 @@ struct BatchDev {
     unsigned long long* nunits;
     unsigned long long* ntiles;
     int64_t hit_cap;  // hit slots (records, vis, lmask) of the batch
+    int64_t tile_cap, mask_cap, unit_cap;  // lengths of tiles, masks and units
     int32_t nframes;
     int32_t tile_w, tile_h;
     int32_t refill;

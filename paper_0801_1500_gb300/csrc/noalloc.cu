@@ -125,6 +125,7 @@ extern "C" GBRT_API int gbrt_render_noalloc(const gbrt_scene* scene, const gbrt_
         bd.units = nullptr;
         bd.nunits = nullptr;
         bd.ntiles = nullptr;
+        bd.tile_cap = bd.mask_cap = bd.unit_cap = 0;
         bd.hit_cap = (int64_t)width * height;
         bd.nframes = 1;
         bd.tile_w = tw;

@@ -653,10 +653,11 @@ __global__ void __launch_bounds__(256) k_primary(const __grid_constant__ BatchDe
             unsigned long long at =
                 atomicAdd(b.ntiles, (unsigned long long)((F.mask_words + F.rec_words - 1) / F.rec_words));
             for (int w = 0; w < F.mask_words; w += F.rec_words, ++at) {
-                b.tiles[at].slot = F.hit_base + (int64_t)base;
-                b.tiles[at].n = __popc(hm);
-                b.tiles[at].frame = f;
-                b.tiles[at].word = w;
+                TileRec& rec = b.tiles[GBRT_INDEX(at, b.tile_cap)];
+                rec.slot = F.hit_base + (int64_t)base;
+                rec.n = __popc(hm);
+                rec.frame = f;
+                rec.word = w;
             }
         }
         if (!mine) continue;
@@ -993,9 +994,10 @@ __global__ void __launch_bounds__(128, 4) k_ao_near(const __grid_constant__ Batc
         if (lane == 0) tile = atomicAdd(b.queue + 2, 1ull);
         tile = __shfl_sync(FULL, tile, 0);
         if (tile >= total) break;
-        const int n = b.tiles[tile].n;
-        const FrameDev& F = b.frames[b.tiles[tile].frame];
-        const int64_t slot = GBRT_INDEX(b.tiles[tile].slot + (lane < n ? lane : 0), b.hit_cap);
+        TileRec& rec = b.tiles[GBRT_INDEX(tile, b.tile_cap)];
+        const int n = rec.n;
+        const FrameDev& F = b.frames[GBRT_INDEX(rec.frame, b.nframes)];
+        const int64_t slot = GBRT_INDEX(rec.slot + (lane < n ? lane : 0), b.hit_cap);
         V3<float> o, nrm, ol = v3(0.0f, 0.0f, 0.0f);
         uint32_t q, own;
         HitIO<float>::load(b.hits32, slot, o, nrm, q, own);
@@ -1072,8 +1074,9 @@ __global__ void __launch_bounds__(128, 4) k_ao_near(const __grid_constant__ Batc
                     if (r0 + lane < rows) {
                         const int y = c0[1] + (r0 + lane) % ny, z = c0[2] + (r0 + lane) / ny;
                         const int64_t row = ((int64_t)z * F.grid.bn[1] + y) * F.grid.bn[0];
-                        k = __ldg(F.grid.bstart + row + c0[0]);
-                        cnt = __ldg(F.grid.bstart + row + c1[0] + 1) - k;
+                        [[maybe_unused]] const int64_t starts = (int64_t)F.grid.bn[0] * F.grid.bn[1] * F.grid.bn[2] + 1;
+                        k = __ldg(F.grid.bstart + GBRT_INDEX(row + c0[0], starts));
+                        cnt = __ldg(F.grid.bstart + GBRT_INDEX(row + c1[0] + 1, starts)) - k;
                     }
                     uint32_t incl = cnt;
 #pragma unroll
@@ -1123,8 +1126,8 @@ __global__ void __launch_bounds__(128, 4) k_ao_near(const __grid_constant__ Batc
             }
             __syncwarp();
         }
-        if (lane == 0) b.tiles[tile].rho = rho;
-        const int w0 = b.tiles[tile].word, w1 = min(w0 + F.rec_words, F.mask_words);
+        if (lane == 0) rec.rho = rho;
+        const int w0 = rec.word, w1 = min(w0 + F.rec_words, F.mask_words);
         for (int w = w0; w < w1; ++w) {
             const int j0 = 16 * w, cnt = F.jobs_per_hit - j0 < 16 ? F.jobs_per_hit - j0 : 16;
             uint32_t todo, start, esc = 0u;
@@ -1150,14 +1153,20 @@ __global__ void __launch_bounds__(128, 4) k_ao_near(const __grid_constant__ Batc
             const uint32_t vis = __popc(esc & ((1u << sp) - 1u));
             if (vis) atomicAdd(b.vis + slot, vis);
             if (esc >> sp) atomicOr(b.lmask + slot, (esc >> sp) << (j0 + sp - F.spp));
-            if (lane < n) b.masks[F.mask_base + (slot - F.hit_base) * F.mask_words + w] = todo | start << 16;
+            if (lane < n) {
+                const int64_t mask = F.mask_base + (slot - F.hit_base) * F.mask_words + w;
+                b.masks[GBRT_INDEX(mask, b.mask_cap)] = todo | start << 16;
+            }
             const uint32_t any = __reduce_or_sync(FULL, todo);
             const uint32_t groups = ((any & 0xFu) != 0u) | ((any & 0xF0u) != 0u) << 1 | ((any & 0xF00u) != 0u) << 2 |
                                     ((any & 0xF000u) != 0u) << 3;
             if (groups && lane == 0) {
                 unsigned long long at = atomicAdd(b.nunits, (unsigned long long)__popc(groups));
                 for (int g = 0; g < 4; ++g)
-                    if ((groups >> g) & 1u) b.units[at++] = tile << 8 | (unsigned)(4 * w + g);
+                    if ((groups >> g) & 1u) {
+                        b.units[GBRT_INDEX(at, b.unit_cap)] = tile << 8 | (unsigned)(4 * w + g);
+                        ++at;
+                    }
             }
         }
         __syncwarp();
@@ -1259,13 +1268,15 @@ __device__ __forceinline__ void unit_take(const BatchDev& b, AoUnit& U, int lane
                 exhausted = true;
                 break;
             }
-            const unsigned long long unit = b.units[at];
+            const unsigned long long unit = b.units[GBRT_INDEX(at, b.unit_cap)];
             const int g = (int)(unit & 0xFFu), sh = 4 * (g & 3);
-            const TileRec T = b.tiles[unit >> 8];
-            const FrameDev& N = b.frames[T.frame];
+            const TileRec T = b.tiles[GBRT_INDEX(unit >> 8, b.tile_cap)];
+            const FrameDev& N = b.frames[GBRT_INDEX(T.frame, b.nframes)];
             uint32_t m = 0u;
-            if (lane < T.n)
-                m = b.masks[N.mask_base + (T.slot - N.hit_base + lane) * N.mask_words + (g >> 2)] >> sh;
+            if (lane < T.n) {
+                const int64_t mask = N.mask_base + (T.slot - N.hit_base + lane) * N.mask_words + (g >> 2);
+                m = b.masks[GBRT_INDEX(mask, b.mask_cap)] >> sh;
+            }
             __syncwarp();
 #pragma unroll
             for (int s = 0; s < 4; ++s) {
@@ -2527,6 +2538,9 @@ int render_frames(Ctx* ctx, FrameDev* frames, int n, bool use_graph) {
     bd.units = near ? (unsigned long long*)((char*)ctx->d_near + units_at) : nullptr;
     bd.masks = near ? (unsigned*)((char*)ctx->d_near + masks_at) : nullptr;
     bd.hit_cap = (int64_t)px;
+    bd.tile_cap = near ? recs : 0;
+    bd.mask_cap = near ? mask_words : 0;
+    bd.unit_cap = near ? 4 * words : 0;
     bd.nframes = n;
     bd.tile_w = tw;
     bd.tile_h = th;
