@@ -1,7 +1,8 @@
 // Device math of the ray tracer: vectors, ray-sphere and ray-cylinder roots,
 // the Amanatides-Woo grid walk, Philox4x32-10, cosine-weighted AO directions,
 // hit refinement and Phong + skylight shading. Templated on the arithmetic
-// type R: float for the FP32 path, double for the plain FP64 path.
+// type R where both precisions share it; walks are FP32 (the FP64 path's start
+// from walk_start_rel and its decisions carry error bounds, see render.cu).
 #pragma once
 
 #include <stdint.h>
@@ -70,12 +71,6 @@ __device__ __forceinline__ R dot(V3<R> a, V3<R> b) { return a.x * b.x + a.y * b.
 // a + s b
 template <class R>
 __device__ __forceinline__ V3<R> madd(V3<R> a, R s, V3<R> b) { return v3(a.x + s * b.x, a.y + s * b.y, a.z + s * b.z); }
-
-template <class R>
-__device__ __forceinline__ V3<R> normalized(V3<R> a) {
-    R l = Num<R>::sqrt_(dot(a, a));
-    return l > R(0) ? v3(a.x / l, a.y / l, a.z / l) : a;
-}
 
 __device__ __forceinline__ V3<float> to_f(V3<double> a) { return v3((float)a.x, (float)a.y, (float)a.z); }
 __device__ __forceinline__ V3<double> to_d(V3<float> a) { return v3((double)a.x, (double)a.y, (double)a.z); }
@@ -178,22 +173,17 @@ __device__ __forceinline__ bool hit_object(const SceneDev& s, uint32_t id, V3<R>
 }
 
 // Whether the same primitive has a root in (0, tmax], without the root itself
-// (shadow and AO rays). The FP64 path multiplies the root conditions through
-// by A = |d_p|^2 > 0: the roots are t = (-B -/+ sqrt(D)) / A with B = w_p.d_p
-// and D = B^2 - A (|w_p|^2 - r^2) (= A times hit_prim's disc), so A t and
-// A s = A (w.a) + (A t)(d.a) are tested against (0, A tmax] and [0, A L],
-// which leaves one square root and no division (FP64 division and square
-// root are instruction sequences on the FP64 pipe). The FP32 path keeps
-// hit_prim, whose reciprocal and square root are single instructions.
-template <class R>
-__device__ __forceinline__ bool any_hit_prim(V3<R> o, V3<R> d, V3<R> p0, V3<R> a, R L, R r, R tmax) {
-    R t;
-    return hit_prim(o, d, p0, a, L, r, R(0), tmax, t);
-}
-
-template <>
-__device__ __forceinline__ bool any_hit_prim<double>(V3<double> o, V3<double> d, V3<double> p0, V3<double> a,
-                                                     double L, double r, double tmax) {
+// (AO and shadow rays that FP64 decides). The root conditions are multiplied
+// through by A = |d_p|^2 > 0: the roots are t = (-B -/+ sqrt(D)) / A with
+// B = w_p.d_p and D = B^2 - A (|w_p|^2 - r^2) (= A times hit_prim's disc), so
+// A t and A s = A (w.a) + (A t)(d.a) are tested against (0, A tmax] and
+// [0, A L], which leaves one square root and no division (FP64 division and
+// square root are instruction sequences on the FP64 pipe).
+__device__ __forceinline__ bool any_hit_object64(const double2* obj, uint32_t id, V3<double> o, V3<double> d,
+                                                 double tmax) {
+    V3<double> p0, a;
+    double L, r;
+    Obj<double>::load(obj, id, p0, a, L, r);
     const V3<double> w = o - p0;
     const double wa = dot(w, a), da = dot(d, a);
     const V3<double> wp = madd(w, -wa, a), dp = madd(d, -da, a);
@@ -207,14 +197,6 @@ __device__ __forceinline__ bool any_hit_prim<double>(V3<double> o, V3<double> d,
     const bool h0 = n0 > 0.0 && n0 <= tA && s0 >= 0.0 && s0 <= LA;
     const bool h1 = n1 > 0.0 && n1 <= tA && s1 >= 0.0 && s1 <= LA;
     return ok && (h0 || h1);
-}
-
-template <class R>
-__device__ __forceinline__ bool any_hit_object(ObjPtr<R> obj, uint32_t id, V3<R> o, V3<R> d, R tmax) {
-    V3<R> p0, a;
-    R L, r;
-    Obj<R>::load(obj, id, p0, a, L, r);
-    return any_hit_prim<R>(o, d, p0, a, L, r, tmax);
 }
 
 // ---------------------------------------------------------------- grid walk

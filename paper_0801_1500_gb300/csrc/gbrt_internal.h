@@ -237,9 +237,9 @@ FrameDev make_frame(const Ctx* ctx, const gbrt_scene* scene, const gbrt_grid* gr
 // caller; tiling and hit-buffer fields are set here).
 int render_frames(Ctx* ctx, FrameDev* frames, int n, bool use_graph);
 // render.cu: for a batch whose descriptors and buffers the caller laid out:
-// opt the AO kernels into their shared memory (once per device), then launch
-// the four wavefront kernels with grids sized for the current device.
-int configure_render_kernels();
+// set the AO kernels' shared-memory preference (once per device), then launch
+// the wavefront kernels with grids sized for the current device.
+void configure_render_kernels();
 int enqueue_prepared(BatchDev bd, int precision, long long tiles, cudaStream_t stream, int block, int num_sms,
                      bool patch);
 

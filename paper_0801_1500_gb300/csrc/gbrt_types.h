@@ -49,7 +49,7 @@ struct SceneDev {
 // scatter pass left them (no result depends on the order).
 struct GridDev {
     float lo[3], hi[3], h[3], inv_h[3];
-    double lo64[3], hi64[3], h64[3], inv_h64[3];
+    double lo64[3];
     // bounding sphere of all objects (centre xyz, radius): walks are clipped to
     // it, so rays skip the empty corners of the grid box
     float bs[4];

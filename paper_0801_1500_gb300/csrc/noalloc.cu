@@ -47,8 +47,7 @@ int setup_device(int dev, unsigned char** base, int* sms) {
         int n = 0;
         if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1)
             return GBRT_EDEVICE;
-        int rc = configure_render_kernels();
-        if (rc != GBRT_OK) return rc;
+        configure_render_kernels();
         g_num_sms[dev] = n;
         g_scratch_addr[dev] = (unsigned char*)p;
     }

@@ -323,7 +323,7 @@ __device__ __forceinline__ void refine_fp32(const FrameDev& f, int i, int j, flo
 // times over: |m| is wrong by at most ~4e-7 (|b| + r) -- w is one rounding of
 // exact floats, b's error only moves m along the ray -- and so is the
 // reference test's own |m|. So x > margin is a miss and, for a sphere,
-// x < -margin a hit that the reference test (hit_prim, or any_hit_prim in
+// x < -margin a hit that the reference test (hit_prim, or any_hit_object64 in
 // FP64) decides the same way; what lies between is left to that test. A miss,
 // nine candidates in ten, costs ~20 instructions instead of ~45, and in the
 // FP64 path no FP64 instruction.
@@ -1768,7 +1768,7 @@ __device__ __forceinline__ void lane_walk(Src& src, LaneScene& A, int refill, ui
 }
 
 // The reference test of one (ray, object) pair of an FP64 frame, from the
-// hit's FP64 record: any_hit_prim on the ray that the sample defines.
+// hit's FP64 record: any_hit_object64 on the ray that the sample defines.
 __device__ __forceinline__ bool ao_exact64(const BatchDev& b, int f, int64_t vslot, uint32_t smp, uint32_t id) {
     const FrameDev& F = b.frames[f];
     V3<double> o, n, d;
@@ -1776,7 +1776,7 @@ __device__ __forceinline__ bool ao_exact64(const BatchDev& b, int f, int64_t vsl
     double tmax;
     HitIO<double>::load(b.hits, vslot, o, n, q, own);
     ao_direction<double>(F, q, smp, n, d, tmax, lbit);
-    return any_hit_object<double>(F.scene.obj64, id, o, d, tmax);
+    return any_hit_object64(F.scene.obj64, id, o, d, tmax);
 }
 
 // The rays of a batch's FP64 frames: the warp's pool claims ao_claim jobs at a
@@ -2041,7 +2041,7 @@ struct ProbeRays {
         V3<double> o, d;
         double tmax;
         probe_ray64(F, pts, nrm, ray.slot, ray.smp, o, d, tmax);
-        return any_hit_object<double>(F.scene.obj64, id, o, d, tmax);
+        return any_hit_object64(F.scene.obj64, id, o, d, tmax);
     }
 
     __device__ __forceinline__ int refill(LaneScene&, int lane, unsigned act, bool free, LaneRay& ray, Walk& w,
@@ -2187,6 +2187,7 @@ static size_t ao_smem(int block) {
 }
 constexpr int NEAR_BLOCK = 128;
 constexpr size_t NEAR_SMEM = NEAR_BLOCK / 32 * sizeof(NearWarp);
+static_assert(NEAR_SMEM <= 48 * 1024, "above this a kernel has to ask for its shared memory");
 
 // Shared-memory share of the SM asked for an AO walk whose CTAs of 256 threads
 // use `smem` bytes: just enough for four of them (and the driver's per-CTA
@@ -2208,7 +2209,7 @@ static cudaError_t prefer_small_carveout(K kernel, size_t smem) {
 
 // A refused preference leaves the driver's choice (and its error is cleared
 // here, so it is not taken for a later launch's).
-static cudaError_t configure_ao() {
+static void configure_ao() {
     if (prefer_small_carveout(k_ao_walk<true, false>, ao_smem<true, false>(256)) != cudaSuccess ||
         prefer_small_carveout(k_ao_walk<false, false>, ao_smem<false, false>(256)) != cudaSuccess ||
         prefer_small_carveout(k_ao_walk<true, true>, ao_smem<true, true>(256)) != cudaSuccess ||
@@ -2216,11 +2217,6 @@ static cudaError_t configure_ao() {
         prefer_small_carveout(k_ao_walk64<false>, 0) != cudaSuccess ||
         prefer_small_carveout(k_ao_walk64<true>, 8 * sizeof(AoUnit)) != cudaSuccess)
         (void)cudaGetLastError();
-    // the near pass's candidate lists exceed the 48 KB default
-    cudaError_t e = cudaFuncSetAttribute(k_ao_near<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)NEAR_SMEM);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_ao_near<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)NEAR_SMEM);
-    return e;
 }
 
 // uni: one scene and grid for the whole batch; near > 0: with a near pass of
@@ -2262,12 +2258,13 @@ static void launch_after_primary(const BatchDev& bd, bool uni, int near, int ao_
     if (resolve) launch_dependent(k_resolve<R>, dim3(resolve_grid, std::min(bd.nframes, 65535)), 256, 0, stream, bd);
 }
 
-static int grids_for(Ctx* ctx, int precision, bool uni, bool near, Grids& g) {
+static Grids grids_for(Ctx* ctx, int precision, bool uni, bool near) {
     const int block = ctx->tuning.block;
     if (!ctx->smem_configured) {
-        if (configure_ao() != cudaSuccess) return GBRT_EDEVICE;
+        configure_ao();
         ctx->smem_configured = true;
     }
+    Grids g;
     g.near = !near ? 0
              : precision == GBRT_FP32 ? persistent_grid(ctx, k_ao_near<false>, NEAR_BLOCK, NEAR_SMEM)
                                       : persistent_grid(ctx, k_ao_near<true>, NEAR_BLOCK, NEAR_SMEM);
@@ -2285,7 +2282,7 @@ static int grids_for(Ctx* ctx, int precision, bool uni, bool near, Grids& g) {
     }
     g.shade = ctx->num_sms * 8;
     g.resolve = ctx->num_sms * 4;
-    return GBRT_OK;
+    return g;
 }
 
 // Every frame of the batch reads the same scene and grid (device-side rebuilt
@@ -2548,8 +2545,7 @@ int render_frames(Ctx* ctx, FrameDev* frames, int n, bool use_graph) {
     ctx->counters_bytes_used = counters_bytes;
 
     if (uni) extra |= EXTRA_UNI;
-    Grids gr;
-    if ((rc = grids_for(ctx, precision, uni, near, gr)) != GBRT_OK) return rc;
+    const Grids gr = grids_for(ctx, precision, uni, near);
     bd.ao_warps = gr.ao * (ctx->tuning.block / 32);
     bd.parts = near ? 1 : ray_parts(tiles, gr.primary * (ctx->tuning.block / 32));
     if (!use_graph) {
@@ -2592,7 +2588,7 @@ int render_frames(Ctx* ctx, FrameDev* frames, int n, bool use_graph) {
     return GBRT_OK;
 }
 
-int configure_render_kernels() { return err_of(configure_ao()); }
+void configure_render_kernels() { configure_ao(); }
 
 int enqueue_prepared(BatchDev bd, int precision, long long tiles, cudaStream_t stream, int block, int num_sms,
                      bool patch) {

@@ -773,12 +773,9 @@ __host__ __device__ inline void grid_geometry(const float slo[3], const float sh
     }
     for (int k = 0; k < 3; ++k) {
         const double nk = (double)d.n[k];
-        d.h64[k] = E[k] / nk;
-        d.inv_h64[k] = nk / E[k];
         d.lo64[k] = (double)d.lo[k];
-        d.hi64[k] = (double)d.hi[k];
-        d.h[k] = (float)d.h64[k];
-        d.inv_h[k] = (float)d.inv_h64[k];
+        d.h[k] = (float)(E[k] / nk);
+        d.inv_h[k] = (float)(nk / E[k]);
         a.p.lo[k] = d.lo[k];
         a.p.inv_h[k] = d.inv_h[k];
         a.p.h[k] = d.h[k];
