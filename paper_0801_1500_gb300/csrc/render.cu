@@ -913,15 +913,19 @@ __device__ __forceinline__ void near_jobs(const FrameDev& F, NearWarp& S, int la
     float d[NS][3], m[NS];
     uint32_t valid = 0u;
     constexpr int W = NS < 8 ? NS : 8;
-    // (unrolled by order: rolled, nvcc 13.0 loses the first eight directions)
-#pragma unroll
-    for (int h = 0; h < NS; h += W) {
+    static_assert(NS <= 2 * W, "two calls fill the directions");
+    // (two calls, not a loop: in a loop that it did not unroll, nvcc 13.0 lost the
+    // first eight directions)
+    auto fill = [&](auto at) {
+        constexpr int h = decltype(at)::value;
         valid |= near_dirs<F64>(F, S, lane, j0 + h, W, nrm, q) << h;
 #pragma unroll
         for (int s = 0; s < W; ++s)
 #pragma unroll
             for (int k = 0; k < 3; ++k) d[h + s][k] = S.dir[s][k][lane];
-    }
+    };
+    fill(std::integral_constant<int, 0>());
+    if constexpr (NS > W) fill(std::integral_constant<int, W>());
     // spheres, then tubes, through the same code (it has to stay in the
     // instruction cache): what a sphere's ball surely stops is hit, what comes
     // close to one or meets a tube's stays open
