@@ -319,22 +319,25 @@ __device__ __forceinline__ void refine_fp32(const FrameDev& f, int i, int j, flo
 // ball's centre (w = o - centre), m = w - b d the ray's offset there and
 // x = |m|^2 + max(b, 0)^2 - r^2, a ray that starts outside or inside the ball
 // meets it ahead exactly when x <= 0 (b > 0: the centre lies behind, and
-// |m|^2 + b^2 = |w|^2). FILTER_EPS r (|b| + r) bounds the rounding of x ten
-// times over: |m| is wrong by at most ~4e-7 (|b| + r) -- w is one rounding of
-// exact floats, b's error only moves m along the ray -- and so is the
-// reference test's own |m|. So x > margin is a miss and, for a sphere,
-// x < -margin a hit that the reference test (hit_prim, or any_hit_object64 in
-// FP64) decides the same way; what lies between is left to that test. A miss,
-// nine candidates in ten, costs ~20 instructions instead of ~45, and in the
-// FP64 path no FP64 instruction.
-constexpr float FILTER_EPS = 1e-5f;
+// |m|^2 + b^2 = |w|^2). filter_margin bounds the rounding of x ten times over:
+// |m| is wrong by at most ~4e-7 (|b| + r) -- w is one rounding of exact floats,
+// b's error only moves m along the ray -- and so is the reference test's own |m|;
+// the square of that counts for a ball that is tiny against its distance (1e-9
+// of it: without the square, 188 of 1,600 pixels were wrong). So x > margin is a
+// miss and, for a sphere, x < -margin a hit that the reference test (hit_prim, or
+// any_hit_object64 in FP64) decides the same way; what lies between is left to
+// that test. A miss, nine candidates in ten, costs ~20 instructions instead of
+// ~45, and in the FP64 path no FP64 instruction.
+// reach: |b| + r, and for coordinates relative to a grid what their rounding adds.
+__device__ __forceinline__ float filter_margin(float r, float reach) {
+    return reach * fmaf(2e-12f, reach, 1e-5f * r);
+}
 
 // What a filter says of one (ray, object) pair.
 enum : int { PAIR_MISS = 0, PAIR_HIT = 1, PAIR_OPEN = 2 };
 
 // A tube in FP32, with error bounds. The arithmetic is hit_prim's; em bounds
-// the error of the offset m (as FILTER_EPS does, four times over), et that of
-// a root's t. On PAIR_HIT t is the nearest root in (0, tmax] and et its error.
+// the error of the offset m (ten times over), et that of a root's t. On PAIR_HIT t is the nearest root in (0, tmax] and et its error.
 // tlim: a root up to tlim - et is surely within tmax.
 __device__ __forceinline__ int tube_root32(V3<float> o, V3<float> d, V3<float> p0, V3<float> a, float L, float r,
                                            float tlim, float tmax, float om, float& t, float& et) {
@@ -477,7 +480,7 @@ __device__ __forceinline__ void nearest_filtered64(const FrameDev& f, int i, int
             const float tc = dot(wv, df) * idd;
             const V3<float> m = madd(wv, tc, df);
             const float r = fabsf(s.w), bp = fminf(tc, 0.0f), x2 = fmaf(-r, r, dot(m, m));
-            const float mg = FILTER_EPS * r * (fabsf(tc) + r + om);
+            const float mg = filter_margin(r, fabsf(tc) + r + om);
             if (!(fmaf(bp, bp, x2) <= mg)) continue;
             float t, et;
             int what;
@@ -1750,7 +1753,7 @@ __device__ __forceinline__ void lane_walk(Src& src, LaneScene& A, int refill, ui
             const V3<float> m = madd(wv, bb, ray.d);
             const float r = fabsf(s.w), bp = fminf(bb, 0.0f), reach = fabsf(bb) + r;
             const float x = fmaf(-r, r, fmaf(bp, bp, dot(m, m)));
-            const float mg = FILTER_EPS * r * (Src::F64 ? reach + A.om : reach);
+            const float mg = filter_margin(r, Src::F64 ? reach + A.om : reach);
             if (x <= mg) {
                 if (s.w > 0.0f && x < -mg && reach <= sure_within(ray.tmax)) {
                     active = false;  // occluded
