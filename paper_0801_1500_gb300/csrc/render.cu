@@ -1020,10 +1020,13 @@ __global__ void __launch_bounds__(128, 4) k_ao_near(const __grid_constant__ Batc
         skip.kind = -1;
         skip.r = 0.0f;
         if (rho > 0.0f) {
-            // The hit's own ball, passed over where the origin is surely outside
-            // the object: a tube's ball may hold it, and with a small eps it is
-            // closer to a sphere than bad allows (1e-6 r keeps clear of the
-            // rounding of |w|^2 and of the walk's own test).
+            // The hit's own ball, passed over where the object surely lies behind
+            // the plane through the origin that the rays start from: a tube's
+            // ball may hold the origin, and with a small eps it is closer to a
+            // sphere than bad allows (1e-6 r keeps clear of the rounding here and
+            // in the walk's own test). Outside alone is not enough: an origin
+            // rounded by more than eps, far from the coordinates' zero, may lie
+            // aside of its normal, and a low ray from there meets the object.
             V3<float> p0, a;
             float L, r;
             own = GBRT_INDEX(own, F.scene.S + F.scene.C);
@@ -1033,7 +1036,7 @@ __global__ void __launch_bounds__(128, 4) k_ao_near(const __grid_constant__ Batc
             const V3<float> wp = madd(w, -dot(w, a), a);  // (a sphere's axis is 0)
             skip.c = v3(c.x, c.y, c.z);
             skip.r = fabsf(c.w);
-            if (c.w != 0.0f && dot(wp, wp) > (L > 0.0f ? 1.0002f : 1.000002f) * r * r) skip.kind = L > 0.0f ? 1 : 0;
+            if (c.w != 0.0f && dot(wp, nrm) > (L > 0.0f ? 1.0001f : 1.000001f) * r) skip.kind = L > 0.0f ? 1 : 0;
             // where the own ball keeps most of the hits from being looked at (an
             // eps of next to nothing, a view from inside) the pass is left out
             const bool kept = skip.kind < 0 && dot(v, v) - c.w * c.w < 1e-4f * c.w * c.w;
