@@ -438,19 +438,34 @@ __device__ __forceinline__ void nearest_consider(Nearest& h, uint32_t id, float 
 
 // A primary ray's walk dealt over `parts` adjacent lanes (SPLIT; else the lane
 // has the ray to itself): lane `sub` visits the cells sub, sub + parts, ... in
-// ray order, and the lanes share their best hit after each of these rounds.
+// ray order, and the lanes share their best hit after each of these rounds. The
+// walk ends with the cell that one lane alone would end with, and what the lanes
+// found in cells behind it is dropped: far from the coordinates' zero such a find
+// may come before the hit, and a ray's result would depend on how many share it.
 // The whole warp calls split_walk together (lanes with nothing to walk pass
-// on = false); next() steps to the next cell, visit() tests the cell's objects
-// and best() is the nearest hit so far.
-template <class Next, class Visit, class Best>
-__device__ __forceinline__ void split_walk(const Walk& w, bool on, int sub, int parts, Next next, Visit visit,
+// on = false); next() steps to the next cell, visit() tests the cell's objects,
+// best() is the nearest hit so far, and h holds what the lane found.
+template <class Hits, class Next, class Visit, class Best>
+__device__ __forceinline__ void split_walk(const Walk& w, bool on, int sub, int parts, Hits& h, Next next, Visit visit,
                                            Best best) {
+    const int group = (threadIdx.x & 31) - sub;
+    float m = Num<float>::inf();
     for (int q = 0; q < sub && on; ++q) on = next();
     while (__any_sync(0xffffffffu, on)) {
+        const Hits before = h;
         if (on) visit();
-        float m = best();
-        for (int x = 1; x < parts; x <<= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, x));
-        if (on && m < Num<float>::inf() && m <= walk_cell_exit(w)) on = false;
+        // m: the nearest of the cells up to the lane's own, in all rounds
+        m = fminf(__shfl_sync(0xffffffffu, m, group + parts - 1), best());
+        for (int x = 1; x < parts; x <<= 1) {
+            const float y = __shfl_up_sync(0xffffffffu, m, x);
+            if (sub >= x) m = fminf(m, y);
+        }
+        const bool last = on && m < Num<float>::inf() && m <= walk_cell_exit(w);
+        const unsigned lasts = (__ballot_sync(0xffffffffu, last) >> group) & ((1u << parts) - 1u);
+        if (lasts) {
+            if (sub >= __ffs(lasts)) h = before;
+            on = false;
+        }
         for (int q = 0; q < parts && on; ++q) on = next();
     }
 }
@@ -472,7 +487,7 @@ __device__ __forceinline__ void trace_nearest(const GridDev& g, const SceneDev& 
         }
     };
     if (SPLIT) {
-        split_walk(w, on, sub, parts, [&] { return walk_next(w, overflow); }, visit, [&] { return h.t1; });
+        split_walk(w, on, sub, parts, h, [&] { return walk_next(w, overflow); }, visit, [&] { return h.t1; });
         return;
     }
     if (!on) return;

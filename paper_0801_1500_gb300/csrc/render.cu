@@ -506,7 +506,7 @@ __device__ __forceinline__ void nearest_filtered64(const FrameDev& f, int i, int
         near64_finish(f, i, j, te0, h);
         return;
     }
-    split_walk(w, on, sub, parts, next, visit, [&] { return h.t + h.e; });
+    split_walk(w, on, sub, parts, h, next, visit, [&] { return h.t + h.e; });
     near64_finish(f, i, j, te0, h);
     // the lanes' hits, merged
     for (int x = 1; x < parts; x <<= 1) {
