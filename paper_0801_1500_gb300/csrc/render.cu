@@ -399,7 +399,7 @@ __device__ __noinline__ double exact_root64(const FrameDev& f, int i, int j, uin
 // before the cell's exit. The object is the one an FP64 walk finds; its FP64 root
 // is formed by the caller, once per hit pixel instead of once per candidate
 // (965 x 1137 frame, this kernel: 2.40 -> 0.205 ms; 256 x 256: 0.39 ->
-// 0.048 ms. The FP64 pipe was the bound; now the walk's load latency and the
+// 0.049 ms. The FP64 pipe was the bound; now the walk's load latency and the
 // winners' ~140 FP64 instructions are).
 struct Near64 {
     uint32_t id;    // GBRT_MISS: none
@@ -978,16 +978,16 @@ __device__ __forceinline__ void near_jobs(const FrameDev& F, NearWarp& S, int la
 // their atoms, so that is one ray in a hundred. The decisions are those of the
 // walk's own test (delta is ten times the rounding of both).
 // Measured (965 x 1137, 16 samples, 9.0 M AO rays): 140 balls a tile; 37% of the
-// rays hit, 13% left the bounds, 1% open; some 240 M warp instructions (gather 39
-// M, directions 48 M, scan 150 M) in 0.31 ms, and the walk 1.00 -> 0.45 ms. 3860 x
-// 4548: frame 15.8 -> 10.3 ms. Instruction issue (16 warps an SM, for the
+// rays hit, 13% left the bounds, 1% open; 258 M warp instructions (some 40 M of the
+// gather, 50 M of the directions, 160 M of the scan) in 0.31 ms, and the walk
+// 1.00 -> 0.45 ms. 3860 x 4548: frame 15.8 -> 10.2 ms. Instruction issue (16 warps an SM, for the
 // directions in registers) and the instruction cache bound it. Tried: the scan as f16-pair
 // m16n8k16 mma.sync (13.7 cycles a 128 pairs, no faster than the FMAs), packed
 // f32x2 FMAs (20% fewer instructions, 10% slower), a row of cells per lane in
 // the gather (55 dependent rounds of loads instead of 16: 0.44 ms).
 // F64: the same for FP64 frames, whose decisions delta covers as well (the
 // directions are the FP32 ones the walk filters with, the origins float pairs):
-// 0.32 ms, and the walk 1.53 -> 0.79 (965 x 1137, frame 1.87 -> 1.46 ms).
+// 0.33 ms, and the walk 1.53 -> 0.80 (965 x 1137, frame 1.87 -> 1.46 ms).
 template <bool F64>
 __global__ void __launch_bounds__(128, 4) k_ao_near(const __grid_constant__ BatchDev b) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1879,11 +1879,11 @@ struct FrameRays {
 // AO walk of FP64 frames, persistent. With every test and step in FP64 (1/64
 // of the FP32 rate) the FP64 pipe was 87% busy and the walk took 15.5 of a
 // 965 x 1137 frame's 17.9 ms; the filter leaves FP64 to one pair in some ten
-// thousand (walk 1.53 ms; 256 x 256 frame at 8 samples 0.57 -> 0.09 ms). One
+// thousand (walk 1.53 ms; 256 x 256 frame at 8 samples 0.57 -> 0.11 ms). One
 // ray a lane rather than the FP32 frames' pair expansion: with a filter this
 // cheap the expansion costs more than the idle lanes (walk 3.8 ms with pairs
 // queued in shared memory). Bound now by instruction issue and load
-// latency. NEAR: after a near pass, over the rays it left (0.79 ms).
+// latency. NEAR: after a near pass, over the rays it left (0.80 ms).
 template <bool NEAR>
 __global__ void __launch_bounds__(256, 3) k_ao_walk64(const __grid_constant__ BatchDev b) {
     __shared__ AoUnit units[NEAR ? 8 : 1];
@@ -2321,11 +2321,10 @@ static bool near_pass_suits(const FrameDev& f) {
 // kernel has warps is bound by the latency of its slowest warp, a chain of
 // dependent loads and tests (cell, item, object): 128 x 96 pixels, 36 us of
 // which the mean warp is busy for 7. Then 2, 4 or 8 lanes walk a ray between
-// them: 29 us with 8 at 128 x 96 (a frame of 520 atoms 66.7 -> 59.4, of 128,200
-// atoms 127 -> 87), a 256 x 256 frame 75.2 -> 72.8 and 145 -> 134 with 2. With
-// more lanes than keep every tile resident at once the cells visited past the
-// hit cost more than they hide (256 x 256: 4 lanes 75.7, 8 lanes 88.6; FP64 195
-// us with one lane, 217 with 4).
+// them: 25 us with 8 at 128 x 96 (a frame of 520 atoms 66.7 -> 54), a 256 x 256
+// frame 79.8 -> 71.9 with 2, FP64 184 -> 179. With more lanes than keep every
+// tile resident at once the cells visited past the hit cost more than they hide
+// in FP32 (256 x 256: 4 lanes 74, 8 lanes 84; FP64 171 and 192).
 static int ray_parts(long long tiles, int warps) {
     int parts = 1;
     while (parts < 8 && 2 * parts * tiles <= warps) parts *= 2;
