@@ -120,3 +120,37 @@ def test_small_offsets(G, fp64):
             for a, b in zip(got, ref):
                 assert torch.equal(a, b), (eps, int((a != b).sum()))
     assert all(times[e] < 2.0 * times[1e-3] for e in times if e >= 4e-6), times
+
+
+@pytest.mark.parametrize("fp64", [False, True])
+@pytest.mark.parametrize("far,eps", [(300.0, 3e-6), (9000.0, 1e-5), (20000.0, 1e-4)])
+def test_origins_on_the_other_side(G, far, eps, fp64):
+    """Far from the coordinates' zero an FP32 origin is rounded by more than eps:
+    one on the inner wall of an open tube may come to lie outside, and its rays,
+    which go inward, do meet that tube."""
+    import torch
+    rng = np.random.default_rng(4)
+    off = np.array([far, -0.7 * far, 0.4 * far])
+    m = rng.uniform(-6.0, 6.0, (150, 3)) + off
+    d = rng.standard_normal((150, 3))
+    d *= 0.6 / np.linalg.norm(d, axis=1, keepdims=True)
+    sc = S.make_scene(np.concatenate([m[:40], np.full((40, 1), 0.2)], 1),
+                      np.concatenate([m - d, m + d, rng.uniform(0.2, 0.5, (150, 1))], 1))
+    cam = S.Camera(eye=tuple(off + [0.0, 0.0, 20.0]), dir=(0.0, 0.0, -1.0), up=(0.0, 1.0, 0.0), right=(1.0, 0.0, 0.0),
+                   half_w=6.5, half_h=6.5)
+    lights = S.default_lights()
+    p = S.Params(ao_samples=16, seed=9, eps=eps, shadows=True,
+                 precision=S.PRECISION_FP64 if fp64 else S.PRECISION_FP32)
+    with G.Renderer(0) as R:
+        scene, grid = R.upload(sc, lam=8.0)
+        got, ref = [[torch.full((H, W, 3), -1.0, device="cuda", dtype=torch.float64 if fp64 else torch.float32)] +
+                    [torch.full((H, W), -7, dtype=torch.int32, device="cuda") for _ in range(2)] for _ in range(2)]
+        n0 = G.gbrt_launch_count(R.ctx)
+        G.gbrt_render(R.ctx, scene, grid, cam, W, H, p.ao_samples, lights, p, *got)
+        assert G.gbrt_launch_count(R.ctx) - n0 == 4
+        for k in range(BANDS):
+            rows = (k * H // BANDS, (k + 1) * H // BANDS)
+            G.gbrt_render_batch(R.ctx, [G.make_item(scene, grid, cam, W, H, p.ao_samples, lights, p, *ref, rows=rows)])
+        G.gbrt_sync(R.ctx)
+        for a, b in zip(got, ref):
+            assert torch.equal(a, b), int((a != b).sum())
