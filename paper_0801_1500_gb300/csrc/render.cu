@@ -1024,9 +1024,10 @@ __global__ void __launch_bounds__(128, 4) k_ao_near(const __grid_constant__ Batc
             // the plane through the origin that the rays start from: a tube's
             // ball may hold the origin, and with a small eps it is closer to a
             // sphere than bad allows (1e-6 r keeps clear of the rounding here and
-            // in the walk's own test). Outside alone is not enough: an origin
-            // rounded by more than eps, far from the coordinates' zero, may lie
-            // aside of its normal, and a low ray from there meets the object.
+            // in the walk's own test). Outside alone is not enough: far from the
+            // coordinates' zero an origin is rounded by more than eps, one on the
+            // inner wall of an open tube to the outside or one on a thin object
+            // aside of its normal, and its rays do meet the object.
             V3<float> p0, a;
             float L, r;
             own = GBRT_INDEX(own, F.scene.S + F.scene.C);
